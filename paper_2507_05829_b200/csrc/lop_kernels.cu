@@ -1,9 +1,5 @@
-// CUDA-core kernels: general convolution (any kernel/stride/padding/dilation/channel count),
-// max pooling, patch gather of a thin chain input (the band "split" step), zero-padding of weight rows.
-//
-// The convolution here is the fp32 path and the fall-back for shapes the tensor-core kernel
-// does not take; it is also the library's second on-GPU opinion (LOP_FLAG_FORCE_SIMT).
-// Operators: Sec. IV-A of the paper (block-wise and element-wise local operators).
+// CUDA-core kernels: max pooling, patch gather of a thin chain input (the band "split" step), zero-padding of weight
+// rows.  Operators: Sec. IV-A of the paper (block-wise and element-wise local operators).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -36,149 +32,6 @@ __device__ __forceinline__ void split_index(long long idx, long long total, int 
         ow = (int)(q % Wo); q /= Wo;
         r = (int)(q % rows);
         n = (int)(q / rows);
-    }
-}
-
-__device__ __forceinline__ float activate(float t, int act)
-{
-    if (act == LOP_ACT_RELU) return fmaxf(t, 0.0f);
-    if (act == LOP_ACT_SILU) return t / (1.0f + expf(-t));
-    if (act == LOP_ACT_GELU) return 0.5f * t * (1.0f + erff(t * 0.70710678f));
-    return t;
-}
-
-// ---------------------------------------------------------------------------------------------
-// Implicit-GEMM convolution on CUDA cores.  M = N*rows*Wo output pixels, N = Cout, K = kh*kw*Cin.
-// 64x64 tile per 256-thread block, 16-wide K slabs staged through shared memory, 4x4 outputs per
-// thread.  K is walked in one fixed order, so a pixel's value does not depend on the band it is in.
-// ---------------------------------------------------------------------------------------------
-constexpr int SM_BK = 16;
-
-// TM: outputs per thread along each tile axis; the tile is (16*TM) pixels x (16*TM) output channels.  TM = 4 for
-// layers with enough tiles to fill the machine, TM = 2 (four times as many CTAs) for small ones.  The next K slab's
-// operands are loaded into registers while the current slab is multiplied, so a slab costs one barrier pair, not a
-// global-memory round trip.  K is walked in ascending order whatever the tile, so a pixel's bits do not depend on it.
-template <typename T, int TM>
-__global__ void __launch_bounds__(256) conv_simt_kernel(ConvArgs p)
-{
-    constexpr int BM = 16 * TM, BN = 16 * TM;
-    __shared__ float As[SM_BK][BM + 4];
-    __shared__ float Bs[SM_BK][BN + 4];
-
-    const T *__restrict__ x = static_cast<const T *>(p.x);
-    const T *__restrict__ w = static_cast<const T *>(p.w);
-    const int rows = p.oh_hi - p.oh_lo;
-    const long long M = (long long)p.N * rows * p.Wo;
-    const int K = p.kh * p.kw * p.Cin;
-    const long long m0 = (long long)blockIdx.x * BM;
-    const int n0 = blockIdx.y * BN;
-    const int t = threadIdx.x;
-    const long long x_elems = (long long)p.N * p.Hin * p.Win * p.Cin, y_elems = (long long)p.N * p.Ho * p.Wo * p.Cout;
-    const int kk = t & 15;              // K index inside the slab this thread stages
-    const int lr = t >> 4;              // 0..15: first of the TM tile rows (stride 16) this thread stages
-
-    // the TM pixels / TM output channels whose operands this thread stages
-    long long xbase[TM];
-    int ih0[TM], iw0[TM];
-    bool mvalid[TM];
-#pragma unroll
-    for (int e = 0; e < TM; ++e) {
-        const long long m = m0 + lr + e * 16;
-        mvalid[e] = m < M;
-        const long long mm = mvalid[e] ? m : 0;
-        const int ow = (int)(mm % p.Wo);
-        const long long q = mm / p.Wo;
-        const int oh = p.oh_lo + (int)(q % rows);
-        const int n = (int)(q / rows);
-        ih0[e] = oh * p.sh - p.ph;
-        iw0[e] = ow * p.sw - p.pw;
-        xbase[e] = (long long)n * p.Hin * p.Win * p.Cin;
-    }
-
-    const int tx = t & 15, ty = t >> 4;
-    float acc[TM][TM];
-#pragma unroll
-    for (int i = 0; i < TM; ++i)
-#pragma unroll
-        for (int j = 0; j < TM; ++j) acc[i][j] = 0.0f;
-
-    // this thread's operand values of the K slab starting at k0
-    float av[TM], wv[TM];
-    auto load_slab = [&](int k0) {
-        const int k = k0 + kk;
-        const bool kvalid = k < K;
-        int ci = 0, a = 0, b = 0;
-        if (kvalid) {
-            ci = k % p.Cin;
-            const int tap = k / p.Cin;
-            b = tap % p.kw;
-            a = tap / p.kw;
-        }
-#pragma unroll
-        for (int e = 0; e < TM; ++e) {
-            float v = 0.0f;
-            if (kvalid && mvalid[e]) {
-                const int ih = ih0[e] + a * p.dh, iw = iw0[e] + b * p.dw;
-                if (ih >= 0 && ih < p.Hin && iw >= 0 && iw < p.Win) {
-                    const long long xo = xbase[e] + ((long long)ih * p.Win + iw) * p.Cin + ci;
-                    if (dbg_in_bounds(p.dbg, xo, 1, x_elems)) v = to_f32(x[xo]);
-                }
-            }
-            av[e] = v;
-            float u = 0.0f;
-            const int co = n0 + lr + e * 16;
-            if (kvalid && co < p.Cout && dbg_in_bounds(p.dbg, (long long)co * K + k, 1, (long long)p.Cout * K)) u = to_f32(w[(long long)co * K + k]);
-            wv[e] = u;
-        }
-    };
-    load_slab(0);
-    for (int k0 = 0; k0 < K; k0 += SM_BK) {
-#pragma unroll
-        for (int e = 0; e < TM; ++e) {
-            As[kk][lr + e * 16] = av[e];
-            Bs[kk][lr + e * 16] = wv[e];
-        }
-        __syncthreads();
-        if (k0 + SM_BK < K) load_slab(k0 + SM_BK);          // in flight while this slab is multiplied
-#pragma unroll
-        for (int q = 0; q < SM_BK; ++q) {
-            float ar[TM], br[TM];
-#pragma unroll
-            for (int i = 0; i < TM; ++i) ar[i] = As[q][ty * TM + i];
-#pragma unroll
-            for (int j = 0; j < TM; ++j) br[j] = Bs[q][tx * TM + j];
-#pragma unroll
-            for (int i = 0; i < TM; ++i)
-#pragma unroll
-                for (int j = 0; j < TM; ++j) acc[i][j] = fmaf(ar[i], br[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
-
-    T *__restrict__ y = static_cast<T *>(p.y);
-    const T *__restrict__ res = static_cast<const T *>(p.res);
-#pragma unroll
-    for (int i = 0; i < TM; ++i) {
-        const long long m = m0 + ty * TM + i;
-        if (m >= M) continue;
-        const int ow = (int)(m % p.Wo);
-        const long long q = m / p.Wo;
-        const int oh = p.oh_lo + (int)(q % rows);
-        const int n = (int)(q / rows);
-        const long long o = (((long long)n * p.Ho + oh) * p.Wo + ow) * p.Cout;
-#pragma unroll
-        for (int j = 0; j < TM; ++j) {
-            const int co = n0 + tx * TM + j;
-            if (co >= p.Cout) continue;
-            // the element inside the tensor, the row inside the rows of this launch (tested as a one-row "tensor")
-            if (!dbg_in_bounds(p.dbg, o + co, 1, y_elems) || !dbg_in_bounds(p.dbg, oh - p.oh_lo, 1, rows)) continue;
-            float v = acc[i][j];
-            v = fmaf(p.scale ? p.scale[co] : 1.0f, v, p.shift ? p.shift[co] : 0.0f);
-            if (res && p.res_pos == LOP_RES_PRE_ACT) v += to_f32(res[o + co]);
-            v = activate(v, p.act);
-            if (res && p.res_pos == LOP_RES_POST_ACT) v += to_f32(res[o + co]);
-            from_f32(y[o + co], v);
-        }
     }
 }
 
@@ -324,24 +177,6 @@ inline int grid_for(long long work_items, int block, int max_blocks = 148 * 8)
 }
 
 }  // namespace
-
-cudaError_t launch_conv_simt(const ConvArgs &a, int dtype, cudaStream_t s)
-{
-    const int rows = a.oh_hi - a.oh_lo;
-    if (rows <= 0) return cudaSuccess;
-    const long long M = (long long)a.N * rows * a.Wo;
-    const long long big_tiles = ((M + 63) / 64) * ((a.Cout + 63) / 64);
-    if (big_tiles >= 2 * 148) {
-        dim3 grid((unsigned)((M + 63) / 64), (unsigned)((a.Cout + 63) / 64));
-        if (dtype == LOP_BF16) conv_simt_kernel<__nv_bfloat16, 4><<<grid, 256, 0, s>>>(a);
-        else conv_simt_kernel<float, 4><<<grid, 256, 0, s>>>(a);
-    } else {
-        dim3 grid((unsigned)((M + 31) / 32), (unsigned)((a.Cout + 31) / 32));
-        if (dtype == LOP_BF16) conv_simt_kernel<__nv_bfloat16, 2><<<grid, 256, 0, s>>>(a);
-        else conv_simt_kernel<float, 2><<<grid, 256, 0, s>>>(a);
-    }
-    return cudaGetLastError();
-}
 
 cudaError_t launch_maxpool(const PoolArgs &a, int dtype, cudaStream_t s)
 {

@@ -1,0 +1,49 @@
+"""Kernel variants and dispatch branches at the sizes where they can go wrong, against the CPU oracle.  Needs a B200."""
+import pytest
+import torch
+
+import lop_inputs as li
+from lop_inputs.workloads import conv
+from paper_2507_05829_b200.chain import DeviceChain
+from test_gpu_parity import check_workload, one_layer
+
+pytestmark = pytest.mark.gpu
+
+
+# ------------------------------------------------------------------------------------ CUDA-core convolution
+SIMT_CASES = [  # k, s, p, d, cin, cout, N, H, W
+    (3, 1, 1, 1, 16, 16, 1, 32, 32),       # small blocks, full
+    (3, 2, 1, 1, 12, 21, 2, 17, 11),       # small blocks: ragged pixels and channels, K with a short last quad row
+    (3, 1, 2, 2, 24, 40, 1, 70, 90),       # too many pixels for small blocks per SM, but Cin is no multiple of 16
+    (1, 1, 0, 1, 16, 9, 1, 200, 161),      # few output channels: small blocks whatever the size
+    (3, 1, 1, 1, 16, 64, 1, 150, 263),     # 128 x 64 tiles, ragged last tile
+    (3, 1, 1, 1, 32, 100, 1, 93, 101),     # 64-wide tiles, ragged channels
+    (1, 2, 0, 1, 48, 33, 2, 51, 77),       # odd channel count: scalar stores
+    (5, 1, 2, 1, 80, 64, 1, 12, 14),       # K = 2000: operands do not fit the small block
+    (7, 2, 3, 1, 3, 70, 1, 45, 52),        # thin input, K = 147 in three filter slices, ragged channels
+    (1, 1, 0, 1, 1, 5, 1, 3, 3),           # the smallest
+]
+
+
+@pytest.mark.parametrize("case", SIMT_CASES)
+def test_cuda_core_convolution_variants(case):
+    k, s, p, d, cin, cout, N, H, W = case
+    wl = one_layer(conv(cin, cout, k, s=s, p=p, d=d, act=li.ACT_SILU), N, H, W, dtype="f32")
+    check_workload(wl, modes=("whole", "banded", "pipelined_copy"))
+
+
+def test_cuda_core_convolution_takes_weights_of_any_alignment():
+    """Weights four bytes off a vector boundary: the scalar kernel, the same bits."""
+    wl = one_layer(conv(16, 24, 3, act=li.ACT_RELU), 1, 40, 33, dtype="f32")
+    dc = DeviceChain(wl)
+    x = dc.input_tensor()
+    want = dc.run_whole(x).clone()
+    l = wl.segments[0].layers[0]
+    buf = torch.zeros(l.weight.size + 1, device="cuda")
+    buf[1:] = torch.from_numpy(l.weight.reshape(-1)).cuda()
+    sc, sh = torch.from_numpy(l.scale).cuda(), torch.from_numpy(l.shift).cuda()
+    dc.plans[0].set_params(0, buf.data_ptr() + 4, sc.data_ptr(), sh.data_ptr())
+    got = dc.run_whole(x)
+    torch.cuda.synchronize()
+    assert torch.equal(got, want)
+
