@@ -205,7 +205,7 @@ int lop_plan_shard(const lop_plan_t *plan, int rank, int world, int *band_lo, in
  * lop_run_banded on one device. */
 int lop_run_shard(lop_plan_t *plan, int band_lo, int band_hi, const void *in_dev, void *out_dev,
                   void *workspace, void *stream);
-/* The same transfer step done by the persistent kernel's fetch warps instead of the copy engine (see lop_run_pipelined:
+/* The same transfer step done by the SMs (the persistent kernel's fetch warps) instead of the copy engine (see lop_run_pipelined:
  * the "fetched" transport), by itself: band >= 0 brings that band's new rows, band == -1 every band's, from
  * in_host_pinned -- which must be mapped into the device's address space and agree with staging_dev modulo 16 bytes,
  * else LOP_EUNSUPPORTED -- to staging_dev.  One launch, no operator runs.  For timing the transmission a pipelined run
@@ -217,9 +217,10 @@ int lop_fetch_band(lop_plan_t *plan, int band, const void *in_host_pinned, void 
  *     cudaHostRegister memory is): the persistent kernel itself reads each band's rows from host memory
  *     and stores them to staging_dev -- fetch stages that precede the band's first operator in the
  *     dependency graph, spread over the SMs -- so the whole request is ONE launch on the caller's stream
- *     with no copy, event or flag command at all;
- *   - copy engine (LOP_FLAG_COPY_ENGINE, unmapped host memory, or plans the persistent kernel does not
- *     take): one asynchronous copy per band on the plan's side stream, forked and joined by CUDA events;
+ *     with no copy, event or flag command at all (plans that run on per-layer kernels: one launch that
+ *     brings the rows, then one per layer);
+ *   - copy engine (LOP_FLAG_COPY_ENGINE, unmapped host memory, or per-layer plans that are timed or
+ *     checked): one asynchronous copy per band on the plan's side stream, forked and joined by CUDA events;
  *     a band's arrival is a 4-byte stream-ordered write behind its copy that the persistent kernel polls
  *     (per-layer launches wait on one event per band instead).
  * Both leave the input in staging_dev and give the same output bits.  Returns after enqueueing; the

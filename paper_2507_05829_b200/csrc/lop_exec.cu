@@ -272,6 +272,37 @@ int first_row(const lop_plan_t *pl, int block_lo, int band, int i)
     return std::min(std::max((int)r.out_lo, done), (int)r.out_hi);
 }
 
+// Operation batching (Sec. IV-C): with the whole input on the device, the bands' operations at a layer are one
+// contiguous run of rows (neighbouring bands' ranges touch or overlap), so each layer is ONE launch over the hull of
+// the bands' rows.  Every row is computed once, with the same bits as band by band.
+int run_batched_impl(lop_plan_t *pl, const void *in, void *out, void *ws, cudaStream_t s)
+{
+    const int L = (int)pl->layers.size();
+    int rc = LOP_OK;
+    for (int i = 0; i < L; ++i) {
+        int lo = 0, hi = 0;
+        bool any = false, contiguous = true;
+        for (int b = 0; b < pl->n_bands; ++b) {
+            const lop_range &r = pl->ranges[(size_t)b * L + i];
+            if (r.out_hi <= r.out_lo) continue;
+            if (any && r.out_lo > hi) contiguous = false;
+            lo = any ? std::min(lo, (int)r.out_lo) : (int)r.out_lo;
+            hi = any ? std::max(hi, (int)r.out_hi) : (int)r.out_hi;
+            any = true;
+        }
+        if (!any) continue;
+        if (contiguous) {
+            if ((rc = run_layer(pl, i, lo, hi, in, out, ws, s, -1)) != LOP_OK) return rc;
+        } else {
+            for (int b = 0; b < pl->n_bands; ++b) {
+                const lop_range &r = pl->ranges[(size_t)b * L + i];
+                if ((rc = run_layer(pl, i, first_row(pl, 0, b, i), r.out_hi, in, out, ws, s, -1)) != LOP_OK) return rc;
+            }
+        }
+    }
+    return LOP_OK;
+}
+
 // block_lo: the first band that runs on this device (0 unless the bands are sharded over devices).
 void band_requests(const lop_plan_t *pl, int seg, int band, bool wait_arrival, std::vector<StageReq> &reqs, int block_lo = 0)
 {
@@ -521,6 +552,25 @@ int copy_rows_impl(lop_plan_t *pl, int lo, int hi, const void *host, void *stagi
     return LOP_OK;
 }
 
+// The transfer step of plans without a persistent program: the rows band `band` needs and no earlier band has brought, or
+// (band == -1) the rows any band needs, by one launch.
+int fetch_rows_impl(lop_plan_t *pl, int band, const void *src, void *staging, cudaStream_t s)
+{
+    int lo = 0, hi = 0;
+    for (int b = band < 0 ? 0 : band; b < (band < 0 ? pl->n_bands : band + 1); ++b) {
+        const lop_range &need = pl->in_need[b];
+        if (need.out_hi <= need.new_lo) continue;
+        lo = hi > lo ? std::min(lo, (int)need.new_lo) : (int)need.new_lo;
+        hi = std::max(hi, (int)need.out_hi);
+    }
+    for (int b = 0; b < pl->n_bands; ++b) pl->exec->copy_issued[b] = 0;
+    pl->exec->copies_timed = false;
+    if (hi <= lo) return LOP_OK;
+    LOP_CUDA(launch_fetch_rows(src, staging, pl->N, pl->H, (long long)pl->W * pl->C * elem_size(pl->dtype), lo, hi, s));
+    pl->exec->launches++;
+    return LOP_OK;
+}
+
 // The single-launch band pipeline on stream s (which may be capturing): fork the side streams, launch the
 // persistent kernel, enqueue every band's copy and arrival write, join.
 // withheld: a band whose copy and arrival write are left out (lop_run_pipelined_withheld), or -1.
@@ -629,32 +679,7 @@ int lop_run_banded(lop_plan_t *pl, const void *in, void *out, void *ws, void *st
             if ((rc = run_band_impl(pl, b, in, out, ws, s)) != LOP_OK) return rc;
         return LOP_OK;
     }
-    // Operation batching (Sec. IV-C): with the whole input on the device, the bands' operations at a layer are one
-    // contiguous run of rows (neighbouring bands' ranges touch or overlap), so each layer is ONE launch over the hull of
-    // the bands' rows.  Every row is computed once, with the same bits as band by band.
-    const int L = (int)pl->layers.size();
-    for (int i = 0; i < L; ++i) {
-        int lo = 0, hi = 0;
-        bool any = false, contiguous = true;
-        for (int b = 0; b < pl->n_bands; ++b) {
-            const lop_range &r = pl->ranges[(size_t)b * L + i];
-            if (r.out_hi <= r.out_lo) continue;
-            if (any && r.out_lo > hi) contiguous = false;
-            lo = any ? std::min(lo, (int)r.out_lo) : (int)r.out_lo;
-            hi = any ? std::max(hi, (int)r.out_hi) : (int)r.out_hi;
-            any = true;
-        }
-        if (!any) continue;
-        if (contiguous) {
-            if ((rc = run_layer(pl, i, lo, hi, in, out, ws, s, -1)) != LOP_OK) return rc;
-        } else {
-            for (int b = 0; b < pl->n_bands; ++b) {
-                const lop_range &r = pl->ranges[(size_t)b * L + i];
-                if ((rc = run_layer(pl, i, first_row(pl, 0, b, i), r.out_hi, in, out, ws, s, -1)) != LOP_OK) return rc;
-            }
-        }
-    }
-    return LOP_OK;
+    return run_batched_impl(pl, in, out, ws, s);
 }
 
 int lop_run_layer(lop_plan_t *pl, int layer, int row_lo, int row_hi, const void *in, void *out, void *ws, void *stream)
@@ -741,12 +766,12 @@ int lop_fetch_band(lop_plan_t *pl, int band, const void *host, void *staging, vo
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     e->launches = e->copies = 0;
     e->last_stream = s;
-    if (!e->wavefront) { set_error("lop_fetch_band: this plan does not run on the persistent kernel; use lop_copy_band"); return LOP_EUNSUPPORTED; }
     const void *src = fetchable(pl, host);
     if (!src || (reinterpret_cast<uintptr_t>(src) & 15) != (reinterpret_cast<uintptr_t>(staging) & 15)) {
         set_error("lop_fetch_band: the host buffer is not mapped into the device's address space, or differs from the staging tensor modulo 16 bytes");
         return LOP_EUNSUPPORTED;
     }
+    if (!e->wavefront) return fetch_rows_impl(pl, band, src, staging, s);
     if ((rc = prepare_workspace(pl, ws, s)) != LOP_OK) return rc;
     Program *p = nullptr;
     if ((rc = get_program(pl, PROG_FETCH_ALONE, staging, staging, ws, &p, src, band)) != LOP_OK) return rc;
@@ -795,6 +820,16 @@ int lop_run_pipelined(lop_plan_t *pl, const void *host, void *staging, void *out
         if (timed) LOP_CUDA(cudaEventRecord(e->ev_end, s));
         e->timing_valid = timed;
         return LOP_OK;
+    }
+    if (!(pl->flags & (LOP_FLAG_TIME_LAYERS | LOP_FLAG_DEBUG_BOUNDS))) {
+        // Per-layer kernels, input in host memory the device can address: one launch brings the rows every band needs,
+        // and each layer is one launch behind it.  Copies band by band hide at most the transfer, and cost four stream
+        // commands and a launch per layer for every band: a 64 KB input in four bands took 60 us that way, 13 us so.
+        const void *src = fetchable(pl, host);
+        if (src && ((reinterpret_cast<uintptr_t>(src) ^ reinterpret_cast<uintptr_t>(staging)) & 15) == 0) {
+            if ((rc = fetch_rows_impl(pl, -1, src, staging, s)) != LOP_OK) return rc;
+            return run_batched_impl(pl, staging, out, ws, s);
+        }
     }
     // the side stream starts after everything already queued on the caller's stream; all transfers are queued
     // up front on it: band i+1 (and later) stream in while band i computes

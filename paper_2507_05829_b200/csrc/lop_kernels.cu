@@ -168,6 +168,39 @@ __global__ void pad_weights_kernel(const uint16_t *__restrict__ w, uint16_t *__r
     }
 }
 
+// ---------------------------------------------------------------------------------------------
+// The transfer step for plans that run on per-layer kernels: rows of the chain input, read straight from page-locked host
+// memory by the SMs (around the caches: the host changes it between launches).  A copy-engine copy costs several
+// microseconds of stream commands whatever its size, and a band of a small input is a microsecond of transfer; this is
+// one launch.  Bound by the host link; four 16-byte loads per thread are in flight.  One 1-D grid of segments per image
+// (blockIdx.y); elements before the first and behind the last 16-byte boundary are moved two bytes at a time.
+// ---------------------------------------------------------------------------------------------
+constexpr int FETCH_THREADS = 128, FETCH_VECS = 4;
+
+__global__ void __launch_bounds__(FETCH_THREADS) fetch_rows_kernel(const uint8_t *__restrict__ src, uint8_t *__restrict__ dst, long long image_bytes,
+                                                                   long long first, long long bytes)
+{
+    const uint8_t *s0 = src + blockIdx.y * image_bytes + first;
+    uint8_t *d0 = dst + blockIdx.y * image_bytes + first;
+    const long long mis = (16 - (reinterpret_cast<uintptr_t>(s0) & 15)) & 15, head = mis < bytes ? mis : bytes;
+    const long long nvec = (bytes - head) >> 4;
+    const uint4 *s4 = reinterpret_cast<const uint4 *>(s0 + head);
+    uint4 *d4 = reinterpret_cast<uint4 *>(d0 + head);
+    const long long v0 = (long long)blockIdx.x * (FETCH_THREADS * FETCH_VECS) + threadIdx.x;
+    uint4 q[FETCH_VECS];
+#pragma unroll
+    for (int u = 0; u < FETCH_VECS; ++u)
+        if (v0 + u * FETCH_THREADS < nvec) q[u] = __ldcv(s4 + v0 + u * FETCH_THREADS);
+#pragma unroll
+    for (int u = 0; u < FETCH_VECS; ++u)
+        if (v0 + u * FETCH_THREADS < nvec) d4[v0 + u * FETCH_THREADS] = q[u];
+    if (blockIdx.x == 0 && threadIdx.x < 16) {
+        const int h = threadIdx.x;                              // lanes 0..7: the head, 8..15: the tail
+        const long long o = h < 8 ? 2 * h : head + (nvec << 4) + 2 * (h - 8);
+        if (o < (h < 8 ? head : bytes)) *reinterpret_cast<uint16_t *>(d0 + o) = __ldcv(reinterpret_cast<const uint16_t *>(s0 + o));
+    }
+}
+
 inline int grid_for(long long work_items, int block, int max_blocks = 148 * 8)
 {
     long long b = (work_items + block - 1) / block;
@@ -204,6 +237,21 @@ cudaError_t launch_stem_gather(const void *x, void *y, const GatherGeom &g, int 
     if (g.Kcol % 8 != 0) return cudaErrorInvalidValue;
     const long long work = (long long)g.N * (hi - lo) * g.Wo * (g.Kcol / 8);
     stem_gather_kernel<<<grid_for(work, 256), 256, 0, s>>>(static_cast<const uint16_t *>(x), static_cast<uint16_t *>(y), g, lo, hi, dbg);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_fetch_rows(const void *src, void *dst, int N, int rows, long long row_bytes, int lo, int hi, cudaStream_t s)
+{
+    if (hi <= lo) return cudaSuccess;
+    long long image = (long long)rows * row_bytes, bytes = (hi - lo) * row_bytes;
+    int images = N;
+    if (lo == 0 && hi == rows) { bytes *= N; images = 1; }                // whole images are one run
+    const long long per_block = 16LL * FETCH_THREADS * FETCH_VECS;
+    for (int n = 0; n < images; n += 65535) {
+        const dim3 grid((unsigned)((bytes + per_block - 1) / per_block), (unsigned)(images - n < 65535 ? images - n : 65535));
+        fetch_rows_kernel<<<grid, FETCH_THREADS, 0, s>>>(static_cast<const uint8_t *>(src) + n * image, static_cast<uint8_t *>(dst) + n * image, image,
+                                                         lo * row_bytes, bytes);
+    }
     return cudaGetLastError();
 }
 

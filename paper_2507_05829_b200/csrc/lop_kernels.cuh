@@ -54,6 +54,9 @@ cudaError_t launch_dw_transpose(const void *w, void *wt, int C, int taps, cudaSt
 struct GatherGeom;
 // dbg: checked execution's status word (see ConvArgs), or nullptr
 cudaError_t launch_stem_gather(const void *x, void *y, const GatherGeom &g, int lo, int hi, cudaStream_t s, unsigned *dbg = nullptr);
+// Rows [lo, hi) of each of N images of `rows` rows of row_bytes bytes: src (host memory as the device addresses it) -> dst.
+// src and dst agree modulo 16.
+cudaError_t launch_fetch_rows(const void *src, void *dst, int N, int rows, long long row_bytes, int lo, int hi, cudaStream_t s);
 // w[rows][C] -> wp[rows][Cpad] zero-padded (bf16 only).
 cudaError_t launch_pad_weights(const void *w, void *wp, long long rows, int C, int Cpad, cudaStream_t s);
 

@@ -3,9 +3,11 @@ import pytest
 import torch
 
 import lop_inputs as li
+import paper_2507_05829_b200 as lop
 from lop_inputs.workloads import conv
-from paper_2507_05829_b200.chain import DeviceChain
-from test_gpu_parity import check_workload, one_layer
+from oracle import chain as ochain
+from paper_2507_05829_b200.chain import DeviceChain, to_host_f32
+from test_gpu_parity import TOL, check_workload, one_layer, rel_err
 
 pytestmark = pytest.mark.gpu
 
@@ -47,3 +49,24 @@ def test_cuda_core_convolution_takes_weights_of_any_alignment():
     torch.cuda.synchronize()
     assert torch.equal(got, want)
 
+
+# ------------------------------------------------------------------------------------ transfer of per-layer plans
+@pytest.mark.parametrize("N,H,W,C,dtype,bands", [(1, 32, 32, 16, "f32", 4), (2, 7, 5, 3, "f32", 3), (3, 9, 13, 5, "bf16", 4), (1, 1, 1, 1, "f32", 1)])
+def test_one_launch_brings_the_input_of_a_per_layer_plan(N, H, W, C, dtype, bands):
+    """Rows of any length (no multiple of 16 bytes, images that start inside a vector), one band and all."""
+    wl = one_layer(conv(C, 8, 1, p=0), N, H, W, dtype=dtype, n_bands=bands)
+    dc = DeviceChain(wl, flags=lop.LOP_FLAG_REUSE_HALO | lop.LOP_FLAG_FORCE_SIMT)
+    x = dc.pinned_input()
+    dc.staging.fill_(float("nan"))
+    dc.run_pipelined(x)
+    torch.cuda.synchronize()
+    assert dc.plans[0].last_copies() == 0 and dc.plans[0].last_launches() == 2
+    assert torch.equal(dc.staging.cpu().view(-1), x.view(-1))
+    assert rel_err(to_host_f32(dc.outs[-1]), ochain.run_workload(wl)) <= TOL[dtype]
+    r = dc.plans[0].get_range(bands - 1, lop.LOP_INPUT)
+    dc.staging.fill_(float("nan"))
+    s = torch.cuda.current_stream().cuda_stream
+    dc.plans[0].fetch_band(bands - 1, x.data_ptr(), dc.staging.data_ptr(), dc.ws[0].data_ptr(), s)
+    torch.cuda.synchronize()
+    assert torch.equal(dc.staging[:, r.new_lo:r.out_hi].cpu(), x[:, r.new_lo:r.out_hi])
+    assert torch.isnan(dc.staging[:, :r.new_lo].float()).all() and torch.isnan(dc.staging[:, r.out_hi:].float()).all()
