@@ -193,7 +193,9 @@ class Plan:
         return lib().lop_plan_flops(self._h)
 
     def run_whole(self, in_dev, out_dev, ws, stream):
-        _check(lib().lop_run_whole(self._h, in_dev, out_dev, ws, stream))
+        rc = _lib.lop_run_whole(self._h, in_dev, out_dev, ws, stream)
+        if rc:
+            _check(rc)
 
     def run_band(self, band, in_dev, out_dev, ws, stream):
         _check(lib().lop_run_band(self._h, band, in_dev, out_dev, ws, stream))
@@ -202,7 +204,9 @@ class Plan:
         _check(lib().lop_run_layer(self._h, layer, row_lo, row_hi, in_dev, out_dev, ws, stream))
 
     def run_banded(self, in_dev, out_dev, ws, stream):
-        _check(lib().lop_run_banded(self._h, in_dev, out_dev, ws, stream))
+        rc = _lib.lop_run_banded(self._h, in_dev, out_dev, ws, stream)
+        if rc:
+            _check(rc)
 
     def copy_band(self, band, in_host, staging_dev, stream):
         _check(lib().lop_copy_band(self._h, band, in_host, staging_dev, stream))
@@ -221,7 +225,9 @@ class Plan:
         _check(lib().lop_run_shard(self._h, band_lo, band_hi, in_dev, out_dev, ws, stream))
 
     def run_pipelined(self, in_host, staging_dev, out_dev, ws, stream):
-        _check(lib().lop_run_pipelined(self._h, in_host, staging_dev, out_dev, ws, stream))
+        rc = _lib.lop_run_pipelined(self._h, in_host, staging_dev, out_dev, ws, stream)
+        if rc:
+            _check(rc)
 
     def last_timing(self):
         t = LopTiming()

@@ -32,6 +32,7 @@ class DeviceChain:
         if not torch.cuda.is_available():
             raise RuntimeError("DeviceChain needs a CUDA device; there is no CPU path")
         self.wl, self.device = wl, torch.device(device)
+        self.index = torch.cuda.current_device() if self.device.index is None else self.device.index
         self.dtype = B.LOP_BF16 if wl.dtype == "bf16" else B.LOP_F32
         self.tdtype = torch.bfloat16 if wl.dtype == "bf16" else torch.float32
         self.keep = []                       # device tensors the plans point into
@@ -79,8 +80,10 @@ class DeviceChain:
         return t.contiguous().pin_memory()
 
     def _stream(self, stream):
-        s = torch.cuda.current_stream(self.device) if stream is None else stream
-        return s.cuda_stream
+        if stream is not None:
+            return stream.cuda_stream
+        # (the stream's handle without building a torch.cuda.Stream object: two microseconds of every small call)
+        return torch._C._cuda_getCurrentRawStream(self.index)
 
     def layer_output(self, seg, layer):
         """The full-size output tensor of one layer of a segment: the segment's output tensor for its last layer, else a
