@@ -8,6 +8,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <map>
 #include <vector>
 
 #include "lop_internal.h"
@@ -46,21 +47,24 @@ namespace {
 #ifndef LOP_FETCH_WINDOW_MAX_BYTES
 #define LOP_FETCH_WINDOW_MAX_BYTES (256 * 1024)
 #endif
-#ifndef LOP_SA_MAX
-#define LOP_SA_MAX 4
+// Bytes one ring entry of a per-tap stage aims at: the issuing thread pays for every entry with a wait and a commit, a
+// third of the MMAs' time at 32 KB (a ResNet-50 of batch 8: 559 us with 32 KB, 516 with 48, 515 with 64), while three
+// entries must fit the ring to keep the loads on their way.
+#ifndef LOP_ENTRY_BYTES
+#define LOP_ENTRY_BYTES (48 * 1024)
 #endif
-#ifndef LOP_SB_MAX
-#define LOP_SB_MAX 8
-#endif
-#ifndef LOP_CPS_MAX
-#define LOP_CPS_MAX 4
+#ifndef LOP_KEEP_BYTES
+#define LOP_KEEP_BYTES (80 * 1024)
 #endif
 constexpr uint32_t A_BOX_MAX = 48u * 1024u;     // largest activation box a ring slot is sized for
 constexpr uint32_t LOP_ROWOP_STAGING_BYTES = 64u * 1024u;    // largest receptive window a depth-wise item stages
-constexpr uint32_t B_BOX_MAX = 32u * 1024u;     // largest weight box
+constexpr uint32_t B_BOX_MAX = 48u * 1024u;     // largest weight box of several taps: a 3x3 filter row of 128 x 64 weights
 
 int ilog2i(int v) { int l = 0; while ((1 << l) < v) ++l; return l; }
 uint32_t round_up_u32(uint32_t v, uint32_t a) { return (v + a - 1) / a * a; }
+
+// Channels of one output unit of a tile bn channels wide: what a swizzled bulk store takes.
+int unit_channels(int bn) { return bn % 64 == 0 ? 64 : (bn % 32 == 0 ? 32 : 16); }
 
 // Tile geometry of one convolution stage.
 struct Geom {
@@ -69,22 +73,23 @@ struct Geom {
     int tw_valid;             // output columns per tile
     int RI;                   // rows of the activation box
     int BN, BK, tb, n_taps, n_chunks;
-    uint32_t a_bytes, b_bytes, a_slot, b_slot;
+    uint32_t a_bytes, b_bytes;
 };
 
 // a: the convolution as its kernel sees it (a gathered stem already reduced to 1x1).
 // even_tiles: tiles must hold whole 2x2 windows (rows and valid columns even, at least two rows).
-Geom choose_geom(const ConvArgs &a, int rows, bool even_tiles)
+// bulk_out: the tile's output leaves by bulk stores (the workers' own copy-out needs every unit of the tile in place).
+// ring: bytes of the operand ring, of which a slab stage needs two activation boxes and a weight box.
+Geom choose_geom(const ConvArgs &a, int rows, bool even_tiles, bool bulk_out, uint32_t ring)
 {
     Geom g{};
     g.BK = a.Cin % 64 == 0 ? 64 : (a.Cin % 32 == 0 ? 32 : 16);
     g.BN = 16;
     for (int bn = 128; bn >= 16; bn -= 16)
-        if (a.Cout % bn == 0) { g.BN = bn; break; }
+        if (a.Cout % bn == 0 && (bulk_out || bn / unit_channels(bn) <= WF_UNITS)) { g.BN = bn; break; }
     // A layer with few pixel tiles (a small map deep in the network) would occupy a handful of SMs, each streaming
-    // all of K for a wide slice of the weights at what one SM can pull from L2 (~40 GB/s measured): narrower
-    // output-channel tiles spread the same weight traffic over more SMs.  Not below 64: an MMA with N = 32 costs the
-    // issuing thread as much as one with N = 64 (measured on a ResNet-50 of batch 8: 669 us with a floor of 64, 732 us with 32).
+    // all of K for a wide slice of the weights: narrower output-channel tiles spread the same weight traffic over more
+    // SMs.  Not below 64: an MMA with N = 32 costs the issuing thread as much as one with N = 64 (45 and 49 cycles).
     const long long layer_tiles = ((long long)a.N * a.Ho * a.Wo + 127) / 128;
     while (g.BN > 64 && g.BN % 32 == 0 && layer_tiles * (a.Cout / g.BN) < 148) g.BN /= 2;
     g.n_taps = a.kh * a.kw;
@@ -100,7 +105,7 @@ Geom choose_geom(const ConvArgs &a, int rows, bool even_tiles)
             const int twv = P - halo_w, TR = 128 / P, RI = TR + halo_h;
             if (twv < 8 || RI > 256 || (even_tiles && (TR < 2 || (twv & 1)))) continue;
             const uint32_t box = (uint32_t)RI * P * row_bytes;
-            if (box > A_BOX_MAX) continue;
+            if (box > A_BOX_MAX || 2u * box + (uint32_t)(a.kw * g.BN) * row_bytes > ring) continue;
             const long long tiles = (long long)((a.Wo + twv - 1) / twv) * ((rows + TR - 1) / TR);
             if (best_tiles < 0 || tiles < best_tiles || (tiles == best_tiles && box < best_box)) {
                 best_tiles = tiles; best_box = box;
@@ -109,8 +114,7 @@ Geom choose_geom(const ConvArgs &a, int rows, bool even_tiles)
             }
         }
     }
-    if (slab || pointwise) g.mode = WF_SLAB;
-    else g.mode = WF_TAP;
+    g.mode = slab ? WF_SLAB : WF_TAP;
     if (!slab) {
         // dense tile: the (TW, TR, TN) split of 128 pixels that needs the fewest tiles
         int nmax = 1;
@@ -127,16 +131,16 @@ Geom choose_geom(const ConvArgs &a, int rows, bool even_tiles)
         g.tw_valid = g.P; g.RI = g.TR;
     }
     g.a_bytes = (uint32_t)g.RI * g.P * g.TN * row_bytes;
-    // a shifted tap reads up to halo_w pixels past the box: the slot's padding takes that
-    g.a_slot = round_up_u32(g.a_bytes + (slab ? (uint32_t)halo_w * row_bytes : 0u), 1024u);
+    // (a shifted tap reads up to halo_w pixels past the box, into whatever follows it in shared memory: those rows of the
+    // accumulator are the dropped anchors of the halo gap)
     g.tb = 1;
-    if (g.mode == WF_SLAB && g.n_taps > 1) {
-        const int cap = std::max(1, (int)(B_BOX_MAX / ((uint32_t)g.BN * row_bytes)));
-        const int nblk = (g.n_taps + cap - 1) / cap;
-        g.tb = (g.n_taps + nblk - 1) / nblk;
+    if (slab) {
+        // whole filter rows where one fits a box, else as many taps as do
+        const uint32_t tap_bytes = (uint32_t)g.BN * row_bytes;
+        const int cap = std::max(1, (int)(B_BOX_MAX / tap_bytes)), nblk = (g.n_taps + cap - 1) / cap;
+        g.tb = a.kw * tap_bytes <= B_BOX_MAX ? a.kw : (g.n_taps + nblk - 1) / nblk;
     }
     g.b_bytes = (uint32_t)g.tb * g.BN * row_bytes;
-    g.b_slot = round_up_u32(g.b_bytes, 1024u);
     return g;
 }
 
@@ -182,6 +186,28 @@ int encode_maps(const ConvArgs &a, const Geom &g, CUtensorMap *out, int *valid_m
         return LOP_ECUDA;
     *valid_mask = mask;
     return LOP_OK;
+}
+
+// Rows below oh_hi of an output-shaped tensor, in boxes of one output unit: `sub` channels of a tile's packed rows.
+int encode_rows_map(const ConvArgs &a, const void *tensor, int sub, int tw, int tr, int tn, CUtensorMap *out)
+{
+    TensorMapEncodeFn enc = tensor_map_encoder();
+    if (!enc) return LOP_ECUDA;
+    const CUtensorMapSwizzle swz = sub == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : (sub == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
+    const cuuint32_t ones[4] = {1, 1, 1, 1};
+    const cuuint64_t dims[4] = {(cuuint64_t)a.Cout, (cuuint64_t)a.Wo, (cuuint64_t)a.oh_hi, (cuuint64_t)a.N};
+    const cuuint64_t strides[3] = {(cuuint64_t)a.Cout * 2, (cuuint64_t)a.Wo * a.Cout * 2, (cuuint64_t)a.Ho * a.Wo * a.Cout * 2};
+    const cuuint32_t box[4] = {(cuuint32_t)sub, (cuuint32_t)tw, (cuuint32_t)tr, (cuuint32_t)tn};
+    return enc(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(tensor), dims, strides, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS ? LOP_OK : LOP_ECUDA;
+}
+
+// Bulk stores go to device memory; a result tensor in mapped host memory is stored by the workers.
+bool in_device_memory(const void *p)
+{
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) { cudaGetLastError(); return false; }
+    return at.type == cudaMemoryTypeDevice;
 }
 
 // Layer i is a tensor-core convolution whose output is read by nothing but a 2x2 stride-2 unpadded max pooling
@@ -522,7 +548,25 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
     std::vector<int> expected;                         // completions per row group, per stage
     int n_ctr = WF_CTR_FIRST;
     bool uses_flags = false;
-    uint32_t a_slot = 1024, b_slot = 1024, stg_bytes = 1024;
+    uint32_t unit_bytes = 1024, stg_bytes = 0;
+    // scratch of the SIMT items, and with it what the operand ring has at least
+    auto gather_scratch = [](const lop_plan_t *pl, const LayerInfo &li) {
+        // the kh image rows an output row reads are staged in shared memory when they fit, else read in place
+        const uint32_t pitch = ((uint32_t)pl->W * pl->C * 2u + 31u + 15u) & ~15u;
+        const uint32_t need = round_up_u32((uint32_t)li.l.kh * pitch + 4u * (uint32_t)li.cin_eff, 1024u);
+        return need <= 48u * 1024u && li.l.kh <= 64 ? need : 0u;
+    };
+    for (const StageReq &rq : reqs) {
+        const lop_plan_t *pl = segs[rq.seg].pl;
+        const LayerInfo &li = pl->layers[rq.layer];
+        rowop::DwTile t{1, 1, 8};
+        if (rq.gather) stg_bytes = std::max(stg_bytes, gather_scratch(pl, li));
+        else if (!rq.fetch && li.l.op == LOP_DWCONV2D && dw_tile(pl, li, &t))
+            stg_bytes = std::max(stg_bytes, round_up_u32((uint32_t)rowop::dw_tile_bytes(li.l.kh, li.l.kw, li.l.sh, li.l.sw, li.l.dh, li.l.dw, t), 1024u));
+    }
+    const uint32_t ring_least = (227u * 1024u - 1024u - WF_FIXED_SMEM - stg_bytes - WF_UNITS * 16u * 1024u) & ~1023u;
+    std::vector<char> out_on_device(segs.size());
+    for (size_t i = 0; i < segs.size(); ++i) out_on_device[i] = in_device_memory(segs[i].out);
 
     std::vector<char> consumed(reqs.size(), 0);            // pooling requests folded into their convolution's stage
     std::vector<int> prod_lo, prod_hi;                     // per stage: rows of the tensor it produces
@@ -557,11 +601,7 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
             st.x = in; st.y = wsb + pl->col_off;
             st.N = pl->N; st.Hin = pl->H; st.Win = pl->W; st.Cin = pl->C; st.Ho = li.Ho; st.Wo = li.Wo; st.Cout = li.cin_eff;
             st.kh = l.kh; st.kw = l.kw; st.sh = l.sh; st.sw = l.sw; st.ph = l.ph; st.pw = l.pw; st.dh = l.dh; st.dw = l.dw;
-            // the kh image rows an output row reads are staged in shared memory when they fit (mode 0), else read in place
-            const uint32_t pitch = ((uint32_t)pl->W * pl->C * 2u + 31u + 15u) & ~15u;
-            const uint32_t need = round_up_u32((uint32_t)l.kh * pitch + 4u * (uint32_t)li.cin_eff, 1024u);
-            if (need <= 48u * 1024u && l.kh <= 64) stg_bytes = std::max(stg_bytes, need);
-            else st.mode = 1;
+            st.mode = gather_scratch(pl, li) ? 0 : 1;
         } else if (l.op == LOP_MAXPOOL2D) {
             const PoolArgs a = pool_args(pl, rq.layer, in, out, ws, rq.lo, rq.hi);
             st.kind = WF_POOL;
@@ -584,7 +624,6 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
                 tiles_r = (rows + t.R - 1) / t.R;
                 tiles_w = (li.Wo + t.tw - 1) / t.tw;
                 cout_tiles = l.cin / t.cc;
-                stg_bytes = std::max(stg_bytes, round_up_u32((uint32_t)rowop::dw_tile_bytes(l.kh, l.kw, l.sh, l.sw, l.dh, l.dw, t), 1024u));
             }
         } else {
             const ConvArgs a = conv_args(pl, rq.layer, in, out, ws, rq.lo, rq.hi);
@@ -595,7 +634,8 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
                     if (!consumed[k] && !reqs[k].gather && reqs[k].seg == rq.seg && reqs[k].band == rq.band &&
                         reqs[k].layer == rq.layer + 1 && rq.lo == 2 * reqs[k].lo && rq.hi == 2 * reqs[k].hi) { rj = k; break; }
             const bool fuse = rj < reqs.size();
-            const Geom g = choose_geom(a, rows, fuse);
+            const bool bulk_out = !fuse && (rq.layer + 1 < (int)pl->layers.size() || out_on_device[rq.seg]);
+            const Geom g = choose_geom(a, rows, fuse, bulk_out, ring_least);
             st.kind = WF_CONV;
             st.mode = g.mode;
             st.x = a.x; st.res = a.res; st.scale = a.scale; st.shift = a.shift; st.y = a.y;
@@ -626,9 +666,21 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
             st.sbo_bytes = 8u * st.row_bytes;
             // instruction descriptor: fp32 accumulate, bf16 x bf16, both operands K-major, N = BN, M = 128
             st.idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(g.BN >> 3) << 17) | ((128u >> 4) << 24);
-            a_slot = std::max(a_slot, g.a_slot);
-            b_slot = std::max(b_slot, g.b_slot);
-            stg_bytes = std::max(stg_bytes, round_up_u32(128u * (uint32_t)g.BN * 2u, 1024u));
+            const int sub = unit_channels(g.BN);
+            st.sub_log = ilog2i(sub);
+            unit_bytes = std::max(unit_bytes, round_up_u32((uint32_t)((128 >> st.p_log) * g.tw_valid * sub * 2), 1024u));
+            st.out_map = st.res_map = -1;
+            CUtensorMap rm;
+            if (a.res) {
+                if (encode_rows_map(a, a.res, sub, g.tw_valid, g.TR, g.TN, &rm) != LOP_OK) { set_error("layer %d: residual map encoding failed", rq.layer); return LOP_ECUDA; }
+                st.res_map = (int)maps.size();
+                maps.push_back(rm);
+            }
+            if (bulk_out) {
+                if (encode_rows_map(a, a.y, sub, g.tw_valid, g.TR, g.TN, &rm) != LOP_OK) { set_error("layer %d: output map encoding failed", rq.layer); return LOP_ECUDA; }
+                st.out_map = (int)maps.size();
+                maps.push_back(rm);
+            }
             if (fuse) {
                 const LayerInfo &pool = pl->layers[rq.layer + 1];
                 consumed[rj] = 1;
@@ -725,28 +777,35 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
     const int n_items = (int)items.size();
     if (n_items == 0 && fetch_items.empty()) { *result = p; return LOP_OK; }          // nothing to do: an empty program
 
-    // ---- shared-memory rings: as many slots as fit beside the staging tile, weights first
-    const size_t fixed = 1024 + stg_bytes + 8 * (2 * 8 + 2 * 8 + 4 + 2 * WF_PUBQ + 4) + 64 + 2048 + 1280 + 64;
-    const size_t budget = 227 * 1024 - fixed;
-    int sa = 2, sb = 2;
-    if ((size_t)sa * a_slot + (size_t)sb * b_slot > budget) { delete p; set_error("tile buffers do not fit shared memory"); return LOP_EUNSUPPORTED; }
-    for (bool grew = true; grew;) {
-        grew = false;
-        if (sb < LOP_SB_MAX && (size_t)sa * a_slot + (size_t)(sb + 1) * b_slot <= budget) { ++sb; grew = true; }
-        if (sa < LOP_SA_MAX && (size_t)(sa + 1) * a_slot + (size_t)sb * b_slot <= budget) { ++sa; grew = true; }
-    }
-
-    // chunks per ring slot of the long pointwise stages (see WfStage::cps), now that the slot sizes are known
+    // ---- shared memory: the operand ring takes what the output units and the SIMT scratch leave
+    const uint32_t ring_bytes = (227u * 1024u - 1024u - WF_FIXED_SMEM - stg_bytes - WF_UNITS * unit_bytes) & ~1023u;
+    std::map<int, long long> tiles_of;                            // convolution tiles per weight map: the layer's stages together
+    for (const int4 &it : items)
+        if (stages[it.x & 0xFFFF].kind == WF_CONV) ++tiles_of[stages[it.x & 0xFFFF].map_base];
     for (WfStage &st : stages) {
         st.cps = 1;
         if (st.kind != WF_CONV) continue;
-        const bool long_pointwise = st.mode == WF_SLAB && st.n_taps == 1 && st.BK == 64 && st.n_chunks > sb;
-        if (!long_pointwise && st.mode != WF_TAP) continue;            // per-tap windows: cps consecutive taps per slot
-        st.cps = std::max(1, std::min({(int)(a_slot / st.a_bytes), (int)(b_slot / st.b_bytes), LOP_CPS_MAX}));
+        const uint32_t a_sz = round_up_u32(st.a_bytes, 1024u), b_sz = round_up_u32(st.b_bytes, 1024u);
+        // Weights stay in shared memory from tile to tile where every CTA gets at least two tiles of the layer, always of
+        // the same output channels (items go round-robin), and they leave room for two activation boxes.
+        const uint32_t boxes = (uint32_t)st.n_chunks * ((st.n_taps + st.tb - 1) / st.tb);
+        const int cout_tiles = st.Cout / st.BN;
+        if (boxes * b_sz <= LOP_KEEP_BYTES && boxes * b_sz + 2u * a_sz <= ring_bytes && 148 % cout_tiles == 0 && tiles_of[st.map_base] >= 2 * 148)
+            st.keep_bytes = (int)(boxes * b_sz);
+        if (2u * a_sz + b_sz > ring_bytes) { delete p; set_error("tile buffers do not fit shared memory"); return LOP_EUNSUPPORTED; }
+        if (st.mode == WF_SLAB && !st.keep_bytes) {
+            // weight boxes per full barrier: the issuing thread stalls at every wait, so it waits once per chunk where the
+            // chunk's weights fit the ring with room for part of the next chunk's
+            const int per_chunk = (st.n_taps + st.tb - 1) / st.tb;
+            const uint32_t most = std::max(b_sz, (ring_bytes - 2u * a_sz) * 7u / 10u);
+            const int groups = (int)((per_chunk * b_sz + most - 1) / most);
+            st.cps = std::min((per_chunk + groups - 1) / groups, (int)(most / b_sz));
+        }
+        if (st.mode == WF_TAP) st.cps = std::max(1, (int)(LOP_ENTRY_BYTES / (st.keep_bytes ? a_sz : a_sz + b_sz)));
     }
 
 #ifdef LOP_WF_TRACE
-    fprintf(stderr, "program: %zu stages, %d items, rings: %d x %u B activations, %d x %u B weights, staging %u B\n", stages.size(), n_items, sa, a_slot, sb, b_slot, stg_bytes);
+    fprintf(stderr, "program: %zu stages, %d items, ring %u B, units %u B, scratch %u B\n", stages.size(), n_items, ring_bytes, unit_bytes, stg_bytes);
 #endif
     // ---- one device allocation for all tables
     auto al = [](size_t v) { return (v + 255) / 256 * 256; };
@@ -783,8 +842,7 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
     P.flag_base = p->flag_base; P.n_flags = p->n_flags;
     P.n_stages = (int)stages.size();
     P.n_items = n_items;
-    P.sa = sa; P.sb = sb;
-    P.a_slot_bytes = a_slot; P.b_slot_bytes = b_slot; P.stg_bytes = stg_bytes;
+    P.ring_bytes = ring_bytes; P.unit_bytes = unit_bytes; P.simt_bytes = stg_bytes;
     P.fetch_items = reinterpret_cast<const int4 *>(d + o_fetch);
     P.fetch_src = fetch_src;
     P.fetch_dst = const_cast<void *>(segs[0].in);

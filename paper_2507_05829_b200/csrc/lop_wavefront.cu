@@ -41,6 +41,7 @@ namespace {
 using namespace ptx;
 
 constexpr int EPI_THREADS = 32 * WF_WORKER_WARPS;
+static_assert(8 * (2 * WF_ENTRIES + 4 + 2 * WF_PUBQ + 4 + 3 * WF_UNITS + 2 + WF_GROUPS) + 128 + 2048 + 8 * (128 + 32) <= WF_FIXED_SMEM, "barriers and tables");
 constexpr int COL_GROUPS = WF_WORKER_WARPS / 4;            // worker warps sharing a TMEM lane group split the columns
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned *p)
@@ -153,12 +154,6 @@ __device__ __forceinline__ void mma_tap_f(uint32_t acc, uint32_t la, uint32_t lb
     else if (ksteps == 2) mma_ksteps_f<2>(acc, la, lb, desc_hi, idesc, accumulate);
     else mma_ksteps_f<1>(acc, la, lb, desc_hi, idesc, accumulate);
 }
-__device__ __forceinline__ void mma_tap(uint32_t acc, uint32_t pa, uint32_t pb, uint32_t desc_hi, uint32_t idesc, int ksteps,
-                                        uint32_t &accumulate)
-{
-    mma_tap_f(acc, desc_lo(pa), desc_lo(pb), desc_hi, idesc, ksteps, accumulate);
-}
-
 // One weight box of three taps of a 3x3 filter row over a 64-channel chunk: twelve MMAs whose descriptors differ
 // from the first one by compile-time constants.  One thread issues every MMA of the CTA and each instruction it
 // executes in between costs as much as a quarter of an N = 64 MMA, so the common case gets straight-line code.
@@ -303,21 +298,25 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t *smem = smem_raw + (base - raw);
-    const int SA = P.sa, SB = P.sb;
-    const uint32_t a_slot_bytes = P.a_slot_bytes, b_slot_bytes = P.b_slot_bytes;
-    const uint32_t a0 = base, b0 = a0 + (uint32_t)SA * a_slot_bytes, stg0 = b0 + (uint32_t)SB * b_slot_bytes;
-    const uint32_t bars = stg0 + P.stg_bytes;
-    const uint32_t full_a = bars, empty_a = full_a + 8u * SA, full_b = empty_a + 8u * SA, empty_b = full_b + 8u * SB;
-    const uint32_t accf0 = empty_b + 8u * SB, acce0 = accf0 + 16u;
-    const uint32_t pubf0 = acce0 + 16u, pube0 = pubf0 + 8u * WF_PUBQ;
+    // shared memory: operand ring | output units | scratch of the SIMT items | barriers | tables
+    const uint32_t ring_bytes = P.ring_bytes, unit_bytes = P.unit_bytes;
+    const uint32_t ring0 = base, unit0 = ring0 + ring_bytes, simt0 = unit0 + WF_UNITS * unit_bytes, bars = simt0 + P.simt_bytes;
+    const uint32_t full0 = bars, empty0 = full0 + 8u * WF_ENTRIES;      // operand entries: loaded / consumed
+    const uint32_t accf0 = empty0 + 8u * WF_ENTRIES, acce0 = accf0 + 16u;   // accumulators: complete / drained
+    const uint32_t pubf0 = acce0 + 16u, pube0 = pubf0 + 8u * WF_PUBQ;    // items the workers stored themselves: stored / published
     const uint32_t ssf0 = pube0 + 8u * WF_PUBQ, sse0 = ssf0 + 16u;      // scale/shift buffers of two tiles: full / empty
-    uint8_t *tail = smem + (sse0 + 16u - base);
+    const uint32_t ugrant0 = sse0 + 16u;                                 // output units: free to write, the residual (if any) in place
+    const uint32_t uready0 = ugrant0 + 8u * WF_UNITS, ufree0 = uready0 + 8u * WF_UNITS;     // ... finished by the workers / read out
+    const uint32_t wfull = ufree0 + 8u * WF_UNITS, wempty = wfull + 8u;  // kept weights: loaded / last used
+    const uint32_t gfull0 = wempty + 8u;                                 // slab stages: a group of boxes is loaded
+    uint8_t *tail = smem + (gfull0 + 8u * WF_GROUPS - base);
     volatile uint32_t *misc = reinterpret_cast<volatile uint32_t *>(tail);      // [0] TMEM base, [1] abort, [2] run, [3] epilogue failure
-    float *s_scale = reinterpret_cast<float *>(tail + 64);                       // [2][128]: per-channel scale of this and the next tile
+    volatile uint32_t *entry_at = misc + 16;                                     // [WF_ENTRIES]: where the ring's entries start (loader only)
+    float *s_scale = reinterpret_cast<float *>(tail + 128);                      // [2][128]: per-channel scale of this and the next tile
     float *s_shift = s_scale + 256;                                              // [2][128]
-    long long *row_pix = reinterpret_cast<long long *>(tail + 64 + 2048);        // [128]: element offset of anchor m's output, or -1
+    long long *row_pix = reinterpret_cast<long long *>(tail + 128 + 2048);       // [128]: element offset of a staged row's output, or -1
     long long *pool_pix = row_pix + 128;                                         // [32]: element offset of a 2x2 window's pooled output, or -1
-    uint8_t *stg = smem + (stg0 - base);
+    uint8_t *units = smem + (unit0 - base), *stg = smem + (simt0 - base);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0 && blockIdx.x < 4) {
@@ -325,13 +324,9 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
         trv(TRACE_ITEMS - 8 + (int)blockIdx.x, 4, (unsigned long long)clock64());
     }
     if (threadIdx.x == 0) {
-        for (int s = 0; s < SA; ++s) {
-            mbar_init(full_a + 8u * s, 1);
-            mbar_init(empty_a + 8u * s, 1);
-        }
-        for (int s = 0; s < SB; ++s) {
-            mbar_init(full_b + 8u * s, 1);
-            mbar_init(empty_b + 8u * s, 1);
+        for (int e = 0; e < WF_ENTRIES; ++e) {
+            mbar_init(full0 + 8u * e, 1);
+            mbar_init(empty0 + 8u * e, 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(accf0 + 8u * b, 1);
@@ -339,6 +334,14 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
             mbar_init(ssf0 + 8u * b, 1);
             mbar_init(sse0 + 8u * b, 1);
         }
+        for (int u = 0; u < WF_UNITS; ++u) {
+            mbar_init(ugrant0 + 8u * u, 1);
+            mbar_init(uready0 + 8u * u, WF_WORKER_WARPS);
+            mbar_init(ufree0 + 8u * u, 1);
+        }
+        mbar_init(wfull, 1);
+        mbar_init(wempty, 1);
+        for (int g = 0; g < WF_GROUPS; ++g) mbar_init(gfull0 + 8u * g, 1);
         for (int q = 0; q < WF_PUBQ; ++q) {
             mbar_init(pubf0 + 8u * q, 1);
             mbar_init(pube0 + 8u * q, 1);
@@ -378,11 +381,15 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
         uint32_t a_bytes = 0, b_bytes = 0;
         const CUtensorMap *maps = nullptr;
         const float *scale = nullptr, *shift = nullptr;
-        int slab_offh = 0, slab_offw = 0, slab_mi = 0, n_boxes = 1, cps = 1;
-        bool slab_have = true;
-        uint32_t a_slot = 0, a_phase = 0, b_slot = 0, b_phase = 0, pc = 0;
-        bool w_kept = false;                                   // (lane 0) the ring holds the weights of tile key w_key
-        long long w_key = -1;
+        int first_offh = 0, first_offw = 0, first_mi = 0, n_boxes = 1, cps = 1, units_n = 0, sub_log = 6, res_map = -1;
+        bool first_have = true;
+        uint32_t a_sz = 0, b_sz = 0, keep_bytes = 0, res_bytes = 0;
+        uint32_t pc = 0, uc = 0;
+        // Operand ring (lane 0).  Entries are allocated and freed in order; positions are counted without wrapping
+        // (head), an entry never straddles the ring's end.  The MMA issuer derives the same places from the same records.
+        uint32_t ring_lim = ring_bytes, head = 0, pos = 0, tail_at = 0, n_alloc = 0, n_freed = 0, n_full = 0, n_group = 0, w_uses = 0;
+        uint32_t slab_sl = 0, slab_end0 = 0, slab_end1 = 0;    // slab stages: next activation box, entry that ended its previous chunk
+        long long cut_key = 0;                                 // how the ring is cut (see below)
         for (; item < NI; item += G) {
             // two items ahead: the record; one item ahead: this lane's dependency entry
             const int4 nn = item + 2 * G < NI ? __ldg(&P.items[item + 2 * G]) : zero4;
@@ -400,13 +407,17 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 ph = __ldg(&sp->ph); pw = __ldg(&sp->pw); dh = __ldg(&sp->dh); dw = __ldg(&sp->dw);
                 scale = ldg_ptr<const float *>(reinterpret_cast<const void *const *>(&sp->scale));
                 shift = ldg_ptr<const float *>(reinterpret_cast<const void *const *>(&sp->shift));
-                // slab mode: the box starts at the first tap's offset; which parity map that is and how far in
-                const int offh = floor_div_i(-ph, sh), offw = floor_div_i(-pw, sw);
-                slab_offh = offh; slab_offw = offw;
-                slab_mi = (-ph - offh * sh) * sw + (-pw - offw * sw);
-                slab_have = (amask >> slab_mi) & 1;
+                // the first tap's offset (slab mode: where the box starts): which parity map that is and how far in
+                first_offh = floor_div_i(-ph, sh); first_offw = floor_div_i(-pw, sw);
+                first_mi = (-ph - first_offh * sh) * sw + (-pw - first_offw * sw);
+                first_have = (amask >> first_mi) & 1;
                 n_boxes = n_chunks * ((n_taps + tbx - 1) / tbx);
                 cps = __ldg(&sp->cps);
+                a_sz = (a_bytes + 1023u) & ~1023u; b_sz = (b_bytes + 1023u) & ~1023u;
+                keep_bytes = (uint32_t)__ldg(&sp->keep_bytes);
+                sub_log = __ldg(&sp->sub_log); units_n = BN >> sub_log;
+                res_map = __ldg(&sp->res_map);
+                res_bytes = (uint32_t)(((128 >> p_log) * tw_valid) << (sub_log + 1));
             }
             if (kind == WF_CONV) {
                 if (lane == 0) tr(item, 0);
@@ -424,9 +435,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 }
                 ok = ok && wait_deps_warp(P, rec_dep0(cur), rec_ndep(cur), dep_cur, run, lane);
                 if (ok) {
-                    // "scale / shift are in place AND the tile's producers (the residual's included) are done": the
-                    // workers fetch the residual tile behind this barrier, while the operands are still on their way
-                    if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(ssf0 + 8u * (pc & 1u)) : "memory");
+                    if (lane == 0) mbar_arrive(ssf0 + 8u * (pc & 1u));          // scale / shift are in place
                     ++pc;
                 }
                 int fail = 0;
@@ -440,82 +449,127 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                     const int oh0 = oh_lo + (rec_tr(cur) << tr_log);
                     const int n0 = rec_tn(cur) * (128 >> (p_log + tr_log));
                     const int co0 = rec_cout(cur) * BN;
-                    // Weights stay in their ring slots from one tile to the next while consecutive tiles of this CTA
-                    // use the same ones (same layer, same output channels) and all their boxes fit the ring: only the
-                    // first such tile loads them.  The MMA issuer takes the same decisions from the same records and
-                    // frees the slots when a tile with other weights comes up.
-                    const long long wkey = (long long)(maps - P.maps) * 65536 + rec_cout(cur);
-                    const bool can_keep = mode == WF_SLAB && n_boxes <= SB;
-                    const bool reuse_w = w_kept && can_keep && wkey == w_key;
-                    w_kept = reuse_w || can_keep;
-                    w_key = wkey;
-                    if (cps > 1 && mode == WF_SLAB) {
-                        for (int ch = 0; ch < n_chunks && !fail; ch += cps) {
-                            const int g = min(cps, n_chunks - ch);
-                            if (!mbar_wait_abortable(empty_a + 8u * a_slot, a_phase ^ 1u, abort_flag) ||
-                                !mbar_wait_abortable(empty_b + 8u * b_slot, b_phase ^ 1u, abort_flag)) { fail = 1; break; }
-                            const uint32_t fa = full_a + 8u * a_slot, fb = full_b + 8u * b_slot;
-                            mbar_expect_tx(fa, (uint32_t)g * a_bytes);
-                            mbar_expect_tx(fb, (uint32_t)g * b_bytes);
-                            for (int u = 0; u < g; ++u) {
-                                tma_load_4d(a0 + a_slot * a_slot_bytes + (uint32_t)u * a_bytes, maps + slab_mi, fa, (ch + u) * BK,
-                                            slab_have ? ow0 + slab_offw : -65536, slab_have ? oh0 + slab_offh : -65536, n0);
-                                tma_load_3d(b0 + b_slot * b_slot_bytes + (uint32_t)u * b_bytes, maps + 4, fb, (ch + u) * BK, co0, 0);
+                    // waits until the oldest entry is consumed
+                    auto free_oldest = [&]() {
+                        const uint32_t e = n_freed & (WF_ENTRIES - 1);
+                        if (!mbar_wait_abortable(empty0 + 8u * e, (n_freed / WF_ENTRIES) & 1u, abort_flag)) return false;
+                        ++n_freed;
+                        tail_at = n_freed == n_alloc ? head : entry_at[n_freed & (WF_ENTRIES - 1)];
+                        return true;
+                    };
+                    // a place of `size` bytes: its address, 0 when a wait ran out
+                    auto place = [&](uint32_t size) -> uint32_t {
+                        if (pos + size > ring_lim) { head += ring_lim - pos; pos = 0; }
+                        if (n_freed == n_alloc) tail_at = head;
+                        while (head + size - tail_at > ring_lim || n_alloc - n_freed == WF_ENTRIES)
+                            if (!free_oldest()) return 0u;
+                        const uint32_t at = ring0 + pos;
+                        entry_at[n_alloc & (WF_ENTRIES - 1)] = head;
+                        ++n_alloc; head += size; pos += size;
+                        return at;
+                    };
+                    // ... with a full barrier of its own, armed for `tx` bytes
+                    uint32_t full_bar = 0;
+                    auto allocate = [&](uint32_t size, uint32_t tx) -> uint32_t {
+                        const uint32_t at = place(size);
+                        full_bar = full0 + 8u * (n_full & (WF_ENTRIES - 1));
+                        if (at) { ++n_full; mbar_expect_tx(full_bar, tx); }
+                        return at;
+                    };
+                    // How the ring is cut.  key > 0, kept weights: where a layer gives every CTA several tiles of the same
+                    // output channels, the tile's weights stay at the ring's end and only the first such tile loads them.
+                    // key < 0, slab stages: two activation boxes at the ring's end beside the weight boxes -- a chunk's
+                    // activation box outlives its weight boxes, so it cannot be an entry among them.  key == 0: one ring.
+                    // When the key changes (the MMA issuer takes the same decision from the same records) the ring is
+                    // drained and cut anew.
+                    const bool kept = keep_bytes != 0;
+                    const long long key = kept ? (((long long)(maps - P.maps) << 16) | rec_cout(cur)) + 1 : (mode == WF_SLAB ? -(long long)a_sz : 0);
+                    if (key != cut_key) {
+                        // (MMAs complete in order: the newest entry stands for all)
+                        if (n_freed != n_alloc) {
+                            const uint32_t last = n_alloc - 1u;
+                            fail = !mbar_wait_abortable(empty0 + 8u * (last & (WF_ENTRIES - 1)), (last / WF_ENTRIES) & 1u, abort_flag);
+                            n_freed = n_alloc;
+                        }
+                        slab_end0 = slab_end1 = n_freed;
+                        if (!fail && cut_key > 0 && !mbar_wait_abortable(wempty, (w_uses - 1u) & 1u, abort_flag)) fail = 1;
+                        cut_key = key;
+                        ring_lim = ring_bytes - (key < 0 ? 2u * a_sz : keep_bytes);
+                        head = pos = tail_at = 0;
+                        if (!fail && kept) {
+                            ++w_uses;
+                            mbar_expect_tx(wfull, (uint32_t)n_boxes * b_bytes);
+                            uint32_t at = ring0 + ring_lim;
+                            for (int ch = 0; ch < n_chunks; ++ch)
+                                for (int t0 = 0; t0 < n_taps; t0 += tbx, at += b_sz) tma_load_3d(at, maps + 4, wfull, ch * BK, co0, t0);
+                        }
+                    }
+                    // the whole receptive window of the tile in one box per chunk: its first tap's offset places it
+                    const int aw = first_have ? ow0 + first_offw : -65536, ah = first_have ? oh0 + first_offh : -65536;
+                    if (mode == WF_SLAB && kept) {
+                        for (int ch = 0; ch < n_chunks && !fail; ++ch) {
+                            const uint32_t at = allocate(a_sz, a_bytes);
+                            if (!at) { fail = 1; break; }
+                            tma_load_4d(at, maps + first_mi, full_bar, ch * BK, aw, ah, n0);
+                        }
+                    } else if (mode == WF_SLAB) {
+                        const int per_chunk = (n_taps + tbx - 1) / tbx;
+                        for (int ch = 0; ch < n_chunks && !fail; ++ch) {
+                            // the activation box of the chunk two back is consumed when that chunk's last entry is
+                            while ((int)(n_freed - slab_end0) < 0)
+                                if (!free_oldest()) { fail = 1; break; }
+                            uint32_t bar = 0;
+                            for (int i = 0, in_group = 0; i < per_chunk && !fail; ++i) {
+                                if (in_group == 0) {
+                                    bar = gfull0 + 8u * (n_group & (WF_GROUPS - 1));
+                                    ++n_group;
+                                    mbar_expect_tx(bar, (uint32_t)min(cps, per_chunk - i) * b_bytes + (i == 0 ? a_bytes : 0u));
+                                    if (i == 0) tma_load_4d(ring0 + ring_lim + slab_sl * a_sz, maps + first_mi, bar, ch * BK, aw, ah, n0);
+                                }
+                                const uint32_t at = place(b_sz);
+                                if (!at) { fail = 1; break; }
+                                tma_load_3d(at, maps + 4, bar, ch * BK, co0, i * tbx);
+                                if (++in_group == cps) in_group = 0;
                             }
-                            if (++a_slot == (uint32_t)SA) { a_slot = 0; a_phase ^= 1u; }
-                            if (++b_slot == (uint32_t)SB) { b_slot = 0; b_phase ^= 1u; }
+                            slab_end0 = slab_end1; slab_end1 = n_alloc;
+                            slab_sl ^= 1u;
                         }
                     } else {
-                    int tap_u = 0, in_slot = 0;                        // per-tap mode: boxes issued so far, boxes in the open slot
-                    for (int ch = 0; ch < n_chunks && !fail; ++ch) {
-                        if (mode == WF_SLAB) {
-                            // the whole receptive window of the tile in one box: its first tap's offset places it
-                            const int mi = slab_mi, offh = slab_offh, offw = slab_offw;
-                            const bool have = slab_have;
-                            if (!mbar_wait_abortable(empty_a + 8u * a_slot, a_phase ^ 1u, abort_flag)) { fail = 1; break; }
-                            const uint32_t fa = full_a + 8u * a_slot;
-                            mbar_expect_tx(fa, a_bytes);
-                            tma_load_4d(a0 + a_slot * a_slot_bytes, maps + mi, fa, ch * BK, have ? ow0 + offw : -65536,
-                                        have ? oh0 + offh : -65536, n0);
-                            if (++a_slot == (uint32_t)SA) { a_slot = 0; a_phase ^= 1u; }
-                            for (int t0 = 0; t0 < n_taps && !reuse_w; t0 += tbx) {
-                                if (!mbar_wait_abortable(empty_b + 8u * b_slot, b_phase ^ 1u, abort_flag)) { fail = 1; break; }
-                                const uint32_t fb = full_b + 8u * b_slot;
-                                mbar_expect_tx(fb, b_bytes);
-                                tma_load_3d(b0 + b_slot * b_slot_bytes, maps + 4, fb, ch * BK, co0, t0);
-                                if (++b_slot == (uint32_t)SB) { b_slot = 0; b_phase ^= 1u; }
-                            }
-                        } else {
-                            // one activation and one weight box per (channel chunk, tap); `cps` consecutive taps share a
-                            // slot of each ring and its barrier (strides are 1 or 2 almost always: no division then)
-                            for (int a = 0; a < kh && !fail; ++a) {
-                                const int qh = a * dh - ph;
-                                const int offh = sh == 1 ? qh : (sh == 2 ? qh >> 1 : floor_div_i(qh, sh)), parh = qh - offh * sh;
-                                for (int b = 0; b < kw; ++b, ++tap_u) {
-                                    const int qw = b * dw - pw;
-                                    const int offw = sw == 1 ? qw : (sw == 2 ? qw >> 1 : floor_div_i(qw, sw)), parw = qw - offw * sw;
-                                    const int mi = parh * sw + parw;
-                                    const bool have = (amask >> mi) & 1;
-                                    if (in_slot == 0) {
-                                        const int g = min(cps, n_chunks * n_taps - tap_u);
-                                        if (!mbar_wait_abortable(empty_a + 8u * a_slot, a_phase ^ 1u, abort_flag) ||
-                                            !mbar_wait_abortable(empty_b + 8u * b_slot, b_phase ^ 1u, abort_flag)) { fail = 1; break; }
-                                        mbar_expect_tx(full_a + 8u * a_slot, (uint32_t)g * a_bytes);
-                                        mbar_expect_tx(full_b + 8u * b_slot, (uint32_t)g * b_bytes);
-                                    }
-                                    tma_load_4d(a0 + a_slot * a_slot_bytes + (uint32_t)in_slot * a_bytes, maps + mi, full_a + 8u * a_slot, ch * BK,
-                                                have ? ow0 + offw : -65536, have ? oh0 + offh : -65536, n0);
-                                    tma_load_3d(b0 + b_slot * b_slot_bytes + (uint32_t)in_slot * b_bytes, maps + 4, full_b + 8u * b_slot, ch * BK, co0,
-                                                a * kw + b);
-                                    if (++in_slot == cps || tap_u + 1 == n_chunks * n_taps) {
-                                        in_slot = 0;
-                                        if (++a_slot == (uint32_t)SA) { a_slot = 0; a_phase ^= 1u; }
-                                        if (++b_slot == (uint32_t)SB) { b_slot = 0; b_phase ^= 1u; }
-                                    }
-                                }
+                        // one activation and one weight box per (channel chunk, tap), `cps` of them per entry
+                        const int steps = n_chunks * n_taps;
+                        int ch = 0, ta = 0, tb = 0;
+                        int offh = first_offh, offw = first_offw, mi = first_mi;
+                        bool have = first_have;
+                        for (int st = 0; st < steps && !fail; st += cps) {
+                            const uint32_t g = (uint32_t)min(cps, steps - st);
+                            uint32_t at = allocate(g * (kept ? a_sz : a_sz + b_sz), g * (kept ? a_bytes : a_bytes + b_bytes));
+                            if (!at) { fail = 1; break; }
+                            uint32_t bt = at + g * a_sz;
+                            for (uint32_t u = 0; u < g; ++u, at += a_sz, bt += b_sz) {
+                                tma_load_4d(at, maps + mi, full_bar, ch * BK, have ? ow0 + offw : -65536, have ? oh0 + offh : -65536, n0);
+                                if (!kept) tma_load_3d(bt, maps + 4, full_bar, ch * BK, co0, ta * kw + tb);
+                                if (n_taps == 1) { ++ch; continue; }
+                                // next tap (strides are 1 or 2 almost always: no division then)
+                                if (++tb == kw) { tb = 0; if (++ta == kh) { ta = 0; ++ch; } }
+                                const int qh = ta * dh - ph, qw = tb * dw - pw;
+                                offh = sh == 1 ? qh : (sh == 2 ? qh >> 1 : floor_div_i(qh, sh));
+                                offw = sw == 1 ? qw : (sw == 2 ? qw >> 1 : floor_div_i(qw, sw));
+                                mi = (qh - offh * sh) * sw + (qw - offw * sw);
+                                have = (amask >> mi) & 1;
                             }
                         }
                     }
+                    // the tile's output units, behind its operands: free (their previous contents are stored), and with
+                    // the residual's rows on their way where there is one
+                    for (int u = 0; u < units_n && !fail; ++u, ++uc) {
+                        const uint32_t sl = uc & (WF_UNITS - 1), gb = ugrant0 + 8u * sl;
+                        if (!mbar_wait_abortable(ufree0 + 8u * sl, ((uc / WF_UNITS) & 1u) ^ 1u, abort_flag)) { fail = 1; break; }
+                        if (res_map >= 0) {
+                            mbar_expect_tx(gb, res_bytes);
+                            tma_load_4d(unit0 + sl * unit_bytes, P.maps + res_map, gb, co0 + (u << sub_log), ow0, oh0, n0);
+                        } else {
+                            mbar_arrive(gb);
+                        }
                     }
                     if (fail) atomicOr(P.status, 0x1u);
                     tr(item, 2);
@@ -538,17 +592,13 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
             int sidx = -1;
             int kind = -1, mode = 0, n_chunks = 1, n_taps = 1, tbx = 1, kw = 1, dh = 1, dw = 1, p_log = 0, ksteps = 1;
             uint32_t idesc = 0, desc_hi = 0, row_bytes = 0, tap_bytes = 0;
-            uint32_t a_slot = 0, a_phase = 0, b_slot = 0, b_phase = 0, cnt = 0;
+            uint32_t cnt = 0, a_sz = 0, b_sz = 0, a_bytes = 0, b_bytes = 0, keep_bytes = 0;
             bool fail = false, row3x64 = false;
-            bool w_kept = false;                               // weights kept in ring slots w_first .. w_first + w_n - 1 for key w_key
-            long long w_key = -1;
-            uint32_t w_first = 0, w_n = 0;
-            int map_base = 0, nblk = 1, cps = 1;               // nblk: weight boxes per channel chunk; cps: chunks per ring slot
-            uint32_t a_bytes = 0, b_bytes = 0;
+            int map_base = 0, cps = 1;
+            // the ring as the loader fills it: the next entry's place and number; the kept weights' loads so far
+            uint32_t ring_lim = ring_bytes, pos = 0, n_used = 0, n_full = 0, n_group = 0, w_uses = 0, slab_sl = 0;
+            long long cut_key = 0;
             uint32_t tap16 = 0, step_w16 = 0, step_h16 = 0;    // descriptor start-field steps: next tap's weights, next filter column / row
-#ifdef LOP_WF_TRACE
-            long long dbg_c0 = 0, dbg_fence = 0, dbg_mma = 0;
-#endif
             for (; item < NI && !fail; item += G) {
                 const int4 nxt = item + G < NI ? __ldg(&P.items[item + G]) : zero4;
                 if (rec_stage(cur) != sidx) {
@@ -558,7 +608,6 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                     n_chunks = __ldg(&sp->n_chunks); n_taps = __ldg(&sp->n_taps); tbx = __ldg(&sp->tb);
                     kw = __ldg(&sp->kw); dh = __ldg(&sp->dh); dw = __ldg(&sp->dw); p_log = __ldg(&sp->p_log);
                     map_base = __ldg(&sp->map_base);
-                    nblk = (n_taps + tbx - 1) / tbx;
                     ksteps = __ldg(&sp->BK) / 16;
                     idesc = __ldg(&sp->idesc);
                     desc_hi = ((__ldg(&sp->sbo_bytes) >> 4) & 0x3FFFu) | (1u << 14) | (__ldg(&sp->layout_code) << 29);
@@ -569,6 +618,8 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                     step_h16 = ((uint32_t)(dh << p_log) * row_bytes) >> 4;
                     row3x64 = mode == WF_SLAB && n_taps == 9 && kw == 3 && tbx == 3 && ksteps == 4 && dw == 1;
                     a_bytes = __ldg(&sp->a_bytes); b_bytes = __ldg(&sp->b_bytes);
+                    a_sz = (a_bytes + 1023u) & ~1023u; b_sz = (b_bytes + 1023u) & ~1023u;
+                    keep_bytes = (uint32_t)__ldg(&sp->keep_bytes);
                     cps = __ldg(&sp->cps);
                 }
                 if (kind == WF_CONV) {
@@ -578,132 +629,139 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                     tr(item, 3);
                     const uint32_t acc = tmem_base + buf * 256u;
                     uint32_t accumulate = 0;
-                    // kept weights (see the loader): used in place by tiles with the same key, freed -- once the MMAs
-                    // that read them are done -- when a tile with another key comes up
-                    // (this thread issues every MMA of the CTA and is bound by its own instruction latencies: no division
-                    // or modulo in these loops)
-                    const uint32_t n_boxes = (uint32_t)(n_chunks * nblk);
-                    const long long wkey = (long long)map_base * 65536 + rec_cout(cur);
-                    const bool can_keep = mode == WF_SLAB && n_boxes <= (uint32_t)SB;
-                    const bool reuse_w = w_kept && can_keep && wkey == w_key;
-                    if (w_kept && !reuse_w) {
-                        for (uint32_t i = 0, sl = w_first; i < w_n; ++i) {
-                            umma_commit(empty_b + 8u * sl);
-                            if (++sl == (uint32_t)SB) sl = 0;
+                    // (this thread issues every MMA of the CTA, some 60 cycles each whatever N up to 128, and every other
+                    // instruction it executes is a bubble of the tensor pipe: addresses are ready before the waits, no
+                    // division or modulo)
+                    const bool kept = keep_bytes != 0;
+                    const long long key = kept ? (((long long)map_base << 16) | rec_cout(cur)) + 1 : (mode == WF_SLAB ? -(long long)a_sz : 0);
+                    if (key != cut_key) {                      // see the loader: the ring is cut anew
+                        if (cut_key > 0) umma_commit(wempty);  // the MMAs so far were the kept weights' last users
+                        cut_key = key;
+                        ring_lim = ring_bytes - (key < 0 ? 2u * a_sz : keep_bytes);
+                        pos = 0;
+                        if (kept) {
+                            if (!mbar_wait_abortable(wfull, w_uses & 1u, abort_flag)) { fail = true; break; }
+                            ++w_uses;
                         }
-                        w_kept = false;
                     }
-                    if (!reuse_w && can_keep) { w_kept = true; w_key = wkey; w_first = b_slot; w_n = n_boxes; }
-                    uint32_t ws = w_first;                                  // kept box of the current (chunk, tap block)
-                    if (reuse_w && row3x64 && n_chunks == 1) {
-                        // the common tile of a 3x3 / 64-channel layer with its weights in place: 36 MMAs, nothing between
-                        // them but the start addresses of the three filter rows
-                        if (!mbar_wait_abortable(full_a + 8u * a_slot, a_phase, abort_flag)) { fail = true; break; }
-                        tr(item, 13);
+                    uint32_t kept_at = ring0 + ring_lim;       // next kept weight box
+                    // the next entry; its empty barrier goes to `eb`
+                    uint32_t eb = 0;
+                    auto next_place = [&](uint32_t size) -> uint32_t {
+                        if (pos + size > ring_lim) pos = 0;
+                        const uint32_t at = ring0 + pos;
+                        eb = empty0 + 8u * (n_used & (WF_ENTRIES - 1));
+                        ++n_used; pos += size;
+                        return at;
+                    };
+                    // waits until the next entry / box group is loaded
+                    auto next_full = [&]() {
+                        if (!mbar_wait_abortable(full0 + 8u * (n_full & (WF_ENTRIES - 1)), (n_full / WF_ENTRIES) & 1u, abort_flag)) return false;
+                        ++n_full;
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        const uint32_t la = (((a0 + a_slot * a_slot_bytes) & 0x3FFFFu) >> 4) | (1u << 16);
-                        const uint32_t row16 = (uint32_t)(dh << p_log) * 8u;          // one filter row further down the slab, in 16-byte units
-                        const uint32_t s0 = w_first, s1 = s0 + 1 == (uint32_t)SB ? 0u : s0 + 1, s2 = s1 + 1 == (uint32_t)SB ? 0u : s1 + 1;
-                        mma_row3x64(acc, la, (((b0 + s0 * b_slot_bytes) & 0x3FFFFu) >> 4) | (1u << 16), tap_bytes >> 4, desc_hi, idesc, accumulate);
-                        mma_row3x64(acc, la + row16, (((b0 + s1 * b_slot_bytes) & 0x3FFFFu) >> 4) | (1u << 16), tap_bytes >> 4, desc_hi, idesc, accumulate);
-                        mma_row3x64(acc, la + 2u * row16, (((b0 + s2 * b_slot_bytes) & 0x3FFFFu) >> 4) | (1u << 16), tap_bytes >> 4, desc_hi, idesc, accumulate);
-                        umma_commit(empty_a + 8u * a_slot);
-                        if (++a_slot == (uint32_t)SA) { a_slot = 0; a_phase ^= 1u; }
-                    } else if (cps > 1 && mode == WF_SLAB) {
-                        for (int ch = 0; ch < n_chunks; ch += cps) {
-                            const int g = min(cps, n_chunks - ch);
-                            if (!mbar_wait_abortable(full_a + 8u * a_slot, a_phase, abort_flag) ||
-                                !mbar_wait_abortable(full_b + 8u * b_slot, b_phase, abort_flag)) { fail = true; break; }
+                        return true;
+                    };
+                    auto next_group = [&]() {
+                        if (!mbar_wait_abortable(gfull0 + 8u * (n_group & (WF_GROUPS - 1)), (n_group / WF_GROUPS) & 1u, abort_flag)) return false;
+                        ++n_group;
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        return true;
+                    };
+                    if (row3x64 && !kept && (cps == 3 || cps == 1)) {
+                        // the common 3x3 chunk, its three weight boxes behind one barrier or behind one each: nothing but the
+                        // commits stands between the MMAs (the general loop below spends some 330 cycles of this thread's
+                        // arithmetic per box, half of a box's MMAs: 3700 -> 2614 cycles per 64-channel chunk)
+                        for (int ch = 0; ch < n_chunks; ++ch) {
+                            const uint32_t la = desc_lo(ring0 + ring_lim + slab_sl * a_sz);
+                            const uint32_t lb0 = desc_lo(next_place(b_sz)), e0 = eb, lb1 = desc_lo(next_place(b_sz)), e1 = eb, lb2 = desc_lo(next_place(b_sz)), e2 = eb;
+                            slab_sl ^= 1u;
+                            if (!next_group()) { fail = true; break; }
+                            if (ch == 0) { tr(item, 13); tr(item, 14); }
+                            mma_row3x64(acc, la, lb0, tap16, desc_hi, idesc, accumulate);
+                            umma_commit(e0);
+                            if (cps == 1 && !next_group()) { fail = true; break; }
+                            mma_row3x64(acc, la + step_h16, lb1, tap16, desc_hi, idesc, accumulate);
+                            umma_commit(e1);
+                            if (cps == 1 && !next_group()) { fail = true; break; }
+                            mma_row3x64(acc, la + 2u * step_h16, lb2, tap16, desc_hi, idesc, accumulate);
+                            umma_commit(e2);
+                        }
+                    } else if (row3x64 && kept) {
+                        // the same with the weights in place
+                        const uint32_t b16 = b_sz >> 4;
+                        for (int ch = 0; ch < n_chunks; ++ch, kept_at += 3u * b_sz) {
+                            const uint32_t la = desc_lo(next_place(a_sz)), lb0 = desc_lo(kept_at);
+                            if (!next_full()) { fail = true; break; }
+                            if (ch == 0) { tr(item, 13); tr(item, 14); }
+                            mma_row3x64(acc, la, lb0, tap16, desc_hi, idesc, accumulate);
+                            mma_row3x64(acc, la + step_h16, lb0 + b16, tap16, desc_hi, idesc, accumulate);
+                            mma_row3x64(acc, la + 2u * step_h16, lb0 + 2u * b16, tap16, desc_hi, idesc, accumulate);
+                            umma_commit(eb);
+                        }
+                    } else if (mode == WF_SLAB) {
+                        for (int ch = 0; ch < n_chunks && !fail; ++ch) {
+                            uint32_t sa, a_empty = 0;
+                            if (kept) {
+                                sa = next_place(a_sz);
+                                a_empty = eb;
+                                if (!next_full()) { fail = true; break; }
+                            } else {
+                                if (!next_group()) { fail = true; break; }
+                                sa = ring0 + ring_lim + slab_sl * a_sz;
+                                slab_sl ^= 1u;
+                            }
                             if (ch == 0) tr(item, 13);
-                            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                            uint32_t la = desc_lo(a0 + a_slot * a_slot_bytes), lb = desc_lo(b0 + b_slot * b_slot_bytes);
-                            for (int u = 0; u < g; ++u, la += a_bytes >> 4, lb += b_bytes >> 4) mma_ksteps_f<4>(acc, la, lb, desc_hi, idesc, accumulate);
-                            umma_commit(empty_a + 8u * a_slot);
-                            umma_commit(empty_b + 8u * b_slot);
-                            if (++a_slot == (uint32_t)SA) { a_slot = 0; a_phase ^= 1u; }
-                            if (++b_slot == (uint32_t)SB) { b_slot = 0; b_phase ^= 1u; }
+                            // start field of the tap's activation operand: one pixel further per filter column, one slab row
+                            // further per filter row (kept incrementally)
+                            uint32_t la_row = desc_lo(sa), la = la_row;
+                            int tb = 0, in_group = 0;                        // filter column of tap t0, boxes used of the group
+                            for (int t0 = 0; t0 < n_taps; t0 += tbx) {
+                                uint32_t sb = kept_at;
+                                if (kept) {
+                                    kept_at += b_sz;
+                                } else {
+                                    if (in_group == cps) {
+                                        if (!next_group()) { fail = true; break; }
+                                        in_group = 0;
+                                    }
+                                    ++in_group;
+                                    sb = next_place(b_sz);
+                                }
+                                if (ch == 0 && t0 == 0) tr(item, 14);
+                                uint32_t lb = desc_lo(sb);
+                                const int t1 = min(t0 + tbx, n_taps);
+                                for (int t = t0; t < t1; ++t, lb += tap16) {
+                                    // tap (a, b): the same box, read (a*dh*P + b*dw) pixels further on
+                                    mma_tap_f(acc, la, lb, desc_hi, idesc, ksteps, accumulate);
+                                    la += step_w16;
+                                    if (++tb == kw) { tb = 0; la_row += step_h16; la = la_row; }
+                                }
+                                if (!kept) umma_commit(eb);
+                            }
+                            if (kept) umma_commit(a_empty);
                         }
                     } else {
-                    int tap_u = 0, in_slot = 0;                        // per-tap mode: boxes consumed so far, boxes used of the open slot
-                    for (int ch = 0; ch < n_chunks && !fail; ++ch) {
-                        if (mode == WF_SLAB) {
-                            if (!mbar_wait_abortable(full_a + 8u * a_slot, a_phase, abort_flag)) { fail = true; break; }
-                            if (ch == 0) tr(item, 13);
-                            const uint32_t sa = a0 + a_slot * a_slot_bytes;
-                            int ta = 0, tb = 0;                             // filter position of tap t0
-                            // start field of the tap's activation operand: one pixel further per filter column, one
-                            // slab row further per filter row (kept incrementally: this thread pays for every instruction)
-                            uint32_t la_row = desc_lo(sa), la = la_row;
-                            for (int t0 = 0; t0 < n_taps; t0 += tbx) {
-                                uint32_t bs = b_slot;
-                                if (reuse_w) {
-                                    bs = ws;
-                                    if (++ws == (uint32_t)SB) ws = 0;
-                                } else if (!mbar_wait_abortable(full_b + 8u * b_slot, b_phase, abort_flag)) { fail = true; break; }
-                                if (ch == 0 && t0 == 0) tr(item, 14);
-#ifdef LOP_WF_TRACE
-                                const long long c0 = clock64();
-                                if (t0 == 0) dbg_c0 = c0;
-#endif
-                                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#ifdef LOP_WF_TRACE
-                                const long long c1 = clock64();
-                                dbg_fence += c1 - c0;
-#endif
-                                const uint32_t sb = b0 + bs * b_slot_bytes;
-                                if (row3x64) {
-                                    // box = one row of a 3x3 filter: the slab row it starts at, then constants
-                                    const uint32_t pa = sa + (uint32_t)((ta * dh) << p_log) * 128u;
-                                    mma_row3x64(acc, ((pa & 0x3FFFFu) >> 4) | (1u << 16), ((sb & 0x3FFFFu) >> 4) | (1u << 16), tap_bytes >> 4,
-                                                desc_hi, idesc, accumulate);
-#ifdef LOP_WF_TRACE
-                                    dbg_mma += clock64() - c1;
-#endif
-                                    ++ta;
-                                } else {
-                                    const int t1 = min(t0 + tbx, n_taps);
-                                    uint32_t lb = desc_lo(sb);
-                                    for (int t = t0; t < t1; ++t, lb += tap16) {
-                                        // tap (ta, tb): the same box, read (ta*dh*P + tb*dw) pixels further on
-                                        mma_tap_f(acc, la, lb, desc_hi, idesc, ksteps, accumulate);
-                                        la += step_w16;
-                                        if (++tb == kw) { tb = 0; la_row += step_h16; la = la_row; }
-                                    }
-                                }
-                                if (!reuse_w) {
-                                    if (!can_keep) umma_commit(empty_b + 8u * b_slot);
-                                    if (++b_slot == (uint32_t)SB) { b_slot = 0; b_phase ^= 1u; }
-                                }
+                        const uint32_t a16 = a_sz >> 4, b16 = b_sz >> 4;
+                        uint32_t lbk = desc_lo(kept_at);
+                        for (int left = n_chunks * n_taps; left > 0; left -= cps) {
+                            const uint32_t g = (uint32_t)min(cps, left);
+                            const uint32_t at = next_place(g * (kept ? a_sz : a_sz + b_sz));
+                            uint32_t la = desc_lo(at), lb = kept ? lbk : desc_lo(at + g * a_sz);
+                            if (!next_full()) { fail = true; break; }
+                            if (left == n_chunks * n_taps) tr(item, 13);
+                            if (ksteps == 4) {
+                                mma_ksteps_f<4>(acc, la, lb, desc_hi, idesc, accumulate);
+                                if (g > 1) mma_ksteps_f<4>(acc, la + a16, lb + b16, desc_hi, idesc, accumulate);
+                                if (g > 2) mma_ksteps_f<4>(acc, la + 2u * a16, lb + 2u * b16, desc_hi, idesc, accumulate);
+                                if (g > 3) mma_ksteps_f<4>(acc, la + 3u * a16, lb + 3u * b16, desc_hi, idesc, accumulate);
+                            } else {
+                                for (uint32_t u = 0; u < g; ++u, la += a16, lb += b16) mma_tap_f(acc, la, lb, desc_hi, idesc, ksteps, accumulate);
                             }
-                            umma_commit(empty_a + 8u * a_slot);
-                            if (++a_slot == (uint32_t)SA) { a_slot = 0; a_phase ^= 1u; }
-                        } else {
-                            for (int t = 0; t < n_taps; ++t, ++tap_u) {
-                                if (in_slot == 0) {
-                                    if (!mbar_wait_abortable(full_a + 8u * a_slot, a_phase, abort_flag) ||
-                                        !mbar_wait_abortable(full_b + 8u * b_slot, b_phase, abort_flag)) { fail = true; break; }
-                                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                                }
-                                mma_tap(acc, a0 + a_slot * a_slot_bytes + (uint32_t)in_slot * a_bytes, b0 + b_slot * b_slot_bytes + (uint32_t)in_slot * b_bytes,
-                                        desc_hi, idesc, ksteps, accumulate);
-                                if (++in_slot == cps || tap_u + 1 == n_chunks * n_taps) {
-                                    in_slot = 0;
-                                    umma_commit(empty_a + 8u * a_slot);
-                                    umma_commit(empty_b + 8u * b_slot);
-                                    if (++a_slot == (uint32_t)SA) { a_slot = 0; a_phase ^= 1u; }
-                                    if (++b_slot == (uint32_t)SB) { b_slot = 0; b_phase ^= 1u; }
-                                }
-                            }
+                            umma_commit(eb);
+                            lbk += g * b16;
                         }
                     }
-                    }
                     if (fail) break;
-#ifdef LOP_WF_TRACE
-                    trv(item, 8, (unsigned long long)dbg_fence);
-                    trv(item, 9, (unsigned long long)dbg_mma);
-                    trv(item, 10, (unsigned long long)(clock64() - dbg_c0));
-                    dbg_fence = dbg_mma = 0;
-#endif
                     tr(item, 15);
                     umma_commit(accf0 + 8u * buf);
                     tr(item, 4);
@@ -724,21 +782,53 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
             // this thread waits for, so its fence orders them before the release increment of the counter.
             int item = blockIdx.x;
             int4 cur = item < NI ? __ldg(&P.items[item]) : zero4;
-            int sidx = -1, ctr_base = 0;
+            // A convolution's output units leave from here too, as bulk stores: this thread issues a unit's store as soon as
+            // the workers have finished it, hands the unit back when it has been read out, and waits for the stores'
+            // completion before the increment -- the workers are at the next tile by then.
+            int sidx = -1, ctr_base = 0, kind = -1, out_map = -1, sub_log = 6, units_n = 0, oh_lo = 0, p_log = 0, tr_log = 0, tw_valid = 0, BN = 0;
+            uint32_t uc = 0, k = 0;
             bool fail = false;
-            for (uint32_t k = 0; item < NI; item += G, ++k) {
+            for (; item < NI; item += G) {
                 const int4 nxt = item + G < NI ? __ldg(&P.items[item + G]) : zero4;
                 if (rec_stage(cur) != sidx) {
                     sidx = rec_stage(cur);
-                    ctr_base = __ldg(&P.stages[sidx].ctr_base);
+                    const WfStage *sp = &P.stages[sidx];
+                    ctr_base = __ldg(&sp->ctr_base); kind = __ldg(&sp->kind); out_map = __ldg(&sp->out_map);
+                    sub_log = __ldg(&sp->sub_log); oh_lo = __ldg(&sp->oh_lo); p_log = __ldg(&sp->p_log); tr_log = __ldg(&sp->tr_log);
+                    tw_valid = __ldg(&sp->tw_valid); BN = __ldg(&sp->BN);
+                    units_n = BN >> sub_log;
                 }
-                const uint32_t q = k % WF_PUBQ, round = k / WF_PUBQ;
-                if (!mbar_wait_abortable(pubf0 + 8u * q, round & 1u, abort_flag)) { fail = !*abort_flag; break; }
-                __threadfence();
-                atomicAdd(P.counters + ctr_base + rec_tr(cur), 1u);
-                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(pube0 + 8u * q) : "memory");
+                if (kind == WF_CONV && out_map >= 0) {
+                    const int ow0 = rec_tw(cur) * tw_valid, oh0 = oh_lo + (rec_tr(cur) << tr_log), n0 = rec_tn(cur) * (128 >> (p_log + tr_log));
+                    for (int u = 0; u < units_n; ++u) {
+                        const uint32_t sl = (uc + u) & (WF_UNITS - 1);
+                        if (!mbar_wait_abortable(uready0 + 8u * sl, ((uc + u) / WF_UNITS) & 1u, abort_flag)) { fail = true; break; }
+                        tma_store_4d(P.maps + out_map, unit0 + sl * unit_bytes, rec_cout(cur) * BN + (u << sub_log), ow0, oh0, n0);
+                        bulk_commit();
+                        if (units_n > WF_UNITS) {              // more units than places: each goes back before the next is needed
+                            bulk_wait_read();
+                            mbar_arrive(ufree0 + 8u * sl);
+                        }
+                    }
+                    bulk_wait_read();
+                    if (fail) { fail = !*abort_flag; break; }
+                    for (int u = 0; u < units_n && units_n <= WF_UNITS; ++u) mbar_arrive(ufree0 + 8u * ((uc + u) & (WF_UNITS - 1)));
+                    uc += units_n;
+                    bulk_wait_all();
+                    __threadfence();
+                    atomicAdd(P.counters + ctr_base + rec_tr(cur), 1u);
+                } else {
+                    if (kind == WF_CONV) uc += units_n;            // stored, and handed back, by the workers
+                    const uint32_t q = k % WF_PUBQ, round = k / WF_PUBQ;
+                    if (!mbar_wait_abortable(pubf0 + 8u * q, round & 1u, abort_flag)) { fail = !*abort_flag; break; }
+                    __threadfence();
+                    atomicAdd(P.counters + ctr_base + rec_tr(cur), 1u);
+                    mbar_arrive(pube0 + 8u * q);
+                    ++k;
+                }
                 cur = nxt;
             }
+            bulk_wait_all();
             if (fail) {
                 atomicOr(P.status, 0x8u);
                 atomicExch(P.counters + 2, 1u);
@@ -795,7 +885,9 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
         int4 nxt = item + G < NI ? __ldg(&P.items[item + G]) : zero4;
         int2 dep_cur = (warp == WF_FIRST_WORKER && item < NI && lane < rec_ndep(cur)) ? __ldg(&P.deps[rec_dep0(cur) + lane]) : make_int2(0, 0);
         int sidx = -1;
-        uint32_t cnt = 0, done_items = 0;
+        uint32_t cnt = 0, done_items = 0, uc = 0;
+        int sub_log = 6, units_n = 0;
+        bool bulk_out = false;
         int kind = -1, oh_lo = 0, oh_hi = 0, p_log = 0, tr_log = 0, tw_valid = 0, BN = 0, gather_direct = 0, fuse_pool = 0, pool_Ho = 0, pool_Wo = 0;
         int N = 0, Hin = 0, Win = 0, Cin = 0, Ho = 0, Wo = 0, Cout = 0, kh = 1, kw = 1, sh = 1, sw = 1, ph = 0, pw = 0, dh = 1,
             dw = 1, act = 0, res_pos = 0;
@@ -819,6 +911,8 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 act = __ldg(&sp->act); res_pos = __ldg(&sp->res_pos);
                 fuse_pool = __ldg(&sp->fuse_pool); pool_Ho = __ldg(&sp->pool_Ho); pool_Wo = __ldg(&sp->pool_Wo);
                 xin = ldg_ptr<const void *>(&sp->x);
+                sub_log = __ldg(&sp->sub_log); units_n = BN >> sub_log;
+                bulk_out = __ldg(&sp->out_map) >= 0;
                 resp = ldg_ptr<const void *>(&sp->res);
                 scale = ldg_ptr<const float *>(reinterpret_cast<const void *const *>(&sp->scale));
                 shift = ldg_ptr<const float *>(reinterpret_cast<const void *const *>(&sp->shift));
@@ -833,61 +927,54 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 const int ow = rec_tw(cur) * tw_valid + c;
                 const int oh = oh_lo + (tile_r << tr_log) + r;
                 const int n = rec_tn(cur) * (128 >> (p_log + tr_log)) + (m >> (p_log + tr_log));
-                const bool valid = c < tw_valid && ow < Wo && oh < oh_hi && n < N;
+                const bool staged = c < tw_valid;                      // the other anchors are the slab's halo gap
+                const bool valid = staged && ow < Wo && oh < oh_hi && n < N;
                 const int co0 = rec_cout(cur) * BN;
-                if (cgrp == 0) row_pix[m] = valid ? (((long long)n * Ho + oh) * Wo + ow) * Cout + co0 : -1LL;
-                if (fuse_pool && cgrp == 0 && !((r | c) & 1)) {
-                    // top-left anchor of a 2x2 window: where its maximum goes, if the whole window is inside the stage
-                    const int q = (((m >> (p_log + tr_log)) << (tr_log - 1)) + (r >> 1)) * ((1 << p_log) >> 1) + (c >> 1);
-                    const bool ok = valid && c + 1 < tw_valid && ow + 1 < Wo && oh + 1 < oh_hi;
-                    pool_pix[q] = ok ? (((long long)n * pool_Ho + (oh >> 1)) * pool_Wo + (ow >> 1)) * Cout + co0 : -1LL;
-                }
-                const float *t_scale = s_scale + 128 * buf, *t_shift = s_shift + 128 * buf;   // filled by warp 0 a tile ahead
-                const int cpr = BN >> 3;                               // 16-byte chunks per staged row
-                const int cpr_log = (cpr & (cpr - 1)) == 0 ? 31 - __clz(cpr) : -1;
-                const uint32_t row_stride = (uint32_t)BN * 2u;
-                const int swz = (cpr & 7) == 0 ? 7 : 0;                // chunk position = chunk ^ (row & 7): conflict-free columns
-                __nv_bfloat16 *y = static_cast<__nv_bfloat16 *>(yout);
-                // the loader warp arrives here once it has seen the tile's producers (the residual's included): the residual
-                // tile is fetched now, under the operands' transfer and the main loop
-                if (!mbar_wait_abortable(ssf0 + 8u * buf, (cnt >> 1) & 1u, abort_flag)) *epi_fail = 1;
-                if (resp) {
-                    epi_bar();                                         // row_pix of every anchor is written
-                    // residual tile -> staging, coalesced; produced inside this launch by other SMs: read through L2
-                    const __nv_bfloat16 *res = static_cast<const __nv_bfloat16 *>(resp);
-#pragma unroll 4
-                    for (int idx = tid; idx < 128 * cpr; idx += EPI_THREADS) {
-                        const int row = cpr_log >= 0 ? idx >> cpr_log : idx / cpr, j = idx - row * cpr;
-                        const long long rp = row_pix[row];
-                        if (rp >= 0)
-                            *reinterpret_cast<uint4 *>(stg + row * row_stride + ((j ^ (row & swz)) << 4)) =
-                                __ldcg(reinterpret_cast<const uint4 *>(res + rp) + j);
+                const int trows = 1 << tr_log;
+                // staged rows are packed: image, row, column below tw_valid (the box of a bulk load or store)
+                const int srow = (((m >> (p_log + tr_log)) << tr_log) + r) * tw_valid + c;
+                if (!bulk_out) {
+                    if (cgrp == 0 && staged) row_pix[srow] = valid ? (((long long)n * Ho + oh) * Wo + ow) * Cout + co0 : -1LL;
+                    if (fuse_pool && cgrp == 0 && !((r | c) & 1)) {
+                        // top-left anchor of a 2x2 window: where its maximum goes, if the whole window is inside the stage
+                        const int q = (((m >> (p_log + tr_log)) << (tr_log - 1)) + (r >> 1)) * ((1 << p_log) >> 1) + (c >> 1);
+                        const bool ok = valid && c + 1 < tw_valid && ow + 1 < Wo && oh + 1 < oh_hi;
+                        pool_pix[q] = ok ? (((long long)n * pool_Ho + (oh >> 1)) * pool_Wo + (ow >> 1)) * Cout + co0 : -1LL;
                     }
                 }
+                const float *t_scale = s_scale + 128 * buf, *t_shift = s_shift + 128 * buf;   // filled by warp 0 a tile ahead
+                const uint32_t row_stride = 2u << sub_log;             // bytes of a staged row in a unit
+                // position of a 16-byte chunk in a staged row: the swizzle of the unit's tensor maps (128, 64 or 32 bytes)
+                const int swz = sub_log == 6 ? srow & 7 : (sub_log == 5 ? (srow >> 1) & 3 : (srow >> 2) & 1);
+                if (!mbar_wait_abortable(ssf0 + 8u * buf, (cnt >> 1) & 1u, abort_flag)) *epi_fail = 1;
                 if (!mbar_wait_abortable(accf0 + 8u * buf, (cnt >> 1) & 1u, abort_flag)) *epi_fail = 1;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 if (tid == 0) tr(item, 5);
-                if (resp) epi_bar();                                   // the staged residual tile is complete
-                {
-                    const uint32_t acc = tmem_base + buf * 256u + ((uint32_t)(g * 32) << 16);
-                    uint8_t *my_row = stg + m * row_stride;
-                    for (int j = 16 * cgrp; j < BN; j += 16 * COL_GROUPS) {
+                for (int u = 0; u < units_n; ++u) {
+                    const uint32_t sl = (uc + u) & (WF_UNITS - 1);
+                    // the unit is free, and the residual's rows are in it where the layer has one
+                    if (!mbar_wait_abortable(ugrant0 + 8u * sl, ((uc + u) / WF_UNITS) & 1u, abort_flag)) *epi_fail = 1;
+                    uint8_t *my_row = units + sl * unit_bytes + srow * row_stride;
+                    const uint32_t acc = tmem_base + buf * 256u + ((uint32_t)(g * 32) << 16) + ((uint32_t)u << sub_log);
+                    // the two warps of a TMEM lane group take alternate 16-column chunks
+                    for (int j = 16 * cgrp; j < (1 << sub_log); j += 16 * COL_GROUPS) {
                         uint32_t rr[16];
                         tmem_ld16(acc + (uint32_t)j, rr);
                         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                        if (!valid) continue;
+                        if (!staged) continue;
+                        const int ct = (u << sub_log) + j;             // channel inside the tile
                         float v[16];
 #pragma unroll
                         for (int i = 0; i < 16; i += 4) {                  // 16-byte broadcast reads of the tile's scale / shift
-                            const float4 sc = *reinterpret_cast<const float4 *>(t_scale + j + i);
-                            const float4 sf = *reinterpret_cast<const float4 *>(t_shift + j + i);
+                            const float4 sc = *reinterpret_cast<const float4 *>(t_scale + ct + i);
+                            const float4 sf = *reinterpret_cast<const float4 *>(t_shift + ct + i);
                             v[i] = fmaf(sc.x, __uint_as_float(rr[i]), sf.x);
                             v[i + 1] = fmaf(sc.y, __uint_as_float(rr[i + 1]), sf.y);
                             v[i + 2] = fmaf(sc.z, __uint_as_float(rr[i + 2]), sf.z);
                             v[i + 3] = fmaf(sc.w, __uint_as_float(rr[i + 3]), sf.w);
                         }
-                        uint4 *c0p = reinterpret_cast<uint4 *>(my_row + ((((j >> 3)) ^ (m & swz)) << 4));
-                        uint4 *c1p = reinterpret_cast<uint4 *>(my_row + ((((j >> 3) + 1) ^ (m & swz)) << 4));
+                        uint4 *c0p = reinterpret_cast<uint4 *>(my_row + (((j >> 3) ^ swz) << 4));
+                        uint4 *c1p = reinterpret_cast<uint4 *>(my_row + ((((j >> 3) + 1) ^ swz) << 4));
                         float rv[16];
                         if (resp) {
                             const uint4 q0 = *c0p, q1 = *c1p;
@@ -908,45 +995,57 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                         *c0p = make_uint4(o[0], o[1], o[2], o[3]);
                         *c1p = make_uint4(o[4], o[5], o[6], o[7]);
                     }
+                    // this warp's part of the unit is done (the publisher stores a bulk unit; the phase advances for all)
+                    if (bulk_out) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(uready0 + 8u * sl);
                 }
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 if (tid == 0) tr(item, 11);
-                epi_bar();                                             // accumulator drained, staging tile complete
+                epi_bar();                                             // accumulator drained, units complete
                 if (tid == 0) {
-                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(acce0 + 8u * buf) : "memory");
-                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(sse0 + 8u * buf) : "memory");
+                    mbar_arrive(acce0 + 8u * buf);
+                    mbar_arrive(sse0 + 8u * buf);
                 }
                 ++cnt;
-                if (!*epi_fail && fuse_pool) {
-                    // 2x2 windows of staged rows -> their maxima (exact in bf16) -> the pooled tensor, 16 bytes per thread
-                    const int P_ = 1 << p_log, half_p = P_ >> 1, half_tr = (1 << tr_log) >> 1;
-                    for (int idx = tid; idx < 32 * cpr; idx += EPI_THREADS) {
-                        const int q = cpr_log >= 0 ? idx >> cpr_log : idx / cpr, j = idx - q * cpr;
-                        const long long pp = pool_pix[q];
-                        if (pp < 0) continue;
-                        const int pc = q % half_p, t = q / half_p;
-                        const int m0 = ((t / half_tr) << (p_log + tr_log)) + ((2 * (t % half_tr)) << p_log) + 2 * pc;
-                        const int rows4[4] = {m0, m0 + 1, m0 + P_, m0 + P_ + 1};
-                        uint4 acc4 = *reinterpret_cast<const uint4 *>(stg + rows4[0] * row_stride + ((j ^ (rows4[0] & swz)) << 4));
+                if (!bulk_out && !*epi_fail) {
+                    __nv_bfloat16 *y = static_cast<__nv_bfloat16 *>(yout);
+                    const int cpr_log = sub_log - 3, rows_n = (128 >> p_log) * tw_valid;     // 16-byte chunks per staged row, staged rows
+                    auto chunk = [&](int u, int row, int j) {          // chunk j of a staged row of unit u
+                        const int sw = sub_log == 6 ? row & 7 : (sub_log == 5 ? (row >> 1) & 3 : (row >> 2) & 1);
+                        return *reinterpret_cast<const uint4 *>(units + ((uc + u) & (WF_UNITS - 1)) * unit_bytes + row * row_stride + ((j ^ sw) << 4));
+                    };
+                    for (int u = 0; u < units_n; ++u) {
+                        if (fuse_pool) {
+                            // 2x2 windows of staged rows -> their maxima (exact in bf16) -> the pooled tensor, 16 bytes per thread
+                            const int half_p = (1 << p_log) >> 1, half_tr = trows >> 1;
+                            for (int idx = tid; idx < 32 << cpr_log; idx += EPI_THREADS) {
+                                const int q = idx >> cpr_log, j = idx - (q << cpr_log);
+                                const long long pp = pool_pix[q];
+                                if (pp < 0) continue;
+                                const int pc = q % half_p, t = q / half_p;
+                                const int s0 = (((t / half_tr) << tr_log) + 2 * (t % half_tr)) * tw_valid + 2 * pc;
+                                const int rows4[4] = {s0, s0 + 1, s0 + tw_valid, s0 + tw_valid + 1};
+                                uint4 acc4 = chunk(u, rows4[0], j);
 #pragma unroll
-                        for (int k = 1; k < 4; ++k) {
-                            const uint4 v4 = *reinterpret_cast<const uint4 *>(stg + rows4[k] * row_stride + ((j ^ (rows4[k] & swz)) << 4));
-                            __nv_bfloat162 *pa = reinterpret_cast<__nv_bfloat162 *>(&acc4);
-                            const __nv_bfloat162 *pv = reinterpret_cast<const __nv_bfloat162 *>(&v4);
+                                for (int k = 1; k < 4; ++k) {
+                                    const uint4 v4 = chunk(u, rows4[k], j);
+                                    __nv_bfloat162 *pa = reinterpret_cast<__nv_bfloat162 *>(&acc4);
+                                    const __nv_bfloat162 *pv = reinterpret_cast<const __nv_bfloat162 *>(&v4);
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) pa[e] = __hmax2(pa[e], pv[e]);
-                        }
-                        *(reinterpret_cast<uint4 *>(y + pp) + j) = acc4;
-                    }
-                } else if (!*epi_fail) {
-                    // staged rows -> global: consecutive threads write consecutive 16 bytes of a pixel's channels
+                                    for (int e = 0; e < 4; ++e) pa[e] = __hmax2(pa[e], pv[e]);
+                                }
+                                *(reinterpret_cast<uint4 *>(y + pp) + (u << cpr_log) + j) = acc4;
+                            }
+                        } else {
+                            // staged rows -> global: consecutive threads write consecutive 16 bytes of a pixel's channels
 #pragma unroll 4
-                    for (int idx = tid; idx < 128 * cpr; idx += EPI_THREADS) {
-                        const int row = cpr_log >= 0 ? idx >> cpr_log : idx / cpr, j = idx - row * cpr;
-                        const long long rp = row_pix[row];
-                        if (rp >= 0)
-                            *(reinterpret_cast<uint4 *>(y + rp) + j) =
-                                *reinterpret_cast<const uint4 *>(stg + row * row_stride + ((j ^ (row & swz)) << 4));
+                            for (int idx = tid; idx < rows_n << cpr_log; idx += EPI_THREADS) {
+                                const int row = idx >> cpr_log, j = idx - (row << cpr_log);
+                                const long long rp = row_pix[row];
+                                if (rp >= 0) *(reinterpret_cast<uint4 *>(y + rp) + (u << cpr_log) + j) = chunk(u, row, j);
+                            }
+                        }
                     }
                 }
                 if (tid == 0) tr(item, 12);
@@ -1118,15 +1217,23 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 }
                 break;
             }
-            if (tid == 0) {
-                // hand the item to the publisher warp, which fences and increments the row group's counter while
-                // the workers go on; it may lag WF_PUBQ items behind
-                const uint32_t q = done_items % WF_PUBQ, round = done_items / WF_PUBQ;
-                if (!mbar_wait_abortable(pube0 + 8u * q, (round & 1u) ^ 1u, abort_flag)) *epi_fail = 1;
-                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(pubf0 + 8u * q) : "memory");
-                tr(item, 6);
+            const bool stored_here = kind != WF_CONV || !bulk_out;
+            if (kind == WF_CONV) {
+                if (stored_here && tid == 0)
+                    for (int u = 0; u < units_n; ++u) mbar_arrive(ufree0 + 8u * ((uc + u) & (WF_UNITS - 1)));
+                uc += units_n;
             }
-            ++done_items;
+            if (stored_here) {
+                if (tid == 0) {
+                    // hand the item to the publisher warp, which fences and increments the row group's counter while
+                    // the workers go on; it may lag WF_PUBQ items behind
+                    const uint32_t q = done_items % WF_PUBQ, round = done_items / WF_PUBQ;
+                    if (!mbar_wait_abortable(pube0 + 8u * q, (round & 1u) ^ 1u, abort_flag)) *epi_fail = 1;
+                    mbar_arrive(pubf0 + 8u * q);
+                }
+                ++done_items;
+            }
+            if (tid == 0) tr(item, 6);
             cur = nxt; dep_cur = dep_nxt; nxt = nn;
         }
     }
@@ -1185,8 +1292,7 @@ extern "C" int lop_debug_trace_copy(void *host, size_t bytes, int clear)
 
 size_t wavefront_smem_bytes(const WfParams &p)
 {
-    return 1024 + (size_t)p.sa * p.a_slot_bytes + (size_t)p.sb * p.b_slot_bytes + p.stg_bytes + 8 * (size_t)(2 * p.sa + 2 * p.sb + 4 + 2 * WF_PUBQ + 4) + 64 +
-           2 * 256 * sizeof(float) + (128 + 32) * sizeof(long long) + 64;
+    return 1024 + (size_t)p.ring_bytes + (size_t)WF_UNITS * p.unit_bytes + p.simt_bytes + WF_FIXED_SMEM;
 }
 
 namespace {

@@ -23,8 +23,8 @@ enum WfKind { WF_GATHER = 0, WF_CONV = 1, WF_POOL = 2, WF_FETCH = 3, WF_DWCONV =
 //   WF_SLAB  one activation box per channel chunk: the output tile's receptive window (tile plus halo),
 //            laid out in shared memory as rows of P pixels; every filter tap is the same box read at a
 //            shifted start address.  Weights arrive as boxes of several taps.
-//   WF_TAP   one activation box and one weight box per (channel chunk, tap): strided windows and
-//            channel chunks narrower than 64.
+//   WF_TAP   one activation box and one weight box per (channel chunk, tap): pointwise layers, strided
+//            windows and channel chunks narrower than 64.
 enum WfMode { WF_SLAB = 0, WF_TAP = 1 };
 
 // One (band, layer) stage: rows [oh_lo, oh_hi) of a bound operator.
@@ -51,13 +51,16 @@ struct WfStage {
     // fuse_pool: the convolution's only consumer is a 2x2 stride-2 max pooling; the tile's epilogue takes the
     // maximum of each 2x2 window of staged rows and writes the pooled tensor [N, pool_Ho, pool_Wo, Cout] instead
     int fuse_pool, pool_Ho, pool_Wo;
-    // cps > 1: a pointwise stage with a long walk over K puts `cps` consecutive channel chunks, a per-tap stage `cps`
-    // consecutive taps, into one ring slot behind one barrier pair (activation boxes in the activation ring, weight
-    // boxes in the weight ring), so that more bytes are on their way at a time: such a walk is bound by the loads'
-    // latency, a few slots deep, not by their rate
+    // per-tap mode: `cps` consecutive (chunk, tap) steps share one ring entry and its barrier pair; slab mode: `cps` weight
+    // boxes of a chunk (the first group with the chunk's activation box) share one full barrier
     int cps;
     const void *w_taps;       // depth-wise stage: the filters as [tap][channel] bf16
-    int pad_[10];
+    // the tile's output leaves shared memory as `BN / sub` units of `sub` channels (64, 32 or 16)
+    int sub_log;
+    int out_map;              // tensor map of the output's rows below oh_hi (a unit is one bulk store), or -1: the workers store it
+    int res_map;              // tensor map of the residual (a unit is one bulk load), or -1
+    int keep_bytes;           // > 0: a tile's weights stay in shared memory (this many bytes at the ring's end) from tile to tile
+    int pad_[6];
 };
 static_assert(sizeof(WfStage) == 256, "WfStage layout");
 
@@ -73,8 +76,9 @@ struct WfParams {
     int flag_base, n_flags;
     unsigned *status;
     int n_stages, n_items;
-    int sa, sb;               // slots of the activation / weight ring
-    uint32_t a_slot_bytes, b_slot_bytes, stg_bytes;
+    uint32_t ring_bytes;      // operand ring
+    uint32_t unit_bytes;      // one of the WF_UNITS output units in flight between the workers and the bulk stores
+    uint32_t simt_bytes;      // scratch of the gather and depth-wise items
     // In-kernel input transfer (Sec. IV-B transmission, done by the kernel itself): every CTA has one more warp that
     // walks this list round-robin; entry j copies z bytes at byte offset (x | y << 32) from fetch_src (host memory
     // the device can address) to fetch_dst and then increments counters[w].  At most fetch_window entries are in
@@ -93,6 +97,10 @@ struct WfParams {
 constexpr int WF_WORKER_WARPS = LOP_WF_WORKER_WARPS;      // epilogue / SIMT warps (a multiple of 4)
 constexpr int WF_FIRST_WORKER = 3;                         // warps 0..2: loader, MMA issuer, publisher
 constexpr int WF_THREADS = 32 * (WF_FIRST_WORKER + WF_WORKER_WARPS);
+constexpr int WF_ENTRIES = 16;                             // operand ring entries in flight at most (a power of two)
+constexpr int WF_GROUPS = 8;                               // slab mode: box groups in flight at most (a power of two)
+constexpr int WF_UNITS = 4;                                // output units in flight (a power of two)
+constexpr uint32_t WF_FIXED_SMEM = 4096;                  // barriers, scale / shift and pixel tables
 constexpr int WF_PUBQ = 4;                                 // finished items the publisher may lag behind the workers
 constexpr int WF_CTR_FIRST = 4;
 constexpr int WF_MAX_DEPS = 4095;

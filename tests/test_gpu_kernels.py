@@ -1,10 +1,11 @@
 """Kernel variants and dispatch branches at the sizes where they can go wrong, against the CPU oracle.  Needs a B200."""
+import numpy as np
 import pytest
 import torch
 
 import lop_inputs as li
 import paper_2507_05829_b200 as lop
-from lop_inputs.workloads import conv
+from lop_inputs.workloads import Segment, Workload, conv
 from oracle import chain as ochain
 from paper_2507_05829_b200.chain import DeviceChain, to_host_f32
 from test_gpu_parity import TOL, check_workload, one_layer, rel_err
@@ -70,3 +71,37 @@ def test_one_launch_brings_the_input_of_a_per_layer_plan(N, H, W, C, dtype, band
     torch.cuda.synchronize()
     assert torch.equal(dc.staging[:, r.new_lo:r.out_hi].cpu(), x[:, r.new_lo:r.out_hi])
     assert torch.isnan(dc.staging[:, :r.new_lo].float()).all() and torch.isnan(dc.staging[:, r.out_hi:].float()).all()
+
+
+# ------------------------------------------------------------------------------------ operand ring and output units
+RING_CASES = [  # k, s, p, cin, cout, N, H, W, residual
+    (3, 1, 1, 64, 64, 1, 150, 143, True),      # kept weights: several tiles per CTA, one cut of the ring
+    (1, 1, 0, 64, 256, 2, 90, 119, True),      # kept pointwise weights, two output units per tile
+    (3, 1, 1, 128, 128, 1, 139, 141, False),   # 128-channel tiles: a filter row per weight box, a wait per row
+    (5, 1, 2, 64, 128, 1, 17, 19, True),       # 40 KB weight boxes, two groups per chunk
+    (3, 1, 1, 256, 80, 2, 9, 12, False),       # five output units of 16 channels: more than are in flight at a time
+    (1, 1, 0, 192, 112, 3, 7, 5, True),        # seven units, tiles that fold images, rows beyond the band
+    (3, 2, 1, 320, 48, 1, 21, 30, False),      # per-tap entries, the last one short
+    (1, 1, 0, 16, 16, 1, 3, 3, True),          # the smallest tile
+]
+
+
+@pytest.mark.parametrize("case", RING_CASES)
+def test_operand_ring_cuts_and_output_units(case):
+    """One layer, then one with other tiles behind it (the ring is cut anew between them), bands and host output."""
+    k, s, p, cin, cout, N, H, W, residual = case
+    layers = [conv(cin, cout, k, s=s, p=p, act=li.ACT_RELU), conv(cout, cout, 1, p=0, act=li.ACT_NONE)]
+    layers[0].input_from, layers[1].input_from = -1, 0
+    if residual:
+        layers[1].residual_from, layers[1].residual_pos = 0, li.RES_PRE_ACT
+    wl = Workload("ring", "bf16", N, H, W, cin, [Segment(layers, 3)], seed=31)
+    li.fill_parameters(wl)
+    li.make_input(wl)
+    want = check_workload(wl, flags=lop.LOP_FLAG_REUSE_HALO, modes=("whole", "banded", "pipelined"))["whole"][-1]
+    dc = DeviceChain(wl, flags=lop.LOP_FLAG_REUSE_HALO)
+    host = torch.zeros(dc.outs[-1].shape, dtype=dc.outs[-1].dtype).pin_memory()
+    for _ in range(2):
+        dc.run_pipelined(dc.pinned_input(), out_pinned=host)
+        torch.cuda.synchronize()
+        dc.check_device()
+        assert np.array_equal(to_host_f32(host), want)
