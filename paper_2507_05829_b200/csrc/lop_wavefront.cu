@@ -41,6 +41,10 @@ namespace {
 using namespace ptx;
 
 constexpr int EPI_THREADS = 32 * WF_WORKER_WARPS;
+#ifndef LOP_PREFETCH
+#define LOP_PREFETCH 32
+#endif
+constexpr int PREFETCH_BOXES = LOP_PREFETCH;                // weight boxes of a tile asked for ahead of its dependencies
 static_assert(8 * (2 * WF_ENTRIES + 4 + 2 * WF_PUBQ + 4 + 3 * WF_UNITS + 2 + WF_GROUPS) + 128 + 2048 + 8 * (128 + 32) <= WF_FIXED_SMEM, "barriers and tables");
 constexpr int COL_GROUPS = WF_WORKER_WARPS / 4;            // worker warps sharing a TMEM lane group split the columns
 
@@ -90,9 +94,11 @@ __device__ __forceinline__ int rec_dep0(const int4 &r) { return r.w; }
 
 // Bounded wait of a whole warp for an item's dependencies: lane j polls entry j of the list (its first
 // 32 entries were prefetched into `mine`).  Counters only grow (compare modulo 2^32).  The result is
-// uniform across the warp.
-__device__ __forceinline__ bool wait_deps_warp(const WfParams &P, int first, int count, int2 mine, unsigned run, int lane)
+// uniform across the warp.  idle() runs once if the first look finds a producer unfinished: there is time then.
+template <typename Idle>
+__device__ __forceinline__ bool wait_deps_warp(const WfParams &P, int first, int count, int2 mine, unsigned run, int lane, Idle idle)
 {
+    bool idled = false;
     for (int j0 = 0; j0 < count; j0 += 32) {
         const bool have = j0 + lane < count;
         int2 d = mine;
@@ -104,6 +110,7 @@ __device__ __forceinline__ bool wait_deps_warp(const WfParams &P, int first, int
         for (uint32_t i = 0;; ++i) {
             if (!done) done = (int)(ld_acquire(ctr) - target) >= 0;
             if (__all_sync(0xffffffffu, done)) break;
+            if (!idled) { idled = true; idle(); }
             if (i >= P.spin_limit) return false;
             if ((i & 63u) == 63u && __any_sync(0xffffffffu, ld_relaxed(P.counters + 2) != 0u)) return false;
             __nanosleep(32);
@@ -433,7 +440,15 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                     }
                     __syncwarp();
                 }
-                ok = ok && wait_deps_warp(P, rec_dep0(cur), rec_ndep(cur), dep_cur, run, lane);
+                // while the tile's producers are still at work: its weights on their way to L2, the maps to the descriptor cache
+                ok = ok && wait_deps_warp(P, rec_dep0(cur), rec_ndep(cur), dep_cur, run, lane, [&] {
+                    if (lane != 0) return;
+                    const int co0 = rec_cout(cur) * BN;
+                    prefetch_map(maps + first_mi);
+                    for (int ch = 0, n = 0; ch < n_chunks && n < PREFETCH_BOXES; ++ch)
+                        for (int t0 = 0; t0 < n_taps && n < PREFETCH_BOXES; t0 += tbx, ++n) tma_prefetch_3d(maps + 4, ch * BK, co0, t0);
+                    if (res_map >= 0) prefetch_map(P.maps + res_map);
+                });
                 if (ok) {
                     if (lane == 0) mbar_arrive(ssf0 + 8u * (pc & 1u));          // scale / shift are in place
                     ++pc;
@@ -1051,7 +1066,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 if (tid == 0) tr(item, 12);
             } else {
                 // pooling or patch gather: one output row of one image per item, all worker threads
-                if (warp == WF_FIRST_WORKER && !wait_deps_warp(P, rec_dep0(cur), rec_ndep(cur), dep_cur, run, lane) && lane == 0) *epi_fail = 1;
+                if (warp == WF_FIRST_WORKER && !wait_deps_warp(P, rec_dep0(cur), rec_ndep(cur), dep_cur, run, lane, [] {}) && lane == 0) *epi_fail = 1;
                 epi_bar();
                 if (tid == 0) tr(item, 1);
                 const int n = rec_tn(cur);
