@@ -280,11 +280,10 @@ int conv_tc_encode(const ConvArgs &a, const ConvTcGeom &g, ConvTcMaps *maps)
             const int idx = ph * a.sw + pw;
             const long long Hp = (a.Hin - ph + a.sh - 1) / a.sh, Wp = (a.Win - pw + a.sw - 1) / a.sw;
             if (a.Hin - ph <= 0 || a.Win - pw <= 0 || Hp <= 0 || Wp <= 0) continue;
-            const cuuint64_t dims[4] = {(cuuint64_t)a.Cin, (cuuint64_t)Wp, (cuuint64_t)Hp, (cuuint64_t)a.N};
-            const cuuint64_t strides[3] = {(cuuint64_t)a.sw * a.Cin * 2, (cuuint64_t)a.sh * a.Win * a.Cin * 2,
-                                           (cuuint64_t)a.Hin * a.Win * a.Cin * 2};
+            const cuuint64_t dims[4] = {(cuuint64_t)a.x_run, (cuuint64_t)Wp, (cuuint64_t)Hp, (cuuint64_t)a.N};
+            const cuuint64_t strides[3] = {(cuuint64_t)a.sw * a.x_pixel * 2, (cuuint64_t)(a.sh * a.x_row * 2), (cuuint64_t)(a.Hin * a.x_row * 2)};
             const cuuint32_t box[4] = {(cuuint32_t)g.BK, (cuuint32_t)g.TW, (cuuint32_t)g.TR, (cuuint32_t)g.TN};
-            void *basep = (void *)(static_cast<const char *>(a.x) + ((size_t)ph * a.Win + pw) * a.Cin * 2);
+            void *basep = (void *)(static_cast<const char *>(a.x) + (ph * a.x_row + (long long)pw * a.x_pixel) * 2);
             CUresult r = enc(&maps->a[idx], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, basep, dims, strides, box, ones,
                              CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);

@@ -1,8 +1,20 @@
-// Patch gather of a thin chain input (the tensor "split" an operator interceptor performs, Sec. III-B
-// of the paper, combined with the block-wise operator's receptive field, Sec. IV-A): for every output
-// pixel of the first convolution its kh*kw*C input values, in (kh, kw, channel) order, zero where a tap
-// falls outside the image and in the tail up to Kcol.  The convolution then is a pointwise product of
-// the [N, Ho, Wo, Kcol] patch tensor with the [Cout, Kcol] zero-padded weights.
+// Gather of a thin chain input (the tensor "split" an operator interceptor performs, Sec. III-B of the
+// paper, combined with the block-wise operator's receptive field, Sec. IV-A), after which the first
+// convolution is a pointwise product of `K` gathered values per output pixel with zero-padded weights.
+// The gathered tensor has one row per output row, and its columns come in one of two layouts:
+//
+//   shared columns   one column per input column (padding included), holding that column's kh values of
+//                    every channel as C' = kh*C rounded up to 8 elements, zero-padded.  An output pixel's
+//                    kw columns are neighbours, so its K = kw*C' values are one contiguous run; the runs
+//                    of neighbouring pixels overlap, and the convolution's tensor map steps sw columns per
+//                    pixel.  Each input value is written kh times instead of kh*kw times: a 7x7 stride-2
+//                    window over 3 channels takes 96 bytes per output pixel, where its patches take 320.
+//   patches          one column per output pixel with its kh*kw*C values in (kh, kw, channel) order:
+//                    dilated windows, whose columns are no neighbours, and windows so small that the
+//                    rounding of C' would make the shared columns the larger tensor.
+//
+// Either way a gathered column is the patch of a window, kh x 1 in the first layout, so one description
+// and one kernel serve both.
 #pragma once
 #include <cuda_runtime.h>
 #include <cstdint>
@@ -11,9 +23,21 @@ namespace lop {
 
 struct GatherGeom {
     int N, H, W, C;           // chain input
-    int Ho, Wo, Kcol;         // patch tensor
-    int kh, kw, sh, sw, ph, pw, dh, dw;
+    int Ho, Wo, Kcol;         // gathered tensor: rows, columns, elements of a column
+    int kh, kw, sh, sw, ph, pw, dh, dw;       // window of a column
 };
+
+// The persistent kernel gathers from input rows staged in shared memory with the padding's zeros around them.  Bytes of
+// zeros in front of a staged row (its data starts up to 15 bytes later, where its 16-byte vectors put it), and from a
+// row to the next.
+__host__ __device__ inline int gather_lead(const GatherGeom &g) { return (g.pw * g.C * 2 + 15) & ~15; }
+__host__ __device__ inline int gather_pitch(const GatherGeom &g)
+{
+    const int end = ((g.Wo - 1) * g.sw - g.pw + (g.kw - 1) * g.dw + 1) * g.C * 2, row = g.W * g.C * 2;
+    return (gather_lead(g) + 15 + (end > row ? end : row) + 15) & ~15;
+}
+// Input rows behind `rows` gathered ones.
+__host__ __device__ inline int gather_rows_in(const GatherGeom &g, int rows) { return (rows - 1) * g.sh + (g.kh - 1) * g.dh + 1; }
 
 // Eight consecutive patch elements k8*8 .. k8*8+7 of output pixel (n, oh, ow), as bf16 bit patterns.
 // THROUGH_L2: read around L1 (for an input that another engine is still writing while the kernel runs,

@@ -16,12 +16,14 @@ struct LayerInfo {
     int Hin = 0, Win = 0;          // spatial extent of the main input
     int Ho = 0, Wo = 0, Co = 0;    // output shape
     int kernel = K_CONV_SIMT;
-    int cin_eff = 0;               // channels the tensor-core kernel sees (= the patch length Kcol for a gathered stem)
+    int cin_eff = 0;               // channels the tensor-core kernel sees (= the gathered values K of a pixel for a stem)
     bool linear = false;           // given as the row-wise operator LOP_LINEAR (runs as the pointwise convolution it is)
-    bool stem_gather = false;      // thin chain input: the layer's receptive patches are gathered into a
-                                   // [N, Ho, Wo, Kcol] tensor first and the convolution runs as 1x1 over it
+    bool stem_gather = false;      // thin chain input: the values its pixels read are gathered into a tensor
+                                   // [N, Ho, stem_w, stem_c] first and the convolution runs as 1x1 over it
+    bool stem_shared = false;      // the gathered columns are shared by neighbouring pixels (see lop_gather.cuh)
+    int stem_w = 0, stem_c = 0;    // columns of the gathered tensor, elements of a column
     size_t out_off = 0;            // workspace offset of the full-size output (unused for the last layer)
-    size_t wpad_off = 0;           // workspace offset of the [cout][Kcol] zero-padded weights (if stem_gather), of the
+    size_t wpad_off = 0;           // workspace offset of the [cout][cin_eff] zero-padded weights (if stem_gather), of the
                                    // [taps][C] transposed filters (if dw_transposed)
     bool dw_transposed = false;    // bf16 depth-wise convolution with C % 8 == 0: the workspace keeps its filters tap-major
 };
@@ -37,7 +39,7 @@ struct lop_plan {
     int stem = -1;                 // index of the stem_gather layer, or -1
     std::vector<lop_range> ranges;     // [band][layer]
     std::vector<lop_range> in_need;    // [band]: chain-input rows (out_lo,out_hi,new_lo)
-    size_t ws_bytes = 0, status_off = 0, col_off = 0;   // col_off: the gathered patch tensor
+    size_t ws_bytes = 0, status_off = 0, col_off = 0;   // col_off: the gathered tensor of the stem
     double flops = 0.0;
     int copy_group = 1;                // bands moved by one copy-engine copy in pipelined runs (see lop_plan.cpp)
     unsigned wait_limit = 0;           // polls a device-side wait may take before the kernel gives up (0: the default)

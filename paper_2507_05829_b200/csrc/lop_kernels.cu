@@ -156,15 +156,17 @@ __global__ void __launch_bounds__(256) stem_gather_kernel(const uint16_t *__rest
     }
 }
 
-__global__ void pad_weights_kernel(const uint16_t *__restrict__ w, uint16_t *__restrict__ wp, long long rows, int C,
-                                   int Cpad)
+__global__ void stem_weights_kernel(const uint16_t *__restrict__ w, uint16_t *__restrict__ wp, int cout, int kh, int kw, int C, int col, int K)
 {
-    const long long total = rows * Cpad;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(i % Cpad);
-        const long long r = i / Cpad;
-        wp[i] = c < C ? w[r * C + c] : (uint16_t)0;
+    const int total = cout * K, taps_c = kh * kw * C;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+        const int k = i % K, co = i / K;
+        int src = k < taps_c ? k : -1;
+        if (col) {
+            const int b = k / col, r = k - b * col, a = r / C;
+            src = b < kw && a < kh ? (a * kw + b) * C + (r - a * C) : -1;
+        }
+        wp[i] = src >= 0 ? w[co * taps_c + src] : (uint16_t)0;
     }
 }
 
@@ -255,10 +257,10 @@ cudaError_t launch_fetch_rows(const void *src, void *dst, int N, int rows, long 
     return cudaGetLastError();
 }
 
-cudaError_t launch_pad_weights(const void *w, void *wp, long long rows, int C, int Cpad, cudaStream_t s)
+cudaError_t launch_stem_weights(const void *w, void *wp, int cout, int kh, int kw, int C, int col, int K, cudaStream_t s)
 {
-    pad_weights_kernel<<<grid_for(rows * Cpad, 256), 256, 0, s>>>(static_cast<const uint16_t *>(w),
-                                                                  static_cast<uint16_t *>(wp), rows, C, Cpad);
+    stem_weights_kernel<<<grid_for((long long)cout * K, 256), 256, 0, s>>>(static_cast<const uint16_t *>(w), static_cast<uint16_t *>(wp), cout, kh, kw,
+                                                                           C, col, K);
     return cudaGetLastError();
 }
 

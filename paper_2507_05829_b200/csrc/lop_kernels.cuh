@@ -16,6 +16,10 @@ struct ConvArgs {
     int kh, kw, sh, sw, ph, pw, dh, dw;
     int act, res_pos;
     int oh_lo, oh_hi;       // rows to compute
+    // the input in elements: a pixel's channels (those up to Cin read as zeros), from a pixel to the next, from a row to
+    // the next.  x_pixel < x_run only for a gathered stem, whose neighbouring pixels share values.
+    int x_run, x_pixel;
+    long long x_row;
     unsigned *dbg;          // checked execution: the status word that takes bit 0x100 on a violation, else nullptr
 };
 
@@ -50,15 +54,16 @@ cudaError_t launch_layernorm(const ConvArgs &a, int dtype, cudaStream_t s);
 cudaError_t launch_concat(const ConvArgs &a, int dtype, cudaStream_t s);
 // depth-wise filters w[C][taps] -> wt[taps][C] (bf16 only), the layout the persistent kernel reads
 cudaError_t launch_dw_transpose(const void *w, void *wt, int C, int taps, cudaStream_t s);
-// rows [lo,hi) of the patch tensor y[N,Ho,Wo,Kcol] of a thin chain input x[N,H,W,C] (bf16 only).
+// rows [lo,hi) of the gathered tensor y[N,Ho,Wo,Kcol] of a thin chain input x[N,H,W,C] (bf16 only).
 struct GatherGeom;
 // dbg: checked execution's status word (see ConvArgs), or nullptr
 cudaError_t launch_stem_gather(const void *x, void *y, const GatherGeom &g, int lo, int hi, cudaStream_t s, unsigned *dbg = nullptr);
 // Rows [lo, hi) of each of N images of `rows` rows of row_bytes bytes: src (host memory as the device addresses it) -> dst.
 // src and dst agree modulo 16.
 cudaError_t launch_fetch_rows(const void *src, void *dst, int N, int rows, long long row_bytes, int lo, int hi, cudaStream_t s);
-// w[rows][C] -> wp[rows][Cpad] zero-padded (bf16 only).
-cudaError_t launch_pad_weights(const void *w, void *wp, long long rows, int C, int Cpad, cudaStream_t s);
+// w[cout][kh][kw][C] -> wp[cout][K], zero-padded, in the order of a gathered stem's values: (kw, kh, C) with each column's
+// kh*C values padded to col elements, or (kh, kw, C) for col = 0 (bf16 only).
+cudaError_t launch_stem_weights(const void *w, void *wp, int cout, int kh, int kw, int C, int col, int K, cudaStream_t s);
 
 // cuTensorMapEncodeTiled, looked up through the runtime (no link-time dependency on the driver library); nullptr if absent.
 typedef CUresult (*TensorMapEncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,

@@ -20,13 +20,14 @@ inline GatherGeom gather_geom(const lop_plan_t *pl, int i)
     const lop_layer &l = li.l;
     GatherGeom g;
     g.N = pl->N; g.H = pl->H; g.W = pl->W; g.C = pl->C;
-    g.Ho = li.Ho; g.Wo = li.Wo; g.Kcol = li.cin_eff;
+    g.Ho = li.Ho; g.Wo = li.stem_w; g.Kcol = li.stem_c;
     g.kh = l.kh; g.kw = l.kw; g.sh = l.sh; g.sw = l.sw; g.ph = l.ph; g.pw = l.pw; g.dh = l.dh; g.dw = l.dw;
+    if (li.stem_shared) g.kw = g.sw = 1;                      // one column of the window per gathered column
     return g;
 }
 
 // Convolution layer i over output rows [lo, hi).  A tensor-core layer is described the way its kernel
-// sees it: a gathered stem is a pointwise convolution over the patch tensor with zero-padded weights.
+// sees it: a gathered stem is a pointwise convolution over the gathered tensor with zero-padded weights.
 inline ConvArgs conv_args(const lop_plan_t *pl, int i, const void *in, void *out, void *ws, int lo, int hi)
 {
     const LayerInfo &li = pl->layers[i];
@@ -42,6 +43,7 @@ inline ConvArgs conv_args(const lop_plan_t *pl, int i, const void *in, void *out
     a.act = l.act; a.res_pos = a.res ? l.residual_pos : LOP_RES_NONE;
     a.oh_lo = lo; a.oh_hi = hi;
     a.dbg = (pl->flags & LOP_FLAG_DEBUG_BOUNDS) ? reinterpret_cast<unsigned *>(static_cast<char *>(ws) + pl->status_off) : nullptr;
+    a.x_run = a.x_pixel = a.Cin; a.x_row = (long long)a.Win * a.Cin;
     if (li.kernel == K_CONV_TC) {
         a.Cin = li.cin_eff;
         if (li.stem_gather) {
@@ -50,6 +52,9 @@ inline ConvArgs conv_args(const lop_plan_t *pl, int i, const void *in, void *out
             a.Hin = li.Ho; a.Win = li.Wo;
             a.kh = a.kw = a.sh = a.sw = a.dh = a.dw = 1;
             a.ph = a.pw = 0;
+            a.x_run = li.stem_shared ? l.kw * li.stem_c : li.stem_c;
+            a.x_pixel = li.stem_shared ? l.sw * li.stem_c : li.stem_c;
+            a.x_row = (long long)li.stem_w * li.stem_c;
         }
     }
     return a;

@@ -226,12 +226,19 @@ static void choose_kernels(lop_plan_t &pl)
         if (l.cout % 16 != 0 || l.sh * l.sw > 4) continue;
         int cin = l.cin;
         if (cin % 16 != 0) {
-            // a thin chain input (an image): gather each output pixel's kh*kw*cin patch, zero-padded to a multiple
-            // of 16, and run the layer as a pointwise convolution over the patches
+            // a thin chain input (an image): gather the kh*kw*cin values each output pixel reads, zero-padded, and run
+            // the layer as a pointwise convolution over them (see lop_gather.cuh)
             const long long patch = (long long)l.kh * l.kw * cin;
             if (l.input_from != LOP_INPUT || cin > 16 || patch > 1024 || pl.stem >= 0) continue;
-            cin = (int)align_up((size_t)patch, 16);
+            const int full = (int)align_up((size_t)patch, 16), col = (int)align_up((size_t)l.kh * cin, 8);
             li.stem_gather = true;
+            // the smaller of the two layouts, per output pixel; a row pitch that is whole pixels of the tensor map
+            li.stem_shared = l.dw == 1 && l.sw * col < full;
+            li.stem_c = li.stem_shared ? col : full;
+            li.stem_w = li.stem_shared ? (int)align_up((size_t)(li.Wo - 1) * l.sw + l.kw, l.sw) : li.Wo;
+            // 64-element chunks: one operand box each and the widest swizzle, for at most 56 zeros more to multiply
+            cin = full;
+            if (li.stem_shared) cin = l.kw * col <= 32 ? (int)align_up((size_t)l.kw * col, 16) : (int)align_up((size_t)l.kw * col, 64);
             pl.stem = i;
         }
         if ((long long)l.kh * l.kw * cin > (1LL << 20)) continue;
@@ -252,7 +259,7 @@ static void choose_kernels(lop_plan_t &pl)
         LayerInfo &li = pl.layers[i];
         if (li.stem_gather) {
             pl.col_off = off;
-            off += align_up((size_t)pl.N * li.Ho * li.Wo * li.cin_eff * es, 1024);
+            off += align_up((size_t)pl.N * li.Ho * li.stem_w * li.stem_c * es, 1024);
             li.wpad_off = off;
             off += align_up((size_t)li.l.cout * li.cin_eff * es, 1024);
         }

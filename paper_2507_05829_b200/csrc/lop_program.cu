@@ -162,11 +162,10 @@ int encode_maps(const ConvArgs &a, const Geom &g, CUtensorMap *out, int *valid_m
             if (idx >= 4) continue;
             const long long Hp = (a.Hin - ph + a.sh - 1) / a.sh, Wp = (a.Win - pw + a.sw - 1) / a.sw;
             if (a.Hin - ph <= 0 || a.Win - pw <= 0 || Hp <= 0 || Wp <= 0) continue;
-            const cuuint64_t dims[4] = {(cuuint64_t)a.Cin, (cuuint64_t)Wp, (cuuint64_t)Hp, (cuuint64_t)a.N};
-            const cuuint64_t strides[3] = {(cuuint64_t)a.sw * a.Cin * 2, (cuuint64_t)a.sh * a.Win * a.Cin * 2,
-                                           (cuuint64_t)a.Hin * a.Win * a.Cin * 2};
+            const cuuint64_t dims[4] = {(cuuint64_t)a.x_run, (cuuint64_t)Wp, (cuuint64_t)Hp, (cuuint64_t)a.N};
+            const cuuint64_t strides[3] = {(cuuint64_t)a.sw * a.x_pixel * 2, (cuuint64_t)(a.sh * a.x_row * 2), (cuuint64_t)(a.Hin * a.x_row * 2)};
             const cuuint32_t box[4] = {(cuuint32_t)g.BK, (cuuint32_t)g.P, (cuuint32_t)g.RI, (cuuint32_t)g.TN};
-            void *basep = (void *)(static_cast<const char *>(a.x) + ((size_t)ph * a.Win + pw) * a.Cin * 2);
+            void *basep = (void *)(static_cast<const char *>(a.x) + (ph * a.x_row + (long long)pw * a.x_pixel) * 2);
             if (enc(&out[idx], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, basep, dims, strides, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
                     CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
                 return LOP_ECUDA;
@@ -550,17 +549,23 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
     bool uses_flags = false;
     uint32_t unit_bytes = 1024, stg_bytes = 0;
     // scratch of the SIMT items, and with it what the operand ring has at least
-    auto gather_scratch = [](const lop_plan_t *pl, const LayerInfo &li) {
-        // the kh image rows an output row reads are staged in shared memory when they fit, else read in place
-        const uint32_t pitch = ((uint32_t)pl->W * pl->C * 2u + 31u + 15u) & ~15u;
-        const uint32_t need = round_up_u32((uint32_t)li.l.kh * pitch + 4u * (uint32_t)li.cin_eff, 1024u);
-        return need <= 48u * 1024u && li.l.kh <= 64 ? need : 0u;
+    auto gather_scratch = [](const lop_plan_t *pl, int layer, int *rows) {
+        // Rows of one gather item: an item's fixed cost (about 2 us: its dependencies, the loads' latency, the hand-over)
+        // is shared by as many rows as leave two items per SM, and the rows of a window are loaded fewer times.
+        const GatherGeom g = gather_geom(pl, layer);
+        const long long all = (long long)g.N * g.Ho;
+        *rows = all >= 8 * 148 ? 4 : (all >= 4 * 148 ? 2 : 1);
+        // the image rows they read are staged in shared memory when they fit, else read in place
+        auto bytes = [&](int r) { return (long long)gather_rows_in(g, r) * gather_pitch(g) + 4 * g.kh * g.kw * g.C; };
+        while (*rows > 1 && bytes(*rows) > 20 * 1024) *rows /= 2;
+        return bytes(*rows) <= 48 * 1024 ? round_up_u32((uint32_t)bytes(*rows), 1024u) : 0u;
     };
     for (const StageReq &rq : reqs) {
         const lop_plan_t *pl = segs[rq.seg].pl;
         const LayerInfo &li = pl->layers[rq.layer];
         rowop::DwTile t{1, 1, 8};
-        if (rq.gather) stg_bytes = std::max(stg_bytes, gather_scratch(pl, li));
+        int gr = 1;
+        if (rq.gather) stg_bytes = std::max(stg_bytes, gather_scratch(pl, rq.layer, &gr));
         else if (!rq.fetch && li.l.op == LOP_DWCONV2D && dw_tile(pl, li, &t))
             stg_bytes = std::max(stg_bytes, round_up_u32((uint32_t)rowop::dw_tile_bytes(li.l.kh, li.l.kw, li.l.sh, li.l.sw, li.l.dh, li.l.dw, t), 1024u));
     }
@@ -599,9 +604,12 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
         } else if (rq.gather) {
             st.kind = WF_GATHER;
             st.x = in; st.y = wsb + pl->col_off;
-            st.N = pl->N; st.Hin = pl->H; st.Win = pl->W; st.Cin = pl->C; st.Ho = li.Ho; st.Wo = li.Wo; st.Cout = li.cin_eff;
-            st.kh = l.kh; st.kw = l.kw; st.sh = l.sh; st.sw = l.sw; st.ph = l.ph; st.pw = l.pw; st.dh = l.dh; st.dw = l.dw;
-            st.mode = gather_scratch(pl, li) ? 0 : 1;
+            const GatherGeom gg = gather_geom(pl, rq.layer);
+            st.N = gg.N; st.Hin = gg.H; st.Win = gg.W; st.Cin = gg.C; st.Ho = gg.Ho; st.Wo = gg.Wo; st.Cout = gg.Kcol;
+            st.kh = gg.kh; st.kw = gg.kw; st.sh = gg.sh; st.sw = gg.sw; st.ph = gg.ph; st.pw = gg.pw; st.dh = gg.dh; st.dw = gg.dw;
+            st.mode = gather_scratch(pl, rq.layer, &group_rows) ? 0 : 1;
+            st.tr_log = ilog2i(group_rows);
+            tiles_r = (rows + group_rows - 1) / group_rows;
         } else if (l.op == LOP_MAXPOOL2D) {
             const PoolArgs a = pool_args(pl, rq.layer, in, out, ws, rq.lo, rq.hi);
             st.kind = WF_POOL;

@@ -118,7 +118,7 @@ extern "C" int lop_run_whole_static(lop_plan_t *pl, const void *in, void *out, u
         }
         if (li.stem_gather) {
             // another plan may have used the array since: padded weights and patches are rebuilt by every call
-            ST_CUDA(launch_pad_weights(l.weight, ws + li.wpad_off, l.cout, l.kh * l.kw * l.cin, li.cin_eff, s));
+            ST_CUDA(launch_stem_weights(l.weight, ws + li.wpad_off, l.cout, l.kh, l.kw, l.cin, li.stem_shared ? li.stem_c : 0, li.cin_eff, s));
             ST_CUDA(launch_stem_gather(in, ws + pl->col_off, gather_geom(pl, i), 0, li.Ho, s, a.dbg));
         }
         const ConvTcGeom g = conv_tc_geometry(a, li.Ho);

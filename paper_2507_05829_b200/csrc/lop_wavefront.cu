@@ -295,7 +295,106 @@ __device__ __forceinline__ void fetch_bytes(const uint8_t *src, uint8_t *dst, in
         *reinterpret_cast<uint16_t *>(dst + i) = __ldcv(reinterpret_cast<const uint16_t *>(src + i));
 }
 
-// FETCH: the program has a fetch list; the CTA then has one more warp, which walks it.
+// Gather of the stem's values (lop_gather.cuh), 1 << tr_log rows per item: Wo columns of Cout elements;
+// x is the chain input, possibly still arriving.  Latency-bound (one round trip for the input rows, and
+// the item's fixed cost): 32 images of 224x224 before a 7x7 stride-2 layer take 43 us, patches took 50.
+__device__ __noinline__ void gather_item(const WfStage *st, int n, int tile_r, int tid, uint8_t *stg)
+{
+    GatherGeom gg;
+    gg.N = __ldg(&st->N); gg.H = __ldg(&st->Hin); gg.W = __ldg(&st->Win); gg.C = __ldg(&st->Cin);
+    gg.Ho = __ldg(&st->Ho); gg.Wo = __ldg(&st->Wo); gg.Kcol = __ldg(&st->Cout);
+    gg.kh = __ldg(&st->kh); gg.kw = __ldg(&st->kw); gg.sh = __ldg(&st->sh); gg.sw = __ldg(&st->sw);
+    gg.ph = __ldg(&st->ph); gg.pw = __ldg(&st->pw); gg.dh = __ldg(&st->dh); gg.dw = __ldg(&st->dw);
+    const int N = gg.N, Hin = gg.H, Win = gg.W, Cin = gg.C, Ho = gg.Ho, Wo = gg.Wo, Cout = gg.Kcol;
+    const int kh = gg.kh, kw = gg.kw, sh = gg.sh, sw = gg.sw, ph = gg.ph, pw = gg.pw, dh = gg.dh, dw = gg.dw;
+    const int tr_log = __ldg(&st->tr_log), oh_lo = __ldg(&st->oh_lo), oh_hi = __ldg(&st->oh_hi), gather_direct = __ldg(&st->mode);
+    const void *xin = ldg_ptr<const void *>(&st->x);
+    void *yout = ldg_ptr<void *>(reinterpret_cast<const void *const *>(&st->y));
+    const int oh0 = oh_lo + (tile_r << tr_log), n_rows = min(1 << tr_log, oh_hi - oh0);
+    const int k8n = Cout >> 3;
+    const uint16_t *x = static_cast<const uint16_t *>(xin);
+    uint16_t *y = static_cast<uint16_t *>(yout) + ((long long)n * Ho + oh0) * Wo * Cout;
+    if (gather_direct) {
+        for (int idx = tid; idx < n_rows * Wo * k8n; idx += EPI_THREADS) {
+            const int q = idx / k8n, r = q / Wo;
+            *reinterpret_cast<uint4 *>(y + (long long)idx * 8) = gather8<true>(x, gg, n, oh0 + r, q - r * Wo, idx - q * k8n);
+        }
+    } else {
+        // The input rows, copied once into shared memory in 16-byte vectors (around L1: they may have arrived
+        // while the kernel was running), zeros where the window reaches past the image
+        const int row_bytes = Win * Cin * 2, lead = gather_lead(gg), pitch = gather_pitch(gg), nvec = pitch >> 4;
+        const int ih0 = oh0 * sh - ph, total = gather_rows_in(gg, n_rows) * nvec;
+        const long long off0 = ((long long)n * Hin + ih0) * row_bytes;        // byte offset of the first staged row's data
+        const int mis0 = (int)(off0 & 15), mis_step = row_bytes & 15;
+        const long long tensor_bytes = (long long)N * Hin * row_bytes;
+        const uint8_t *xb = reinterpret_cast<const uint8_t *>(x);
+        for (int idx0 = tid; idx0 < total; idx0 += 4 * EPI_THREADS) {
+            uint4 q[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int idx = idx0 + u * EPI_THREADS, row = idx / nvec;
+                const int mis = (mis0 + row * mis_step) & 15;
+                const int at = (idx - row * nvec) * 16 - lead - mis;              // first byte of the vector, from the row's data
+                const long long o = off0 + (long long)row * row_bytes + at;
+                q[u] = make_uint4(0u, 0u, 0u, 0u);
+                if (idx >= total || ih0 + row < 0 || ih0 + row >= Hin || at <= -16 || at >= row_bytes) continue;
+                if (o + 16 <= tensor_bytes) {
+                    q[u] = __ldcg(reinterpret_cast<const uint4 *>(xb + o));
+                } else {                                          // the tensor ends inside this vector
+                    uint32_t h[8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        h[e] = o + 2 * e < tensor_bytes ? (uint32_t)__ldcg(reinterpret_cast<const uint16_t *>(xb + o + 2 * e)) : 0u;
+                    q[u] = make_uint4(h[0] | (h[1] << 16), h[2] | (h[3] << 16), h[4] | (h[5] << 16), h[6] | (h[7] << 16));
+                }
+                if (at < 0 || at + 16 > row_bytes) {              // the row starts or ends inside it
+                    uint32_t *w = reinterpret_cast<uint32_t *>(&q[u]);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        if (at + 4 * e < 0 || at + 4 * e >= row_bytes) w[e] &= 0xFFFF0000u;
+                        if (at + 4 * e + 2 < 0 || at + 4 * e + 2 >= row_bytes) w[e] &= 0xFFFFu;
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (idx0 + u * EPI_THREADS < total) *reinterpret_cast<uint4 *>(stg + (idx0 + u * EPI_THREADS) * 16) = q[u];
+        }
+        // where a column's values lie: staged row << 16 | byte offset from the pixel's first input column (kept
+        // even where that is negative: the window's left padding is part of the lead)
+        int *tab = reinterpret_cast<int *>(stg + gather_rows_in(gg, 1 << tr_log) * pitch);
+        for (int k = tid; k < kh * kw * Cin; k += EPI_THREADS) {
+            const int tap = k / Cin, a = tap / kw;
+            tab[k] = ((a * dh) << 16) | (((tap - a * kw) * dw * Cin + k - tap * Cin) * 2);
+        }
+        epi_bar();
+        // A thread keeps to one vector of the columns: where its eight values lie in the staged rows changes
+        // with the row only, so a column costs eight 2-byte reads and the store.
+        const int per = EPI_THREADS / k8n, k8 = tid % k8n, k_left = kh * kw * Cin - k8 * 8;
+        int p = tid / k8n, r = 0, j = p;
+        bool moved = true;
+        int ad[8];
+        for (const int end = tid < per * k8n ? n_rows * Wo : 0; p < end; p += per) {
+            while (j >= Wo) { j -= Wo; ++r; moved = true; }
+            if (moved) {
+                moved = false;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const int t = tab[k8 * 8 + min(e, k_left - 1)], row = r * sh + (t >> 16);
+                    ad[e] = row * pitch + lead + ((mis0 + row * mis_step) & 15) + (t & 0xFFFF) - pw * Cin * 2;
+                }
+            }
+            uint32_t h[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                h[e] = e < k_left ? (uint32_t)*reinterpret_cast<const uint16_t *>(stg + ad[e] + j * sw * Cin * 2) : 0u;
+            *reinterpret_cast<uint4 *>(y + ((long long)p * k8n + k8) * 8) =
+                make_uint4(h[0] | (h[1] << 16), h[2] | (h[3] << 16), h[4] | (h[5] << 16), h[6] | (h[7] << 16));
+            j += per;
+        }
+    }
+}
+
 // FETCH: one more warp per CTA brings the chain input from host memory.  ROWOPS: the program has depth-wise /
 // normalisation / concatenation stages; programs without them run an instantiation that does not carry their code.
 template <bool FETCH, bool ROWOPS>
@@ -903,7 +1002,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
         uint32_t cnt = 0, done_items = 0, uc = 0;
         int sub_log = 6, units_n = 0;
         bool bulk_out = false;
-        int kind = -1, oh_lo = 0, oh_hi = 0, p_log = 0, tr_log = 0, tw_valid = 0, BN = 0, gather_direct = 0, fuse_pool = 0, pool_Ho = 0, pool_Wo = 0;
+        int kind = -1, oh_lo = 0, oh_hi = 0, p_log = 0, tr_log = 0, tw_valid = 0, BN = 0, fuse_pool = 0, pool_Ho = 0, pool_Wo = 0;
         int N = 0, Hin = 0, Win = 0, Cin = 0, Ho = 0, Wo = 0, Cout = 0, kh = 1, kw = 1, sh = 1, sw = 1, ph = 0, pw = 0, dh = 1,
             dw = 1, act = 0, res_pos = 0;
         const void *xin = nullptr, *resp = nullptr;
@@ -916,7 +1015,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
             if (rec_stage(cur) != sidx) {
                 sidx = rec_stage(cur);
                 const WfStage *sp = &P.stages[sidx];
-                kind = __ldg(&sp->kind); gather_direct = __ldg(&sp->mode); oh_lo = __ldg(&sp->oh_lo); oh_hi = __ldg(&sp->oh_hi);
+                kind = __ldg(&sp->kind); oh_lo = __ldg(&sp->oh_lo); oh_hi = __ldg(&sp->oh_hi);
                 p_log = __ldg(&sp->p_log); tr_log = __ldg(&sp->tr_log); tw_valid = __ldg(&sp->tw_valid);
                 BN = __ldg(&sp->BN);
                 N = __ldg(&sp->N); Hin = __ldg(&sp->Hin); Win = __ldg(&sp->Win); Cin = __ldg(&sp->Cin);
@@ -1141,85 +1240,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 } else if (ROWOPS && kind == WF_CONCAT) {
                     concat_item(&P.stages[sidx], n, oh, tid);
                 } else {
-                    // patch gather: Cout holds the patch length Kcol; x is the chain input, possibly still arriving
-                    GatherGeom gg;
-                    gg.N = N; gg.H = Hin; gg.W = Win; gg.C = Cin; gg.Ho = Ho; gg.Wo = Wo; gg.Kcol = Cout;
-                    gg.kh = kh; gg.kw = kw; gg.sh = sh; gg.sw = sw; gg.ph = ph; gg.pw = pw; gg.dh = dh; gg.dw = dw;
-                    const int k8n = Cout >> 3;
-                    const int total = Wo * k8n;
-                    const uint16_t *x = static_cast<const uint16_t *>(xin);
-                    uint16_t *y = static_cast<uint16_t *>(yout);
-                    if (gather_direct) {
-                        for (int idx = tid; idx < total; idx += EPI_THREADS) {
-                            const int ow = idx / k8n, k8 = idx - ow * k8n;
-                            *reinterpret_cast<uint4 *>(y + (((long long)n * Ho + oh) * Wo + ow) * Cout + k8 * 8) =
-                                gather8<true>(x, gg, n, oh, ow, k8);
-                        }
-                    } else {
-                        // the kh image rows this output row reads, copied once into the staging tile with 16-byte
-                        // loads (around L1: the rows may have arrived while the kernel was running), then the
-                        // patches are put together from shared memory
-                        const int row_bytes_in = Win * Cin * 2;
-                        const int pitch = (row_bytes_in + 31 + 15) & ~15;
-                        const long long tensor_bytes = (long long)N * Hin * row_bytes_in;
-                        int *s_mis = reinterpret_cast<int *>(row_pix);       // per filter row: byte offset of the row's first element in staging, or -1
-                        const uint8_t *xb = reinterpret_cast<const uint8_t *>(x);
-                        const int nvec_max = (row_bytes_in + 30) >> 4;
-                        for (int idx = tid; idx < kh * nvec_max; idx += EPI_THREADS) {
-                            const int a = idx / nvec_max, v = idx - a * nvec_max;
-                            const int ih = oh * sh - ph + a * dh;
-                            const bool have = ih >= 0 && ih < Hin;
-                            const long long off = ((long long)n * Hin + ih) * row_bytes_in;
-                            const int mis = (int)(off & 15);
-                            if (v == 0) s_mis[a] = have ? a * pitch + mis : -1;
-                            if (!have || v >= ((mis + row_bytes_in + 15) >> 4)) continue;
-                            const long long off_al = off - mis;
-                            uint4 q;
-                            if (off_al + 16LL * (v + 1) <= tensor_bytes) {
-                                q = __ldcg(reinterpret_cast<const uint4 *>(xb + off_al) + v);
-                            } else {                                          // the tensor ends inside this vector
-                                uint32_t h[8];
-#pragma unroll
-                                for (int e = 0; e < 8; ++e) {
-                                    const long long o = off_al + 16LL * v + 2 * e;
-                                    h[e] = o < tensor_bytes ? (uint32_t)__ldcg(reinterpret_cast<const uint16_t *>(xb + o)) : 0u;
-                                }
-                                q = make_uint4(h[0] | (h[1] << 16), h[2] | (h[3] << 16), h[4] | (h[5] << 16), h[6] | (h[7] << 16));
-                            }
-                            *reinterpret_cast<uint4 *>(stg + a * pitch + 16 * v) = q;
-                        }
-                        // per patch element: filter row << 16 | element offset inside that row's run of kw*C values, or -1
-                        int *tab = reinterpret_cast<int *>(stg + kh * pitch);
-                        const int klen = kh * kw * Cin;
-                        for (int k = tid; k < Cout; k += EPI_THREADS) {
-                            int t = -1;
-                            if (k < klen) {
-                                const int tap = k / Cin, ci = k - tap * Cin;
-                                const int a = tap / kw, b = tap - a * kw;
-                                t = (a << 16) | (b * dw * Cin + ci);
-                            }
-                            tab[k] = t;
-                        }
-                        epi_bar();
-                        const int row_elems = Win * Cin;
-                        for (int idx = tid; idx < total; idx += EPI_THREADS) {
-                            const int ow = idx / k8n, k8 = idx - ow * k8n;
-                            const int base_e = (ow * sw - pw) * Cin;                  // first element of the pixel's runs
-                            const int4 t0 = *reinterpret_cast<const int4 *>(tab + k8 * 8);
-                            const int4 t1 = *reinterpret_cast<const int4 *>(tab + k8 * 8 + 4);
-                            const int tt[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
-                            uint32_t h[8];
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) {
-                                const int fa = tt[e] >> 16, src = base_e + (tt[e] & 0xFFFF);
-                                const int rowoff = s_mis[fa < 0 ? 0 : fa];          // byte offset of the row in staging, or -1
-                                const bool ok = tt[e] >= 0 && rowoff >= 0 && src >= 0 && src < row_elems;
-                                h[e] = ok ? (uint32_t)*reinterpret_cast<const uint16_t *>(stg + rowoff + src * 2) : 0u;
-                            }
-                            *reinterpret_cast<uint4 *>(y + (((long long)n * Ho + oh) * Wo + ow) * Cout + k8 * 8) =
-                                make_uint4(h[0] | (h[1] << 16), h[2] | (h[3] << 16), h[4] | (h[5] << 16), h[6] | (h[7] << 16));
-                        }
-                    }
+                    gather_item(&P.stages[sidx], n, tile_r, tid, stg);
                 }
             }
             if (kind != WF_CONV && tid == 0) tr(item, 12);

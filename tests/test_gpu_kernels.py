@@ -105,3 +105,30 @@ def test_operand_ring_cuts_and_output_units(case):
         torch.cuda.synchronize()
         dc.check_device()
         assert np.array_equal(to_host_f32(host), want)
+
+
+# ------------------------------------------------------------------------------------ gathered stems
+STEM_CASES = [  # k, s, p, dilation, cin, cout, N, H, W
+    (7, 2, 3, 1, 3, 64, 16, 150, 21),      # shared columns, four rows per gather item, a last item of three
+    (7, 2, 3, 1, 3, 48, 5, 241, 33),       # two rows per item, rows whose bytes are no multiple of 16
+    (3, 1, 1, 1, 3, 64, 1, 19, 1),         # one pixel wide
+    (3, 1, 1, 1, 1, 16, 2, 9, 40),         # the shortest column: 3 of 8 values, runs of 24
+    (3, 1, 1, 1, 8, 32, 1, 12, 17),        # 72 values in two chunks
+    (5, 1, 4, 2, 3, 16, 1, 20, 23),        # dilated: patches
+    (3, 2, 1, 1, 3, 32, 3, 33, 47),        # shared columns would be no smaller: patches
+    (1, 2, 0, 1, 3, 16, 1, 11, 13),        # a pointwise stem
+]
+
+
+@pytest.mark.parametrize("case", STEM_CASES)
+def test_gathered_stem_layouts(case):
+    """Whole, band by band and streamed runs of the persistent kernel, and the per-layer kernels, on both layouts."""
+    k, s, p, d, cin, cout, N, H, W = case
+    layers = [conv(cin, cout, k, s=s, p=p, act=li.ACT_RELU)]
+    layers[0].dh = layers[0].dw = d
+    layers[0].input_from = -1
+    wl = Workload("stem", "bf16", N, H, W, cin, [Segment(layers, 3)], seed=37)
+    li.fill_parameters(wl)
+    li.make_input(wl)
+    check_workload(wl, flags=lop.LOP_FLAG_REUSE_HALO, modes=("whole", "banded", "pipelined"))
+    check_workload(wl, flags=lop.LOP_FLAG_REUSE_HALO | lop.LOP_FLAG_PER_LAYER, modes=("whole", "banded"))
