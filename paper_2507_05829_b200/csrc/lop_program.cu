@@ -87,11 +87,6 @@ Geom choose_geom(const ConvArgs &a, int rows, bool even_tiles, bool bulk_out, ui
     g.BN = 16;
     for (int bn = 128; bn >= 16; bn -= 16)
         if (a.Cout % bn == 0 && (bulk_out || bn / unit_channels(bn) <= WF_UNITS)) { g.BN = bn; break; }
-    // A layer with few pixel tiles (a small map deep in the network) would occupy a handful of SMs, each streaming
-    // all of K for a wide slice of the weights: narrower output-channel tiles spread the same weight traffic over more
-    // SMs.  Not below 64: an MMA with N = 32 costs the issuing thread as much as one with N = 64 (45 and 49 cycles).
-    const long long layer_tiles = ((long long)a.N * a.Ho * a.Wo + 127) / 128;
-    while (g.BN > 64 && g.BN % 32 == 0 && layer_tiles * (a.Cout / g.BN) < 148) g.BN /= 2;
     g.n_taps = a.kh * a.kw;
     g.n_chunks = a.Cin / g.BK;
     const uint32_t row_bytes = (uint32_t)g.BK * 2u;
@@ -130,6 +125,13 @@ Geom choose_geom(const ConvArgs &a, int rows, bool even_tiles, bool bulk_out, ui
             }
         g.tw_valid = g.P; g.RI = g.TR;
     }
+    // Output channels per tile: the widest tile reads its activations once and its MMAs do the most work each, but a layer
+    // with few of them leaves SMs idle.  A tile half as wide takes about 1 / 1.4 of the time (an MMA with N = 64 costs the
+    // issuing thread 48 cycles, one with N = 128 65; the epilogue 1.5 and 2.2 us), so the width follows from the number of
+    // rounds the layer's tiles take on 148 SMs.  Not below 64: an MMA with N = 32 costs as much as one with N = 64.
+    const long long pixel_tiles = (long long)((a.Wo + g.tw_valid - 1) / g.tw_valid) * ((a.Ho + g.TR - 1) / g.TR) * ((a.N + g.TN - 1) / g.TN);
+    auto rounds = [&](int bn) { return (pixel_tiles * (a.Cout / bn) + 147) / 148; };
+    while (g.BN > 64 && g.BN % 32 == 0 && rounds(g.BN / 2) < 1.4 * rounds(g.BN)) g.BN /= 2;
     g.a_bytes = (uint32_t)g.RI * g.P * g.TN * row_bytes;
     // (a shifted tap reads up to halo_w pixels past the box, into whatever follows it in shared memory: those rows of the
     // accumulator are the dropped anchors of the halo gap)
@@ -309,201 +311,130 @@ Reads reads_of(const Ctx &cx, const StageReq &rq, int o0, int o1)
     return r;
 }
 
-// Rough shape of a stage for the ordering below: how many items it is cut into and how long one takes (microseconds;
-// measured: ~1.2 us fixed per convolution tile plus ~0.035 us per tensor-core instruction and ~0.2 us per operand box, each
-// issued by one thread; ~4 us more until the tile's epilogue has run and its rows are visible;
-// ~2.5 us per pooling / gather row).  A fetch is not run by the CTAs: items = 0, item_us = its time on the host link.
-struct StageShape { int items; double item_us; double tail_us; };   // tail_us: from an item's end on its CTA to its result being visible
-StageShape stage_shape(const Ctx &cx, const StageReq &rq)
-{
-    const lop_plan_t *pl = cx.segs[rq.seg].pl;
-    const LayerInfo &li = pl->layers[rq.layer];
-    const double rows = rq.hi - rq.lo;
-    if (rq.fetch) return StageShape{0, rows * pl->W * pl->C * 2.0 * pl->N / 24e3, 0.0};      // ~24 GB/s measured for SM-issued reads
-    if (rq.gather || li.l.op == LOP_MAXPOOL2D || li.l.op == LOP_CONCAT) return StageShape{(int)rows * pl->N, 2.5, 0.5};
-    if (li.l.op == LOP_LAYERNORM) return StageShape{(int)rows * pl->N, 4.0, 0.5};
-    if (li.l.op == LOP_DWCONV2D) {
-        rowop::DwTile t{1, 1, 8};
-        dw_tile(pl, li, &t);
-        return StageShape{(int)((rows + t.R - 1) / t.R) * pl->N * ((li.Wo + t.tw - 1) / t.tw) * (li.l.cin / t.cc), 4.0, 0.5};
-    }
-    const double tiles = std::ceil(rows * li.Wo * pl->N / 128.0) * std::max(1, li.l.cout / 128);
-    // operand boxes, ~0.2 us each (issue, and the wait for a free ring slot): one per (tap, 64-channel chunk) and operand for strided windows, one
-    // activation box and a few weight boxes per chunk otherwise
-    const int taps = li.stem_gather ? 1 : li.l.kh * li.l.kw;
-    const double chunks = std::ceil(li.cin_eff / 64.0);
-    const bool per_tap = taps > 1 && (li.l.sh != 1 || li.l.sw != 1 || li.cin_eff % 64 != 0);
-    const double boxes = per_tap ? 2.0 * taps * chunks : (1.0 + std::ceil(taps / 3.0)) * chunks;
-    // a CTA overlaps a tile's epilogue with the next tile's loads and MMAs: the epilogue is latency, not occupancy
-    return StageShape{(int)tiles, 1.2 + 0.2 * boxes + 0.035 * taps * (li.cin_eff / 16.0), 4.0};
-}
-
-// Puts the requests into program order.  Resident programs: ascending priority as far as dependencies allow (a
-// stable topological order).  Programs whose input arrives while they run (arrival_us: when each band of plan 0 is
-// expected on the device; or fetch requests): the order in which a model of the machine would start the stages.
-int order_requests(const Ctx &cx, std::vector<StageReq> &reqs, bool reuse, const std::vector<double> *arrival_us)
+// Puts the requests into ascending priority as far as dependencies allow (a stable topological order).
+int order_requests(const Ctx &cx, std::vector<StageReq> &reqs, bool reuse)
 {
     const size_t n = reqs.size();
     std::vector<int> produces(n);
     for (size_t i = 0; i < n; ++i)
         produces[i] = reqs[i].fetch ? cx.raw : (reqs[i].gather ? cx.patches_id(reqs[i].seg) : cx.tensor_id(reqs[i].seg, reqs[i].layer));
-    const bool by_start = arrival_us != nullptr || cx.raw >= 0;
-    bool sorted_already = !by_start;
+    bool sorted_already = true;
     for (size_t i = 1; i < n; ++i)
         if (reqs[i].prio < reqs[i - 1].prio) sorted_already = false;
-    std::vector<std::vector<int>> users(n), prods(n);
-    std::vector<char> raw(n, 0);
+    std::vector<std::vector<int>> users(n);
+    std::vector<int> pending(n, 0), heap;
     for (size_t i = 0; i < n; ++i) {
         const Reads r = reads_of(cx, reqs[i], reqs[i].lo, reqs[i].hi);
-        raw[i] = r.raw;
         for (int q = 0; q < r.n; ++q)
             for (size_t j = 0; j < n; ++j) {
                 if (j == i || produces[j] != r.need[q].tensor) continue;
                 if (!reuse && r.need[q].same_seg && reqs[j].band != reqs[i].band) continue;
                 if (std::max(r.need[q].lo, reqs[j].lo) >= std::min(r.need[q].hi, reqs[j].hi)) continue;
                 users[j].push_back((int)i);
-                prods[i].push_back((int)j);
+                ++pending[i];
                 if (j > i) sorted_already = false;
             }
     }
     if (sorted_already) return LOP_OK;
-    auto kahn = [&](std::vector<int> &order) {
-        auto later = [&](int x, int y) { return reqs[x].prio != reqs[y].prio ? reqs[x].prio > reqs[y].prio : x > y; };
-        std::vector<int> pending(n), heap;
-        for (size_t i = 0; i < n; ++i) {
-            pending[i] = (int)prods[i].size();
-            if (!pending[i]) heap.push_back((int)i);
-        }
-        std::make_heap(heap.begin(), heap.end(), later);
-        order.clear();
-        while (!heap.empty()) {
-            std::pop_heap(heap.begin(), heap.end(), later);
-            const int i = heap.back();
-            heap.pop_back();
-            order.push_back(i);
-            for (int u : users[i])
-                if (--pending[u] == 0) { heap.push_back(u); std::push_heap(heap.begin(), heap.end(), later); }
-        }
-        return order.size() == n;
-    };
-    std::vector<int> order;
-    if (!by_start) {
-        if (!kahn(order)) { set_error("the stage requests depend on each other in a cycle"); return LOP_EINVAL; }
-    } else {
-        // A model of the machine as it really runs: items go round-robin to n_cta CTAs in program order and each
-        // CTA takes its items in order, waiting for an item's stage to be ready; fetches queue on the host link.
-        struct Machine {
-            std::vector<double> cta_free;
-            double link_free = 0.0, makespan = 0.0;
-            long long rr = 0;                                   // items placed so far: the round-robin position
-            explicit Machine(int n_cta) : cta_free(n_cta, 0.0) {}
-            double run(const StageShape &sh, bool fetch, double ready)
-            {
-                double fin = ready;
-                if (fetch) {
-                    const double start = std::max(ready, link_free);
-                    link_free = start + sh.item_us;
-                    fin = link_free + 3.0;                      // + the link's latency
-                } else {
-                    for (int it = 0; it < sh.items; ++it, ++rr) {
-                        double &f = cta_free[rr % (long long)cta_free.size()];
-                        f = std::max(f, ready) + sh.item_us;
-                        fin = std::max(fin, f + sh.tail_us);
-                    }
-                }
-                makespan = std::max(makespan, fin);
-                return fin;
-            }
-        };
-        const int n_cta = 148;
-        const double hop_us = 1.0;                              // producer's last store -> consumer sees the counter
-        std::vector<StageShape> shape(n);
-        for (size_t i = 0; i < n; ++i) shape[i] = stage_shape(cx, reqs[i]);
-        auto arrival_of = [&](int i) {
-            return (arrival_us && raw[i] && reqs[i].wait_arrival && reqs[i].band < (int)arrival_us->size()) ? (*arrival_us)[reqs[i].band] : 0.0;
-        };
-        // Candidate 1, greedy list scheduling: repeatedly append, among the stages whose producers are all placed,
-        // the one that is ready first, and let the model run it.  While the machine waits for input this follows
-        // each band down its layers (the pipeline of Sec. IV-B); once the machine is saturated, finish times slip,
-        // stages of other bands become ready first and the order turns layer-major by itself.
-        double span_greedy = 0.0;
-        {
-            Machine mc(n_cta);
-            std::vector<double> ready(n, 0.0);
-            std::vector<int> pending(n), heap;
-            auto later = [&](int x, int y) {
-                if (ready[x] != ready[y]) return ready[x] > ready[y];
-                if (reqs[x].prio != reqs[y].prio) return reqs[x].prio > reqs[y].prio;
-                return x > y;
-            };
-            for (size_t i = 0; i < n; ++i) {
-                pending[i] = (int)prods[i].size();
-                if (!pending[i]) { ready[i] = arrival_of((int)i); heap.push_back((int)i); }
-            }
-            std::make_heap(heap.begin(), heap.end(), later);
-            while (!heap.empty()) {
-                std::pop_heap(heap.begin(), heap.end(), later);
-                const int i = heap.back();
-                heap.pop_back();
-                order.push_back(i);
-                const double fin = mc.run(shape[i], reqs[i].fetch, ready[i]);
-                for (int u : users[i]) {
-                    ready[u] = std::max(ready[u], fin + hop_us);
-                    if (--pending[u] == 0) {
-                        ready[u] = std::max(ready[u], arrival_of(u));
-                        heap.push_back(u);
-                        std::push_heap(heap.begin(), heap.end(), later);
-                    }
-                }
-            }
-            if (order.size() != n) { set_error("the stage requests depend on each other in a cycle"); return LOP_EINVAL; }
-            span_greedy = mc.makespan;
-        }
-        // Candidate 2, layer-major (operation batching, Sec. IV-C): all bands' stages of one depth together, the
-        // way resident programs run; the input's transfer is then hidden only behind the first layers.  Deep
-        // chains of many thin bands do better this way: their late stages have too few tiles to fill the machine
-        // band by band.  The model decides.
-        {
-            std::vector<int> depth(n, 0);
-            for (int i : order)
-                for (int j : prods[i]) depth[i] = std::max(depth[i], depth[j] + 1);
-            std::vector<long long> keep(n);
-            for (size_t i = 0; i < n; ++i) { keep[i] = reqs[i].prio; reqs[i].prio = (long long)depth[i] * 65536 + reqs[i].band; }
-            std::vector<int> batched;
-            kahn(batched);
-            for (size_t i = 0; i < n; ++i) reqs[i].prio = keep[i];
-            Machine mc(n_cta);
-            std::vector<double> fin(n, 0.0);
-            for (int i : batched) {
-                double ready = arrival_of(i);
-                for (int j : prods[i]) ready = std::max(ready, fin[j] + hop_us);
-                fin[i] = mc.run(shape[i], reqs[i].fetch, ready);
-            }
-#ifdef LOP_WF_TRACE
-            fprintf(stderr, "order model: greedy %.1f us, layer-major %.1f us (%zu stages)\n", span_greedy, mc.makespan, n);
-#endif
-            // The model is too coarse to separate the two when they come out close, and measurements did: where the
-            // input's transfer is a small part of the run (under a fifth), the layer-major order wins by running the
-            // bulk of the work the way resident programs do (a ResNet-50 of batch 8: 836 vs 862 us); where the transfer is a large
-            // part, following the arrivals wins (one 224x224 image through a VGG block: 38 vs 51 us).
-            double transfer = 0.0;
-            for (size_t i = 0; i < n; ++i)
-                if (reqs[i].fetch) transfer += shape[i].item_us;
-            if (arrival_us && !arrival_us->empty()) transfer = std::max(transfer, arrival_us->back());
-            const bool compute_bound = transfer < 0.2 * mc.makespan;
-            // (a resident program, nothing arriving: the greedy order unless the model clearly prefers layer-major --
-            // it moves late layers of early bands in front of early layers of late bands where that shortens waits)
-            const bool resident = transfer == 0.0;
-            if (batched.size() == n && (resident ? mc.makespan < 0.98 * span_greedy
-                                                 : (mc.makespan < 0.95 * span_greedy || (compute_bound && mc.makespan < 1.05 * span_greedy))))
-                order.swap(batched);
-        }
-    }
+    auto later = [&](int x, int y) { return reqs[x].prio != reqs[y].prio ? reqs[x].prio > reqs[y].prio : x > y; };
+    for (size_t i = 0; i < n; ++i)
+        if (!pending[i]) heap.push_back((int)i);
+    std::make_heap(heap.begin(), heap.end(), later);
     std::vector<StageReq> out;
-    out.reserve(n);
-    for (int i : order) out.push_back(reqs[i]);
+    while (!heap.empty()) {
+        std::pop_heap(heap.begin(), heap.end(), later);
+        const int i = heap.back();
+        heap.pop_back();
+        out.push_back(reqs[i]);
+        for (int u : users[i])
+            if (--pending[u] == 0) { heap.push_back(u); std::push_heap(heap.begin(), heap.end(), later); }
+    }
+    if (out.size() != n) { set_error("the stage requests depend on each other in a cycle"); return LOP_EINVAL; }
     reqs.swap(out);
     return LOP_OK;
+}
+
+// A row group of a stage: consecutive items that wait for the same producers and count as one dependency, its counter
+// being counters[WF_CTR_FIRST + its index].
+struct Unit {
+    int first_item, items, first_dep, deps;
+    double item_us, tail_us;      // a CTA's time for one item; from an item's end on its CTA to its result being visible
+    double fetch_us;              // time on the host link (a fetch unit: no items), else 0
+};
+
+// Order in which the units' items are dealt out: that in which a model of the machine could start them.  Items go
+// round-robin to the CTAs and each CTA takes its items in order, waiting for an item's unit to be ready; fetches queue
+// on the host link.  A list of units in stage order (layer by layer, operation batching of Sec. IV-C) is right while
+// every layer fills the machine; where the input is still arriving, or layers are too small to fill it, units of later
+// layers over early rows have to come in between (the pipeline of Sec. IV-B). Dealing out, whenever
+// a CTA is free, the ready unit with the longest chain of readers behind it does either: while the machine waits the
+// order follows the rows down the layers, and once it is saturated it turns layer by layer by itself.
+// arrival_us: expected arrival of each band a negative dependency names.
+void schedule_units(const std::vector<Unit> &units, const std::vector<int2> &deps, const std::vector<double> *arrival_us, std::vector<int> &order)
+{
+    const int n = (int)units.size(), n_cta = 148;
+    // producer's last store -> consumer sees the counter: about 1 us, and a margin, because a unit dealt out too early makes
+    // a CTA wait with everything behind it, one dealt out too late costs next to nothing (1 -> 4: a ResNet-50 of batch 32
+    // 1091 -> 1063 us, a 1024x1024 stack streamed 314 -> 302)
+    const double hop_us = 4.0;
+    std::vector<int> pending(n, 0), start(n + 1, 0), users, heap;
+    std::vector<double> ready(n, 0.0);
+    for (int i = 0; i < n; ++i)
+        for (int d = units[i].first_dep; d < units[i].first_dep + units[i].deps; ++d) {
+            if (deps[d].x >= WF_CTR_FIRST) { ++start[deps[d].x - WF_CTR_FIRST + 1]; ++pending[i]; }
+            else if (arrival_us && -1 - deps[d].x < (int)arrival_us->size()) ready[i] = std::max(ready[i], (*arrival_us)[-1 - deps[d].x]);
+        }
+    for (int i = 0; i < n; ++i) start[i + 1] += start[i];
+    users.resize(start[n]);
+    {
+        std::vector<int> at(start.begin(), start.end() - 1);
+        for (int i = 0; i < n; ++i)
+            for (int d = units[i].first_dep; d < units[i].first_dep + units[i].deps; ++d)
+                if (deps[d].x >= WF_CTR_FIRST) users[at[deps[d].x - WF_CTR_FIRST]++] = i;
+    }
+    // time from a unit's start to the end of the longest chain behind it (producers come before their readers in `units`)
+    std::vector<double> path(n, 0.0);
+    for (int i = n - 1; i >= 0; --i) {
+        double behind = 0.0;
+        for (int u = start[i]; u < start[i + 1]; ++u) behind = std::max(behind, path[users[u]]);
+        path[i] = behind + hop_us + units[i].item_us + units[i].tail_us;
+    }
+    auto later = [&](int x, int y) { return ready[x] != ready[y] ? ready[x] > ready[y] : x > y; };
+    auto shorter = [&](int x, int y) { return path[x] != path[y] ? path[x] < path[y] : x > y; };
+    for (int i = 0; i < n; ++i)
+        if (!pending[i]) heap.push_back(i);
+    std::make_heap(heap.begin(), heap.end(), later);        // by the time they are ready
+    std::vector<int> now;                                   // ready when the next CTA is free: longest chain first
+    std::vector<double> cta_free(n_cta, 0.0);
+    double link_free = 0.0;
+    size_t rr = 0;                                          // items placed so far: the round-robin position
+    order.clear();
+    while (!heap.empty() || !now.empty()) {
+        while (!heap.empty() && (now.empty() || ready[heap.front()] <= cta_free[rr % n_cta])) {
+            now.push_back(heap.front());
+            std::pop_heap(heap.begin(), heap.end(), later);
+            heap.pop_back();
+            std::push_heap(now.begin(), now.end(), shorter);
+        }
+        std::pop_heap(now.begin(), now.end(), shorter);
+        const int i = now.back();
+        now.pop_back();
+        order.push_back(i);
+        double fin = ready[i];
+        if (units[i].items == 0) {
+            link_free = std::max(link_free, fin) + units[i].fetch_us;
+            fin = link_free + 3.0;                          // + the link's latency
+        }
+        for (int it = 0; it < units[i].items; ++it) {
+            double &f = cta_free[rr++ % n_cta];
+            f = std::max(f, ready[i]) + units[i].item_us;
+            fin = std::max(fin, f + units[i].tail_us);
+        }
+        for (int u = start[i]; u < start[i + 1]; ++u) {
+            ready[users[u]] = std::max(ready[users[u]], fin + hop_us);
+            if (--pending[users[u]] == 0) { heap.push_back(users[u]); std::push_heap(heap.begin(), heap.end(), later); }
+        }
+    }
 }
 
 }  // namespace
@@ -534,7 +465,7 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
             if (rq.hi > rq.lo) live.push_back(rq);
         reqs.swap(live);
     }
-    int orc = order_requests(cx, reqs, reuse, arrival_us);
+    int orc = order_requests(cx, reqs, reuse);
     if (orc != LOP_OK) return orc;
 
     std::vector<WfStage> stages;
@@ -545,6 +476,7 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
     std::vector<int2> deps;
     std::vector<std::vector<int>> by_tensor(n_tensors);   // stage indices per produced tensor
     std::vector<int> expected;                         // completions per row group, per stage
+    std::vector<Unit> units;
     int n_ctr = WF_CTR_FIRST;
     bool uses_flags = false;
     uint32_t unit_bytes = 1024, stg_bytes = 0;
@@ -591,6 +523,7 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
         int group_rows = 1, tiles_r = rows, tiles_w = 1, tiles_n = pl->N, cout_tiles = 1;
         int produces = rq.fetch ? cx.raw : (rq.gather ? cx.patches_id(rq.seg) : cx.tensor_id(rq.seg, rq.layer));
         int out_lo = rq.lo, out_hi = rq.hi;                    // rows of the produced tensor
+        double item_us = 4.0, tail_us = 0.5;                   // for the schedule (measured, microseconds)
         if (rq.fetch) {
             // a stage only in the book-keeping sense (row-group counters its readers wait for): its work goes to the
             // fetch list.  Entries of about 3 KB, whole rows: a warp has that much in flight at a time.
@@ -609,10 +542,12 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
             st.kh = gg.kh; st.kw = gg.kw; st.sh = gg.sh; st.sw = gg.sw; st.ph = gg.ph; st.pw = gg.pw; st.dh = gg.dh; st.dw = gg.dw;
             st.mode = gather_scratch(pl, rq.layer, &group_rows) ? 0 : 1;
             st.tr_log = ilog2i(group_rows);
+            item_us = 1.0 + 0.9 * group_rows;
             tiles_r = (rows + group_rows - 1) / group_rows;
         } else if (l.op == LOP_MAXPOOL2D) {
             const PoolArgs a = pool_args(pl, rq.layer, in, out, ws, rq.lo, rq.hi);
             st.kind = WF_POOL;
+            item_us = 3.4;
             st.x = a.x; st.y = a.y;
             st.N = a.N; st.Hin = a.Hin; st.Win = a.Win; st.Cin = a.C; st.Ho = a.Ho; st.Wo = a.Wo; st.Cout = a.C;
             st.kh = a.kh; st.kw = a.kw; st.sh = a.sh; st.sw = a.sw; st.ph = a.ph; st.pw = a.pw; st.dh = a.dh; st.dw = a.dw;
@@ -697,6 +632,9 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
                 produces = cx.tensor_id(rq.seg, rq.layer + 1);
                 out_lo = reqs[rj].lo; out_hi = reqs[rj].hi;
             }
+            // an MMA costs the issuing thread 0.05 to 0.09 us with its share of the waits, the epilogue runs beside the next tile's
+            item_us = std::max(g.BN > 64 ? 2.2 : 1.5, 0.6 + 0.07 * g.n_chunks * g.n_taps * (g.BK / 16));
+            tail_us = 3.0;
             group_rows = g.TR;
             tiles_r = (rows + g.TR - 1) / g.TR;
             tiles_w = (a.Wo + g.tw_valid - 1) / g.tw_valid;
@@ -749,8 +687,10 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
                 }
             const int count = (int)deps.size() - first;
             if (count > WF_MAX_DEPS) { set_error("layer %d: a tile depends on too many row groups", rq.layer); return LOP_EUNSUPPORTED; }
+            units.push_back(Unit{(int)items.size(), rq.fetch ? 0 : exp_here, first, count, item_us, tail_us, 0.0});
             if (rq.fetch) {
                 const long long row_b = (long long)pl->W * pl->C * 2;
+                units.back().fetch_us = (double)(o1 - o0) * row_b * pl->N / 48e3;      // ~48 GB/s measured for SM-issued reads
                 for (int n = 0; n < pl->N; ++n) {
                     const unsigned long long off = (unsigned long long)(((long long)n * pl->H + o0) * row_b);
                     fetch_items.push_back(make_int4((int)(unsigned)(off & 0xffffffffu), (int)(unsigned)(off >> 32), (int)((o1 - o0) * row_b),
@@ -772,6 +712,15 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
         expected.push_back(exp_here);
     }
 
+    if (arrival_us || cx.raw >= 0) {
+        std::vector<int> order;
+        schedule_units(units, deps, arrival_us, order);
+        if (order.size() != units.size()) { set_error("the stages depend on each other in a cycle"); return LOP_EINVAL; }
+        std::vector<int4> dealt;
+        dealt.reserve(items.size());
+        for (int u : order) dealt.insert(dealt.end(), items.begin() + units[u].first_item, items.begin() + units[u].first_item + units[u].items);
+        items.swap(dealt);
+    }
     lop_plan_t *pl0 = segs[0].pl;
     Program *p = new (std::nothrow) Program();
     if (!p) { set_error("out of host memory"); return LOP_ENOMEM; }
