@@ -295,6 +295,121 @@ __device__ __forceinline__ void fetch_bytes(const uint8_t *src, uint8_t *dst, in
         *reinterpret_cast<uint16_t *>(dst + i) = __ldcv(reinterpret_cast<const uint16_t *>(src + i));
 }
 
+// The functions below are kept out of line: inlined, they cost the epilogue's path registers and instruction cache (a
+// ResNet-50 of batch 32: 998 us with pooling and gather inside the kernel's body, 974 outside; a ConvNeXt block 47 -> 45).
+
+// 16-byte chunk j of staged row `row` of an output unit (the swizzle of the unit's tensor maps).
+__device__ __forceinline__ uint4 unit_chunk(const uint8_t *unit, int row, int j, int sub_log)
+{
+    const int sw = sub_log == 6 ? row & 7 : (sub_log == 5 ? (row >> 1) & 3 : (row >> 2) & 1);
+    return *reinterpret_cast<const uint4 *>(unit + (row << (sub_log + 1)) + ((j ^ sw) << 4));
+}
+
+// Staged rows of a unit -> global: consecutive threads write consecutive 16 bytes of a pixel's channels.
+__device__ __noinline__ void copy_unit(const uint8_t *unit, const long long *row_pix, uint4 *y, int rows_n, int sub_log, int tid)
+{
+    const int cpr_log = sub_log - 3;                           // 16-byte chunks per staged row
+#pragma unroll 4
+    for (int idx = tid; idx < rows_n << cpr_log; idx += EPI_THREADS) {
+        const int row = idx >> cpr_log, j = idx - (row << cpr_log);
+        const long long rp = row_pix[row];
+        if (rp >= 0) y[(rp >> 3) + j] = unit_chunk(unit, row, j, sub_log);
+    }
+}
+
+// 2x2 windows of staged rows -> their maxima (exact in bf16) -> the pooled tensor, 16 bytes per thread.
+__device__ __noinline__ void pool_unit(const uint8_t *unit, const long long *pool_pix, uint4 *y, int p_log, int tr_log, int tw_valid, int sub_log, int tid)
+{
+    const int cpr_log = sub_log - 3;
+#pragma unroll 2
+    for (int idx = tid; idx < 32 << cpr_log; idx += EPI_THREADS) {
+        const int q = idx >> cpr_log, j = idx - (q << cpr_log);
+        const long long pp = pool_pix[q];
+        if (pp < 0) continue;
+        const int pc = q & ((1 << (p_log - 1)) - 1), t = q >> (p_log - 1);
+        const int s0 = (((t >> (tr_log - 1)) << tr_log) + 2 * (t & ((1 << (tr_log - 1)) - 1))) * tw_valid + 2 * pc;
+        const int rows4[4] = {s0, s0 + 1, s0 + tw_valid, s0 + tw_valid + 1};
+        uint4 acc4 = unit_chunk(unit, rows4[0], j, sub_log);
+#pragma unroll
+        for (int k = 1; k < 4; ++k) {
+            const uint4 v4 = unit_chunk(unit, rows4[k], j, sub_log);
+            __nv_bfloat162 *pa = reinterpret_cast<__nv_bfloat162 *>(&acc4);
+            const __nv_bfloat162 *pv = reinterpret_cast<const __nv_bfloat162 *>(&v4);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) pa[e] = __hmax2(pa[e], pv[e]);
+        }
+        y[(pp >> 3) + j] = acc4;
+    }
+}
+
+// One output row of one image of a max pooling over channel vectors of eight.
+__device__ __noinline__ void pool_item(const WfStage *st, int n, int oh, int tid)
+{
+    const int Hin = __ldg(&st->Hin), Win = __ldg(&st->Win), Cin = __ldg(&st->Cin), Ho = __ldg(&st->Ho), Wo = __ldg(&st->Wo);
+    const int kh = __ldg(&st->kh), kw = __ldg(&st->kw), sh = __ldg(&st->sh), sw = __ldg(&st->sw);
+    const int ph = __ldg(&st->ph), pw = __ldg(&st->pw), dh = __ldg(&st->dh), dw = __ldg(&st->dw);
+    const int cg = Cin >> 3;
+    const int total = Wo * cg;
+    const __nv_bfloat16 *x = static_cast<const __nv_bfloat16 *>(ldg_ptr<const void *>(&st->x));
+    __nv_bfloat16 *y = static_cast<__nv_bfloat16 *>(ldg_ptr<void *>(reinterpret_cast<const void *const *>(&st->y)));
+    // two channel-group vectors per thread
+    for (int idx0 = 0; idx0 < total; idx0 += 2 * EPI_THREADS) {
+        int gch[2], ow[2];
+        bool live[2];
+        float mx[2][8];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int idx = idx0 + u * EPI_THREADS + tid;
+            live[u] = idx < total;
+            ow[u] = idx / cg;
+            gch[u] = idx - ow[u] * cg;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) mx[u][i] = -INFINITY;
+        }
+        const int nt = kh * kw;
+        for (int t0 = 0; t0 < nt; t0 += 4) {                 // four filter taps of both vectors in flight
+            uint4 q4[2][4];
+            bool ok[2][4];
+#pragma unroll
+            for (int tt = 0; tt < 4; ++tt) {
+                const int t = t0 + tt;
+                const int a = t / kw, b = t - a * kw;
+                const int ih = oh * sh - ph + a * dh;
+                const bool rowok = t < nt && ih >= 0 && ih < Hin;
+                const long long rowbase = ((long long)n * Hin + ih) * Win;
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int iw = ow[u] * sw - pw + b * dw;
+                    ok[u][tt] = live[u] && rowok && iw >= 0 && iw < Win;
+                    if (ok[u][tt]) q4[u][tt] = __ldcg(reinterpret_cast<const uint4 *>(x + (rowbase + iw) * Cin + gch[u] * 8));
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+#pragma unroll
+                for (int tt = 0; tt < 4; ++tt)
+                    if (ok[u][tt]) {
+                        const uint32_t w4[4] = {q4[u][tt].x, q4[u][tt].y, q4[u][tt].z, q4[u][tt].w};
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            mx[u][2 * i] = fmaxf(mx[u][2 * i], __uint_as_float(w4[i] << 16));
+                            mx[u][2 * i + 1] = fmaxf(mx[u][2 * i + 1], __uint_as_float(w4[i] & 0xFFFF0000u));
+                        }
+                    }
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+            if (live[u]) {
+                uint32_t o[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i)      // values are bf16 already: truncation is exact
+                    o[i] = (__float_as_uint(mx[u][2 * i]) >> 16) | (__float_as_uint(mx[u][2 * i + 1]) & 0xFFFF0000u);
+                *reinterpret_cast<uint4 *>(y + (((long long)n * Ho + oh) * Wo + ow[u]) * Cin + gch[u] * 8) =
+                    make_uint4(o[0], o[1], o[2], o[3]);
+            }
+    }
+}
+
 // Gather of the stem's values (lop_gather.cuh), 1 << tr_log rows per item: Wo columns of Cout elements;
 // x is the chain input, possibly still arriving.  Latency-bound (one round trip for the input rows, and
 // the item's fixed cost): 32 images of 224x224 before a 7x7 stride-2 layer take 43 us, patches took 50.
@@ -496,6 +611,8 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
         uint32_t ring_lim = ring_bytes, head = 0, pos = 0, tail_at = 0, n_alloc = 0, n_freed = 0, n_full = 0, n_group = 0, w_uses = 0;
         uint32_t slab_sl = 0, slab_end0 = 0, slab_end1 = 0;    // slab stages: next activation box, entry that ended its previous chunk
         long long cut_key = 0;                                 // how the ring is cut (see below)
+        int ss_key[2] = {-1, -1};                              // whose scale / shift the two buffers hold: stage, first channel
+        int ss_co[2] = {0, 0};
         for (; item < NI; item += G) {
             // two items ahead: the record; one item ahead: this lane's dependency entry
             const int4 nn = item + 2 * G < NI ? __ldg(&P.items[item + 2 * G]) : zero4;
@@ -530,9 +647,10 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 // the tile's per-channel scale / shift go to shared memory from here, a tile ahead of the epilogue
                 // that uses them: their load latency is off the workers' path
                 bool ok = __all_sync(0xffffffffu, mbar_wait_abortable(sse0 + 8u * (pc & 1u), ((pc >> 1) & 1u) ^ 1u, abort_flag));
-                if (ok) {
+                const int c0 = rec_cout(cur) * BN;
+                if (ok && (((pc & 1u) ? ss_key[1] : ss_key[0]) != sidx || ((pc & 1u) ? ss_co[1] : ss_co[0]) != c0)) {
                     float *ds = s_scale + 128 * (pc & 1u), *dsh = s_shift + 128 * (pc & 1u);
-                    const int c0 = rec_cout(cur) * BN;
+                    if (pc & 1u) { ss_key[1] = sidx; ss_co[1] = c0; } else { ss_key[0] = sidx; ss_co[0] = c0; }
                     for (int i = lane; i < BN; i += 32) {
                         ds[i] = scale ? __ldg(scale + c0 + i) : 1.0f;
                         dsh[i] = shift ? __ldg(shift + c0 + i) : 0.0f;
@@ -1003,10 +1121,8 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
         int sub_log = 6, units_n = 0;
         bool bulk_out = false;
         int kind = -1, oh_lo = 0, oh_hi = 0, p_log = 0, tr_log = 0, tw_valid = 0, BN = 0, fuse_pool = 0, pool_Ho = 0, pool_Wo = 0;
-        int N = 0, Hin = 0, Win = 0, Cin = 0, Ho = 0, Wo = 0, Cout = 0, kh = 1, kw = 1, sh = 1, sw = 1, ph = 0, pw = 0, dh = 1,
-            dw = 1, act = 0, res_pos = 0;
-        const void *xin = nullptr, *resp = nullptr;
-        const float *scale = nullptr, *shift = nullptr;
+        int N = 0, Ho = 0, Wo = 0, Cout = 0, act = 0, res_pos = 0;
+        const void *resp = nullptr;
         void *yout = nullptr;
         for (; item < NI; item += G) {
             const int4 nn = item + 2 * G < NI ? __ldg(&P.items[item + 2 * G]) : zero4;
@@ -1018,18 +1134,12 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 kind = __ldg(&sp->kind); oh_lo = __ldg(&sp->oh_lo); oh_hi = __ldg(&sp->oh_hi);
                 p_log = __ldg(&sp->p_log); tr_log = __ldg(&sp->tr_log); tw_valid = __ldg(&sp->tw_valid);
                 BN = __ldg(&sp->BN);
-                N = __ldg(&sp->N); Hin = __ldg(&sp->Hin); Win = __ldg(&sp->Win); Cin = __ldg(&sp->Cin);
-                Ho = __ldg(&sp->Ho); Wo = __ldg(&sp->Wo); Cout = __ldg(&sp->Cout);
-                kh = __ldg(&sp->kh); kw = __ldg(&sp->kw); sh = __ldg(&sp->sh); sw = __ldg(&sp->sw);
-                ph = __ldg(&sp->ph); pw = __ldg(&sp->pw); dh = __ldg(&sp->dh); dw = __ldg(&sp->dw);
+                N = __ldg(&sp->N); Ho = __ldg(&sp->Ho); Wo = __ldg(&sp->Wo); Cout = __ldg(&sp->Cout);
                 act = __ldg(&sp->act); res_pos = __ldg(&sp->res_pos);
                 fuse_pool = __ldg(&sp->fuse_pool); pool_Ho = __ldg(&sp->pool_Ho); pool_Wo = __ldg(&sp->pool_Wo);
-                xin = ldg_ptr<const void *>(&sp->x);
                 sub_log = __ldg(&sp->sub_log); units_n = BN >> sub_log;
                 bulk_out = __ldg(&sp->out_map) >= 0;
                 resp = ldg_ptr<const void *>(&sp->res);
-                scale = ldg_ptr<const float *>(reinterpret_cast<const void *const *>(&sp->scale));
-                shift = ldg_ptr<const float *>(reinterpret_cast<const void *const *>(&sp->shift));
                 yout = ldg_ptr<void *>(reinterpret_cast<const void *const *>(&sp->y));
             }
             const int tile_r = rec_tr(cur);
@@ -1044,7 +1154,6 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 const bool staged = c < tw_valid;                      // the other anchors are the slab's halo gap
                 const bool valid = staged && ow < Wo && oh < oh_hi && n < N;
                 const int co0 = rec_cout(cur) * BN;
-                const int trows = 1 << tr_log;
                 // staged rows are packed: image, row, column below tw_valid (the box of a bulk load or store)
                 const int srow = (((m >> (p_log + tr_log)) << tr_log) + r) * tw_valid + c;
                 if (!bulk_out) {
@@ -1123,43 +1232,11 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 }
                 ++cnt;
                 if (!bulk_out && !*epi_fail) {
-                    __nv_bfloat16 *y = static_cast<__nv_bfloat16 *>(yout);
-                    const int cpr_log = sub_log - 3, rows_n = (128 >> p_log) * tw_valid;     // 16-byte chunks per staged row, staged rows
-                    auto chunk = [&](int u, int row, int j) {          // chunk j of a staged row of unit u
-                        const int sw = sub_log == 6 ? row & 7 : (sub_log == 5 ? (row >> 1) & 3 : (row >> 2) & 1);
-                        return *reinterpret_cast<const uint4 *>(units + ((uc + u) & (WF_UNITS - 1)) * unit_bytes + row * row_stride + ((j ^ sw) << 4));
-                    };
                     for (int u = 0; u < units_n; ++u) {
-                        if (fuse_pool) {
-                            // 2x2 windows of staged rows -> their maxima (exact in bf16) -> the pooled tensor, 16 bytes per thread
-                            const int half_p = (1 << p_log) >> 1, half_tr = trows >> 1;
-                            for (int idx = tid; idx < 32 << cpr_log; idx += EPI_THREADS) {
-                                const int q = idx >> cpr_log, j = idx - (q << cpr_log);
-                                const long long pp = pool_pix[q];
-                                if (pp < 0) continue;
-                                const int pc = q % half_p, t = q / half_p;
-                                const int s0 = (((t / half_tr) << tr_log) + 2 * (t % half_tr)) * tw_valid + 2 * pc;
-                                const int rows4[4] = {s0, s0 + 1, s0 + tw_valid, s0 + tw_valid + 1};
-                                uint4 acc4 = chunk(u, rows4[0], j);
-#pragma unroll
-                                for (int k = 1; k < 4; ++k) {
-                                    const uint4 v4 = chunk(u, rows4[k], j);
-                                    __nv_bfloat162 *pa = reinterpret_cast<__nv_bfloat162 *>(&acc4);
-                                    const __nv_bfloat162 *pv = reinterpret_cast<const __nv_bfloat162 *>(&v4);
-#pragma unroll
-                                    for (int e = 0; e < 4; ++e) pa[e] = __hmax2(pa[e], pv[e]);
-                                }
-                                *(reinterpret_cast<uint4 *>(y + pp) + (u << cpr_log) + j) = acc4;
-                            }
-                        } else {
-                            // staged rows -> global: consecutive threads write consecutive 16 bytes of a pixel's channels
-#pragma unroll 4
-                            for (int idx = tid; idx < rows_n << cpr_log; idx += EPI_THREADS) {
-                                const int row = idx >> cpr_log, j = idx - (row << cpr_log);
-                                const long long rp = row_pix[row];
-                                if (rp >= 0) *(reinterpret_cast<uint4 *>(y + rp) + (u << cpr_log) + j) = chunk(u, row, j);
-                            }
-                        }
+                        const uint8_t *unit = units + ((uc + u) & (WF_UNITS - 1)) * unit_bytes;
+                        uint4 *y = static_cast<uint4 *>(yout) + (u << (sub_log - 3));
+                        if (fuse_pool) pool_unit(unit, pool_pix, y, p_log, tr_log, tw_valid, sub_log, tid);
+                        else copy_unit(unit, row_pix, y, (128 >> p_log) * tw_valid, sub_log, tid);
                     }
                 }
                 if (tid == 0) tr(item, 12);
@@ -1173,66 +1250,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 if (*epi_fail) {
                     // fall through to the common exit below
                 } else if (kind == WF_POOL) {
-                    const int cg = Cin >> 3;
-                    const int total = Wo * cg;
-                    const __nv_bfloat16 *x = static_cast<const __nv_bfloat16 *>(xin);
-                    __nv_bfloat16 *y = static_cast<__nv_bfloat16 *>(yout);
-                    // two channel-group vectors per thread
-                    for (int idx0 = 0; idx0 < total; idx0 += 2 * EPI_THREADS) {
-                        int gch[2], ow[2];
-                        bool live[2];
-                        float mx[2][8];
-#pragma unroll
-                        for (int u = 0; u < 2; ++u) {
-                            const int idx = idx0 + u * EPI_THREADS + tid;
-                            live[u] = idx < total;
-                            ow[u] = idx / cg;
-                            gch[u] = idx - ow[u] * cg;
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) mx[u][i] = -INFINITY;
-                        }
-                        const int nt = kh * kw;
-                        for (int t0 = 0; t0 < nt; t0 += 4) {                 // four filter taps of both vectors in flight
-                            uint4 q4[2][4];
-                            bool ok[2][4];
-#pragma unroll
-                            for (int tt = 0; tt < 4; ++tt) {
-                                const int t = t0 + tt;
-                                const int a = t / kw, b = t - a * kw;
-                                const int ih = oh * sh - ph + a * dh;
-                                const bool rowok = t < nt && ih >= 0 && ih < Hin;
-                                const long long rowbase = ((long long)n * Hin + ih) * Win;
-#pragma unroll
-                                for (int u = 0; u < 2; ++u) {
-                                    const int iw = ow[u] * sw - pw + b * dw;
-                                    ok[u][tt] = live[u] && rowok && iw >= 0 && iw < Win;
-                                    if (ok[u][tt]) q4[u][tt] = __ldcg(reinterpret_cast<const uint4 *>(x + (rowbase + iw) * Cin + gch[u] * 8));
-                                }
-                            }
-#pragma unroll
-                            for (int u = 0; u < 2; ++u)
-#pragma unroll
-                                for (int tt = 0; tt < 4; ++tt)
-                                    if (ok[u][tt]) {
-                                        const uint32_t w4[4] = {q4[u][tt].x, q4[u][tt].y, q4[u][tt].z, q4[u][tt].w};
-#pragma unroll
-                                        for (int i = 0; i < 4; ++i) {
-                                            mx[u][2 * i] = fmaxf(mx[u][2 * i], __uint_as_float(w4[i] << 16));
-                                            mx[u][2 * i + 1] = fmaxf(mx[u][2 * i + 1], __uint_as_float(w4[i] & 0xFFFF0000u));
-                                        }
-                                    }
-                        }
-#pragma unroll
-                        for (int u = 0; u < 2; ++u)
-                            if (live[u]) {
-                                uint32_t o[4];
-#pragma unroll
-                                for (int i = 0; i < 4; ++i)      // values are bf16 already: truncation is exact
-                                    o[i] = (__float_as_uint(mx[u][2 * i]) >> 16) | (__float_as_uint(mx[u][2 * i + 1]) & 0xFFFF0000u);
-                                *reinterpret_cast<uint4 *>(y + (((long long)n * Ho + oh) * Wo + ow[u]) * Cin + gch[u] * 8) =
-                                    make_uint4(o[0], o[1], o[2], o[3]);
-                            }
-                    }
+                    pool_item(&P.stages[sidx], n, oh, tid);
                 } else if (ROWOPS && kind == WF_DWCONV) {
                     dwconv_item(&P.stages[sidx], n, tile_r, rec_tw(cur), rec_cout(cur), tid, stg);
                 } else if (ROWOPS && kind == WF_LAYERNORM) {
