@@ -481,12 +481,12 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
     bool uses_flags = false;
     uint32_t unit_bytes = 1024, stg_bytes = 0;
     // scratch of the SIMT items, and with it what the operand ring has at least
-    auto gather_scratch = [](const lop_plan_t *pl, int layer, int *rows) {
-        // Rows of one gather item: an item's fixed cost (about 2 us: its dependencies, the loads' latency, the hand-over)
-        // is shared by as many rows as leave two items per SM, and the rows of a window are loaded fewer times.
+    // Rows of one gather or pooling item: an item's fixed cost (about 2 us: its dependencies, the loads' latency, the
+    // hand-over) is shared by as many rows as leave two items per SM, and the rows of a window are loaded fewer times.
+    auto rows_per_item = [](long long all) { return all >= 8 * 148 ? 4 : (all >= 4 * 148 ? 2 : 1); };
+    auto gather_scratch = [&](const lop_plan_t *pl, int layer, int *rows) {
         const GatherGeom g = gather_geom(pl, layer);
-        const long long all = (long long)g.N * g.Ho;
-        *rows = all >= 8 * 148 ? 4 : (all >= 4 * 148 ? 2 : 1);
+        *rows = rows_per_item((long long)g.N * g.Ho);
         // the image rows they read are staged in shared memory when they fit, else read in place
         auto bytes = [&](int r) { return (long long)gather_rows_in(g, r) * gather_pitch(g) + 4 * g.kh * g.kw * g.C; };
         while (*rows > 1 && bytes(*rows) > 20 * 1024) *rows /= 2;
@@ -547,7 +547,13 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
         } else if (l.op == LOP_MAXPOOL2D) {
             const PoolArgs a = pool_args(pl, rq.layer, in, out, ws, rq.lo, rq.hi);
             st.kind = WF_POOL;
-            item_us = 3.4;
+            // 3x3 windows: several rows per item where they leave two items per SM (a window's rows are loaded fewer times, and
+            // an item's fixed cost is shared); st.mode says which of the two pooling routines runs
+            st.mode = a.kh == 3 && a.kw == 3 && a.dh == 1 && a.dw == 1;
+            if (st.mode) group_rows = rows_per_item((long long)a.N * a.Ho);
+            st.tr_log = ilog2i(group_rows);
+            tiles_r = (rows + group_rows - 1) / group_rows;
+            item_us = st.mode ? 1.5 + group_rows : 3.4;
             st.x = a.x; st.y = a.y;
             st.N = a.N; st.Hin = a.Hin; st.Win = a.Win; st.Cin = a.C; st.Ho = a.Ho; st.Wo = a.Wo; st.Cout = a.C;
             st.kh = a.kh; st.kw = a.kw; st.sh = a.sh; st.sw = a.sw; st.ph = a.ph; st.pw = a.pw; st.dh = a.dh; st.dw = a.dw;

@@ -5,7 +5,7 @@ import torch
 
 import lop_inputs as li
 import paper_2507_05829_b200 as lop
-from lop_inputs.workloads import Segment, Workload, conv
+from lop_inputs.workloads import Segment, Workload, conv, pool
 from oracle import chain as ochain
 from paper_2507_05829_b200.chain import DeviceChain, to_host_f32
 from test_gpu_parity import TOL, check_workload, one_layer, rel_err
@@ -132,3 +132,20 @@ def test_gathered_stem_layouts(case):
     li.make_input(wl)
     check_workload(wl, flags=lop.LOP_FLAG_REUSE_HALO, modes=("whole", "banded", "pipelined"))
     check_workload(wl, flags=lop.LOP_FLAG_REUSE_HALO | lop.LOP_FLAG_PER_LAYER, modes=("whole", "banded"))
+
+
+# ------------------------------------------------------------------------------------ 3x3 pooling, rows per item
+POOL3_CASES = [  # s, p, C, N, H, W
+    (2, 1, 8, 16, 151, 9),                 # four rows per item, the last item shorter
+    (2, 0, 24, 9, 140, 21),                # two rows per item, no padding
+    (1, 1, 64, 1, 12, 17),                 # one row per item, stride one
+    (3, 1, 16, 16, 230, 7),                # four rows that share nothing
+    (2, 1, 264, 1, 5, 3),                  # more channel vectors than a pass over the threads, columns next to both borders
+]
+
+
+@pytest.mark.parametrize("case", POOL3_CASES)
+def test_pooling_rows_per_item(case):
+    s, p, C, N, H, W = case
+    wl = one_layer(pool(C, 3, s, p=p), N, H, W, n_bands=3)
+    check_workload(wl, flags=lop.LOP_FLAG_REUSE_HALO, modes=("whole", "banded", "pipelined"))
