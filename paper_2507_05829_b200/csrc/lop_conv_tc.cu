@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(TC_THREADS) conv_tc_kernel(const __grid_consta
                         rv[2 * i + 1] = __uint_as_float(rw[i] & 0xFFFF0000u);
                     }
                 }
-                finish16(v, rv, res ? p.res_pos : LOP_RES_NONE, p.act);
+                finish16<2>(v, rv, res ? p.res_pos : LOP_RES_NONE, p.act);
                 uint32_t o[8];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {

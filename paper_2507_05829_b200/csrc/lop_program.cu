@@ -810,9 +810,10 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
     P.fetch_src = fetch_src;
     P.fetch_dst = const_cast<void *>(segs[0].in);
     P.n_fetch = (int)fetch_items.size();
-    P.row_ops = 0;
+    P.row_ops = P.smooth = 0;
     for (const WfStage &st : stages)
         if (st.kind == WF_DWCONV || st.kind == WF_LAYERNORM || st.kind == WF_CONCAT) P.row_ops = 1;
+        else if (st.kind == WF_CONV && (st.act == LOP_ACT_SILU || st.act == LOP_ACT_GELU)) P.smooth = 1;
     // entries in flight: about the link's bandwidth-delay product (some 25 GB/s x 3 us), at least a few warps' worth
     if (P.n_fetch > 0) {
         long long bytes = 0;

@@ -149,44 +149,67 @@ __device__ __forceinline__ float activate_t(float t)
     return t;
 }
 
-// Eight SiLU or GELU values.  Out of line: sixteen inlined evaluations of each, once per place of the residual, are several
-// thousand instructions in the middle of an epilogue that mostly needs none of them.
+// Eight GELU values, out of line: sixteen inlined evaluations are a thousand instructions in the middle of an epilogue that
+// mostly needs none of them.
 struct Float8 { float4 a, b; };
-static __device__ __noinline__ Float8 smooth8(Float8 x, int act)
+static __device__ __noinline__ Float8 gelu8(Float8 x)
 {
     float v[8] = {x.a.x, x.a.y, x.a.z, x.a.w, x.b.x, x.b.y, x.b.z, x.b.w};
-    if (act == LOP_ACT_SILU) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = activate_t<LOP_ACT_SILU>(v[i]);
-    } else {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = activate_t<LOP_ACT_GELU>(v[i]);
-    }
+    for (int i = 0; i < 8; ++i) v[i] = activate_t<LOP_ACT_GELU>(v[i]);
     return Float8{make_float4(v[0], v[1], v[2], v[3]), make_float4(v[4], v[5], v[6], v[7])};
 }
 
-// Last step of the fused epilogue on 16 channels: v = scale*acc + shift already; rv = residual values.
-// res_pos must be LOP_RES_NONE when there is no residual (rv is then not read).
-__device__ __forceinline__ void finish16(float (&v)[16], const float (&rv)[16], int res_pos, int act)
+template <int ACT>
+__device__ __forceinline__ void finish16_t(float (&v)[16], const float (&rv)[16], int res_pos)
 {
     if (res_pos == LOP_RES_PRE_ACT) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] += rv[i];
+        for (int i = 0; i < 16; ++i) v[i] = activate_t<ACT>(__fadd_rn(v[i], rv[i]));
+    } else if (res_pos == LOP_RES_POST_ACT) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = __fadd_rn(activate_t<ACT>(v[i]), rv[i]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = activate_t<ACT>(v[i]);
+    }
+}
+// Last step of the fused epilogue on 16 channels: v = scale*acc + shift already; rv = residual values.
+// res_pos must be LOP_RES_NONE when there is no residual (rv is then not read).  FORM: 0 has neither SiLU nor GELU, 1 has
+// GELU by calls (both for the persistent kernel, whose roles compete for registers and instruction cache), 2 has everything inlined and chosen
+// first (a stand-alone kernel: 51.3 us for a VGG block where form 1 takes 54.2).
+// The additions are kept from being contracted into an activation's last product: both forms give the same bits.
+template <int FORM>
+__device__ __forceinline__ void finish16(float (&v)[16], const float (&rv)[16], int res_pos, int act)
+{
+    if (FORM == 2) {
+        if (act == LOP_ACT_RELU) finish16_t<LOP_ACT_RELU>(v, rv, res_pos);
+        else if (act == LOP_ACT_SILU) finish16_t<LOP_ACT_SILU>(v, rv, res_pos);
+        else if (act == LOP_ACT_GELU) finish16_t<LOP_ACT_GELU>(v, rv, res_pos);
+        else finish16_t<LOP_ACT_NONE>(v, rv, res_pos);
+        return;
+    }
+    if (res_pos == LOP_RES_PRE_ACT) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = __fadd_rn(v[i], rv[i]);
     }
     if (act == LOP_ACT_RELU) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = fmaxf(v[i], 0.0f);
-    } else if (act != LOP_ACT_NONE) {
+        for (int i = 0; i < 16; ++i) v[i] = activate_t<LOP_ACT_RELU>(v[i]);
+    } else if (FORM > 0 && act == LOP_ACT_SILU) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = activate_t<LOP_ACT_SILU>(v[i]);
+    } else if (FORM > 0 && act == LOP_ACT_GELU) {
 #pragma unroll
         for (int h = 0; h < 16; h += 8) {
-            const Float8 f = smooth8(Float8{make_float4(v[h], v[h + 1], v[h + 2], v[h + 3]), make_float4(v[h + 4], v[h + 5], v[h + 6], v[h + 7])}, act);
+            const Float8 f = gelu8(Float8{make_float4(v[h], v[h + 1], v[h + 2], v[h + 3]), make_float4(v[h + 4], v[h + 5], v[h + 6], v[h + 7])});
             v[h] = f.a.x; v[h + 1] = f.a.y; v[h + 2] = f.a.z; v[h + 3] = f.a.w;
             v[h + 4] = f.b.x; v[h + 5] = f.b.y; v[h + 6] = f.b.z; v[h + 7] = f.b.w;
         }
     }
     if (res_pos == LOP_RES_POST_ACT) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] += rv[i];
+        for (int i = 0; i < 16; ++i) v[i] = __fadd_rn(v[i], rv[i]);
     }
 }
 

@@ -555,8 +555,9 @@ __device__ __noinline__ void gather_item(const WfStage *st, int n, int tile_r, i
 }
 
 // FETCH: one more warp per CTA brings the chain input from host memory.  ROWOPS: the program has depth-wise /
-// normalisation / concatenation stages; programs without them run an instantiation that does not carry their code.
-template <bool FETCH, bool ROWOPS>
+// normalisation / concatenation stages, SMOOTH: a convolution of it has SiLU or GELU; programs without them run an
+// instantiation that does not carry their code.
+template <bool FETCH, bool ROWOPS, bool SMOOTH>
 __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavefront_kernel(const WfParams P)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -1252,7 +1253,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                                 rv[2 * i + 1] = __uint_as_float(rw[i] & 0xFFFF0000u);
                             }
                         }
-                        finish16(v, rv, resp ? res_pos : LOP_RES_NONE, act);
+                        finish16<SMOOTH ? 1 : 0>(v, rv, resp ? res_pos : LOP_RES_NONE, act);
                         uint32_t o[8];
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
@@ -1398,11 +1399,14 @@ size_t wavefront_smem_bytes(const WfParams &p)
 namespace {
 
 typedef void (*WfKernel)(const WfParams);
-WfKernel kernel_for(const WfParams &p)
+template <bool FETCH, bool ROWOPS>
+WfKernel with_activations(bool smooth) { return smooth ? wavefront_kernel<FETCH, ROWOPS, true> : wavefront_kernel<FETCH, ROWOPS, false>; }
+WfKernel kernel_for(bool fetch, bool row_ops, bool smooth)
 {
-    if (p.n_fetch > 0) return p.row_ops ? wavefront_kernel<true, true> : wavefront_kernel<true, false>;
-    return p.row_ops ? wavefront_kernel<false, true> : wavefront_kernel<false, false>;
+    if (fetch) return row_ops ? with_activations<true, true>(smooth) : with_activations<true, false>(smooth);
+    return row_ops ? with_activations<false, true>(smooth) : with_activations<false, false>(smooth);
 }
+WfKernel kernel_for(const WfParams &p) { return kernel_for(p.n_fetch > 0, p.row_ops != 0, p.smooth != 0); }
 
 }  // namespace
 
@@ -1432,9 +1436,8 @@ cudaError_t launch_wavefront(const WfParams &p, int grid, cudaStream_t s)
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64 || !configured[dev].load(std::memory_order_acquire)) {
-        WfKernel all[4] = {wavefront_kernel<false, false>, wavefront_kernel<false, true>, wavefront_kernel<true, false>, wavefront_kernel<true, true>};
-        for (WfKernel k : all) {
-            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        for (int k = 0; k < 8; ++k) {
+            e = cudaFuncSetAttribute(kernel_for(k & 4, k & 2, k & 1), cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
             if (e != cudaSuccess) return e;
         }
         if (dev >= 0 && dev < 64) configured[dev].store(true, std::memory_order_release);

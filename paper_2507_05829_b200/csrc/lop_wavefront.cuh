@@ -89,6 +89,7 @@ struct WfParams {
     void *fetch_dst;
     int n_fetch, fetch_window;
     int row_ops;              // the program has WF_DWCONV / WF_LAYERNORM / WF_CONCAT stages
+    int smooth;               // a convolution of the program is activated by SiLU or GELU
 };
 
 #ifndef LOP_WF_WORKER_WARPS
