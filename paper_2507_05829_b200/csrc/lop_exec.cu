@@ -185,7 +185,7 @@ int prepare_workspace(lop_plan_t *pl, void *ws, cudaStream_t s)
         LayerInfo &li = pl->layers[i];
         if (!li.stem_gather && !li.dw_transposed) continue;
         if (!fresh && e->prepared_w[i] == li.l.weight) continue;
-        if (li.stem_gather) LOP_CUDA(launch_stem_weights(li.l.weight, base + li.wpad_off, li.l.cout, li.l.kh, li.l.kw, li.l.cin, li.stem_shared ? li.stem_c : 0, li.cin_eff, s));
+        if (li.stem_gather) LOP_CUDA(launch_stem_weights(stem_weights_args(pl, i, ws), s));
         else LOP_CUDA(launch_dw_transpose(li.l.weight, base + li.wpad_off, li.l.cin, li.l.kh * li.l.kw, s));
         e->prepared_w[i] = li.l.weight;
         e->launches++;

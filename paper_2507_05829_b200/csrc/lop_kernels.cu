@@ -136,39 +136,43 @@ __global__ void __launch_bounds__(256) maxpool_bf16x8_kernel(PoolArgs p)
 // Patch gather for a thin chain input, rows [lo, hi) of the patch tensor (see lop_gather.cuh).
 // One thread per 16-byte group of eight patch elements: consecutive threads write consecutive
 // 16 bytes, reads hit the few image rows of the band in L1/L2.  HBM-bound on the write.
+// The same launch brings the convolution's weights into the order of the gathered values where wp is given (a launch of
+// its own costs two microseconds for a few kilobytes).
 // ---------------------------------------------------------------------------------------------
+__device__ __forceinline__ void stem_weights(const StemWeights &g, int first, int stride)
+{
+    const int total = g.cout * g.K, taps_c = g.kh * g.kw * g.C;
+    for (int i = first; i < total; i += stride) {
+        const int k = i % g.K, co = i / g.K;
+        int src = k < taps_c ? k : -1;
+        if (g.col) {
+            const int b = k / g.col, r = k - b * g.col, a = r / g.C;
+            src = b < g.kw && a < g.kh ? (a * g.kw + b) * g.C + (r - a * g.C) : -1;
+        }
+        static_cast<uint16_t *>(g.wp)[i] = src >= 0 ? static_cast<const uint16_t *>(g.w)[co * taps_c + src] : (uint16_t)0;
+    }
+}
+
+template <typename Index>
 __global__ void __launch_bounds__(256) stem_gather_kernel(const uint16_t *__restrict__ x, uint16_t *__restrict__ y,
-                                                          GatherGeom g, int lo, int hi, unsigned *dbg)
+                                                          GatherGeom g, int lo, int hi, StemWeights wt, unsigned *dbg)
 {
     const int k8n = g.Kcol >> 3;
-    const long long total = (long long)g.N * (hi - lo) * g.Wo * k8n;
-    for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int k8 = (int)(idx % k8n);
-        long long q = idx / k8n;
-        const int ow = (int)(q % g.Wo);
-        q /= g.Wo;
-        const int oh = lo + (int)(q % (hi - lo));
-        const int n = (int)(q / (hi - lo));
+    const Index total = (Index)g.N * (hi - lo) * g.Wo * k8n;
+    for (Index idx = (Index)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (Index)gridDim.x * blockDim.x) {
+        Index q = idx / k8n;
+        const int k8 = (int)(idx - q * k8n);
+        const Index row = q / g.Wo;
+        const int ow = (int)(q - row * g.Wo);
+        const int n = (int)(row / (hi - lo)), oh = lo + (int)(row - (Index)n * (hi - lo));
         const uint4 v = gather8<false>(x, g, n, oh, ow, k8);        // reads in-bounds taps only, by construction of the patch
         const long long yo = (((long long)n * g.Ho + oh) * g.Wo + ow) * g.Kcol + k8 * 8;
         if (dbg_in_bounds(dbg, yo, 8, (long long)g.N * g.Ho * g.Wo * g.Kcol)) *reinterpret_cast<uint4 *>(y + yo) = v;
     }
+    if (wt.wp) stem_weights(wt, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
-__global__ void stem_weights_kernel(const uint16_t *__restrict__ w, uint16_t *__restrict__ wp, int cout, int kh, int kw, int C, int col, int K)
-{
-    const int total = cout * K, taps_c = kh * kw * C;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-        const int k = i % K, co = i / K;
-        int src = k < taps_c ? k : -1;
-        if (col) {
-            const int b = k / col, r = k - b * col, a = r / C;
-            src = b < kw && a < kh ? (a * kw + b) * C + (r - a * C) : -1;
-        }
-        wp[i] = src >= 0 ? w[co * taps_c + src] : (uint16_t)0;
-    }
-}
+__global__ void stem_weights_kernel(StemWeights wt) { stem_weights(wt, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x); }
 
 // ---------------------------------------------------------------------------------------------
 // The transfer step for plans that run on per-layer kernels: rows of the chain input, read straight from page-locked host
@@ -233,12 +237,17 @@ cudaError_t launch_maxpool(const PoolArgs &a, int dtype, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_stem_gather(const void *x, void *y, const GatherGeom &g, int lo, int hi, cudaStream_t s, unsigned *dbg)
+cudaError_t launch_stem_gather(const void *x, void *y, const GatherGeom &g, int lo, int hi, cudaStream_t s, unsigned *dbg, const StemWeights &wt)
 {
     if (hi <= lo) return cudaSuccess;
     if (g.Kcol % 8 != 0) return cudaErrorInvalidValue;
     const long long work = (long long)g.N * (hi - lo) * g.Wo * (g.Kcol / 8);
-    stem_gather_kernel<<<grid_for(work, 256), 256, 0, s>>>(static_cast<const uint16_t *>(x), static_cast<uint16_t *>(y), g, lo, hi, dbg);
+    const int blocks = grid_for(work, 256);
+    const uint16_t *xi = static_cast<const uint16_t *>(x);
+    uint16_t *yi = static_cast<uint16_t *>(y);
+    // (a 64-bit division is a routine of several dozen instructions, and a thread has four of them)
+    if (work < (1LL << 30)) stem_gather_kernel<int><<<blocks, 256, 0, s>>>(xi, yi, g, lo, hi, wt, dbg);
+    else stem_gather_kernel<long long><<<blocks, 256, 0, s>>>(xi, yi, g, lo, hi, wt, dbg);
     return cudaGetLastError();
 }
 
@@ -257,10 +266,9 @@ cudaError_t launch_fetch_rows(const void *src, void *dst, int N, int rows, long 
     return cudaGetLastError();
 }
 
-cudaError_t launch_stem_weights(const void *w, void *wp, int cout, int kh, int kw, int C, int col, int K, cudaStream_t s)
+cudaError_t launch_stem_weights(const StemWeights &wt, cudaStream_t s)
 {
-    stem_weights_kernel<<<grid_for((long long)cout * K, 256), 256, 0, s>>>(static_cast<const uint16_t *>(w), static_cast<uint16_t *>(wp), cout, kh, kw,
-                                                                           C, col, K);
+    stem_weights_kernel<<<grid_for((long long)wt.cout * wt.K, 256), 256, 0, s>>>(wt);
     return cudaGetLastError();
 }
 

@@ -26,6 +26,16 @@ inline GatherGeom gather_geom(const lop_plan_t *pl, int i)
     return g;
 }
 
+inline StemWeights stem_weights_args(const lop_plan_t *pl, int i, void *ws)
+{
+    const LayerInfo &li = pl->layers[i];
+    StemWeights t;
+    t.w = li.l.weight; t.wp = static_cast<char *>(ws) + li.wpad_off;
+    t.cout = li.l.cout; t.kh = li.l.kh; t.kw = li.l.kw; t.C = li.l.cin; t.K = li.cin_eff;
+    t.col = li.stem_shared ? li.stem_c : 0;
+    return t;
+}
+
 // Convolution layer i over output rows [lo, hi).  A tensor-core layer is described the way its kernel
 // sees it: a gathered stem is a pointwise convolution over the gathered tensor with zero-padded weights.
 inline ConvArgs conv_args(const lop_plan_t *pl, int i, const void *in, void *out, void *ws, int lo, int hi)
