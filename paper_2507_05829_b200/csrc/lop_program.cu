@@ -481,12 +481,25 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
     bool uses_flags = false;
     uint32_t unit_bytes = 1024, stg_bytes = 0;
     // scratch of the SIMT items, and with it what the operand ring has at least
-    // Rows of one gather or pooling item: an item's fixed cost (about 2 us: its dependencies, the loads' latency, the
-    // hand-over) is shared by as many rows as leave two items per SM, and the rows of a window are loaded fewer times.
-    auto rows_per_item = [](long long all) { return all >= 8 * 148 ? 4 : (all >= 4 * 148 ? 2 : 1); };
+    // Rows of one gather or pooling item: an item's fixed cost (about 1.5 us: its dependencies, the loads' latency, the
+    // hand-over) is shared by its rows, and the rows of a window are loaded fewer times, but the items have to go round 148
+    // SMs.  A row costs about 1 us per 600 vectors of 16 bytes written (measured at 32 images of 112x230x24).  Where the
+    // input is still arriving, larger items hold up the rows behind them: several rows only where there are many items
+    // (a ResNet-50 of batch 8 streamed: 490 us so, 527 with four rows).
+    bool arriving = cx.raw >= 0;
+    for (const StageReq &rq : reqs) arriving = arriving || rq.wait_arrival;
+    auto rows_per_item = [arriving](long long all, double row_us) {
+        if (arriving) return all >= 8 * 148 ? 4 : (all >= 4 * 148 ? 2 : 1);
+        int best = 1;
+        auto time = [&](int r) { return (double)((all + 148LL * r - 1) / (148LL * r)) * (1.5 + row_us * r); };
+        for (int r = 2; r <= 4; r *= 2)
+            if (time(r) < time(best)) best = r;
+        return best;
+    };
+    auto row_us = [](long long w, long long c) { return (double)(w * c / 8) / 600.0; };
     auto gather_scratch = [&](const lop_plan_t *pl, int layer, int *rows) {
         const GatherGeom g = gather_geom(pl, layer);
-        *rows = rows_per_item((long long)g.N * g.Ho);
+        *rows = rows_per_item((long long)g.N * g.Ho, row_us(g.Wo, g.Kcol));
         // the image rows they read are staged in shared memory when they fit, else read in place
         auto bytes = [&](int r) { return (long long)gather_rows_in(g, r) * gather_pitch(g) + 4 * g.kh * g.kw * g.C; };
         while (*rows > 1 && bytes(*rows) > 20 * 1024) *rows /= 2;
@@ -542,7 +555,7 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
             st.kh = gg.kh; st.kw = gg.kw; st.sh = gg.sh; st.sw = gg.sw; st.ph = gg.ph; st.pw = gg.pw; st.dh = gg.dh; st.dw = gg.dw;
             st.mode = gather_scratch(pl, rq.layer, &group_rows) ? 0 : 1;
             st.tr_log = ilog2i(group_rows);
-            item_us = 1.0 + 0.9 * group_rows;
+            item_us = 1.5 + group_rows * row_us(gg.Wo, gg.Kcol);
             tiles_r = (rows + group_rows - 1) / group_rows;
         } else if (l.op == LOP_MAXPOOL2D) {
             const PoolArgs a = pool_args(pl, rq.layer, in, out, ws, rq.lo, rq.hi);
@@ -550,10 +563,10 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
             // 3x3 windows: several rows per item where they leave two items per SM (a window's rows are loaded fewer times, and
             // an item's fixed cost is shared); st.mode says which of the two pooling routines runs
             st.mode = a.kh == 3 && a.kw == 3 && a.dh == 1 && a.dw == 1;
-            if (st.mode) group_rows = rows_per_item((long long)a.N * a.Ho);
+            if (st.mode) group_rows = rows_per_item((long long)a.N * a.Ho, row_us(a.Wo, a.C));
             st.tr_log = ilog2i(group_rows);
             tiles_r = (rows + group_rows - 1) / group_rows;
-            item_us = st.mode ? 1.5 + group_rows : 3.4;
+            item_us = st.mode ? 1.5 + group_rows * row_us(a.Wo, a.C) : 3.4;
             st.x = a.x; st.y = a.y;
             st.N = a.N; st.Hin = a.Hin; st.Win = a.Win; st.Cin = a.C; st.Ho = a.Ho; st.Wo = a.Wo; st.Cout = a.C;
             st.kh = a.kh; st.kw = a.kw; st.sh = a.sh; st.sw = a.sw; st.ph = a.ph; st.pw = a.pw; st.dh = a.dh; st.dw = a.dw;
