@@ -273,26 +273,31 @@ __device__ __forceinline__ void fetch_bytes(const uint8_t *src, uint8_t *dst, in
 {
     int head = (16 - (int)(reinterpret_cast<uintptr_t>(src) & 15)) & 15;
     if (head > len) head = len;
-    for (int i = 2 * lane; i < head; i += 64)
-        *reinterpret_cast<uint16_t *>(dst + i) = __ldcv(reinterpret_cast<const uint16_t *>(src + i));
-    const int nvec = (len - head) >> 4;
+    const int nvec = (len - head) >> 4, tail = head + (nvec << 4);
+    // elements before the first and behind the last 16-byte boundary: lanes 0..7 and 8..15, on their way with the vectors
+    const int edge = lane < 8 ? 2 * lane : tail + 2 * (lane - 8);
+    const bool has_edge = lane < 16 && edge < (lane < 8 ? head : len);
+    uint16_t edge_value = 0;
+    if (has_edge) edge_value = __ldcv(reinterpret_cast<const uint16_t *>(src + edge));
     const uint4 *s4 = reinterpret_cast<const uint4 *>(src + head);
     uint4 *d4 = reinterpret_cast<uint4 *>(dst + head);
-    for (int v0 = 0; v0 < nvec; v0 += FETCH_DEPTH * 32) {
+    // A warp's loads start at 128-byte lines of the source.  (Rows of 4656 bytes, read from where they start, came at 11 GB/s
+    // for the lines that two loads shared, from line starts at twice that and more: a 674x777 stack streamed 457 -> 278 us.)
+    const int skew = (int)(reinterpret_cast<uintptr_t>(s4) & 127) >> 4;
+    for (int v0 = -skew; v0 < nvec; v0 += FETCH_DEPTH * 32) {
         uint4 q[FETCH_DEPTH];
 #pragma unroll
         for (int u = 0; u < FETCH_DEPTH; ++u) {
             const int v = v0 + u * 32 + lane;
-            if (v < nvec) q[u] = __ldcv(s4 + v);
+            if (v >= 0 && v < nvec) q[u] = __ldcv(s4 + v);
         }
 #pragma unroll
         for (int u = 0; u < FETCH_DEPTH; ++u) {
             const int v = v0 + u * 32 + lane;
-            if (v < nvec) d4[v] = q[u];
+            if (v >= 0 && v < nvec) d4[v] = q[u];
         }
     }
-    for (int i = head + (nvec << 4) + 2 * lane; i < len; i += 64)
-        *reinterpret_cast<uint16_t *>(dst + i) = __ldcv(reinterpret_cast<const uint16_t *>(src + i));
+    if (has_edge) *reinterpret_cast<uint16_t *>(dst + edge) = edge_value;
 }
 
 // The functions below are kept out of line: inlined, they cost the epilogue's path registers and instruction cache (a

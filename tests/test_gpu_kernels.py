@@ -149,3 +149,11 @@ def test_pooling_rows_per_item(case):
     s, p, C, N, H, W = case
     wl = one_layer(pool(C, 3, s, p=p), N, H, W, n_bands=3)
     check_workload(wl, flags=lop.LOP_FLAG_REUSE_HALO, modes=("whole", "banded", "pipelined"))
+
+
+# ------------------------------------------------------------------------------------ input fetched by the persistent kernel
+@pytest.mark.parametrize("W", [1, 5, 8, 171, 777, 1000])
+def test_fetched_rows_of_any_alignment(W):
+    """Rows that start anywhere in a 128-byte line, shorter and longer than what a warp has in flight."""
+    wl = one_layer(conv(3, 16, 3, act=li.ACT_RELU), 2, 11, W)
+    check_workload(wl, flags=lop.LOP_FLAG_REUSE_HALO, modes=("pipelined",))
