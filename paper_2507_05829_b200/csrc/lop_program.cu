@@ -9,6 +9,7 @@
 #include <cmath>
 #include <cstdio>
 #include <map>
+#include <numeric>
 #include <vector>
 
 #include "lop_internal.h"
@@ -758,26 +759,49 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
     std::map<int, long long> tiles_of;                            // convolution tiles per weight map: the layer's stages together
     for (const int4 &it : items)
         if (stages[it.x & 0xFFFF].kind == WF_CONV) ++tiles_of[stages[it.x & 0xFFFF].map_base];
+    auto slot = [](uint32_t bytes) { return round_up_u32(bytes, 1024u); };
+    std::map<uint32_t, uint32_t> box_step;                        // slab stages that share a cut of the ring: divisor of their weight boxes
+    for (WfStage &st : stages) {
+        if (st.kind != WF_CONV) continue;
+        const uint32_t a_sz = slot(st.a_bytes), b_sz = slot(st.b_bytes);
+        // Weights stay in shared memory from tile to tile where every CTA gets at least two tiles of the layer, always of
+        // the same output channels (items go round-robin), and they leave room for two activation boxes and a full entry (a
+        // ResNet-50 of four 640x1152 images, whose gather leaves the ring 112 KB: 1602 us so, 1611 with 64 KB of weights kept
+        // beside entries of two boxes).
+        const uint32_t boxes = (uint32_t)st.n_chunks * ((st.n_taps + st.tb - 1) / st.tb);
+        const uint32_t beside = std::max(2u * a_sz, st.mode == WF_TAP ? LOP_ENTRY_BYTES / a_sz * a_sz : 0u);
+        const int cout_tiles = st.Cout / st.BN;
+        if (boxes * b_sz <= LOP_KEEP_BYTES && boxes * b_sz + beside <= ring_bytes && 148 % cout_tiles == 0 && tiles_of[st.map_base] >= 2 * 148)
+            st.keep_bytes = (int)(boxes * b_sz);
+        if (2u * a_sz + b_sz > ring_bytes) { delete p; set_error("tile buffers do not fit shared memory"); return LOP_EUNSUPPORTED; }
+        if (st.mode == WF_SLAB && !st.keep_bytes) box_step[a_sz] = std::gcd(box_step[a_sz], b_sz);
+    }
     for (WfStage &st : stages) {
         st.cps = 1;
         if (st.kind != WF_CONV) continue;
-        const uint32_t a_sz = round_up_u32(st.a_bytes, 1024u), b_sz = round_up_u32(st.b_bytes, 1024u);
-        // Weights stay in shared memory from tile to tile where every CTA gets at least two tiles of the layer, always of
-        // the same output channels (items go round-robin), and they leave room for two activation boxes.
-        const uint32_t boxes = (uint32_t)st.n_chunks * ((st.n_taps + st.tb - 1) / st.tb);
-        const int cout_tiles = st.Cout / st.BN;
-        if (boxes * b_sz <= LOP_KEEP_BYTES && boxes * b_sz + 2u * a_sz <= ring_bytes && 148 % cout_tiles == 0 && tiles_of[st.map_base] >= 2 * 148)
-            st.keep_bytes = (int)(boxes * b_sz);
-        if (2u * a_sz + b_sz > ring_bytes) { delete p; set_error("tile buffers do not fit shared memory"); return LOP_EUNSUPPORTED; }
+        const uint32_t a_sz = slot(st.a_bytes), b_sz = slot(st.b_bytes);
+        // what the stage's entries share: the ring without the kept weights, or without a slab stage's activation boxes
+        const uint32_t lim = ring_bytes - (st.keep_bytes ? (uint32_t)st.keep_bytes : (st.mode == WF_SLAB ? 2u * a_sz : 0u));
         if (st.mode == WF_SLAB && !st.keep_bytes) {
             // weight boxes per full barrier: the issuing thread stalls at every wait, so it waits once per chunk where the
             // chunk's weights fit the ring with room for part of the next chunk's
             const int per_chunk = (st.n_taps + st.tb - 1) / st.tb;
-            const uint32_t most = std::max(b_sz, (ring_bytes - 2u * a_sz) * 7u / 10u);
+            const uint32_t most = std::max(b_sz, lim * 7u / 10u);
             const int groups = (int)((per_chunk * b_sz + most - 1) / most);
-            st.cps = std::min((per_chunk + groups - 1) / groups, (int)(most / b_sz));
+            st.cps = std::min({(per_chunk + groups - 1) / groups, (int)(most / b_sz), WF_ENTRIES});
+            // The loader places a group's boxes before any of them can be consumed.  A box does not straddle the ring's end,
+            // and boxes start at multiples of the divisor of all sizes in this cut: what is skipped there and the group
+            // have to fit together.
+            while (st.cps > 1 && (st.cps + 1) * b_sz - box_step[a_sz] > lim) --st.cps;
         }
-        if (st.mode == WF_TAP) st.cps = std::max(1, (int)(LOP_ENTRY_BYTES / (st.keep_bytes ? a_sz : a_sz + b_sz)));
+        if (st.mode == WF_TAP) {
+            const uint32_t step = st.keep_bytes ? a_sz : a_sz + b_sz;
+            st.cps = (int)std::max(1u, std::min<uint32_t>(LOP_ENTRY_BYTES, lim) / step);
+        }
+        // (an entry larger than its ring would be waited for in vain)
+        const uint32_t entry = st.keep_bytes ? (st.mode == WF_TAP ? (uint32_t)st.cps * a_sz : a_sz)
+                                             : (uint32_t)st.cps * (st.mode == WF_TAP ? a_sz + b_sz : b_sz);
+        if (entry > lim) { delete p; set_error("an operand ring entry of %u bytes does not fit %u", entry, lim); return LOP_EUNSUPPORTED; }
     }
 
 #ifdef LOP_WF_TRACE

@@ -107,6 +107,45 @@ def test_operand_ring_cuts_and_output_units(case):
         assert np.array_equal(to_host_f32(host), want)
 
 
+def _stack(layers, N, H, W, n_bands=3):
+    for i, l in enumerate(layers):
+        l.input_from = i - 1
+    wl = Workload("stack", "bf16", N, H, W, layers[0].cin, [Segment(layers, n_bands)], seed=31)
+    li.fill_parameters(wl)
+    li.make_input(wl)
+    return wl
+
+
+@pytest.mark.parametrize("name", ["kept weights beside a wide image's gather scratch", "more boxes per chunk than entries"])
+def test_operand_rings_with_little_room(name):
+    """Rings that hold less than a full entry beside what is cut off them (tests/test_host_side.py walks them without a GPU)."""
+    if name.startswith("kept"):
+        wl = _stack([conv(3, 64, 7, s=2), conv(64, 32, 1), conv(32, 256, 3)], 1, 80, 1150)
+    else:
+        l = conv(512, 16, 1)
+        l.kh, l.ph = 17, 8
+        wl = _stack([l], 1, 26, 200)
+    check_workload(wl, flags=lop.LOP_FLAG_REUSE_HALO, modes=("whole", "banded", "pipelined"))
+
+
+def test_wide_resnet50_is_the_same_by_both_executors():
+    """1152 columns: the gather's scratch takes 48 KB of the operand ring."""
+    wl = li.build("resnet50", N=1, H=640, W=1152)
+    outs = []
+    for flags in (lop.LOP_FLAG_REUSE_HALO, lop.LOP_FLAG_REUSE_HALO | lop.LOP_FLAG_PER_LAYER):
+        dc = DeviceChain(wl, flags=flags)
+        dc.run_banded(dc.input_tensor())
+        torch.cuda.synchronize()
+        dc.check_device()
+        outs.append(dc.outs[-1].clone())
+        if not flags & lop.LOP_FLAG_PER_LAYER:
+            dc.run_pipelined(dc.pinned_input())
+            torch.cuda.synchronize()
+            dc.check_device()
+            assert torch.equal(dc.outs[-1], outs[0])
+    assert torch.equal(outs[0], outs[1])
+
+
 # ------------------------------------------------------------------------------------ gathered stems
 STEM_CASES = [  # k, s, p, dilation, cin, cout, N, H, W
     (7, 2, 3, 1, 3, 64, 16, 150, 21),      # shared columns, four rows per gather item, a last item of three
