@@ -146,6 +146,25 @@ def test_wide_resnet50_is_the_same_by_both_executors():
     assert torch.equal(outs[0], outs[1])
 
 
+def test_units_that_workers_copy_out_are_taken_by_residual_loads():
+    """Folded poolings and host output leave their units by the workers; residuals then arrive in the same units by bulk loads.
+    Some seven tiles of each layer per CTA, four units."""
+    layers = [conv(64, 64, 3, act=li.ACT_RELU), pool(64, 2, 2, 0), conv(64, 64, 1, act=li.ACT_RELU), conv(64, 64, 3, act=li.ACT_NONE)]
+    wl = _stack(layers, 4, 368, 368, n_bands=8)
+    layers[3].residual_from, layers[3].residual_pos = 1, li.RES_PRE_ACT
+    ref = DeviceChain(wl, flags=lop.LOP_FLAG_REUSE_HALO | lop.LOP_FLAG_PER_LAYER)
+    want = ref.run_banded(ref.input_tensor()).cpu()
+    dc = DeviceChain(wl, flags=lop.LOP_FLAG_REUSE_HALO)
+    x = dc.pinned_input()
+    host = torch.zeros(dc.outs[-1].shape, dtype=dc.outs[-1].dtype).pin_memory()
+    for _ in range(4):
+        host.zero_()
+        dc.run_pipelined(x, out_pinned=host)
+        torch.cuda.synchronize()
+        dc.check_device()
+        assert torch.equal(host, want)
+
+
 # ------------------------------------------------------------------------------------ gathered stems
 STEM_CASES = [  # k, s, p, dilation, cin, cout, N, H, W
     (7, 2, 3, 1, 3, 64, 16, 150, 21),      # shared columns, four rows per gather item, a last item of three
