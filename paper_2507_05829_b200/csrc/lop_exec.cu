@@ -63,7 +63,6 @@ struct ExecState {
     int copies = 0;                                            // async copies enqueued by it
     bool timing_valid = false;
     bool copies_timed = false;                                 // per-band copy events were recorded by the last pipelined run
-    const void *mapped_host = nullptr, *mapped_dev = nullptr;  // last host buffer looked up and its device-side address (or nullptr)
     std::vector<char> copy_issued;
 };
 
@@ -522,22 +521,17 @@ int get_program(lop_plan_t *pl, int kind, const void *in, void *out, void *ws, P
 }
 
 // The address under which the device reads the host buffer, when it can (page-locked memory is mapped into the
-// unified address space) and the plan does not insist on the copy engine; nullptr otherwise.
-const void *fetchable(lop_plan_t *pl, const void *host)
+// unified address space) and the plan does not insist on the copy engine; nullptr otherwise.  Looked up by every call
+// (0.1 us): a buffer that was page-locked may have been freed since, and its address be an ordinary allocation's now.
+const void *fetchable(const lop_plan_t *pl, const void *host)
 {
     if (pl->flags & LOP_FLAG_COPY_ENGINE) return nullptr;
-    ExecState *e = pl->exec;
-    if (e->mapped_host == host) return e->mapped_dev;
     cudaPointerAttributes at{};
-    const void *dev = nullptr;
-    if (cudaPointerGetAttributes(&at, host) == cudaSuccess) {
-        if (at.type == cudaMemoryTypeHost && at.devicePointer) dev = at.devicePointer;
-    } else {
+    if (cudaPointerGetAttributes(&at, host) != cudaSuccess) {
         cudaGetLastError();                                  // an unknown pointer is no error here: it gets copies
+        return nullptr;
     }
-    e->mapped_host = host;
-    e->mapped_dev = dev;
-    return dev;
+    return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
 }
 
 int run_program(lop_plan_t *pl, int kind, const void *in, void *out, void *ws, cudaStream_t s)

@@ -71,6 +71,8 @@ class Chain:
 
     def pipelined(self, host_out=None):
         outs = self.outs[:-1] + [host_out or self.outs[-1]]
+        if len(self.plans) == 1:
+            return self.plans[0].run_pipelined(HOST, self.staging, outs[0], self.ws[0], None)
         binding.run_chain_pipelined(self.plans, HOST, self.staging, outs, self.ws, None)
 
 
@@ -118,3 +120,21 @@ def test_a_group_of_boxes_fits_the_rings_entries(host):
     l.kh, l.ph, l.input_from = 17, 8, -1
     wl = Workload("column", "bf16", 1, 26, 200, 512, [Segment([l], 2), Segment([conv(16, 16, 1, input_from=-1)], 1)])
     check_rings(host, wl)
+
+
+# ------------------------------------------------------------------------------------ the streamed input's transport
+def commands(host, run):
+    """The stream commands and launches of one call, as (command, stream, ...) tuples."""
+    host.lib.host_side_clear()
+    run()
+    return [tuple(line.split()) for line in host.lib.host_side_log().decode().splitlines()]
+
+
+@pytest.mark.parametrize("name", ["single_conv", "vgg_block", "resnet18"])
+def test_an_address_that_is_no_longer_page_locked_is_copied_from(host, name):
+    """The same address, page-locked, then an ordinary allocation's, then page-locked again: fp32, bf16, a chain of plans."""
+    c = host.chain(li.build(name, with_data=False))
+    for pinned in (True, False, True):
+        host.lib.host_side_pin(HOST, (1 << 30) if pinned else 0)
+        copies = [x for x in commands(host, c.pipelined) if x[0] == "copy"]
+        assert bool(copies) == (not pinned), (name, pinned)
