@@ -217,8 +217,9 @@ int lop_fetch_band(lop_plan_t *plan, int band, const void *in_host_pinned, void 
  *     cudaHostRegister memory is): the persistent kernel itself reads each band's rows from host memory
  *     and stores them to staging_dev -- fetch stages that precede the band's first operator in the
  *     dependency graph, spread over the SMs -- so the whole request is ONE launch on the caller's stream
- *     with no copy, event or flag command at all (plans that run on per-layer kernels: one launch that
- *     brings the rows, then one per layer);
+ *     with no copy, event or flag command at all.  Plans that run on per-layer kernels: one launch that
+ *     brings the rows, then one per layer; an input of 8 MB or more comes in two pieces, of 32 MB or more in
+ *     four, each some neighbouring bands copied on the side stream with the layers' launches behind it;
  *   - copy engine (LOP_FLAG_COPY_ENGINE, unmapped host memory, or per-layer plans that are timed or
  *     checked): one asynchronous copy per band on the plan's side stream, forked and joined by CUDA events;
  *     a band's arrival is a 4-byte stream-ordered write behind its copy that the persistent kernel polls

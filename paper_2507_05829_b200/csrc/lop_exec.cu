@@ -271,19 +271,21 @@ int first_row(const lop_plan_t *pl, int block_lo, int band, int i)
     return std::min(std::max((int)r.out_lo, done), (int)r.out_hi);
 }
 
-// Operation batching (Sec. IV-C): with the whole input on the device, the bands' operations at a layer are one
-// contiguous run of rows (neighbouring bands' ranges touch or overlap), so each layer is ONE launch over the hull of
-// the bands' rows.  Every row is computed once, with the same bits as band by band.
-int run_batched_impl(lop_plan_t *pl, const void *in, void *out, void *ws, cudaStream_t s)
+// Operation batching (Sec. IV-C): with their input on the device, the operations of bands [b0, b1) at a layer are one
+// contiguous run of rows (neighbouring bands' ranges touch or overlap), so each layer is ONE launch over the hull of the
+// bands' rows, without those that bands before b0 have computed.  Every row is computed once, with the same bits as band by
+// band.
+int run_batched_impl(lop_plan_t *pl, int b0, int b1, const void *in, void *out, void *ws, cudaStream_t s)
 {
     const int L = (int)pl->layers.size();
     int rc = LOP_OK;
     for (int i = 0; i < L; ++i) {
-        int lo = 0, hi = 0;
+        int lo = 0, hi = 0, done = 0;
         bool any = false, contiguous = true;
-        for (int b = 0; b < pl->n_bands; ++b) {
+        for (int b = 0; b < b1; ++b) {
             const lop_range &r = pl->ranges[(size_t)b * L + i];
             if (r.out_hi <= r.out_lo) continue;
+            if (b < b0) { done = std::max(done, (int)r.out_hi); continue; }
             if (any && r.out_lo > hi) contiguous = false;
             lo = any ? std::min(lo, (int)r.out_lo) : (int)r.out_lo;
             hi = any ? std::max(hi, (int)r.out_hi) : (int)r.out_hi;
@@ -291,9 +293,9 @@ int run_batched_impl(lop_plan_t *pl, const void *in, void *out, void *ws, cudaSt
         }
         if (!any) continue;
         if (contiguous) {
-            if ((rc = run_layer(pl, i, lo, hi, in, out, ws, s, -1)) != LOP_OK) return rc;
+            if ((rc = run_layer(pl, i, std::max(lo, done), hi, in, out, ws, s, -1)) != LOP_OK) return rc;
         } else {
-            for (int b = 0; b < pl->n_bands; ++b) {
+            for (int b = b0; b < b1; ++b) {
                 const lop_range &r = pl->ranges[(size_t)b * L + i];
                 if ((rc = run_layer(pl, i, first_row(pl, 0, b, i), r.out_hi, in, out, ws, s, -1)) != LOP_OK) return rc;
             }
@@ -574,22 +576,68 @@ int copy_rows_impl(lop_plan_t *pl, int lo, int hi, const void *host, void *stagi
     return LOP_OK;
 }
 
+// The rows that bands [b0, b1) need and no earlier band has brought: one contiguous run.  false: none.
+bool new_input_rows(const lop_plan_t *pl, int b0, int b1, int *lo, int *hi)
+{
+    *lo = *hi = 0;
+    for (int b = b0; b < b1; ++b) {
+        const lop_range &need = pl->in_need[b];
+        if (need.out_hi <= need.new_lo) continue;
+        *lo = *hi > *lo ? std::min(*lo, (int)need.new_lo) : (int)need.new_lo;
+        *hi = std::max(*hi, (int)need.out_hi);
+    }
+    return *hi > *lo;
+}
+
 // The transfer step of plans without a persistent program: the rows band `band` needs and no earlier band has brought, or
 // (band == -1) the rows any band needs, by one launch.
 int fetch_rows_impl(lop_plan_t *pl, int band, const void *src, void *staging, cudaStream_t s)
 {
-    int lo = 0, hi = 0;
-    for (int b = band < 0 ? 0 : band; b < (band < 0 ? pl->n_bands : band + 1); ++b) {
-        const lop_range &need = pl->in_need[b];
-        if (need.out_hi <= need.new_lo) continue;
-        lo = hi > lo ? std::min(lo, (int)need.new_lo) : (int)need.new_lo;
-        hi = std::max(hi, (int)need.out_hi);
-    }
+    int lo, hi;
+    const bool any = new_input_rows(pl, band < 0 ? 0 : band, band < 0 ? pl->n_bands : band + 1, &lo, &hi);
     for (int b = 0; b < pl->n_bands; ++b) pl->exec->copy_issued[b] = 0;
     pl->exec->copies_timed = false;
-    if (hi <= lo) return LOP_OK;
+    if (!any) return LOP_OK;
     LOP_CUDA(launch_fetch_rows(src, staging, pl->N, pl->H, (long long)pl->W * pl->C * elem_size(pl->dtype), lo, hi, s));
     pl->exec->launches++;
+    return LOP_OK;
+}
+
+// Into how many pieces a streamed run of the per-layer kernels cuts its input, at band borders.  One: a launch that reads host
+// memory brings all rows and every layer is one launch behind it; a copy, its event and a partial launch per layer would cost
+// more than they hide.  More: neighbouring bands are joined, all copies are queued on the side stream, and a piece's layers
+// follow its arrival.  Measured in fp32, one piece / two / four, microseconds:
+//                                   4 MB              8 MB              16 MB               32 MB
+//   3x3 convolution 16->16    126 / 110 / 111   234 / 207 / 196   458 / 383 / 363    904 /  746 /  694
+//   two 3x3 (3->16) and pool  328 / 333 / 338   635 / 580 / 607  1250 / 1100 / 1062  2475 / 2170 / 2029
+//   eight 3x3 8->8            350 / 368 / 447   644 / 615 / 657  1242 / 1128 / 1154  2438 / 2147 / 2094
+//   2x2 pooling                93 /  94 / 103   178 / 171 / 180   350 / 323 / 331    693 /  625 /  633
+// (A copy per band, 16 bands: 1423 us for a 3x3 convolution of 64 MB, four pieces 1361; 1078 and 809 for the second at 12 MB.)
+int input_pieces(const lop_plan_t *pl)
+{
+    const size_t bytes = lop_plan_staging_bytes(pl);
+    return std::min(pl->n_bands, bytes < (8u << 20) ? 1 : (bytes < (32u << 20) ? 2 : 4));
+}
+
+// Sec. IV-B's pipeline with per-layer kernels: see input_pieces.
+int run_pieces_impl(lop_plan_t *pl, int pieces, const void *host, void *staging, void *out, void *ws, cudaStream_t s)
+{
+    ExecState *e = pl->exec;
+    int rc = LOP_OK, lo, hi;
+    auto first_band = [&](int p) { return (int)((long long)p * pl->n_bands / pieces); };
+    LOP_CUDA(cudaEventRecord(e->ev_fork, s));               // the copies start after everything already queued on the caller's stream
+    LOP_CUDA(cudaStreamWaitEvent(e->copy_stream, e->ev_fork, 0));
+    for (int b = 0; b < pl->n_bands; ++b) e->copy_issued[b] = 0;
+    e->copies_timed = false;
+    for (int p = 0; p < pieces; ++p) {
+        const int last = first_band(p + 1) - 1;
+        if (new_input_rows(pl, first_band(p), last + 1, &lo, &hi) && (rc = copy_rows_impl(pl, lo, hi, host, staging, e->copy_stream)) != LOP_OK) return rc;
+        LOP_CUDA(cudaEventRecord(e->ev_arrive[last], e->copy_stream));
+    }
+    for (int p = 0; p < pieces; ++p) {
+        LOP_CUDA(cudaStreamWaitEvent(s, e->ev_arrive[first_band(p + 1) - 1], 0));
+        if ((rc = run_batched_impl(pl, first_band(p), first_band(p + 1), staging, out, ws, s)) != LOP_OK) return rc;
+    }
     return LOP_OK;
 }
 
@@ -615,18 +663,11 @@ int enqueue_pipelined(lop_plan_t *pl, Program *p, const void *host, void *stagin
     LOP_CUDA(cudaStreamWaitEvent(e->signal_stream, e->ev_fork, 0));
     const int G = std::max(1, pl->copy_group);
     for (int b0 = 0; b0 < pl->n_bands; b0 += G) {
-        // one copy for the bands [b0, b1): their new rows are one contiguous run; the arrival is written for the last band
+        // one copy for the bands [b0, b1); the arrival is written for the last band
         const int b1 = std::min(pl->n_bands, b0 + G), b = b1 - 1;
-        int lo = 0, hi = 0;
-        bool any = false;
-        for (int q = b0; q < b1; ++q) {
-            const lop_range &need = pl->in_need[q];
-            e->copy_issued[q] = 0;
-            if (need.out_hi <= need.new_lo) continue;
-            lo = any ? std::min(lo, (int)need.new_lo) : (int)need.new_lo;
-            hi = any ? std::max(hi, (int)need.out_hi) : (int)need.out_hi;
-            any = true;
-        }
+        int lo, hi;
+        const bool any = new_input_rows(pl, b0, b1, &lo, &hi);
+        for (int q = b0; q < b1; ++q) e->copy_issued[q] = 0;
         if (withheld >= b0 && withheld < b1) continue;
         e->copy_issued[b] = any;
         if (any && (rc = copy_rows_impl(pl, lo, hi, host, staging, e->copy_stream)) != LOP_OK) return rc;
@@ -701,7 +742,7 @@ int lop_run_banded(lop_plan_t *pl, const void *in, void *out, void *ws, void *st
             if ((rc = run_band_impl(pl, b, in, out, ws, s)) != LOP_OK) return rc;
         return LOP_OK;
     }
-    return run_batched_impl(pl, in, out, ws, s);
+    return run_batched_impl(pl, 0, pl->n_bands, in, out, ws, s);
 }
 
 int lop_run_layer(lop_plan_t *pl, int layer, int row_lo, int row_hi, const void *in, void *out, void *ws, void *stream)
@@ -844,13 +885,13 @@ int lop_run_pipelined(lop_plan_t *pl, const void *host, void *staging, void *out
         return LOP_OK;
     }
     if (!(pl->flags & (LOP_FLAG_TIME_LAYERS | LOP_FLAG_DEBUG_BOUNDS))) {
-        // Per-layer kernels, input in host memory the device can address: one launch brings the rows every band needs,
-        // and each layer is one launch behind it.  Copies band by band hide at most the transfer, and cost four stream
-        // commands and a launch per layer for every band: a 64 KB input in four bands took 60 us that way, 13 us so.
+        // per-layer kernels, input in page-locked memory
         const void *src = fetchable(pl, host);
+        const int pieces = input_pieces(pl);
+        if (src && pieces > 1) return run_pieces_impl(pl, pieces, host, staging, out, ws, s);
         if (src && ((reinterpret_cast<uintptr_t>(src) ^ reinterpret_cast<uintptr_t>(staging)) & 15) == 0) {
             if ((rc = fetch_rows_impl(pl, -1, src, staging, s)) != LOP_OK) return rc;
-            return run_batched_impl(pl, staging, out, ws, s);
+            return run_batched_impl(pl, 0, pl->n_bands, staging, out, ws, s);
         }
     }
     // the side stream starts after everything already queued on the caller's stream; all transfers are queued

@@ -73,6 +73,28 @@ def test_one_launch_brings_the_input_of_a_per_layer_plan(N, H, W, C, dtype, band
     assert torch.isnan(dc.staging[:, :r.new_lo].float()).all() and torch.isnan(dc.staging[:, r.out_hi:].float()).all()
 
 
+@pytest.mark.parametrize("dtype,C,N,H,W,bands,flags,copies", [
+    ("f32", 8, 1, 512, 512, 5, lop.LOP_FLAG_REUSE_HALO, 2),                # the smallest input that comes in pieces
+    ("f32", 8, 2, 519, 263, 7, 0, 2),                                      # odd sizes, bands that recompute their halo
+    ("bf16", 12, 1, 611, 650, 3, lop.LOP_FLAG_FORCE_SIMT, 2),
+    ("f32", 8, 1, 1024, 1024, 16, lop.LOP_FLAG_REUSE_HALO, 4),
+])
+def test_large_inputs_of_the_per_layer_kernels_come_in_pieces(dtype, C, N, H, W, bands, flags, copies):
+    layers = [conv(C, C, 3, s=2, act=li.ACT_RELU), conv(C, C, 3, act=li.ACT_NONE), pool(C, 2, 2, 0)]
+    layers[0].input_from, layers[1].input_from, layers[2].input_from = -1, 0, 1
+    wl = Workload("pieces", dtype, N, H, W, C, [Segment(layers, bands)], seed=41)
+    li.fill_parameters(wl)
+    li.make_input(wl)
+    check_workload(wl, flags=flags, modes=("banded", "pipelined"))
+    dc = DeviceChain(wl, flags=flags)
+    x = dc.pinned_input()
+    for _ in range(3):                       # the staging tensor is written again only after the run before has read it
+        dc.run_pipelined(x)
+    torch.cuda.synchronize()
+    assert dc.plans[0].last_copies() == copies
+    assert torch.equal(dc.staging.cpu().view(-1), x.view(-1))
+
+
 # ------------------------------------------------------------------------------------ operand ring and output units
 RING_CASES = [  # k, s, p, cin, cout, N, H, W, residual
     (3, 1, 1, 64, 64, 1, 150, 143, True),      # kept weights: several tiles per CTA, one cut of the ring

@@ -138,3 +138,36 @@ def test_an_address_that_is_no_longer_page_locked_is_copied_from(host, name):
         host.lib.host_side_pin(HOST, (1 << 30) if pinned else 0)
         copies = [x for x in commands(host, c.pipelined) if x[0] == "copy"]
         assert bool(copies) == (not pinned), (name, pinned)
+
+
+@pytest.mark.parametrize("flags", [0, lop.LOP_FLAG_REUSE_HALO])
+@pytest.mark.parametrize("N,H,bands,pieces", [(1, 511, 8, 1), (1, 512, 8, 2), (2, 517, 3, 2), (1, 2047, 5, 2), (1, 2048, 32, 4), (3, 2048, 2, 2),
+                                              (1, 4096, 1, 1), (1, 2050, 4000, 4)])
+def test_a_large_input_of_the_per_layer_kernels_arrives_while_it_is_computed(host, N, H, bands, pieces, flags):
+    """From 8 MB on, a 512-column fp32 input of 8 channels comes in pieces, and each layer's rows are computed once, as
+    far as the rows that have arrived allow."""
+    layers = [conv(8, 8, 5, s=2), conv(8, 8, 3)]
+    layers[0].input_from, layers[1].input_from = -1, 0
+    c = host.chain(Workload("two", "f32", N, H, 512, 8, [Segment(layers, bands)]), flags=flags)
+    plan, log = c.plans[0], commands(host, c.pipelined)
+    side = {x[1] for x in log if x[0] == "copy"}
+    copies = [int(x[2]) for x in log if x[0] == "copy"]
+    convs = [(int(x[3]), int(x[4])) for x in log if x[0] == "conv"]
+    fetches = [x for x in log if x[0] == "fetch"]
+    assert (len(copies), len(fetches)) == ((0, 1) if pieces == 1 else (pieces, 0))
+    assert sum(copies) == (N * H * 512 * 32 if copies else 0) and side.isdisjoint({"0"}) and len(convs) == 2 * pieces
+    assert (plan.last_copies(), plan.last_launches()) == (len(copies), len(convs) + len(fetches))
+    for layer in range(2):
+        rows = convs[layer::2]
+        assert rows[0][0] == 0 and rows[-1][1] == plan.out_shape(layer)[0]
+        assert all(a[1] == b[0] for a, b in zip(rows, rows[1:]))
+    # a piece's layers follow the wait for its copy, and need no row that comes later
+    arrived, row, waited, recorded = {}, 0, 0, [x[2] for x in log if x[0] == "record" and x[1] in side]
+    for e, n in zip(recorded, copies):
+        row += n // (N * 512 * 32)
+        arrived[e] = row
+    for x in log:
+        if x[0] == "wait" and x[1] == "0":
+            waited = arrived[x[2]]
+        elif x[0] == "conv" and copies and int(x[4]) == convs[2 * list(arrived.values()).index(waited)][1]:
+            assert min(H, (int(x[4]) - 1) * 2 - 2 + 5) <= waited
