@@ -14,6 +14,10 @@ from . import binding as B
 _FIELDS = ("op", "cin", "cout", "kh", "kw", "sh", "sw", "ph", "pw", "dh", "dw", "act", "input_from",
            "residual_from", "residual_pos")
 
+# the current stream's handle without building a torch.cuda.Stream object: two microseconds of every small call.  Not a public
+# name of torch: without it the public way is taken
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
 
 def to_device(a, dtype, device):
     """float32 numpy array -> device tensor in the storage dtype (bf16 values must be representable)."""
@@ -82,8 +86,9 @@ class DeviceChain:
     def _stream(self, stream):
         if stream is not None:
             return stream.cuda_stream
-        # (the stream's handle without building a torch.cuda.Stream object: two microseconds of every small call)
-        return torch._C._cuda_getCurrentRawStream(self.index)
+        if _raw_stream is not None:
+            return _raw_stream(self.index)
+        return torch.cuda.current_stream(self.device).cuda_stream
 
     def layer_output(self, seg, layer):
         """The full-size output tensor of one layer of a segment: the segment's output tensor for its last layer, else a

@@ -123,6 +123,18 @@ def test_row_wise_operator_must_not_carry_a_window():
         assert e.value.status == -1 and "row-wise" in str(e.value)
 
 
+def test_the_stream_handle_does_not_depend_on_a_private_name_of_torch(monkeypatch):
+    from types import SimpleNamespace
+    import torch
+    from paper_2507_05829_b200 import chain
+    monkeypatch.setattr(chain, "_raw_stream", None)              # as under a torch that has dropped it
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda device: SimpleNamespace(cuda_stream=("handle", device)))
+    dc = chain.DeviceChain.__new__(chain.DeviceChain)
+    dc.device, dc.index = "cuda:3", 3
+    assert dc._stream(None) == ("handle", "cuda:3")
+    assert dc._stream(SimpleNamespace(cuda_stream=7)) == 7
+
+
 def test_the_developer_trace_build_compiles(tmp_path):
     """-DLOP_WF_TRACE adds per-item time stamps of the persistent kernel's roles and the lop_debug_* readers (a developer
     build, never the shipped library): it must keep compiling for sm_100a as the kernel changes."""
