@@ -338,15 +338,15 @@ bool hull_requests(const lop_plan_t *pl, int seg, bool wait_arrival, std::vector
     return true;
 }
 
-// Operation batching across thin bands (Sec. IV-C): deep in a network a band is a row or two of a small map, far less
-// than the rows one tile covers, so every band would pay for a mostly empty tile -- and stream the layer's weights once
-// more.  In reuse mode consecutive bands compute consecutive rows, so at a layer whose bands have fewer than eight rows
+// Operation batching across thin bands (Sec. IV-C), for reuse-mode programs whose layers are cut at the bands' borders: a
+// block of bands on one of several devices, and chains whose bands leave rows out.  Deep in a network a band is a row or two
+// of a small map, far less than the rows one tile covers, so every band would pay for a mostly empty tile -- and stream the
+// layer's weights once more.  In reuse mode consecutive bands compute consecutive rows, so at a layer whose bands have fewer than eight rows
 // the requests of g neighbouring bands are joined into one wherever their row ranges touch (g: about eight rows per
 // group; a tile of a 16-pixel-wide map has eight).  The rows computed, and their bits, stay the same.
-// keep_plan0: leave the first plan's bands alone (they are gated by the arrival of their input).
-void merge_thin_bands(const std::vector<SegBind> &segs, std::vector<StageReq> &reqs, bool keep_plan0)
+void merge_thin_bands(const std::vector<SegBind> &segs, std::vector<StageReq> &reqs)
 {
-    for (int sg = keep_plan0 ? 1 : 0; sg < (int)segs.size(); ++sg) {
+    for (int sg = 0; sg < (int)segs.size(); ++sg) {
         const lop_plan_t *pl = segs[sg].pl;
         if (!(pl->flags & LOP_FLAG_REUSE_HALO) || pl->n_bands < 2) continue;
         const int L = (int)pl->layers.size();
@@ -420,17 +420,14 @@ int get_program(const std::vector<SegBind> &segs, int kind, Program **prog, cons
                 }
             }
         } else if (kind == PROG_ALL_BANDS || kind == PROG_PIPELINED || kind == PROG_FETCHED) {
-            // ALL_BANDS (input resident): the bands' operations of one layer do not depend on each other, so they are
-            // batched layer by layer (operation batching, Sec. IV-C); dependencies stay per band row group.
-            // PIPELINED: bands arrive one after the other and each band's stages form a dependency chain, so the
-            // stages are ordered along the diagonals of the (band, stage) grid: while band b is at its first stage,
-            // band b-1 is at its second, and so on -- the pipeline of Sec. IV-B -- and the plans of a chain follow
-            // one another on the same diagonals (a later plan's band needs the previous plan's rows around it, so it
-            // lags by a band; the builder moves a stage back wherever its producers come later still).  Inside a
-            // diagonal the deeper stages come first, so a CTA does not sit on a band that has not arrived while
-            // older bands have work.
-            // FETCHED: the same, each band of plan 0 preceded by the fetch of its new input rows; the builder orders
-            // these programs by earliest start.
+            // The order here is the stages' numbering: a topological order, and what decides between row groups that the
+            // builder's schedule (schedule_units) finds equally urgent; the schedule itself follows the rows' arrival.
+            // Where a layer is one request over all bands (reuse mode) the stages follow one another layer by layer.
+            // Where every band recomputes its halo, or the bands leave rows out, each band has stages of its own: layer by
+            // layer with the input resident (operation batching, Sec. IV-C), else along the diagonals of the (band, stage)
+            // grid (while band b is at its first stage, band b-1 is at its second: the pipeline of Sec. IV-B; the plans of
+            // a chain follow one another on the same diagonals, the deeper stage of a diagonal first).
+            // FETCHED: each band of plan 0 is preceded by the fetch of its new input rows.
             long long joff = 0;
             for (int sg = 0; sg < (int)segs.size(); ++sg) {
                 const lop_plan_t *pl = segs[sg].pl;
@@ -504,10 +501,7 @@ int get_program(const std::vector<SegBind> &segs, int kind, Program **prog, cons
                 for (int b = b0; b < b1; ++b) arrival.push_back(t + 5.0);       // the bands of one copy arrive together
             }
         }
-        if (kind == PROG_ALL_BANDS || kind <= PROG_BLOCK0) merge_thin_bands(segs, reqs, false);
-        // (also in the first plan, whose bands are gated by their arrival: a 12-layer stack cut into 32 one-row bands ran
-        // 389 -> 352 us pipelined with its deep layers joined, the other configurations unchanged)
-        else if (kind == PROG_PIPELINED || kind == PROG_FETCHED) merge_thin_bands(segs, reqs, false);
+        merge_thin_bands(segs, reqs);
         Program *p = nullptr;
         int rc = program_build(segs, reqs, &p, (kind == PROG_PIPELINED || kind == PROG_ALL_BANDS) ? &arrival : nullptr, fetch_src);
         if (rc != LOP_OK) return rc;

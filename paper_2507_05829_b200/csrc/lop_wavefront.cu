@@ -3,14 +3,14 @@
 // CTA layout (three special warps + WF_WORKER_WARPS worker warps, one CTA per SM):
 //   warp 0      all lanes poll the item's producer row groups in parallel (the dependency list of the
 //               next item is prefetched while this one runs); lane 0 then streams the item's activation
-//               and weight boxes by TMA into two shared-memory rings that live across items
+//               and weight boxes by TMA into a shared-memory ring of entries that lives across items
 //   warp 1      one lane issues tcgen05.mma into one of two fp32 accumulators in tensor memory, so the
 //               next item's main loop overlaps this item's epilogue
-//   warp 2      one lane publishes finished items: after the workers' barrier it fences and does the release
-//               increment of the item's row-group counter, so that memory-fence latency is off the workers' path
-//   workers     epilogue of convolution items: TMEM -> scale/shift/residual/activation -> bf16 rows in a
-//               shared staging tile -> coalesced 16-byte stores; and the whole of pooling, patch-gather,
-//               depth-wise convolution, layer-normalisation and concatenation items.
+//   warp 2      one lane issues the bulk stores of finished output units and publishes finished items: it fences and does
+//               the release increment of the item's row-group counter, so that this latency is off the workers' path
+//   workers     epilogue of convolution items: TMEM -> scale/shift/residual/activation -> bf16 rows in an output
+//               unit in shared memory (results in host memory and folded poolings they copy out themselves); and
+//               the whole of pooling, patch-gather, depth-wise convolution, layer-normalisation and concatenation items.
 //               Many of them because straight-line per-element code needs several warps per scheduler to
 //               hide its own latency; the four warps that share a TMEM lane group split a tile's columns.
 //
@@ -20,7 +20,8 @@
 // so one TMA box per 64-channel chunk serves all taps (the shared-memory matrix descriptor simply starts
 // later: the swizzle is a function of the address).  Anchors in the last (kw-1)*dw columns of a
 // pitch would wrap into the next row; they are computed and dropped.  K is walked as (channel chunk, kh,
-// kw, 16-channel step) whatever the tile, so a pixel's bits do not depend on who computes it.
+// kw, 16-channel step) whatever the tile, so a pixel's bits do not depend on who computes it.  (A gathered stem is a
+// pointwise layer here: its K is the order of the gathered values, lop_gather.cuh.)
 //
 // Deadlock freedom: items are numbered in a topological order, every CTA is resident and takes its
 // items in increasing order, so the lowest unfinished item never waits on an unstarted one.  All
@@ -1293,7 +1294,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 }
                 if (tid == 0) tr(item, 12);
             } else {
-                // pooling or patch gather: one output row of one image per item, all worker threads
+                // an item of the worker warps alone: output rows of one image (or a depth-wise tile)
                 if (warp == WF_FIRST_WORKER && !wait_deps_warp(P, rec_dep0(cur), rec_ndep(cur), dep_cur, run, lane, [] {}) && lane == 0) *epi_fail = 1;
                 epi_bar();
                 if (tid == 0) tr(item, 1);

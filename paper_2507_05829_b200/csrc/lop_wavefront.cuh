@@ -16,8 +16,9 @@ namespace lop {
 // WF_FETCH: rows of the chain input brought from host memory by the CTAs' fetch warps.  Such a stage has row-group
 // counters like any producer but no items in the main list: its work is the program's fetch list.
 // WF_DWCONV / WF_LAYERNORM / WF_CONCAT: the memory-bound operators, run by the worker warps like pooling.  A depth-wise
-// item is one output row of one image, tw_valid columns wide and BN channels deep (its receptive window is staged in
-// shared memory); a normalisation or concatenation item is one whole output row of one image.
+// item is 1 << tr_log output rows of one image, tw_valid columns wide and BN channels deep (its receptive window is staged
+// in shared memory); a normalisation or concatenation item is one whole output row of one image; a gather or 3x3 pooling
+// item is 1 << tr_log of them.
 enum WfKind { WF_GATHER = 0, WF_CONV = 1, WF_POOL = 2, WF_FETCH = 3, WF_DWCONV = 4, WF_LAYERNORM = 5, WF_CONCAT = 6 };
 // How a convolution stage feeds the tensor cores.
 //   WF_SLAB  one activation box per channel chunk: the output tile's receptive window (tile plus halo),
