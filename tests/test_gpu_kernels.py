@@ -95,6 +95,30 @@ def test_large_inputs_of_the_per_layer_kernels_come_in_pieces(dtype, C, N, H, W,
     assert torch.equal(dc.staging.cpu().view(-1), x.view(-1))
 
 
+@pytest.mark.parametrize("dtype,C,H,W", [("f32", 16, 32, 32), ("f32", 8, 512, 512), ("bf16", 3, 60, 44)])
+def test_streamed_runs_are_captured_in_a_graph(dtype, C, H, W):
+    """One launch and one per layer, pieces on the side stream, the persistent kernel: replayed on another input."""
+    wl = one_layer(conv(C, 16, 3, act=li.ACT_RELU), 1, H, W, dtype=dtype)
+    dc = DeviceChain(wl, flags=lop.LOP_FLAG_REUSE_HALO)
+    x = dc.pinned_input()
+    dc.run_pipelined(x)                      # the first call makes streams, events and tables
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        dc.run_pipelined(x)
+    other = torch.flip(x, [1]).clone()
+    x.copy_(other)
+    for _ in range(2):
+        dc.outs[-1].zero_()
+        graph.replay()
+    torch.cuda.synchronize()
+    dc.check_device()
+    got = dc.outs[-1].clone()
+    dc.run_banded(other.cuda())
+    torch.cuda.synchronize()
+    assert torch.equal(got, dc.outs[-1])
+
+
 # ------------------------------------------------------------------------------------ operand ring and output units
 RING_CASES = [  # k, s, p, cin, cout, N, H, W, residual
     (3, 1, 1, 64, 64, 1, 150, 143, True),      # kept weights: several tiles per CTA, one cut of the ring
