@@ -754,11 +754,13 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
     const int n_items = (int)items.size();
     if (n_items == 0 && fetch_items.empty()) { *result = p; return LOP_OK; }          // nothing to do: an empty program
 
-    // ---- shared memory: the operand ring takes what the output units and the SIMT scratch leave
-    const uint32_t ring_bytes = (227u * 1024u - 1024u - WF_FIXED_SMEM - stg_bytes - WF_UNITS * unit_bytes) & ~1023u;
     std::map<int, long long> tiles_of;                            // convolution tiles per weight map: the layer's stages together
     for (const int4 &it : items)
         if (stages[it.x & 0xFFFF].kind == WF_CONV) ++tiles_of[stages[it.x & 0xFFFF].map_base];
+    // ---- shared memory: the operand ring takes what the output units and the SIMT scratch leave.  Without a convolution
+    // there is none: what is not asked for stays L1, which the loads of the memory-bound items go through (8x224x224x64 with
+    // the whole of it asked for and without: depth-wise 7x7 289 and 238 us, normalisation 115 and 98, concatenation 260 and 222).
+    const uint32_t ring_bytes = tiles_of.empty() ? 0u : (227u * 1024u - 1024u - WF_FIXED_SMEM - stg_bytes - WF_UNITS * unit_bytes) & ~1023u;
     auto slot = [](uint32_t bytes) { return round_up_u32(bytes, 1024u); };
     std::map<uint32_t, uint32_t> box_step;                        // slab stages that share a cut of the ring: divisor of their weight boxes
     for (WfStage &st : stages) {

@@ -201,7 +201,7 @@ cudaError_t launch_conv_tc(const ConvArgs &a, const ConvTcGeom &, const ConvTcMa
 TensorMapEncodeFn tensor_map_encoder() { return encode; }
 size_t wavefront_smem_bytes(const WfParams &p) { return 1024 + (size_t)p.ring_bytes + (size_t)WF_UNITS * p.unit_bytes + p.simt_bytes + WF_FIXED_SMEM; }
 cudaError_t wavefront_resident_ctas(const WfParams &, int *ctas) { *ctas = 148; return cudaSuccess; }
-cudaError_t launch_wavefront(const WfParams &p, int, cudaStream_t s) { g_last = p; return note("persistent %llx", id(s)); }
+cudaError_t launch_wavefront(const WfParams &p, int, cudaStream_t s) { g_last = p; return note("persistent %llx %zu", id(s), wavefront_smem_bytes(p)); }
 }  // namespace lop
 
 extern "C" int lop_run_whole_static(lop_plan_t *, const void *, void *, unsigned *, void *) { return LOP_EUNSUPPORTED; }

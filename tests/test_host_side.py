@@ -10,7 +10,7 @@ import pytest
 
 import lop_inputs as li
 import paper_2507_05829_b200 as lop
-from lop_inputs.workloads import Segment, Workload, conv
+from lop_inputs.workloads import Segment, Workload, conv, pool
 from paper_2507_05829_b200 import binding
 from paper_2507_05829_b200.chain import _FIELDS
 
@@ -122,12 +122,24 @@ def test_a_group_of_boxes_fits_the_rings_entries(host):
     check_rings(host, wl)
 
 
-# ------------------------------------------------------------------------------------ the streamed input's transport
 def commands(host, run):
     """The stream commands and launches of one call, as (command, stream, ...) tuples."""
     host.lib.host_side_clear()
     run()
     return [tuple(line.split()) for line in host.lib.host_side_log().decode().splitlines()]
+
+
+@pytest.mark.parametrize("layer", [li.dwconv(64, 7), li.layernorm(64), pool(64, 3, 2, 1), conv(64, 64, 1)])
+def test_a_program_without_a_convolution_leaves_shared_memory_to_l1(host, layer):
+    layer.input_from = -1
+    c = host.chain(Workload("one", "bf16", 2, 56, 56, 64, [Segment([layer], 4)]))
+    for run in (c.banded, c.pipelined):
+        smem = [int(x[2]) for x in commands(host, run) if x[0] == "persistent"]
+        assert len(smem) == 1 and (smem[0] > 200 * 1024) == (layer.op == conv(1, 1, 1).op) and smem[0] <= 227 * 1024
+        assert layer.op == conv(1, 1, 1).op or smem[0] <= (1 + 4 + 4 + 64) * 1024          # alignment, tables, units, scratch
+
+
+# ------------------------------------------------------------------------------------ the streamed input's transport
 
 
 @pytest.mark.parametrize("name", ["single_conv", "vgg_block", "resnet18"])
