@@ -57,7 +57,7 @@ namespace {
 #ifndef LOP_KEEP_BYTES
 #define LOP_KEEP_BYTES (80 * 1024)
 #endif
-constexpr uint32_t A_BOX_MAX = 48u * 1024u;     // largest activation box a ring slot is sized for
+constexpr uint32_t A_BOX_MAX = 48u * 1024u;     // largest activation box of a slab stage: two of them and a weight box share the ring
 constexpr uint32_t LOP_ROWOP_STAGING_BYTES = 64u * 1024u;    // largest receptive window a depth-wise item stages
 constexpr uint32_t B_BOX_MAX = 48u * 1024u;     // largest weight box of several taps: a 3x3 filter row of 128 x 64 weights
 

@@ -26,9 +26,9 @@ bool program_supported(const lop_plan_t *pl);
 // convolution's epilogue (its own output tensor is then never written).
 bool program_folds_pool(const lop_plan_t *pl, int layer);
 // arrival_us (optional): expected arrival time of each band of plan 0 (empty: all there); the row groups of all stages are then
-// dealt out by their earliest possible start under that schedule instead of stage by stage.  fetch_src: the chain input in
-// host memory as the device addresses it, source of the fetch requests (segs[0].in is their destination); programs with
-// fetch requests are ordered by earliest start as well, the host link taken as a serial resource.
+// dealt out in the order of a schedule on a model of the machine (schedule_units) instead of stage by stage.  fetch_src: the
+// chain input in host memory as the device addresses it, source of the fetch requests (segs[0].in is their destination);
+// programs with fetch requests are scheduled likewise, the host link taken as a serial resource.
 int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, Program **result,
                   const std::vector<double> *arrival_us = nullptr, const void *fetch_src = nullptr);
 int program_launch(Program *p, cudaStream_t s);
