@@ -9,7 +9,8 @@ by pooling items of the persistent kernel), ``gather`` (patch gather + 7x7 strid
 the stand-alone kernels; ``gather:persistent`` inside the persistent kernel), ``convnext_block`` / ``dense_layer``
 (depth-wise convolution, layer normalisation, concatenation: items of the persistent kernel; ``<name>:per_layer``
 runs the stand-alone kernels, one launch per layer), ``dwconv`` / ``layernorm`` / ``concat`` (one such operator on an
-8 x 224 x 224 x 64 tensor, stand-alone kernel or ``:persistent``).  The L2 is flushed before every run.
+8 x 224 x 224 x 64 tensor, stand-alone kernel or ``:persistent``), ``vgg_block_f32``
+(the CUDA-core convolutions).  The L2 is flushed before every run.
 """
 import sys
 
@@ -28,6 +29,8 @@ def build_case(name):
         if mode == "per_layer":                                   # one stand-alone kernel per layer, whole tensors
             return li.build(base), "whole", B.LOP_FLAG_PER_LAYER
         return li.build(base), (mode or "banded"), 0
+    if base == "vgg_block_f32":                                   # the CUDA-core convolutions
+        return li.build("vgg_block", dtype="f32"), (mode or "banded"), 0
     if base == "pool":
         l = pool(64, 3, 2, 1)
         l.input_from = -1
