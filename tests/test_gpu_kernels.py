@@ -261,3 +261,26 @@ def test_fetched_rows_of_any_alignment(W):
     """Rows that start anywhere in a 128-byte line, shorter and longer than what a warp has in flight."""
     wl = one_layer(conv(3, 16, 3, act=li.ACT_RELU), 2, 11, W)
     check_workload(wl, flags=lop.LOP_FLAG_REUSE_HALO, modes=("pipelined",))
+
+
+# ------------------------------------------------------------------------------------ GELU of the tensor-core epilogues
+@pytest.mark.parametrize("flags", [0, lop.LOP_FLAG_PER_LAYER])
+def test_gelu_over_its_whole_range(flags):
+    """An identity layer: every output is the GELU of a bf16 value.  The epilogue's fp32 value is off by less than 1e-6 (its
+    polynomial, and a handful of roundings near one), then it is rounded to bf16 once: half a unit in the last place."""
+    from math import erfc
+    C, x = 16, np.concatenate([np.linspace(-20.0, 20.0, 4001), np.logspace(-30, 30, 183), -np.logspace(-30, 30, 183), [0.0, -0.0, np.inf]])
+    x = li.round_to_bf16(np.resize(x, 16 * 18 * C).astype(np.float32)).reshape(1, 16, 18, C)
+    l = conv(C, C, 1, p=0, act=li.ACT_GELU)
+    wl = one_layer(l, 1, 16, 18, dtype="bf16")
+    l.weight = np.eye(C, dtype=np.float32).reshape(l.weight.shape)
+    l.scale, l.shift = np.ones(C, np.float32), np.zeros(C, np.float32)
+    # (0 times infinity is a NaN in the other channels of an infinite value's pixel)
+    finite = np.isfinite(x).all(-1)
+    got = to_host_f32((lambda dc: dc.run_whole(dc.input_tensor(x)))(DeviceChain(wl, flags=flags)))
+    v = x.astype(np.float64)
+    with np.errstate(invalid="ignore", over="ignore"):
+        want = v * np.vectorize(lambda t: 0.5 * erfc(-t / np.sqrt(2.0)))(v)
+    g, w = got[finite], want[finite]
+    assert (np.abs(g - w) <= 2.0 ** -8 * np.abs(w) * (1 + 1e-3) + 1e-6 * np.minimum(np.abs(w), 1.0) + 1e-9).all()
+    assert np.isposinf(got[np.isposinf(x)]).all()
