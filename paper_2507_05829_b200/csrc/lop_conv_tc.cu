@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(TC_THREADS) conv_tc_kernel(const __grid_consta
     const int slabs = p.cin / p.BK;
     const int n_iter = p.kh * p.kw * slabs;
 
-    if (warp == 0 && lane == 0) {
+    if (warp == 0 && elect_one()) {
         // ---------------- TMA producer ----------------
         // K is walked as (channel slab, kh, kw): the order every executor of this library uses, so that a
         // pixel's value does not depend on which of them computed it
@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(TC_THREADS) conv_tc_kernel(const __grid_consta
                 }
             }
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1 && elect_one()) {
         // ---------------- MMA issuer ----------------
         for (int it = 0; it < n_iter; ++it) {
             const int s = it % p.stages;

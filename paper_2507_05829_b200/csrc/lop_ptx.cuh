@@ -16,6 +16,22 @@ constexpr uint32_t WAIT_LIMIT = 1u << 23;
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// True in one lane of a converged warp, the same one every time.  The single-thread roles are entered by this and not by a
+// comparison with a lane number: the compiler knows then that one thread is active, and hands addresses and descriptors to
+// the TMA and tensor-core instructions without a loop over the warp's active lanes.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "elect.sync _|p, 0xffffffff;\n"
+        "selp.u32 %0, 1, 0, p;\n"
+        "}\n"
+        : "=r"(p));
+    return p != 0u;
+}
+
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");

@@ -725,7 +725,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 if (!ok) {
                     if (lane == 0) atomicOr(P.status, 0x10u);
                     fail = 1;
-                } else if (lane == 0) {
+                } else if (elect_one()) {
                     tr(item, 1);
                     asm volatile("fence.proxy.async.global;" ::: "memory");       // producers' generic-proxy writes -> our TMA reads
                     const int ow0 = rec_tw(cur) * tw_valid;
@@ -868,7 +868,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
             cur = nxt; dep_cur = dep_nxt; nxt = nn;
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ---------------- MMA issuer ----------------
             int item = blockIdx.x;
             int4 cur = item < NI ? __ldg(&P.items[item]) : zero4;
@@ -1059,7 +1059,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
             }
         }
     } else if (warp == 2) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ---------------- publisher ----------------
             // Makes finished items visible: the workers' stores happen before their barrier and the arrive that
             // this thread waits for, so its fence orders them before the release increment of the counter.
