@@ -269,6 +269,7 @@ __global__ void __launch_bounds__(SMALL_THREADS) conv_simt_small_kernel(const __
     const long long m0 = (long long)blockIdx.x * SMALL_PX;
     const int n0 = blockIdx.y * SMALL_CO;
     const long long x_elems = (long long)p.N * p.Hin * p.Win * p.Cin, y_elems = (long long)p.N * p.Ho * p.Wo * p.Cout;
+    grid_release();
     float *As = small_sm, *Bs = small_sm + SMALL_PX * pitch;
     const float *__restrict__ x = static_cast<const float *>(p.x);
     const float *__restrict__ w = static_cast<const float *>(p.w);
@@ -284,6 +285,7 @@ __global__ void __launch_bounds__(SMALL_THREADS) conv_simt_small_kernel(const __
         copy16(Bs + r * pitch + 4 * k4, live ? w + wo : w, live);
     }
     // patches: four threads per pixel, each every fourth filter tap
+    grid_wait();                                               // (no launch before this one writes weights)
     {
         const int px = threadIdx.x >> 2;
         const bool ok = m0 + px < M;
@@ -425,6 +427,8 @@ cudaError_t launch_tiles(const ConvArgs &a, long long M, cudaStream_t s)
 {
     const dim3 grid((unsigned)((M + BM - 1) / BM), (unsigned)((a.Cout + BN - 1) / BN));
     constexpr int NT = (BM / TM) * (BN / TN);
+    // (not begun before the launch in front has ended: its blocks, a few per SM, would go to the SMs that are free first, three
+    // on some and one on others -- a VGG block of 181x203 pixels 94 us so, 125 begun early)
     conv_simt_kernel<T, BM, BN, TM, TN><<<grid, NT, 0, s>>>(a);
     return cudaGetLastError();
 }
@@ -468,8 +472,7 @@ cudaError_t launch_conv_simt(const ConvArgs &a, int dtype, cudaStream_t s)
     const bool aligned = ((reinterpret_cast<uintptr_t>(a.x) | reinterpret_cast<uintptr_t>(a.w)) & 15) == 0;
     if (a.Cin % 4 == 0 && aligned && small_bytes <= 48u * 1024u && (small_blocks <= 4 * 148 || a.Cout <= SMALL_CO || a.Cin % SM_BK != 0)) {
         const dim3 grid((unsigned)((M + SMALL_PX - 1) / SMALL_PX), (unsigned)((a.Cout + SMALL_CO - 1) / SMALL_CO));
-        conv_simt_small_kernel<<<grid, SMALL_THREADS, small_bytes, s>>>(a);
-        return cudaGetLastError();
+        return launch_after(conv_simt_small_kernel, grid, SMALL_THREADS, small_bytes, s, a);
     }
     return launch_typed<float>(a, M, s);
 }

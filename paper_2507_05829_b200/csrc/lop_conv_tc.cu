@@ -88,6 +88,8 @@ __global__ void __launch_bounds__(TC_THREADS) conv_tc_kernel(const __grid_consta
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_acc = *tmem_slot;
+    grid_release();
+    grid_wait();
 
     // which output tile
     const int TW = 1 << p.tw_log, TR = 1 << p.tr_log;
@@ -344,8 +346,7 @@ cudaError_t launch_conv_tc(const ConvArgs &a, const ConvTcGeom &g, const ConvTcM
         if (dev >= 0 && dev < 64) configured[dev].store(true, std::memory_order_release);
     }
     dim3 grid((unsigned)(p.tiles_w * p.tiles_r * tiles_n), (unsigned)(a.Cout / g.BN));
-    conv_tc_kernel<<<grid, TC_THREADS, smem, s>>>(maps, p);
-    return cudaGetLastError();
+    return launch_after(conv_tc_kernel, grid, TC_THREADS, smem, s, maps, p);
 }
 
 }  // namespace lop

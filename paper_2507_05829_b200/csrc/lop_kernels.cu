@@ -48,10 +48,12 @@ struct alignas(sizeof(T) * VEC) Pack {
 template <typename T, int VEC>
 __global__ void __launch_bounds__(256) maxpool_kernel(PoolArgs p)
 {
+    grid_release();
     const int rows = p.oh_hi - p.oh_lo;
     const int cg = p.C / VEC;
     const long long total = (long long)p.N * rows * p.Wo * cg;
-    const T *__restrict__ x = static_cast<const T *>(p.x);
+    grid_wait();
+    const T *__restrict__ x = from_here(static_cast<const T *>(p.x));
     T *__restrict__ y = static_cast<T *>(p.y);
     for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
          idx += (long long)gridDim.x * blockDim.x) {
@@ -88,12 +90,14 @@ __global__ void __launch_bounds__(256) maxpool_kernel(PoolArgs p)
 template <int KH, int KW>
 __global__ void __launch_bounds__(256) maxpool_bf16x8_kernel(PoolArgs p)
 {
+    grid_release();
     const int rows = p.oh_hi - p.oh_lo;
     const int cg = p.C >> 3;
     const long long total = (long long)p.N * rows * p.Wo * cg;
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    grid_wait();
     if (idx >= total) return;
-    const uint4 *__restrict__ x = static_cast<const uint4 *>(p.x);
+    const uint4 *__restrict__ x = from_here(static_cast<const uint4 *>(p.x));
     int g, ow, r, n;
     split_index(idx, total, cg, p.Wo, rows, g, ow, r, n);
     const int oh = p.oh_lo + r;
@@ -154,9 +158,13 @@ __device__ __forceinline__ void stem_weights(const StemWeights &g, int first, in
 }
 
 template <typename Index>
-__global__ void __launch_bounds__(256) stem_gather_kernel(const uint16_t *__restrict__ x, uint16_t *__restrict__ y,
-                                                          GatherGeom g, int lo, int hi, StemWeights wt, unsigned *dbg)
+__global__ void __launch_bounds__(256) stem_gather_kernel(const uint16_t *x_given, uint16_t *__restrict__ y,
+                                                          GatherGeom g, int lo, int hi, StemWeights wt, unsigned *dbg, unsigned *clear)
 {
+    grid_release();
+    grid_wait();
+    const uint16_t *__restrict__ x = from_here(x_given);
+    if (clear && blockIdx.x == 0 && threadIdx.x == 0) *clear = 0u;
     const int k8n = g.Kcol >> 3;
     const Index total = (Index)g.N * (hi - lo) * g.Wo * k8n;
     for (Index idx = (Index)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (Index)gridDim.x * blockDim.x) {
@@ -186,6 +194,8 @@ constexpr int FETCH_THREADS = 128, FETCH_VECS = 4;
 __global__ void __launch_bounds__(FETCH_THREADS) fetch_rows_kernel(const uint8_t *__restrict__ src, uint8_t *__restrict__ dst, long long image_bytes,
                                                                    long long first, long long bytes)
 {
+    grid_release();
+    grid_wait();                                                // the input tensor may still be read by the run before this one
     const uint8_t *s0 = src + blockIdx.y * image_bytes + first;
     uint8_t *d0 = dst + blockIdx.y * image_bytes + first;
     const long long mis = (16 - (reinterpret_cast<uintptr_t>(s0) & 15)) & 15, head = mis < bytes ? mis : bytes;
@@ -226,18 +236,19 @@ cudaError_t launch_maxpool(const PoolArgs &a, int dtype, cudaStream_t s)
         const long long vecs = pix * (a.C / 8);
         const bool aligned = (reinterpret_cast<uintptr_t>(a.x) & 15) == 0 && (reinterpret_cast<uintptr_t>(a.y) & 15) == 0;
         const unsigned blocks = (unsigned)((vecs + 255) / 256);
-        if (a.C % 8 == 0 && aligned && vecs < (1LL << 38) && a.kh == 2 && a.kw == 2) maxpool_bf16x8_kernel<2, 2><<<blocks, 256, 0, s>>>(a);
-        else if (a.C % 8 == 0 && aligned && vecs < (1LL << 38) && a.kh == 3 && a.kw == 3) maxpool_bf16x8_kernel<3, 3><<<blocks, 256, 0, s>>>(a);
-        else if (a.C % 8 == 0) maxpool_kernel<__nv_bfloat16, 8><<<grid_for(pix * (a.C / 8), 256), 256, 0, s>>>(a);
-        else maxpool_kernel<__nv_bfloat16, 1><<<grid_for(pix * a.C, 256), 256, 0, s>>>(a);
+        if (a.C % 8 == 0 && aligned && vecs < (1LL << 38) && a.kh == 2 && a.kw == 2) return launch_after(maxpool_bf16x8_kernel<2, 2>, dim3(blocks), 256, 0, s, a);
+        else if (a.C % 8 == 0 && aligned && vecs < (1LL << 38) && a.kh == 3 && a.kw == 3) return launch_after(maxpool_bf16x8_kernel<3, 3>, dim3(blocks), 256, 0, s, a);
+        else if (a.C % 8 == 0) return launch_after(maxpool_kernel<__nv_bfloat16, 8>, dim3(grid_for(pix * (a.C / 8), 256)), 256, 0, s, a);
+        else return launch_after(maxpool_kernel<__nv_bfloat16, 1>, dim3(grid_for(pix * a.C, 256)), 256, 0, s, a);
     } else {
-        if (a.C % 4 == 0) maxpool_kernel<float, 4><<<grid_for(pix * (a.C / 4), 256), 256, 0, s>>>(a);
-        else maxpool_kernel<float, 1><<<grid_for(pix * a.C, 256), 256, 0, s>>>(a);
+        if (a.C % 4 == 0) return launch_after(maxpool_kernel<float, 4>, dim3(grid_for(pix * (a.C / 4), 256)), 256, 0, s, a);
+        return launch_after(maxpool_kernel<float, 1>, dim3(grid_for(pix * a.C, 256)), 256, 0, s, a);
     }
     return cudaGetLastError();
 }
 
-cudaError_t launch_stem_gather(const void *x, void *y, const GatherGeom &g, int lo, int hi, cudaStream_t s, unsigned *dbg, const StemWeights &wt)
+cudaError_t launch_stem_gather(const void *x, void *y, const GatherGeom &g, int lo, int hi, cudaStream_t s, unsigned *dbg, const StemWeights &wt,
+                               unsigned *clear)
 {
     if (hi <= lo) return cudaSuccess;
     if (g.Kcol % 8 != 0) return cudaErrorInvalidValue;
@@ -246,8 +257,8 @@ cudaError_t launch_stem_gather(const void *x, void *y, const GatherGeom &g, int 
     const uint16_t *xi = static_cast<const uint16_t *>(x);
     uint16_t *yi = static_cast<uint16_t *>(y);
     // (a 64-bit division is a routine of several dozen instructions, and a thread has four of them)
-    if (work < (1LL << 30)) stem_gather_kernel<int><<<blocks, 256, 0, s>>>(xi, yi, g, lo, hi, wt, dbg);
-    else stem_gather_kernel<long long><<<blocks, 256, 0, s>>>(xi, yi, g, lo, hi, wt, dbg);
+    if (work < (1LL << 30)) return launch_after(stem_gather_kernel<int>, dim3(blocks), 256, 0, s, xi, yi, g, lo, hi, wt, dbg, clear);
+    else return launch_after(stem_gather_kernel<long long>, dim3(blocks), 256, 0, s, xi, yi, g, lo, hi, wt, dbg, clear);
     return cudaGetLastError();
 }
 
@@ -260,10 +271,11 @@ cudaError_t launch_fetch_rows(const void *src, void *dst, int N, int rows, long 
     const long long per_block = 16LL * FETCH_THREADS * FETCH_VECS;
     for (int n = 0; n < images; n += 65535) {
         const dim3 grid((unsigned)((bytes + per_block - 1) / per_block), (unsigned)(images - n < 65535 ? images - n : 65535));
-        fetch_rows_kernel<<<grid, FETCH_THREADS, 0, s>>>(static_cast<const uint8_t *>(src) + n * image, static_cast<uint8_t *>(dst) + n * image, image,
-                                                         lo * row_bytes, bytes);
+        const cudaError_t e = launch_after(fetch_rows_kernel, grid, FETCH_THREADS, 0, s, static_cast<const uint8_t *>(src) + n * image,
+                                           static_cast<uint8_t *>(dst) + n * image, image, lo * row_bytes, bytes);
+        if (e != cudaSuccess) return e;
     }
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 
 cudaError_t launch_stem_weights(const StemWeights &wt, cudaStream_t s)

@@ -32,6 +32,36 @@ struct PoolArgs {
     unsigned *dbg;          // as in ConvArgs
 };
 
+// Consecutive launches on a stream overlap where the second one's start allows it (programmatic dependent launch): a kernel's
+// blocks are set up while the one before it drains, and everything that kernel reads or writes comes after grid_wait().
+// Every thread of every kernel started by launch_after() calls it, so that a kernel's end still means that all before it
+// have ended.  grid_release() lets the next launch begin; it stands behind a tensor-memory allocation, or a block of the next
+// kernel could take the columns that a block of this one waits for.  A launch without the attribute, a copy or an event
+// orders the stream as ever.  (About 2 us per launch: a DenseNet layer called in a row 18.2 -> 16.2 us,
+// a VGG block by per-layer kernels 46.7 -> 39.7.)
+#ifdef __CUDACC__
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// A pointer whose loads the compiler must not take to before this place: those of read-only data move across grid_wait().
+template <typename T>
+__device__ __forceinline__ T *from_here(T *p)
+{
+    asm volatile("" : "+l"(p)::"memory");
+    return p;
+}
+#endif
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, const A &...args)
+{
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid; cfg.blockDim = dim3(block); cfg.dynamicSmemBytes = smem; cfg.stream = s;
+    cfg.attrs = &attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Checked execution (LOP_FLAG_DEBUG_BOUNDS): elements [first, first + count) must lie inside a tensor of `limit`
 // elements.  Without a status word the test costs one predictable branch.
 #ifdef __CUDACC__
@@ -61,8 +91,9 @@ cudaError_t launch_stem_weights(const StemWeights &wt, cudaStream_t s);
 // rows [lo,hi) of the gathered tensor y[N,Ho,Wo,Kcol] of a thin chain input x[N,H,W,C] (bf16 only).
 struct GatherGeom;
 // dbg: checked execution's status word (see ConvArgs), or nullptr.  wt: weights to bring along by the same launch, if any.
+// clear: a word the launch sets to zero, or nullptr.
 cudaError_t launch_stem_gather(const void *x, void *y, const GatherGeom &g, int lo, int hi, cudaStream_t s, unsigned *dbg = nullptr,
-                               const StemWeights &wt = StemWeights());
+                               const StemWeights &wt = StemWeights(), unsigned *clear = nullptr);
 // Rows [lo, hi) of each of N images of `rows` rows of row_bytes bytes: src (host memory as the device addresses it) -> dst.
 // src and dst agree modulo 16.
 cudaError_t launch_fetch_rows(const void *src, void *dst, int N, int rows, long long row_bytes, int lo, int hi, cudaStream_t s);

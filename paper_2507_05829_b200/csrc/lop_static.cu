@@ -87,9 +87,13 @@ extern "C" int lop_run_whole_static(lop_plan_t *pl, const void *in, void *out, u
     if (rc != LOP_OK) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
 
-    // the previous call's leftovers: the status word must read 0 before any kernel can raise it
+    // the previous call's leftovers: the status word must read 0 before any kernel can raise it.  A gathered stem's first
+    // launch, which raises nothing unless execution is checked, clears it by the way (a memset would be a stream command
+    // that no launch overlaps).
     unsigned *status = status_dev ? status_dev : reinterpret_cast<unsigned *>(ws + pl->status_off);
-    ST_CUDA(cudaMemsetAsync(status, 0, sizeof(unsigned), s));
+    const bool stem_clears = L > 0 && pl->layers[0].l.op != LOP_MAXPOOL2D && pl->layers[0].kernel == K_CONV_TC && pl->layers[0].stem_gather &&
+                             !conv_args(pl, 0, in, out, ws, 0, pl->layers[0].Ho).dbg;
+    if (!stem_clears) ST_CUDA(cudaMemsetAsync(status, 0, sizeof(unsigned), s));
     for (int i = 0; i < L; ++i) {
         const LayerInfo &li = pl->layers[i];
         const lop_layer &l = li.l;
@@ -118,7 +122,8 @@ extern "C" int lop_run_whole_static(lop_plan_t *pl, const void *in, void *out, u
         }
         if (li.stem_gather) {
             // another plan may have used the array since: padded weights and patches are rebuilt by every call
-            ST_CUDA(launch_stem_gather(in, ws + pl->col_off, gather_geom(pl, i), 0, li.Ho, s, a.dbg, stem_weights_args(pl, i, ws)));
+            ST_CUDA(launch_stem_gather(in, ws + pl->col_off, gather_geom(pl, i), 0, li.Ho, s, a.dbg, stem_weights_args(pl, i, ws),
+                                       i == 0 && stem_clears ? status : nullptr));
         }
         const ConvTcGeom g = conv_tc_geometry(a, li.Ho);
         ConvTcMaps maps;                                   // encoded on the stack: nothing is cached between calls

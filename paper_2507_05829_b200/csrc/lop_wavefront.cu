@@ -31,6 +31,7 @@
 #include <cuda_bf16.h>
 
 #include "lop_gather.cuh"
+#include "lop_kernels.cuh"
 #include "lop_ptx.cuh"
 #include "lop_rowops.cuh"
 #include "lop_wavefront.cuh"
@@ -619,6 +620,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
             mbar_init(pube0 + 8u * q, 1);
         }
         misc[1] = 0;
+        grid_wait();
         misc[2] = ld_acquire(P.counters) + 1u;                 // this launch is run number (completed runs + 1)
         misc[3] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -632,6 +634,8 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    grid_release();
+    grid_wait();                                               // (all threads: thread 0 waited for what it read)
     if (threadIdx.x == 0 && blockIdx.x < 4) tr(TRACE_ITEMS - 8 + (int)blockIdx.x, 1);
     const uint32_t tmem_base = misc[0];
     const unsigned run = misc[2];
@@ -1455,8 +1459,14 @@ cudaError_t launch_wavefront(const WfParams &p, int grid, cudaStream_t s)
 #ifdef LOP_WF_TRACE
     g_last_params = p;
 #endif
-    kernel_for(p)<<<grid, p.n_fetch > 0 ? WF_THREADS + 32 : WF_THREADS, smem, s>>>(p);
-    return cudaGetLastError();
+    // A program that fetches its input does not begin early: its CTAs would take the SMs in the order in which the previous
+    // launch leaves them, which costs a long one more than the launch's two microseconds (ResNet-18 streamed 169.8 us so,
+    // 170.9 begun early; a ResNet-50 of batch 8 442.6 and 445.5).
+    if (p.n_fetch > 0) {
+        kernel_for(p)<<<grid, WF_THREADS + 32, smem, s>>>(p);
+        return cudaGetLastError();
+    }
+    return launch_after(kernel_for(p), dim3(grid), WF_THREADS, smem, s, p);
 }
 
 }  // namespace lop

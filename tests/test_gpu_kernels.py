@@ -284,3 +284,28 @@ def test_gelu_over_its_whole_range(flags):
     g, w = got[finite], want[finite]
     assert (np.abs(g - w) <= 2.0 ** -8 * np.abs(w) * (1 + 1e-3) + 1e-6 * np.minimum(np.abs(w), 1.0) + 1e-9).all()
     assert np.isposinf(got[np.isposinf(x)]).all()
+
+
+# ------------------------------------------------------------------------------------ launches that begin before the previous one ended
+@pytest.mark.parametrize("dtype,C,H,W,flags", [("bf16", 64, 40, 36, 0), ("bf16", 64, 40, 36, lop.LOP_FLAG_PER_LAYER), ("f32", 16, 32, 32, 0),
+                                               ("f32", 64, 70, 61, 0), ("bf16", 5, 19, 23, lop.LOP_FLAG_FORCE_SIMT)])
+def test_calls_in_a_row_wait_for_what_they_read(dtype, C, H, W, flags):
+    """Two chains that read each other's output, called in turn with nothing between: the bits of calls with a
+    synchronisation between them."""
+    def chain(seed):
+        wl = Workload("row", dtype, 1, H, W, C, [Segment([conv(C, C, 3, input_from=-1), pool(C, 3, 1, 1, input_from=0), conv(C, C, 1, p=0, input_from=1)], 2)], seed=seed)
+        li.fill_parameters(wl)
+        li.make_input(wl)
+        return DeviceChain(wl, flags=flags)
+    a, b = chain(5), chain(6)
+    runs = []
+    for between in (torch.cuda.synchronize, lambda: None):
+        x = a.input_tensor()
+        for call in range(6):
+            x = (b if call % 2 else a).run_whole(x)
+            between()
+        torch.cuda.synchronize()
+        runs.append((a.outs[-1].clone(), b.outs[-1].clone()))
+    assert torch.isfinite(runs[0][1].float()).all() and runs[0][1].float().abs().max() > 0
+    assert torch.equal(runs[0][0], runs[1][0]) and torch.equal(runs[0][1], runs[1][1])
+
