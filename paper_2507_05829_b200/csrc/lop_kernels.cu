@@ -159,12 +159,12 @@ __device__ __forceinline__ void stem_weights(const StemWeights &g, int first, in
 
 template <typename Index>
 __global__ void __launch_bounds__(256) stem_gather_kernel(const uint16_t *x_given, uint16_t *__restrict__ y,
-                                                          GatherGeom g, int lo, int hi, StemWeights wt, unsigned *dbg, unsigned *clear)
+                                                          GatherGeom g, int lo, int hi, StemWeights wt, unsigned *dbg)
 {
     grid_release();
     grid_wait();
     const uint16_t *__restrict__ x = from_here(x_given);
-    if (clear && blockIdx.x == 0 && threadIdx.x == 0) *clear = 0u;
+    if (wt.clear && blockIdx.x == 0 && threadIdx.x == 0) *wt.clear = 0u;
     const int k8n = g.Kcol >> 3;
     const Index total = (Index)g.N * (hi - lo) * g.Wo * k8n;
     for (Index idx = (Index)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (Index)gridDim.x * blockDim.x) {
@@ -247,8 +247,7 @@ cudaError_t launch_maxpool(const PoolArgs &a, int dtype, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_stem_gather(const void *x, void *y, const GatherGeom &g, int lo, int hi, cudaStream_t s, unsigned *dbg, const StemWeights &wt,
-                               unsigned *clear)
+cudaError_t launch_stem_gather(const void *x, void *y, const GatherGeom &g, int lo, int hi, cudaStream_t s, unsigned *dbg, const StemWeights &wt)
 {
     if (hi <= lo) return cudaSuccess;
     if (g.Kcol % 8 != 0) return cudaErrorInvalidValue;
@@ -257,8 +256,8 @@ cudaError_t launch_stem_gather(const void *x, void *y, const GatherGeom &g, int 
     const uint16_t *xi = static_cast<const uint16_t *>(x);
     uint16_t *yi = static_cast<uint16_t *>(y);
     // (a 64-bit division is a routine of several dozen instructions, and a thread has four of them)
-    if (work < (1LL << 30)) return launch_after(stem_gather_kernel<int>, dim3(blocks), 256, 0, s, xi, yi, g, lo, hi, wt, dbg, clear);
-    else return launch_after(stem_gather_kernel<long long>, dim3(blocks), 256, 0, s, xi, yi, g, lo, hi, wt, dbg, clear);
+    if (work < (1LL << 30)) return launch_after(stem_gather_kernel<int>, dim3(blocks), 256, 0, s, xi, yi, g, lo, hi, wt, dbg);
+    else return launch_after(stem_gather_kernel<long long>, dim3(blocks), 256, 0, s, xi, yi, g, lo, hi, wt, dbg);
     return cudaGetLastError();
 }
 

@@ -85,15 +85,14 @@ cudaError_t launch_concat(const ConvArgs &a, int dtype, cudaStream_t s);
 // depth-wise filters w[C][taps] -> wt[taps][C] (bf16 only), the layout the persistent kernel reads
 cudaError_t launch_dw_transpose(const void *w, void *wt, int C, int taps, cudaStream_t s);
 // w[cout][kh][kw][C] -> wp[cout][K], zero-padded, in the order of a gathered stem's values: (kw, kh, C) with each column's
-// kh*C values padded to col elements, or (kh, kw, C) for col = 0 (bf16 only).
-struct StemWeights { const void *w = nullptr; void *wp = nullptr; int cout = 0, kh = 0, kw = 0, C = 0, col = 0, K = 0; };
+// kh*C values padded to col elements, or (kh, kw, C) for col = 0 (bf16 only).  clear: a word to set to zero, if any.
+struct StemWeights { const void *w = nullptr; void *wp = nullptr; int cout = 0, kh = 0, kw = 0, C = 0, col = 0, K = 0; unsigned *clear = nullptr; };
 cudaError_t launch_stem_weights(const StemWeights &wt, cudaStream_t s);
 // rows [lo,hi) of the gathered tensor y[N,Ho,Wo,Kcol] of a thin chain input x[N,H,W,C] (bf16 only).
 struct GatherGeom;
 // dbg: checked execution's status word (see ConvArgs), or nullptr.  wt: weights to bring along by the same launch, if any.
-// clear: a word the launch sets to zero, or nullptr.
 cudaError_t launch_stem_gather(const void *x, void *y, const GatherGeom &g, int lo, int hi, cudaStream_t s, unsigned *dbg = nullptr,
-                               const StemWeights &wt = StemWeights(), unsigned *clear = nullptr);
+                               const StemWeights &wt = StemWeights());
 // Rows [lo, hi) of each of N images of `rows` rows of row_bytes bytes: src (host memory as the device addresses it) -> dst.
 // src and dst agree modulo 16.
 cudaError_t launch_fetch_rows(const void *src, void *dst, int N, int rows, long long row_bytes, int lo, int hi, cudaStream_t s);

@@ -122,8 +122,9 @@ extern "C" int lop_run_whole_static(lop_plan_t *pl, const void *in, void *out, u
         }
         if (li.stem_gather) {
             // another plan may have used the array since: padded weights and patches are rebuilt by every call
-            ST_CUDA(launch_stem_gather(in, ws + pl->col_off, gather_geom(pl, i), 0, li.Ho, s, a.dbg, stem_weights_args(pl, i, ws),
-                                       i == 0 && stem_clears ? status : nullptr));
+            StemWeights wt = stem_weights_args(pl, i, ws);
+            if (i == 0 && stem_clears) wt.clear = status;
+            ST_CUDA(launch_stem_gather(in, ws + pl->col_off, gather_geom(pl, i), 0, li.Ho, s, a.dbg, wt));
         }
         const ConvTcGeom g = conv_tc_geometry(a, li.Ho);
         ConvTcMaps maps;                                   // encoded on the stack: nothing is cached between calls
