@@ -954,8 +954,8 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         return true;
                     };
-                    if (row3x64 && !kept && (cps == 3 || cps == 1)) {
-                        // the common 3x3 chunk, its three weight boxes behind one barrier or behind one each: nothing but the
+                    if (row3x64 && !kept) {
+                        // the common 3x3 chunk, its three weight boxes behind one barrier, two or three: nothing but the
                         // commits stands between the MMAs (the general loop below spends some 330 cycles of this thread's
                         // arithmetic per box, half of a box's MMAs: 3700 -> 2614 cycles per 64-channel chunk)
                         for (int ch = 0; ch < n_chunks; ++ch) {
@@ -969,7 +969,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                             if (cps == 1 && !next_group()) { fail = true; break; }
                             mma_row3x64(acc, la + step_h16, lb1, tap16, desc_hi, idesc, accumulate);
                             umma_commit(e1);
-                            if (cps == 1 && !next_group()) { fail = true; break; }
+                            if (cps < 3 && !next_group()) { fail = true; break; }
                             mma_row3x64(acc, la + 2u * step_h16, lb2, tap16, desc_hi, idesc, accumulate);
                             umma_commit(e2);
                         }
