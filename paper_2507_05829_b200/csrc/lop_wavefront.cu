@@ -56,6 +56,11 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned *p)
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
+// An increment behind everything this thread has done or seen done.
+__device__ __forceinline__ void add_release(unsigned *p)
+{
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
+}
 __device__ __forceinline__ unsigned ld_relaxed(const unsigned *p)
 {
     unsigned v;
@@ -96,7 +101,8 @@ __device__ __forceinline__ int rec_dep0(const int4 &r) { return r.w; }
 
 // Bounded wait of a whole warp for an item's dependencies: lane j polls entry j of the list (its first
 // 32 entries were prefetched into `mine`).  Counters only grow (compare modulo 2^32).  The result is
-// uniform across the warp.  idle() runs once if the first look finds a producer unfinished: there is time then.
+// uniform across the warp.  idle() runs once if the first look finds a producer unfinished: there is time then.  (No
+// sleep between two looks: a ResNet-50 of batch 8 442 us with 32 ns, 439 without.)
 template <typename Idle>
 __device__ __forceinline__ bool wait_deps_warp(const WfParams &P, int first, int count, int2 mine, unsigned run, int lane, Idle idle)
 {
@@ -115,7 +121,6 @@ __device__ __forceinline__ bool wait_deps_warp(const WfParams &P, int first, int
             if (!idled) { idled = true; idle(); }
             if (i >= P.spin_limit) return false;
             if ((i & 63u) == 63u && __any_sync(0xffffffffu, ld_relaxed(P.counters + 2) != 0u)) return false;
-            __nanosleep(32);
         }
     }
     __syncwarp();            // every lane's acquire now orders the whole warp's later reads
@@ -1102,14 +1107,12 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                     for (int u = 0; u < units_n && units_n <= WF_UNITS; ++u) mbar_arrive(ufree0 + 8u * ((uc + u) & (WF_UNITS - 1)));
                     uc += units_n;
                     bulk_wait_all();
-                    __threadfence();
-                    atomicAdd(P.counters + ctr_base + rec_tr(cur), 1u);
+                    add_release(P.counters + ctr_base + rec_tr(cur));
                 } else {
                     if (kind == WF_CONV) uc += units_n;            // stored, and handed back, by the workers
                     const uint32_t q = k % WF_PUBQ, round = k / WF_PUBQ;
                     if (!mbar_wait_abortable(pubf0 + 8u * q, round & 1u, abort_flag)) { fail = !*abort_flag; break; }
-                    __threadfence();
-                    atomicAdd(P.counters + ctr_base + rec_tr(cur), 1u);
+                    add_release(P.counters + ctr_base + rec_tr(cur));
                     mbar_arrive(pube0 + 8u * q);
                     ++k;
                 }
@@ -1155,9 +1158,8 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
             __syncwarp();
             if (lane == 0) {
                 tr(TRACE_FETCH0 + j, 1);
-                __threadfence();                                   // the warp's stores, then the release increments
-                atomicAdd(P.counters + rec.w, 1u);
-                atomicAdd(P.counters + 3, 1u);
+                add_release(P.counters + rec.w);                   // the warp's stores, then the increments
+                add_release(P.counters + 3);
                 tr(TRACE_FETCH0 + j, 2);
             }
         }
