@@ -16,8 +16,8 @@
 // A strided window (stride 2) reads every other row/column: the activation is exposed through
 // one tensor map per (row parity, column parity) whose base is offset by the parity and whose
 // strides are doubled, so each tap is again a dense box.  K is always walked in the order
-// (channel slab, kh, kw), whatever the tile position, so a pixel's value does not depend on the
-// band that computes it.  Every wait is bounded; a wait that runs out sets the status word.
+// (channel slab, kh, kw), whatever the tile position, and a plan that sums K in parts has one
+// accumulator per part, so a pixel's value does not depend on the band that computes it.  Every wait is bounded; a wait that runs out sets the status word.
 #include <cuda.h>
 #include <atomic>
 
@@ -48,6 +48,7 @@ struct TcParams {
     uint32_t a_stage_bytes, b_stage_bytes, tmem_cols;
     uint32_t layout_code, sbo_bytes;
     uint32_t idesc;
+    int k_split;                   // accumulators: the channel slabs are summed in this many parts
 };
 
 constexpr int TC_THREADS = 192;
@@ -102,7 +103,7 @@ __global__ void __launch_bounds__(TC_THREADS) conv_tc_kernel(const __grid_consta
     const int n0 = tile_n * (128 >> (p.tw_log + p.tr_log));
     const int co0 = blockIdx.y * p.BN;
     const int slabs = p.cin / p.BK;
-    const int n_iter = p.kh * p.kw * slabs;
+    const int n_iter = p.kh * p.kw * slabs, n_part = n_iter / p.k_split;
 
     if (warp == 0 && elect_one()) {
         // ---------------- TMA producer ----------------
@@ -138,7 +139,9 @@ __global__ void __launch_bounds__(TC_THREADS) conv_tc_kernel(const __grid_consta
         }
     } else if (warp == 1 && elect_one()) {
         // ---------------- MMA issuer ----------------
-        for (int it = 0; it < n_iter; ++it) {
+        uint32_t acc = tmem_acc;
+        for (int it = 0, in_part = 0; it < n_iter; ++it, ++in_part) {
+            if (in_part == n_part) { in_part = 0; acc += (uint32_t)p.BN; }     // the next part has an accumulator of its own
             const int s = it % p.stages;
             const uint32_t round = (uint32_t)(it / p.stages);
             if (*abort_flag || !mbar_wait(full0 + 8u * s, round & 1)) {
@@ -151,7 +154,7 @@ __global__ void __launch_bounds__(TC_THREADS) conv_tc_kernel(const __grid_consta
             for (int k = 0; k < p.BK / 16; ++k) {
                 const uint64_t ad = smem_desc(sa + 32u * k, p.sbo_bytes, p.layout_code);
                 const uint64_t bd = smem_desc(sb + 32u * k, p.sbo_bytes, p.layout_code);
-                umma_bf16(tmem_acc, ad, bd, p.idesc, (it > 0 || k > 0) ? 1u : 0u);
+                umma_bf16(acc, ad, bd, p.idesc, (in_part > 0 || k > 0) ? 1u : 0u);
             }
             umma_commit(empty0 + 8u * s);                     // stage reusable once these MMAs retire
         }
@@ -179,6 +182,13 @@ __global__ void __launch_bounds__(TC_THREADS) conv_tc_kernel(const __grid_consta
                 uint32_t r[16];
                 tmem_ld16(tmem_acc + ((uint32_t)(g * 32) << 16) + (uint32_t)j, r);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                for (int q = 1; q < p.k_split; ++q) {              // the parts in order
+                    uint32_t part[16];
+                    tmem_ld16(tmem_acc + ((uint32_t)(g * 32) << 16) + (uint32_t)(q * p.BN + j), part);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) r[i] = __float_as_uint(__fadd_rn(__uint_as_float(r[i]), __uint_as_float(part[i])));
+                }
                 if (!valid) continue;
                 float v[16];
 #pragma unroll
@@ -199,7 +209,7 @@ __global__ void __launch_bounds__(TC_THREADS) conv_tc_kernel(const __grid_consta
                         rv[2 * i + 1] = __uint_as_float(rw[i] & 0xFFFF0000u);
                     }
                 }
-                finish16<2>(v, rv, res ? p.res_pos : LOP_RES_NONE, p.act);
+                finish_n<2>(v, rv, res ? p.res_pos : LOP_RES_NONE, p.act);
                 uint32_t o[8];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
@@ -260,6 +270,7 @@ ConvTcGeom conv_tc_geometry(const ConvArgs &a, int rows, bool fill_sms)
             if (best < 0 || tiles < best) { best = tiles; g.TW = tw; g.TR = tr; g.TN = tn; }
         }
     // with few pixel tiles, narrower channel tiles give more CTAs to fill the 148 SMs
+    if (a.k_split > 1 && g.BN > 64) g.BN = 64;                // (an accumulator per part; Cout is a multiple of 64)
     while (fill_sms && best * (a.Cout / g.BN) < 148 && g.BN % 32 == 0 && g.BN > 32) g.BN /= 2;
     const int stage = 128 * g.BK * 2 + ((g.BN * g.BK * 2 + 1023) / 1024) * 1024;
     int stages = (100 * 1024) / stage;
@@ -328,7 +339,8 @@ cudaError_t launch_conv_tc(const ConvArgs &a, const ConvTcGeom &g, const ConvTcM
     p.a_stage_bytes = 128u * g.BK * 2u;
     p.b_stage_bytes = ((uint32_t)(g.BN * g.BK * 2) + 1023u) / 1024u * 1024u;
     uint32_t cols = 32;
-    while (cols < (uint32_t)g.BN) cols *= 2;
+    p.k_split = a.k_split;
+    while (cols < (uint32_t)(g.BN * a.k_split)) cols *= 2;
     p.tmem_cols = cols;
     p.layout_code = g.BK == 64 ? 2u : (g.BK == 32 ? 4u : 6u);
     p.sbo_bytes = 8u * g.BK * 2u;

@@ -16,6 +16,7 @@ struct LayerInfo {
     int Hin = 0, Win = 0;          // spatial extent of the main input
     int Ho = 0, Wo = 0, Co = 0;    // output shape
     int kernel = K_CONV_SIMT;
+    int k_split = 1;               // parts the tensor-core kernels sum K in (1, 2 or 4), each part in fp32, then the parts in order
     int cin_eff = 0;               // channels the tensor-core kernel sees (= the gathered values K of a pixel for a stem)
     bool linear = false;           // given as the row-wise operator LOP_LINEAR (runs as the pointwise convolution it is)
     bool stem_gather = false;      // thin chain input: the values its pixels read are gathered into a tensor

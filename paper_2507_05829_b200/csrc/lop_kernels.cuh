@@ -16,6 +16,7 @@ struct ConvArgs {
     int kh, kw, sh, sw, ph, pw, dh, dw;
     int act, res_pos;
     int oh_lo, oh_hi;       // rows to compute
+    int k_split;            // tensor-core kernels: parts of the channel chunks that are summed on their own, then in order
     // the input in elements: a pixel's channels (those up to Cin read as zeros), from a pixel to the next, from a row to
     // the next.  x_pixel < x_run only for a gathered stem, whose neighbouring pixels share values.
     int x_run, x_pixel;

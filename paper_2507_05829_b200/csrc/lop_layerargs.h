@@ -52,6 +52,7 @@ inline ConvArgs conv_args(const lop_plan_t *pl, int i, const void *in, void *out
     a.kh = l.kh; a.kw = l.kw; a.sh = l.sh; a.sw = l.sw; a.ph = l.ph; a.pw = l.pw; a.dh = l.dh; a.dw = l.dw;
     a.act = l.act; a.res_pos = a.res ? l.residual_pos : LOP_RES_NONE;
     a.oh_lo = lo; a.oh_hi = hi;
+    a.k_split = li.k_split;
     a.dbg = (pl->flags & LOP_FLAG_DEBUG_BOUNDS) ? reinterpret_cast<unsigned *>(static_cast<char *>(ws) + pl->status_off) : nullptr;
     a.x_run = a.x_pixel = a.Cin; a.x_row = (long long)a.Win * a.Cin;
     if (li.kernel == K_CONV_TC) {

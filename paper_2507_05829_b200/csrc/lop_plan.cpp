@@ -6,6 +6,7 @@
 // an output is used) and the contiguous-interval rule of Sec. IV-C ("Computational Efficiency"):
 // the operations one executor runs for an operator form one interval, so a band is one row
 // interval per layer and one kernel launch.
+#include <algorithm>
 #include <atomic>
 #include <cstdarg>
 #include <cstdio>
@@ -204,6 +205,73 @@ static void plan_bands(lop_plan_t &pl)
     }
 }
 
+// In how many parts a tensor-core convolution sums its K.  Layers with few output tiles and a long K (the 7x7 maps of a
+// single image: eight tiles of 9 us each) leave the chip idle, so the persistent kernel gives the parts of a tile to the CTAs
+// of a cluster, which exchange their partial sums.  The choice is part of the plan, not of the launch: every executor sums in
+// the same parts, and a tensor's bits do not depend on which of them computed it, nor on the band.
+// The estimate, in microseconds: a (64-channel chunk, filter tap) step takes 0.125 where one box serves all taps, 0.28 with a
+// box per tap, 0.19 for pointwise layers (what arrives per step at the 80-100 GB/s of an SM's operand loads); 2.2 go to the
+// first operands' latency and the epilogue, 1.7 to the exchange; 148 CTAs, of which clusters of four can use 132.
+// A kernel that knows split tiles takes 0.1 to 0.2 longer for every other tile, those of the chain's earlier layers too, of
+// which a plan knows nothing but that there are several times as many.  So the layers of a plan are split together, and only
+// where that saves a good deal per 148 of the plan's own tiles -- less where most of its windows are split: then its deeper
+// neighbour's are too, and the price is paid once for all.
+// Measured, resident, without and with: ResNet-18 of 224x224 142 -> 117 us for one image, 147 -> 132 for four, 173 -> 172 for
+// eight (with one layer of four split 202 -> 212 for twelve: left alone); ResNet-50 336 -> 286 for one, 365 -> 325 for four, 404 -> 397 for eight.
+static int split_of_k(const lop_plan_t &pl, int i, double *saves, double *rounds)
+{
+    const LayerInfo &li = pl.layers[i];
+    const lop_layer &l = li.l;
+    *saves = *rounds = 0.0;
+    if (li.stem_gather || l.cout % 64 != 0 || l.cin % 64 != 0) return 1;
+    const bool window = l.kh * l.kw > 1, slab = window && l.sh == 1 && l.sw == 1;
+    const int halo = (l.kw - 1) * l.dw;
+    long long pixel_tiles = -1;
+    for (int p = slab ? 16 : 1; p <= 128; p *= 2)
+        for (int r = slab ? 128 / p : 1; r <= 128 / p; r *= 2) {
+            const int cols = slab ? p - halo : p, n = 128 / (p * r);
+            if (cols < 1 || n > pl.N) continue;
+            const long long t = (long long)((li.Wo + cols - 1) / cols) * ((li.Ho + r - 1) / r) * ((pl.N + n - 1) / n);
+            if (pixel_tiles < 0 || t < pixel_tiles) pixel_tiles = t;
+        }
+    if (pixel_tiles < 0) return 1;
+    const int chunks = l.cin / 64;
+    const double walk = (double)chunks * l.kh * l.kw * (slab ? 0.125 : (window ? 0.28 : 0.19));
+    auto time = [&](int s) {
+        const long long ctas = s == 4 ? 132 : 148, tiles = pixel_tiles * (l.cout / 64) * s, wide = pixel_tiles * (l.cout / 128);
+        const double t = (double)((tiles + ctas - 1) / ctas) * (walk / s + 2.2) + (s > 1 ? 1.7 : 0.0);
+        // (a tile that is not split may be 128 channels wide, which takes about half as long again)
+        return s > 1 || l.cout % 128 != 0 ? t : std::min(t, (double)((wide + ctas - 1) / ctas) * (1.5 * walk + 2.9));
+    };
+    *rounds = (double)pixel_tiles * (l.cout / 64) / 148.0;
+    for (size_t j = i + 1; j < pl.layers.size(); ++j)
+        if (pl.layers[j].l.op == LOP_MAXPOOL2D && pl.layers[j].l.input_from == i) return 1;       // (may be pooled in the epilogue)
+    int best = 1;
+    for (int s = 2; s <= 4; s *= 2)
+        if (chunks % s == 0 && time(s) < time(best) - (best == 1 ? 0.5 : 0.0)) best = s;
+    *saves = time(1) - time(best);
+    return best;
+}
+static void choose_splits(lop_plan_t &pl)
+{
+    double saves = 0.0, rounds = 0.0;
+    int windows = 0, split = 0;
+    for (size_t i = 0; i < pl.layers.size(); ++i) {
+        LayerInfo &li = pl.layers[i];
+        if (li.kernel != K_CONV_TC) continue;
+        double s, r;
+        li.k_split = split_of_k(pl, (int)i, &s, &r);
+        saves += s;
+        rounds += r;
+        if (li.l.kh * li.l.kw == 1) continue;
+        ++windows;
+        if (li.k_split > 1) ++split;
+    }
+    const bool most = windows > 0 && 2 * split >= windows;
+    if (saves < (most ? 0.35 : 1.5) * rounds)
+        for (LayerInfo &li : pl.layers) li.k_split = 1;
+}
+
 // Decide which kernel serves each layer and lay the workspace out.
 static void choose_kernels(lop_plan_t &pl)
 {
@@ -246,6 +314,7 @@ static void choose_kernels(lop_plan_t &pl)
         li.kernel = K_CONV_TC;
     }
 
+    choose_splits(pl);
     // Copy-engine band pipeline: every copy costs a few microseconds of stream commands whatever its size, so an input
     // of megabytes cut into many bands is moved a few neighbouring bands per copy (at most LOP_MAX_BAND_COPIES copies);
     // the bands of one copy arrive together.  Small inputs keep one copy per band.

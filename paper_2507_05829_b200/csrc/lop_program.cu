@@ -80,8 +80,8 @@ struct Geom {
 // a: the convolution as its kernel sees it (a gathered stem already reduced to 1x1).
 // even_tiles: tiles must hold whole 2x2 windows (rows and valid columns even, at least two rows).
 // bulk_out: the tile's output leaves by bulk stores (the workers' own copy-out needs every unit of the tile in place).
-// ring: bytes of the operand ring, of which a slab stage needs two activation boxes and a weight box.
-Geom choose_geom(const ConvArgs &a, int rows, bool even_tiles, bool bulk_out, uint32_t ring)
+// ring: bytes of the operand ring, of which a slab stage needs two activation boxes and a weight box.  n_cta: the program's CTAs.
+Geom choose_geom(const ConvArgs &a, int rows, bool even_tiles, bool bulk_out, uint32_t ring, int n_cta)
 {
     Geom g{};
     g.BK = a.Cin % 64 == 0 ? 64 : (a.Cin % 32 == 0 ? 32 : 16);
@@ -131,8 +131,9 @@ Geom choose_geom(const ConvArgs &a, int rows, bool even_tiles, bool bulk_out, ui
     // issuing thread 48 cycles, one with N = 128 65; the epilogue 1.5 and 2.2 us), so the width follows from the number of
     // rounds the layer's tiles take on 148 SMs.  Not below 64: an MMA with N = 32 costs as much as one with N = 64.
     const long long pixel_tiles = (long long)((a.Wo + g.tw_valid - 1) / g.tw_valid) * ((a.Ho + g.TR - 1) / g.TR) * ((a.N + g.TN - 1) / g.TN);
-    auto rounds = [&](int bn) { return (pixel_tiles * (a.Cout / bn) + 147) / 148; };
+    auto rounds = [&](int bn) { return (pixel_tiles * (a.Cout / bn) + n_cta - 1) / n_cta; };
     while (g.BN > 64 && g.BN % 32 == 0 && rounds(g.BN / 2) < 1.4 * rounds(g.BN)) g.BN /= 2;
+    if (a.k_split > 1) g.BN = (int)WF_SPLIT_BN;
     g.a_bytes = (uint32_t)g.RI * g.P * g.TN * row_bytes;
     // (a shifted tap reads up to halo_w pixels past the box, into whatever follows it in shared memory: those rows of the
     // accumulator are the dropped anchors of the halo gap)
@@ -370,10 +371,10 @@ struct Unit {
 // layers over early rows have to come in between (the pipeline of Sec. IV-B). Dealing out, whenever
 // a CTA is free, the ready unit with the longest chain of readers behind it does either: while the machine waits the
 // order follows the rows down the layers, and once it is saturated it turns layer by layer by itself.
-// arrival_us: expected arrival of each band a negative dependency names.
-void schedule_units(const std::vector<Unit> &units, const std::vector<int2> &deps, const std::vector<double> *arrival_us, std::vector<int> &order)
+// arrival_us: expected arrival of each band a negative dependency names.  n_cta: how many CTAs there will be.
+void schedule_units(const std::vector<Unit> &units, const std::vector<int2> &deps, const std::vector<double> *arrival_us, int n_cta, std::vector<int> &order)
 {
-    const int n = (int)units.size(), n_cta = 148;
+    const int n = (int)units.size();
     // producer's last store -> consumer sees the counter: about 1 us, and a margin, because a unit dealt out too early makes
     // a CTA wait with everything behind it, one dealt out too late costs next to nothing (1 -> 4: a ResNet-50 of batch 32
     // 1091 -> 1063 us, a 1024x1024 stack streamed 314 -> 302)
@@ -515,6 +516,12 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
         else if (!rq.fetch && li.l.op == LOP_DWCONV2D && dw_tile(pl, li, &t))
             stg_bytes = std::max(stg_bytes, round_up_u32((uint32_t)rowop::dw_tile_bytes(li.l.kh, li.l.kw, li.l.sh, li.l.sw, li.l.dh, li.l.dw, t), 1024u));
     }
+    // CTAs per cluster: as many as the most finely split tile has parts.  Clusters of four leave some SMs out (33 of them fit).
+    int cluster = 1;
+    for (const StageReq &rq : reqs)
+        if (!rq.fetch && !rq.gather) cluster = std::max(cluster, segs[rq.seg].pl->layers[rq.layer].k_split);
+    const int n_cta = cluster == 4 ? 132 : 148;
+    if (cluster > 1) unit_bytes = std::max(unit_bytes, WF_SPLIT_UNIT);
     const uint32_t ring_least = (227u * 1024u - 1024u - WF_FIXED_SMEM - stg_bytes - WF_UNITS * 16u * 1024u) & ~1023u;
     std::vector<char> out_on_device(segs.size());
     for (size_t i = 0; i < segs.size(); ++i) out_on_device[i] = in_device_memory(segs[i].out);
@@ -598,7 +605,7 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
                         reqs[k].layer == rq.layer + 1 && rq.lo == 2 * reqs[k].lo && rq.hi == 2 * reqs[k].hi) { rj = k; break; }
             const bool fuse = rj < reqs.size();
             const bool bulk_out = !fuse && (rq.layer + 1 < (int)pl->layers.size() || out_on_device[rq.seg]);
-            const Geom g = choose_geom(a, rows, fuse, bulk_out, ring_least);
+            const Geom g = choose_geom(a, rows, fuse, bulk_out, ring_least, n_cta);
             st.kind = WF_CONV;
             st.mode = g.mode;
             st.x = a.x; st.res = a.res; st.scale = a.scale; st.shift = a.shift; st.y = a.y;
@@ -629,7 +636,11 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
             st.sbo_bytes = 8u * st.row_bytes;
             // instruction descriptor: fp32 accumulate, bf16 x bf16, both operands K-major, N = BN, M = 128
             st.idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(g.BN >> 3) << 17) | ((128u >> 4) << 24);
-            const int sub = unit_channels(g.BN);
+            // a split tile's items: each walks its share of the chunks and finishes its slice of the channels
+            st.s_log = ilog2i(a.k_split);
+            st.n_chunks = g.n_chunks >> st.s_log;
+            const int out_channels = g.BN >> st.s_log;
+            const int sub = unit_channels(out_channels);
             st.sub_log = ilog2i(sub);
             unit_bytes = std::max(unit_bytes, round_up_u32((uint32_t)((128 >> st.p_log) * g.tw_valid * sub * 2), 1024u));
             st.out_map = st.res_map = -1;
@@ -653,13 +664,13 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
                 out_lo = reqs[rj].lo; out_hi = reqs[rj].hi;
             }
             // an MMA costs the issuing thread 0.05 to 0.09 us with its share of the waits, the epilogue runs beside the next tile's
-            item_us = std::max(g.BN > 64 ? 2.2 : 1.5, 0.6 + 0.07 * g.n_chunks * g.n_taps * (g.BK / 16));
+            item_us = std::max(g.BN > 64 ? 2.2 : 1.5, 0.6 + 0.07 * st.n_chunks * g.n_taps * (g.BK / 16)) + (st.s_log ? 0.9 : 0.0);
             tail_us = 3.0;
             group_rows = g.TR;
             tiles_r = (rows + g.TR - 1) / g.TR;
             tiles_w = (a.Wo + g.tw_valid - 1) / g.tw_valid;
             tiles_n = (a.N + g.TN - 1) / g.TN;
-            cout_tiles = a.Cout / g.BN;
+            cout_tiles = a.Cout / out_channels;
         }
         if (tiles_w > 65535 || tiles_n > 65535 || cout_tiles > 65535 || tiles_r >= (1 << 20)) {
             set_error("layer %d: too many tiles for one stage", rq.layer);
@@ -734,12 +745,28 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
 
     if (arrival_us || cx.raw >= 0) {
         std::vector<int> order;
-        schedule_units(units, deps, arrival_us, order);
+        schedule_units(units, deps, arrival_us, n_cta, order);
         if (order.size() != units.size()) { set_error("the stages depend on each other in a cycle"); return LOP_EINVAL; }
         std::vector<int4> dealt;
         dealt.reserve(items.size());
         for (int u : order) dealt.insert(dealt.end(), items.begin() + units[u].first_item, items.begin() + units[u].first_item + units[u].items);
         items.swap(dealt);
+    }
+    if (cluster > 1) {
+        // a split tile's items start at the first CTA of its part of a cluster: items without work fill what is missing
+        std::vector<int4> placed;
+        placed.reserve(items.size() + items.size() / 8);
+        for (size_t i = 0; i < items.size();) {
+            const size_t parts = (size_t)1 << stages[items[i].x & 0xFFFF].s_log;
+            while (placed.size() % parts) placed.push_back(make_int4((int)stages.size(), 0, 0, 0));
+            for (size_t e = i + parts; i < e; ++i) placed.push_back(items[i]);
+        }
+        items.swap(placed);
+        if (stages.size() >= 65535) { set_error("program has too many stages"); return LOP_EUNSUPPORTED; }
+        WfStage none{};
+        none.kind = WF_NONE;
+        none.kh = none.kw = none.sh = none.sw = none.tb = 1;
+        stages.push_back(none);
     }
     lop_plan_t *pl0 = segs[0].pl;
     Program *p = new (std::nothrow) Program();
@@ -773,7 +800,7 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
         const uint32_t boxes = (uint32_t)st.n_chunks * ((st.n_taps + st.tb - 1) / st.tb);
         const uint32_t beside = std::max(2u * a_sz, st.mode == WF_TAP ? LOP_ENTRY_BYTES / a_sz * a_sz : 0u);
         const int cout_tiles = st.Cout / st.BN;
-        if (boxes * b_sz <= LOP_KEEP_BYTES && boxes * b_sz + beside <= ring_bytes && 148 % cout_tiles == 0 && tiles_of[st.map_base] >= 2 * 148)
+        if (st.s_log == 0 && boxes * b_sz <= LOP_KEEP_BYTES && boxes * b_sz + beside <= ring_bytes && n_cta % cout_tiles == 0 && tiles_of[st.map_base] >= 2 * n_cta)
             st.keep_bytes = (int)(boxes * b_sz);
         if (2u * a_sz + b_sz > ring_bytes) { delete p; set_error("tile buffers do not fit shared memory"); return LOP_EUNSUPPORTED; }
         if (st.mode == WF_SLAB && !st.keep_bytes) box_step[a_sz] = std::gcd(box_step[a_sz], b_sz);
@@ -849,6 +876,7 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
     P.fetch_src = fetch_src;
     P.fetch_dst = const_cast<void *>(segs[0].in);
     P.n_fetch = (int)fetch_items.size();
+    P.cluster = cluster;
     P.row_ops = P.smooth = 0;
     for (const WfStage &st : stages)
         if (st.kind == WF_DWCONV || st.kind == WF_LAYERNORM || st.kind == WF_CONCAT) P.row_ops = 1;
@@ -873,7 +901,8 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
     int resident = 0;
     e = wavefront_resident_ctas(P, &resident);
     if (e != cudaSuccess) { program_destroy(p); set_error("occupancy query failed: %s", cudaGetErrorString(e)); return LOP_ECUDA; }
-    if (resident < p->grid) {
+    if (cluster > 1) p->grid = std::min((n_items + cluster - 1) / cluster * cluster, resident / cluster * cluster);
+    if (resident < p->grid || p->grid == 0) {
         program_destroy(p);
         set_error("the device holds %d CTAs of the persistent kernel at a time, the program needs %d", resident, p->grid);
         return LOP_EUNSUPPORTED;

@@ -40,6 +40,36 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes)
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
+// Distributed shared memory: an address of this CTA's shared memory in CTA `rank` of the cluster; stores there whose bytes
+// count on one of that CTA's barriers.
+__device__ __forceinline__ uint32_t map_to_cta(uint32_t addr, uint32_t rank)
+{
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ uint32_t cta_rank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void st_async(uint32_t remote, uint32_t value, uint32_t remote_bar)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(remote), "r"(value), "r"(remote_bar) : "memory");
+}
+__device__ __forceinline__ void st_async4(uint32_t remote, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t remote_bar)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(remote), "r"(a), "r"(b), "r"(c), "r"(d),
+                 "r"(remote_bar)
+                 : "memory");
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive;" ::: "memory");
+    asm volatile("barrier.cluster.wait;" ::: "memory");
+}
+
 // Bounded wait on an mbarrier phase; false when the limit ran out.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
 {
@@ -142,6 +172,13 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16])
         : "memory");
 }
 
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr)
+                 : "memory");
+}
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32])
 {
     asm volatile(
@@ -210,58 +247,58 @@ __device__ __forceinline__ float2 activate2_t(float t0, float t1)
     if (ACT == LOP_ACT_GELU) return gelu2(t0, t1);
     return make_float2(t0, t1);
 }
-template <int ACT>
-__device__ __forceinline__ void activate16(float (&v)[16])
+template <int ACT, int N>
+__device__ __forceinline__ void activate_n(float (&v)[N])
 {
 #pragma unroll
-    for (int i = 0; i < 16; i += 2) {
+    for (int i = 0; i < N; i += 2) {
         const float2 f = activate2_t<ACT>(v[i], v[i + 1]);
         v[i] = f.x; v[i + 1] = f.y;
     }
 }
 
-template <int ACT>
-__device__ __forceinline__ void finish16_t(float (&v)[16], const float (&rv)[16], int res_pos)
+template <int ACT, int N>
+__device__ __forceinline__ void finish_n_t(float (&v)[N], const float (&rv)[N], int res_pos)
 {
     if (res_pos == LOP_RES_PRE_ACT) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = __fadd_rn(v[i], rv[i]);
+        for (int i = 0; i < N; ++i) v[i] = __fadd_rn(v[i], rv[i]);
     }
-    activate16<ACT>(v);
+    activate_n<ACT>(v);
     if (res_pos == LOP_RES_POST_ACT) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = __fadd_rn(v[i], rv[i]);
+        for (int i = 0; i < N; ++i) v[i] = __fadd_rn(v[i], rv[i]);
     }
 }
-// Last step of the fused epilogue on 16 channels: v = scale*acc + shift already; rv = residual values.
+// Last step of the fused epilogue on N channels: v = scale*acc + shift already; rv = residual values.
 // res_pos must be LOP_RES_NONE when there is no residual (rv is then not read).  FORM: 0 has neither SiLU nor GELU, 1 has
 // both (the persistent kernel, whose roles compete for registers and instruction cache), 2 has a copy of the whole for each
 // activation (a stand-alone kernel: 51.3 us for a VGG block where form 1 takes 54.2).
 // The additions are kept from being contracted into an activation's last product: both forms give the same bits.
-template <int FORM>
-__device__ __forceinline__ void finish16(float (&v)[16], const float (&rv)[16], int res_pos, int act)
+template <int FORM, int N>
+__device__ __forceinline__ void finish_n(float (&v)[N], const float (&rv)[N], int res_pos, int act)
 {
     if (FORM == 2) {
-        if (act == LOP_ACT_RELU) finish16_t<LOP_ACT_RELU>(v, rv, res_pos);
-        else if (act == LOP_ACT_SILU) finish16_t<LOP_ACT_SILU>(v, rv, res_pos);
-        else if (act == LOP_ACT_GELU) finish16_t<LOP_ACT_GELU>(v, rv, res_pos);
-        else finish16_t<LOP_ACT_NONE>(v, rv, res_pos);
+        if (act == LOP_ACT_RELU) finish_n_t<LOP_ACT_RELU>(v, rv, res_pos);
+        else if (act == LOP_ACT_SILU) finish_n_t<LOP_ACT_SILU>(v, rv, res_pos);
+        else if (act == LOP_ACT_GELU) finish_n_t<LOP_ACT_GELU>(v, rv, res_pos);
+        else finish_n_t<LOP_ACT_NONE>(v, rv, res_pos);
         return;
     }
     if (res_pos == LOP_RES_PRE_ACT) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = __fadd_rn(v[i], rv[i]);
+        for (int i = 0; i < N; ++i) v[i] = __fadd_rn(v[i], rv[i]);
     }
     if (act == LOP_ACT_RELU) {
-        activate16<LOP_ACT_RELU>(v);
+        activate_n<LOP_ACT_RELU>(v);
     } else if (FORM > 0 && act == LOP_ACT_SILU) {
-        activate16<LOP_ACT_SILU>(v);
+        activate_n<LOP_ACT_SILU>(v);
     } else if (FORM > 0 && act == LOP_ACT_GELU) {
-        activate16<LOP_ACT_GELU>(v);
+        activate_n<LOP_ACT_GELU>(v);
     }
     if (res_pos == LOP_RES_POST_ACT) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = __fadd_rn(v[i], rv[i]);
+        for (int i = 0; i < N; ++i) v[i] = __fadd_rn(v[i], rv[i]);
     }
 }
 

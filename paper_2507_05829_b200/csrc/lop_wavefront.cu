@@ -47,7 +47,7 @@ constexpr int EPI_THREADS = 32 * WF_WORKER_WARPS;
 #define LOP_PREFETCH 32
 #endif
 constexpr int PREFETCH_BOXES = LOP_PREFETCH;                // weight boxes of a tile asked for ahead of its dependencies
-static_assert(8 * (2 * WF_ENTRIES + 4 + 2 * WF_PUBQ + 4 + 3 * WF_UNITS + 2 + WF_GROUPS) + 128 + 2048 + 8 * (128 + 32) <= WF_FIXED_SMEM, "barriers and tables");
+static_assert(8 * (2 * WF_ENTRIES + 4 + 2 * WF_PUBQ + 4 + 3 * WF_UNITS + 2 + WF_GROUPS + 2) + 128 + 2048 + 8 * (128 + 32) <= WF_FIXED_SMEM, "barriers and tables");
 constexpr int COL_GROUPS = WF_WORKER_WARPS / 4;            // worker warps sharing a TMEM lane group split the columns
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned *p)
@@ -566,10 +566,189 @@ __device__ __noinline__ void gather_item(const WfStage *st, int n, int tile_r, i
     }
 }
 
+// ---- split tiles: the CTAs of a cluster (or half of one) sum a tile's channel chunks in parts and exchange slices of the sums.
+// Places in shared memory that the two functions below need, from the address of the first barrier on.
+constexpr uint32_t BAR_ACCF = 16u * WF_ENTRIES;                                // accumulators complete
+constexpr uint32_t BAR_SSF = BAR_ACCF + 32u + 16u * WF_PUBQ;                   // scale / shift in place
+constexpr uint32_t BAR_UGRANT = BAR_SSF + 32u;                                 // output units: granted, ready, free
+constexpr uint32_t BAR_UREADY = BAR_UGRANT + 8u * WF_UNITS, BAR_UFREE = BAR_UREADY + 8u * WF_UNITS;
+constexpr uint32_t BAR_XOK = BAR_UFREE + 8u * WF_UNITS + 16u + 8u * WF_GROUPS; // the others take partial sums
+constexpr uint32_t BAR_XFULL = BAR_XOK + 8u;                                   // the others' partial sums are here
+constexpr uint32_t BAR_MISC = BAR_XFULL + 8u;                                  // words: [1] abort, [8 + q] the unit part q takes sums in
+
+__device__ __forceinline__ uint32_t ld_shared(uint32_t addr)
+{
+    uint32_t v;
+    asm volatile("ld.volatile.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+}
+// Bounded wait on a barrier that other CTAs of the cluster may complete; gives up when this CTA's abort flag is raised.
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, uint32_t abort_at)
+{
+    for (uint32_t i = 0; i < WAIT_LIMIT; ++i) {
+        uint32_t done;
+        asm volatile(
+            "{\n"
+            ".reg .pred p;\n"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+            "selp.u32 %0, 1, 0, p;\n"
+            "}\n"
+            : "=r"(done)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        if (done) return true;
+        if ((i & 255u) == 255u && ld_shared(abort_at)) return false;
+    }
+    return false;
+}
+
+// The loader's side, by its one thread: once the units that partial sums arrive in are free, the barriers are armed and the
+// other CTAs told where to write.  cout: the item's slice; uc: output units before these; n_split: split tiles before this one.
+// (Barriers whose phase is not over cannot be armed again: with two parts the next tile's units are free before this one's
+// exchange is done.)
+__device__ __noinline__ bool take_partial_sums(uint32_t bars, uint32_t cout, uint32_t s_log, uint32_t uc, uint32_t n_split)
+{
+    const uint32_t others = (1u << s_log) - 1u, part = cout & others, base_rank = cta_rank() & ~others, abort_at = bars + BAR_MISC + 4u;
+    if (n_split > 0 && (!mbar_wait_cluster(bars + BAR_XOK, (n_split - 1u) & 1u, abort_at) || !mbar_wait_cluster(bars + BAR_XFULL, (n_split - 1u) & 1u, abort_at)))
+        return false;
+    for (uint32_t u = uc; u < uc + ((others + 1u) >> 1); ++u) {
+        const uint32_t sl = 8u * (u & (WF_UNITS - 1));
+        if (!mbar_wait_cluster(bars + BAR_UFREE + sl, ((u / WF_UNITS) & 1u) ^ 1u, abort_at)) return false;
+        mbar_arrive(bars + BAR_UGRANT + sl);                                   // (its phase; nobody waits for it)
+    }
+    mbar_expect_tx(bars + BAR_XOK, 4u * others);
+    mbar_expect_tx(bars + BAR_XFULL, others * (512u * (WF_SPLIT_BN >> s_log)));
+    for (uint32_t q = 0; q <= others; ++q)
+        if (q != part)
+            st_async(map_to_cta(bars + BAR_MISC + 4u * (8u + part), base_rank + q), uc & (WF_UNITS - 1), map_to_cta(bars + BAR_XOK, base_rank + q));
+    return true;
+}
+
+// The workers' side, by every worker thread, and the whole of a split tile's epilogue: this CTA's partial sums of the other
+// CTAs' channel slices go to those CTAs, the others' sums of this CTA's slice are added to its own, part by part in order (the
+// order in which every executor of the plan sums), and the slice is finished.  A unit holds 64 / parts channels x 128 rows of
+// fp32 from each of one or two senders, as [four channels][row]: neighbouring lanes write and read neighbouring 16 bytes.
+// acc: the accumulator; uc: units before the tile's, of which it has as many as are returned; a wait that runs out sets the
+// epilogue's failure word.
+// Bound by latency: about 1.7 us from the last MMA to the slice's first sum, of which the slowest CTA's lag is a part.
+// An epilogue of its own, out of line: with the exchange in front of the other tiles' epilogue, those took 0.2 us longer each
+// (a ResNet-50 of batch 32, which has no split tile, 830 -> 873 us).
+template <bool SMOOTH>
+__device__ __noinline__ uint32_t split_item(const WfStage *sp, int4 rec, uint8_t *smem_bars, uint32_t unit0, uint32_t unit_bytes, uint32_t acc, uint32_t uc, uint32_t cnt)
+{
+    const uint32_t n_split = ld_shared(smem_u32(smem_bars) + BAR_MISC + 16u);  // split tiles before this one
+    const uint32_t bars = smem_u32(smem_bars), s_log = (uint32_t)__ldg(&sp->s_log), parts = 1u << s_log, part = (uint32_t)rec_cout(rec) & (parts - 1u);
+    const uint32_t slice = WF_SPLIT_BN >> s_log, base_rank = cta_rank() & ~(parts - 1u), abort_at = bars + BAR_MISC + 4u, rx = uc + 1u;
+    const uint32_t per_unit = parts >> 1, from_bytes = 512u * slice;           // senders per unit (two parts: one, four: two)
+    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u, row = (warp & 3u) * 32u + lane, cgrp = (warp - WF_FIRST_WORKER) >> 2, buf = cnt & 1u;
+    auto sums_at = [&](uint32_t first_unit, uint32_t from) { return unit0 + ((first_unit + from / per_unit) & (WF_UNITS - 1)) * unit_bytes + (from & (per_unit - 1u)) * from_bytes + 16u * row; };
+    const int p_log = __ldg(&sp->p_log), tr_log = __ldg(&sp->tr_log), tw_valid = __ldg(&sp->tw_valid), sub_log = __ldg(&sp->sub_log);
+    const int act = __ldg(&sp->act), res_pos = ldg_ptr<const void *>(&sp->res) ? __ldg(&sp->res_pos) : LOP_RES_NONE;
+    const bool bulk_out = __ldg(&sp->out_map) >= 0;
+    acc += ((warp & 3u) * 32u) << 16;
+    bool ok = mbar_wait_cluster(bars + BAR_ACCF + 8u * buf, (cnt >> 1) & 1u, abort_at);
+    ok = ok && mbar_wait_cluster(bars + BAR_XOK, n_split & 1u, abort_at);
+    ok = __all_sync(0xffffffffu, ok);
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    uint32_t r[8];                                                             // (eight columns at a time: what this needs, the kernel around the call has not)
+#pragma unroll 1
+    for (uint32_t c = 0, k = 0; ok && c < WF_SPLIT_BN; c += 8) {
+        const uint32_t q = c / slice;
+        if (q == part) continue;
+        if (((++k + 1u) >> 1 & 1u) != cgrp) continue;                          // (the first and third 16 columns: the warps without a chunk to finish)
+        tmem_ld8(acc + c, r);
+        const uint32_t to = map_to_cta(sums_at(ld_shared(bars + BAR_MISC + 4u * (8u + q)), part < q ? part : part - 1u) + (c - q * slice) * 512u, base_rank + q);
+        const uint32_t bar = map_to_cta(bars + BAR_XFULL, base_rank + q);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        st_async4(to, r[0], r[1], r[2], r[3], bar);
+        st_async4(to + 2048u, r[4], r[5], r[6], r[7], bar);
+    }
+    // while they travel: where this row goes
+    const int m = (int)row, c = m & ((1 << p_log) - 1), rr = (m >> p_log) & ((1 << tr_log) - 1), img = m >> (p_log + tr_log);
+    const bool staged = c < tw_valid;
+    const int srow = ((img << tr_log) + rr) * tw_valid + c;
+    const int swz = sub_log == 5 ? (srow >> 1) & 3 : (srow >> 2) & 1;          // (a slice is 32 or 16 channels)
+    long long *row_pix = reinterpret_cast<long long *>(smem_bars + BAR_MISC + 128 + 2048);
+    if (!bulk_out && cgrp == 0 && staged) {
+        const int Ho = __ldg(&sp->Ho), Wo = __ldg(&sp->Wo), oh = __ldg(&sp->oh_lo) + (rec_tr(rec) << tr_log) + rr, ow = rec_tw(rec) * tw_valid + c;
+        const int n = rec_tn(rec) * (128 >> (p_log + tr_log)) + img, Cout = __ldg(&sp->Cout);
+        row_pix[srow] = ow < Wo && oh < __ldg(&sp->oh_hi) && n < __ldg(&sp->N) ? (((long long)n * Ho + oh) * Wo + ow) * Cout + rec_cout(rec) * (int)slice : -1LL;
+    }
+    const uint32_t sl = uc & (WF_UNITS - 1);
+    ok = ok && mbar_wait_cluster(bars + BAR_UGRANT + 8u * sl, (uc / WF_UNITS) & 1u, abort_at);
+    ok = ok && mbar_wait_cluster(bars + BAR_SSF + 8u * buf, (cnt >> 1) & 1u, abort_at);
+    ok = ok && mbar_wait_cluster(bars + BAR_XFULL, n_split & 1u, abort_at);
+    ok = __all_sync(0xffffffffu, ok);
+#pragma unroll 1
+    for (uint32_t j = 16u * cgrp; ok && j < min(slice, 16u * cgrp + 16u); j += 8) {
+        tmem_ld8(acc + part * slice + j, r);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (!staged) continue;
+        float v[8], rv[8];
+        for (uint32_t q = 0; q < parts; ++q) {
+            const uint32_t sums = sums_at(rx, q < part ? q : q - 1u) + j * 512u;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                uint32_t w[4] = {r[4 * e], r[4 * e + 1], r[4 * e + 2], r[4 * e + 3]};
+                if (q != part)
+                    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(sums + 2048u * e) : "memory");
+#pragma unroll
+                for (int i = 0; i < 4; ++i) v[4 * e + i] = q == 0 ? __uint_as_float(w[i]) : __fadd_rn(v[4 * e + i], __uint_as_float(w[i]));
+            }
+        }
+        const float *scale = reinterpret_cast<const float *>(smem_bars + BAR_MISC + 128) + 128 * buf + j, *shift = scale + 256;
+        uint8_t *my_row = smem_bars - bars + unit0 + sl * unit_bytes + (srow << (sub_log + 1));
+        uint4 *cp = reinterpret_cast<uint4 *>(my_row + (((int)(j >> 3) ^ swz) << 4));
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = fmaf(scale[i], v[i], shift[i]);
+        if (res_pos != LOP_RES_NONE) {
+            const uint4 q = *cp;
+            const uint32_t rw[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                rv[2 * i] = __uint_as_float(rw[i] << 16);
+                rv[2 * i + 1] = __uint_as_float(rw[i] & 0xFFFF0000u);
+            }
+        }
+        finish_n<SMOOTH ? 1 : 0>(v, rv, res_pos, act);
+        uint32_t o[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+            o[i] = *reinterpret_cast<const uint32_t *>(&h);
+        }
+        *cp = make_uint4(o[0], o[1], o[2], o[3]);
+    }
+    if (!ok) *reinterpret_cast<volatile uint32_t *>(smem_bars + BAR_MISC + 12) = 1u;
+    if (bulk_out) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    // (the units of the partial sums first: the publisher waits for the output unit only)
+    __syncwarp();
+    if (lane == 0) {
+        for (uint32_t u = rx; u < rx + (parts >> 1); ++u) mbar_arrive(bars + BAR_UREADY + 8u * (u & (WF_UNITS - 1)));
+        mbar_arrive(bars + BAR_UREADY + 8u * sl);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    epi_bar();                                                                 // accumulator drained, sums read, slice complete
+    if (threadIdx.x == 32u * WF_FIRST_WORKER) {
+        mbar_arrive(bars + BAR_ACCF + 16u + 8u * buf);
+        mbar_arrive(bars + BAR_SSF + 16u + 8u * buf);
+        for (uint32_t u = rx; u < rx + (parts >> 1); ++u) mbar_arrive(bars + BAR_UFREE + 8u * (u & (WF_UNITS - 1)));
+        *reinterpret_cast<volatile uint32_t *>(smem_bars + BAR_MISC + 16) = n_split + 1u;
+    }
+    if (!bulk_out && ld_shared(bars + BAR_MISC + 12) == 0u) {
+        copy_unit(smem_bars - bars + unit0 + sl * unit_bytes, row_pix, static_cast<uint4 *>(ldg_ptr<void *>(reinterpret_cast<const void *const *>(&sp->y))),
+                  (128 >> p_log) * tw_valid, sub_log, (int)threadIdx.x - 32 * WF_FIRST_WORKER);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");           // (as behind the other tiles' copy-out)
+        epi_bar();
+        if (threadIdx.x == 32u * WF_FIRST_WORKER) mbar_arrive(bars + BAR_UFREE + 8u * sl);
+    }
+    return 1u + (parts >> 1);
+}
+
 // FETCH: one more warp per CTA brings the chain input from host memory.  ROWOPS: the program has depth-wise /
 // normalisation / concatenation stages, SMOOTH: a convolution of it has SiLU or GELU; programs without them run an
-// instantiation that does not carry their code.
-template <bool FETCH, bool ROWOPS, bool SMOOTH>
+// instantiation that does not carry their code.  SPLIT: the CTAs are launched in clusters and the program has split tiles.
+template <bool FETCH, bool ROWOPS, bool SMOOTH, bool SPLIT>
 __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavefront_kernel(const WfParams P)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -580,15 +759,17 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
     const uint32_t ring_bytes = P.ring_bytes, unit_bytes = P.unit_bytes;
     const uint32_t ring0 = base, unit0 = ring0 + ring_bytes, simt0 = unit0 + WF_UNITS * unit_bytes, bars = simt0 + P.simt_bytes;
     const uint32_t full0 = bars, empty0 = full0 + 8u * WF_ENTRIES;      // operand entries: loaded / consumed
-    const uint32_t accf0 = empty0 + 8u * WF_ENTRIES, acce0 = accf0 + 16u;   // accumulators: complete / drained
+    const uint32_t accf0 = bars + BAR_ACCF, acce0 = accf0 + 16u;         // accumulators: complete / drained
     const uint32_t pubf0 = acce0 + 16u, pube0 = pubf0 + 8u * WF_PUBQ;    // items the workers stored themselves: stored / published
-    const uint32_t ssf0 = pube0 + 8u * WF_PUBQ, sse0 = ssf0 + 16u;      // scale/shift buffers of two tiles: full / empty
-    const uint32_t ugrant0 = sse0 + 16u;                                 // output units: free to write, the residual (if any) in place
-    const uint32_t uready0 = ugrant0 + 8u * WF_UNITS, ufree0 = uready0 + 8u * WF_UNITS;     // ... finished by the workers / read out
+    const uint32_t ssf0 = bars + BAR_SSF, sse0 = ssf0 + 16u;                 // scale/shift buffers of two tiles: full / empty
+    const uint32_t ugrant0 = bars + BAR_UGRANT;                          // output units: free to write, the residual (if any) in place
+    const uint32_t uready0 = bars + BAR_UREADY, ufree0 = bars + BAR_UFREE;  // ... finished by the workers / read out
     const uint32_t wfull = ufree0 + 8u * WF_UNITS, wempty = wfull + 8u;  // kept weights: loaded / last used
     const uint32_t gfull0 = wempty + 8u;                                 // slab stages: a group of boxes is loaded
-    uint8_t *tail = smem + (gfull0 + 8u * WF_GROUPS - base);
-    volatile uint32_t *misc = reinterpret_cast<volatile uint32_t *>(tail);      // [0] TMEM base, [1] abort, [2] run, [3] epilogue failure
+    const uint32_t xok = bars + BAR_XOK, xfull = bars + BAR_XFULL;       // split tiles
+    uint8_t *tail = smem + (bars + BAR_MISC - base);
+    volatile uint32_t *misc = reinterpret_cast<volatile uint32_t *>(tail);      // [0] TMEM base, [1] abort, [2] run, [3] epilogue failure,
+                                                                                // [8..11] the units the other parts of a split tile take sums in
     volatile uint32_t *entry_at = misc + 16;                                     // [WF_ENTRIES]: where the ring's entries start (loader only)
     float *s_scale = reinterpret_cast<float *>(tail + 128);                      // [2][128]: per-channel scale of this and the next tile
     float *s_shift = s_scale + 256;                                              // [2][128]
@@ -620,6 +801,8 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
         mbar_init(wfull, 1);
         mbar_init(wempty, 1);
         for (int g = 0; g < WF_GROUPS; ++g) mbar_init(gfull0 + 8u * g, 1);
+        mbar_init(xok, 1);
+        mbar_init(xfull, 1);
         for (int q = 0; q < WF_PUBQ; ++q) {
             mbar_init(pubf0 + 8u * q, 1);
             mbar_init(pube0 + 8u * q, 1);
@@ -627,7 +810,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
         misc[1] = 0;
         grid_wait();
         misc[2] = ld_acquire(P.counters) + 1u;                 // this launch is run number (completed runs + 1)
-        misc[3] = 0;
+        misc[3] = misc[4] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -639,6 +822,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (SPLIT) cluster_sync();                                 // the other CTAs' barriers are ready too
     grid_release();
     grid_wait();                                               // (all threads: thread 0 waited for what it read)
     if (threadIdx.x == 0 && blockIdx.x < 4) tr(TRACE_ITEMS - 8 + (int)blockIdx.x, 1);
@@ -657,14 +841,15 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
         int4 nxt = item + G < NI ? __ldg(&P.items[item + G]) : zero4;
         int2 dep_cur = (item < NI && lane < rec_ndep(cur)) ? __ldg(&P.deps[rec_dep0(cur) + lane]) : make_int2(0, 0);
         int sidx = -1;
-        int kind = -1, mode = 0, oh_lo = 0, tr_log = 0, p_log = 0, tw_valid = 0, BN = 0, BK = 0, n_chunks = 1, n_taps = 1, tbx = 1,
-            amask = 0, kh = 1, kw = 1, sh = 1, sw = 1, ph = 0, pw = 0, dh = 1, dw = 1;
+        // (what only some tiles need is read from the stage's record where it is needed: registers are what this kernel is short of)
+        int kind = -1, mode = 0, oh_lo = 0, tr_log = 0, p_log = 0, tw_valid = 0, BN = 0, BK = 0, n_chunks = 1, n_taps = 1, tbx = 1;
         uint32_t a_bytes = 0, b_bytes = 0;
         const CUtensorMap *maps = nullptr;
-        const float *scale = nullptr, *shift = nullptr;
-        int first_offh = 0, first_offw = 0, first_mi = 0, n_boxes = 1, cps = 1, units_n = 0, sub_log = 6, res_map = -1;
+        int s_log = 0;
+        uint32_t n_split = 0;                                  // split tiles so far
+        int first_offh = 0, first_offw = 0, first_mi = 0, cps = 1, units_n = 0, sub_log = 6, res_map = -1;
         bool first_have = true;
-        uint32_t a_sz = 0, b_sz = 0, keep_bytes = 0, res_bytes = 0;
+        uint32_t a_sz = 0, b_sz = 0, keep_bytes = 0;
         uint32_t pc = 0, uc = 0;
         // Operand ring (lane 0).  Entries are allocated and freed in order; positions are counted without wrapping
         // (head), an entry never straddles the ring's end.  The MMA issuer derives the same places from the same records.
@@ -683,35 +868,35 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 kind = __ldg(&sp->kind); mode = __ldg(&sp->mode); oh_lo = __ldg(&sp->oh_lo);
                 tr_log = __ldg(&sp->tr_log); p_log = __ldg(&sp->p_log); tw_valid = __ldg(&sp->tw_valid);
                 BN = __ldg(&sp->BN); BK = __ldg(&sp->BK); n_chunks = __ldg(&sp->n_chunks); n_taps = __ldg(&sp->n_taps);
-                tbx = __ldg(&sp->tb); amask = __ldg(&sp->a_valid_mask);
+                tbx = __ldg(&sp->tb);
                 a_bytes = __ldg(&sp->a_bytes); b_bytes = __ldg(&sp->b_bytes);
                 maps = P.maps + __ldg(&sp->map_base);
-                kh = __ldg(&sp->kh); kw = __ldg(&sp->kw); sh = __ldg(&sp->sh); sw = __ldg(&sp->sw);
-                ph = __ldg(&sp->ph); pw = __ldg(&sp->pw); dh = __ldg(&sp->dh); dw = __ldg(&sp->dw);
-                scale = ldg_ptr<const float *>(reinterpret_cast<const void *const *>(&sp->scale));
-                shift = ldg_ptr<const float *>(reinterpret_cast<const void *const *>(&sp->shift));
+                const int sh = __ldg(&sp->sh), sw = __ldg(&sp->sw), ph = __ldg(&sp->ph), pw = __ldg(&sp->pw);
                 // the first tap's offset (slab mode: where the box starts): which parity map that is and how far in
                 first_offh = floor_div_i(-ph, sh); first_offw = floor_div_i(-pw, sw);
                 first_mi = (-ph - first_offh * sh) * sw + (-pw - first_offw * sw);
-                first_have = (amask >> first_mi) & 1;
-                n_boxes = n_chunks * ((n_taps + tbx - 1) / tbx);
+                first_have = (__ldg(&sp->a_valid_mask) >> first_mi) & 1;
                 cps = __ldg(&sp->cps);
                 a_sz = (a_bytes + 1023u) & ~1023u; b_sz = (b_bytes + 1023u) & ~1023u;
                 keep_bytes = (uint32_t)__ldg(&sp->keep_bytes);
-                sub_log = __ldg(&sp->sub_log); units_n = BN >> sub_log;
+                if (SPLIT) s_log = __ldg(&sp->s_log);
+                sub_log = __ldg(&sp->sub_log); units_n = (BN >> s_log) >> sub_log;
                 res_map = __ldg(&sp->res_map);
-                res_bytes = (uint32_t)(((128 >> p_log) * tw_valid) << (sub_log + 1));
             }
             if (kind == WF_CONV) {
                 if (lane == 0) tr(item, 0);
                 // the tile's per-channel scale / shift go to shared memory from here, a tile ahead of the epilogue
                 // that uses them: their load latency is off the workers' path
                 bool ok = __all_sync(0xffffffffu, mbar_wait_abortable(sse0 + 8u * (pc & 1u), ((pc >> 1) & 1u) ^ 1u, abort_flag));
-                const int c0 = rec_cout(cur) * BN;
+                // a split tile: the item finishes channels c0 on, of the BN whose sums over chunks ch0 on it takes part in
+                const int c0 = rec_cout(cur) * (BN >> s_log);
+                const int co0 = SPLIT ? (rec_cout(cur) >> s_log) * BN : c0, ch0 = SPLIT ? (rec_cout(cur) & ((1 << s_log) - 1)) * n_chunks : 0;
                 if (ok && (((pc & 1u) ? ss_key[1] : ss_key[0]) != sidx || ((pc & 1u) ? ss_co[1] : ss_co[0]) != c0)) {
                     float *ds = s_scale + 128 * (pc & 1u), *dsh = s_shift + 128 * (pc & 1u);
+                    const float *scale = ldg_ptr<const float *>(reinterpret_cast<const void *const *>(&P.stages[sidx].scale));
+                    const float *shift = ldg_ptr<const float *>(reinterpret_cast<const void *const *>(&P.stages[sidx].shift));
                     if (pc & 1u) { ss_key[1] = sidx; ss_co[1] = c0; } else { ss_key[0] = sidx; ss_co[0] = c0; }
-                    for (int i = lane; i < BN; i += 32) {
+                    for (int i = lane; i < BN >> s_log; i += 32) {
                         ds[i] = scale ? __ldg(scale + c0 + i) : 1.0f;
                         dsh[i] = shift ? __ldg(shift + c0 + i) : 0.0f;
                     }
@@ -720,10 +905,9 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 // while the tile's producers are still at work: its weights on their way to L2, the maps to the descriptor cache
                 ok = ok && wait_deps_warp(P, rec_dep0(cur), rec_ndep(cur), dep_cur, run, lane, [&] {
                     if (lane != 0) return;
-                    const int co0 = rec_cout(cur) * BN;
                     prefetch_map(maps + first_mi);
                     for (int ch = 0, n = 0; ch < n_chunks && n < PREFETCH_BOXES; ++ch)
-                        for (int t0 = 0; t0 < n_taps && n < PREFETCH_BOXES; t0 += tbx, ++n) tma_prefetch_3d(maps + 4, ch * BK, co0, t0);
+                        for (int t0 = 0; t0 < n_taps && n < PREFETCH_BOXES; t0 += tbx, ++n) tma_prefetch_3d(maps + 4, (ch0 + ch) * BK, co0, t0);
                     if (res_map >= 0) prefetch_map(P.maps + res_map);
                 });
                 if (ok) {
@@ -740,7 +924,6 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                     const int ow0 = rec_tw(cur) * tw_valid;
                     const int oh0 = oh_lo + (rec_tr(cur) << tr_log);
                     const int n0 = rec_tn(cur) * (128 >> (p_log + tr_log));
-                    const int co0 = rec_cout(cur) * BN;
                     // waits until the oldest entry is consumed
                     auto free_oldest = [&]() {
                         const uint32_t e = n_freed & (WF_ENTRIES - 1);
@@ -790,7 +973,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                         head = pos = tail_at = 0;
                         if (!fail && kept) {
                             ++w_uses;
-                            mbar_expect_tx(wfull, (uint32_t)n_boxes * b_bytes);
+                            mbar_expect_tx(wfull, (uint32_t)(n_chunks * ((n_taps + tbx - 1) / tbx)) * b_bytes);
                             uint32_t at = ring0 + ring_lim;
                             for (int ch = 0; ch < n_chunks; ++ch)
                                 for (int t0 = 0; t0 < n_taps; t0 += tbx, at += b_sz) tma_load_3d(at, maps + 4, wfull, ch * BK, co0, t0);
@@ -802,7 +985,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                         for (int ch = 0; ch < n_chunks && !fail; ++ch) {
                             const uint32_t at = allocate(a_sz, a_bytes);
                             if (!at) { fail = 1; break; }
-                            tma_load_4d(at, maps + first_mi, full_bar, ch * BK, aw, ah, n0);
+                            tma_load_4d(at, maps + first_mi, full_bar, ch * BK, aw, ah, n0);          // (not split: kept)
                         }
                     } else if (mode == WF_SLAB) {
                         const int per_chunk = (n_taps + tbx - 1) / tbx;
@@ -816,11 +999,11 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                                     bar = gfull0 + 8u * (n_group & (WF_GROUPS - 1));
                                     ++n_group;
                                     mbar_expect_tx(bar, (uint32_t)min(cps, per_chunk - i) * b_bytes + (i == 0 ? a_bytes : 0u));
-                                    if (i == 0) tma_load_4d(ring0 + ring_lim + slab_sl * a_sz, maps + first_mi, bar, ch * BK, aw, ah, n0);
+                                    if (i == 0) tma_load_4d(ring0 + ring_lim + slab_sl * a_sz, maps + first_mi, bar, (ch0 + ch) * BK, aw, ah, n0);
                                 }
                                 const uint32_t at = place(b_sz);
                                 if (!at) { fail = 1; break; }
-                                tma_load_3d(at, maps + 4, bar, ch * BK, co0, i * tbx);
+                                tma_load_3d(at, maps + 4, bar, (ch0 + ch) * BK, co0, i * tbx);
                                 if (++in_group == cps) in_group = 0;
                             }
                             slab_end0 = slab_end1; slab_end1 = n_alloc;
@@ -829,7 +1012,10 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                     } else {
                         // one activation and one weight box per (channel chunk, tap), `cps` of them per entry
                         const int steps = n_chunks * n_taps;
-                        int ch = 0, ta = 0, tb = 0;
+                        const WfStage *sp = &P.stages[sidx];
+                        const int kh = __ldg(&sp->kh), kw = __ldg(&sp->kw), sh = __ldg(&sp->sh), sw = __ldg(&sp->sw);
+                        const int ph = __ldg(&sp->ph), pw = __ldg(&sp->pw), dh = __ldg(&sp->dh), dw = __ldg(&sp->dw), amask = __ldg(&sp->a_valid_mask);
+                        int ch = ch0, ta = 0, tb = 0;
                         int offh = first_offh, offw = first_offw, mi = first_mi;
                         bool have = first_have;
                         for (int st = 0; st < steps && !fail; st += cps) {
@@ -857,11 +1043,16 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                         const uint32_t sl = uc & (WF_UNITS - 1), gb = ugrant0 + 8u * sl;
                         if (!mbar_wait_abortable(ufree0 + 8u * sl, ((uc / WF_UNITS) & 1u) ^ 1u, abort_flag)) { fail = 1; break; }
                         if (res_map >= 0) {
-                            mbar_expect_tx(gb, res_bytes);
-                            tma_load_4d(unit0 + sl * unit_bytes, P.maps + res_map, gb, co0 + (u << sub_log), ow0, oh0, n0);
+                            mbar_expect_tx(gb, (uint32_t)(((128 >> p_log) * tw_valid) << (sub_log + 1)));
+                            tma_load_4d(unit0 + sl * unit_bytes, P.maps + res_map, gb, c0 + (u << sub_log), ow0, oh0, n0);
                         } else {
                             mbar_arrive(gb);
                         }
+                    }
+                    if (SPLIT && s_log > 0 && !fail) {
+                        fail = !take_partial_sums(bars, (uint32_t)rec_cout(cur), (uint32_t)s_log, uc, n_split);
+                        uc += (1u << s_log) >> 1;
+                        ++n_split;
                     }
                     if (fail) atomicOr(P.status, 0x1u);
                     tr(item, 2);
@@ -1078,6 +1269,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
             // the workers have finished it, hands the unit back when it has been read out, and waits for the stores'
             // completion before the increment -- the workers are at the next tile by then.
             int sidx = -1, ctr_base = 0, kind = -1, out_map = -1, sub_log = 6, units_n = 0, oh_lo = 0, p_log = 0, tr_log = 0, tw_valid = 0, BN = 0;
+            uint32_t rx_units = 0;                             // units of a tile that partial sums arrive in
             uint32_t uc = 0, k = 0;
             bool fail = false;
             for (; item < NI; item += G) {
@@ -1088,7 +1280,16 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                     ctr_base = __ldg(&sp->ctr_base); kind = __ldg(&sp->kind); out_map = __ldg(&sp->out_map);
                     sub_log = __ldg(&sp->sub_log); oh_lo = __ldg(&sp->oh_lo); p_log = __ldg(&sp->p_log); tr_log = __ldg(&sp->tr_log);
                     tw_valid = __ldg(&sp->tw_valid); BN = __ldg(&sp->BN);
+                    if (SPLIT) {
+                        const int s_log = __ldg(&sp->s_log);
+                        BN >>= s_log;                          // (the channels the item finishes)
+                        rx_units = (1u << s_log) >> 1;
+                    }
                     units_n = BN >> sub_log;
+                }
+                if (SPLIT && kind == WF_NONE) {
+                    cur = nxt;
+                    continue;
                 }
                 if (kind == WF_CONV && out_map >= 0) {
                     const int ow0 = rec_tw(cur) * tw_valid, oh0 = oh_lo + (rec_tr(cur) << tr_log), n0 = rec_tn(cur) * (128 >> (p_log + tr_log));
@@ -1105,11 +1306,11 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                     bulk_wait_read();
                     if (fail) { fail = !*abort_flag; break; }
                     for (int u = 0; u < units_n && units_n <= WF_UNITS; ++u) mbar_arrive(ufree0 + 8u * ((uc + u) & (WF_UNITS - 1)));
-                    uc += units_n;
+                    uc += units_n + rx_units;
                     bulk_wait_all();
                     add_release(P.counters + ctr_base + rec_tr(cur));
                 } else {
-                    if (kind == WF_CONV) uc += units_n;            // stored, and handed back, by the workers
+                    if (kind == WF_CONV) uc += units_n + rx_units; // stored, and handed back, by the workers
                     const uint32_t q = k % WF_PUBQ, round = k / WF_PUBQ;
                     if (!mbar_wait_abortable(pubf0 + 8u * q, round & 1u, abort_flag)) { fail = !*abort_flag; break; }
                     add_release(P.counters + ctr_base + rec_tr(cur));
@@ -1177,10 +1378,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
         uint32_t cnt = 0, done_items = 0, uc = 0;
         int sub_log = 6, units_n = 0;
         bool bulk_out = false;
-        int kind = -1, oh_lo = 0, oh_hi = 0, p_log = 0, tr_log = 0, tw_valid = 0, BN = 0, fuse_pool = 0, pool_Ho = 0, pool_Wo = 0;
-        int N = 0, Ho = 0, Wo = 0, Cout = 0, act = 0, res_pos = 0;
-        const void *resp = nullptr;
-        void *yout = nullptr;
+        int kind = -1, p_log = 0, tr_log = 0, tw_valid = 0, act = 0, res_pos = 0;
         for (; item < NI; item += G) {
             const int4 nn = item + 2 * G < NI ? __ldg(&P.items[item + 2 * G]) : zero4;
             const int2 dep_nxt =
@@ -1188,16 +1386,12 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
             if (rec_stage(cur) != sidx) {
                 sidx = rec_stage(cur);
                 const WfStage *sp = &P.stages[sidx];
-                kind = __ldg(&sp->kind); oh_lo = __ldg(&sp->oh_lo); oh_hi = __ldg(&sp->oh_hi);
+                kind = SPLIT && __ldg(&sp->s_log) > 0 ? (int)WF_SPLIT : __ldg(&sp->kind);
                 p_log = __ldg(&sp->p_log); tr_log = __ldg(&sp->tr_log); tw_valid = __ldg(&sp->tw_valid);
-                BN = __ldg(&sp->BN);
-                N = __ldg(&sp->N); Ho = __ldg(&sp->Ho); Wo = __ldg(&sp->Wo); Cout = __ldg(&sp->Cout);
-                act = __ldg(&sp->act); res_pos = __ldg(&sp->res_pos);
-                fuse_pool = __ldg(&sp->fuse_pool); pool_Ho = __ldg(&sp->pool_Ho); pool_Wo = __ldg(&sp->pool_Wo);
-                sub_log = __ldg(&sp->sub_log); units_n = BN >> sub_log;
+                act = __ldg(&sp->act);
+                res_pos = ldg_ptr<const void *>(&sp->res) ? __ldg(&sp->res_pos) : LOP_RES_NONE;
+                sub_log = __ldg(&sp->sub_log); units_n = __ldg(&sp->BN) >> sub_log;
                 bulk_out = __ldg(&sp->out_map) >= 0;
-                resp = ldg_ptr<const void *>(&sp->res);
-                yout = ldg_ptr<void *>(reinterpret_cast<const void *const *>(&sp->y));
             }
             const int tile_r = rec_tr(cur);
             if (tid == 0) tr(item, 7);
@@ -1205,17 +1399,19 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 const uint32_t buf = cnt & 1u;
                 const int c = m & ((1 << p_log) - 1);
                 const int r = (m >> p_log) & ((1 << tr_log) - 1);
-                const int ow = rec_tw(cur) * tw_valid + c;
-                const int oh = oh_lo + (tile_r << tr_log) + r;
-                const int n = rec_tn(cur) * (128 >> (p_log + tr_log)) + (m >> (p_log + tr_log));
                 const bool staged = c < tw_valid;                      // the other anchors are the slab's halo gap
-                const bool valid = staged && ow < Wo && oh < oh_hi && n < N;
-                const int co0 = rec_cout(cur) * BN;
                 // staged rows are packed: image, row, column below tw_valid (the box of a bulk load or store)
                 const int srow = (((m >> (p_log + tr_log)) << tr_log) + r) * tw_valid + c;
                 if (!bulk_out) {
+                    const WfStage *sp = &P.stages[sidx];
+                    const int oh_hi = __ldg(&sp->oh_hi), Ho = __ldg(&sp->Ho), Wo = __ldg(&sp->Wo), Cout = __ldg(&sp->Cout);
+                    const int pool_Ho = __ldg(&sp->pool_Ho), pool_Wo = __ldg(&sp->pool_Wo), co0 = rec_cout(cur) * (units_n << sub_log);
+                    const int ow = rec_tw(cur) * tw_valid + c;
+                    const int oh = __ldg(&sp->oh_lo) + (tile_r << tr_log) + r;
+                    const int n = rec_tn(cur) * (128 >> (p_log + tr_log)) + (m >> (p_log + tr_log));
+                    const bool valid = staged && ow < Wo && oh < oh_hi && n < __ldg(&sp->N);
                     if (cgrp == 0 && staged) row_pix[srow] = valid ? (((long long)n * Ho + oh) * Wo + ow) * Cout + co0 : -1LL;
-                    if (fuse_pool && cgrp == 0 && !((r | c) & 1)) {
+                    if (__ldg(&sp->fuse_pool) && cgrp == 0 && !((r | c) & 1)) {
                         // top-left anchor of a 2x2 window: where its maximum goes, if the whole window is inside the stage
                         const int q = (((m >> (p_log + tr_log)) << (tr_log - 1)) + (r >> 1)) * ((1 << p_log) >> 1) + (c >> 1);
                         const bool ok = valid && c + 1 < tw_valid && ow + 1 < Wo && oh + 1 < oh_hi;
@@ -1256,7 +1452,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                         uint4 *c0p = reinterpret_cast<uint4 *>(my_row + (((j >> 3) ^ swz) << 4));
                         uint4 *c1p = reinterpret_cast<uint4 *>(my_row + ((((j >> 3) + 1) ^ swz) << 4));
                         float rv[16];
-                        if (resp) {
+                        if (res_pos != LOP_RES_NONE) {
                             const uint4 q0 = *c0p, q1 = *c1p;
                             const uint32_t rw[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
 #pragma unroll
@@ -1265,7 +1461,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                                 rv[2 * i + 1] = __uint_as_float(rw[i] & 0xFFFF0000u);
                             }
                         }
-                        finish16<SMOOTH ? 1 : 0>(v, rv, resp ? res_pos : LOP_RES_NONE, act);
+                        finish_n<SMOOTH ? 1 : 0>(v, rv, res_pos, act);
                         uint32_t o[8];
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
@@ -1289,6 +1485,9 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 }
                 ++cnt;
                 if (!bulk_out && !*epi_fail) {
+                    const WfStage *sp = &P.stages[sidx];
+                    const int fuse_pool = __ldg(&sp->fuse_pool);
+                    void *yout = ldg_ptr<void *>(reinterpret_cast<const void *const *>(&sp->y));
                     for (int u = 0; u < units_n; ++u) {
                         const uint8_t *unit = units + ((uc + u) & (WF_UNITS - 1)) * unit_bytes;
                         uint4 *y = static_cast<uint4 *>(yout) + (u << (sub_log - 3));
@@ -1302,16 +1501,17 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 if (tid == 0) tr(item, 12);
             } else {
                 // an item of the worker warps alone: output rows of one image (or a depth-wise tile)
-                if (warp == WF_FIRST_WORKER && !wait_deps_warp(P, rec_dep0(cur), rec_ndep(cur), dep_cur, run, lane, [] {}) && lane == 0) *epi_fail = 1;
-                epi_bar();
+                if (!SPLIT || kind < WF_NONE) {
+                    if (warp == WF_FIRST_WORKER && !wait_deps_warp(P, rec_dep0(cur), rec_ndep(cur), dep_cur, run, lane, [] {}) && lane == 0) *epi_fail = 1;
+                    epi_bar();
+                }
                 if (tid == 0) tr(item, 1);
-                const int n = rec_tn(cur);
-                const int oh = oh_lo + tile_r;
+                const int n = rec_tn(cur), oh_lo = __ldg(&P.stages[sidx].oh_lo), oh = oh_lo + tile_r;
                 if (*epi_fail) {
                     // fall through to the common exit below
                 } else if (kind == WF_POOL) {
                     const int oh0 = oh_lo + (tile_r << tr_log);
-                    if (__ldg(&P.stages[sidx].mode)) pool3_item(&P.stages[sidx], n, oh0, min(1 << tr_log, oh_hi - oh0), tid);
+                    if (__ldg(&P.stages[sidx].mode)) pool3_item(&P.stages[sidx], n, oh0, min(1 << tr_log, __ldg(&P.stages[sidx].oh_hi) - oh0), tid);
                     else pool_item(&P.stages[sidx], n, oh, tid);
                 } else if (ROWOPS && kind == WF_DWCONV) {
                     dwconv_item(&P.stages[sidx], n, tile_r, rec_tw(cur), rec_cout(cur), tid, stg);
@@ -1319,6 +1519,10 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                     layernorm_item(&P.stages[sidx], n, oh, tid);
                 } else if (ROWOPS && kind == WF_CONCAT) {
                     concat_item(&P.stages[sidx], n, oh, tid);
+                } else if (SPLIT && kind == WF_SPLIT) {
+                    uc += split_item<SMOOTH>(&P.stages[sidx], cur, smem + (bars - base), unit0, unit_bytes, tmem_base + (cnt & 1u) * 256u, uc, cnt);
+                    ++cnt;
+                } else if (SPLIT && kind == WF_NONE) {
                 } else {
                     gather_item(&P.stages[sidx], n, tile_r, tid, stg);
                 }
@@ -1333,7 +1537,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 }
                 break;
             }
-            const bool stored_here = kind != WF_CONV || !bulk_out;
+            const bool stored_here = kind == WF_CONV || (SPLIT && kind == WF_SPLIT) ? !bulk_out : !SPLIT || kind != WF_NONE;
             if (kind == WF_CONV) {
                 if (stored_here && tid == 0)
                     for (int u = 0; u < units_n; ++u) mbar_arrive(ufree0 + 8u * ((uc + u) & (WF_UNITS - 1)));
@@ -1363,6 +1567,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
         tr(TRACE_ITEMS - 8 + (int)blockIdx.x, 2);
         trv(TRACE_ITEMS - 8 + (int)blockIdx.x, 5, (unsigned long long)clock64());
     }
+    if (SPLIT) cluster_sync();                                 // no CTA's shared memory goes while another may write to it
     if (threadIdx.x == 0) {
         __threadfence();
         const unsigned done = atomicAdd(P.counters + 1, 1u);
@@ -1414,14 +1619,19 @@ size_t wavefront_smem_bytes(const WfParams &p)
 namespace {
 
 typedef void (*WfKernel)(const WfParams);
-template <bool FETCH, bool ROWOPS>
-WfKernel with_activations(bool smooth) { return smooth ? wavefront_kernel<FETCH, ROWOPS, true> : wavefront_kernel<FETCH, ROWOPS, false>; }
-WfKernel kernel_for(bool fetch, bool row_ops, bool smooth)
+template <bool FETCH, bool SMOOTH>
+WfKernel kernel_with(bool row_ops, bool split)
 {
-    if (fetch) return row_ops ? with_activations<true, true>(smooth) : with_activations<true, false>(smooth);
-    return row_ops ? with_activations<false, true>(smooth) : with_activations<false, false>(smooth);
+    if (row_ops) return split ? wavefront_kernel<FETCH, true, SMOOTH, true> : wavefront_kernel<FETCH, true, SMOOTH, false>;
+    return split ? wavefront_kernel<FETCH, false, SMOOTH, true> : wavefront_kernel<FETCH, false, SMOOTH, false>;
 }
-WfKernel kernel_for(const WfParams &p) { return kernel_for(p.n_fetch > 0, p.row_ops != 0, p.smooth != 0); }
+WfKernel kernel_for(bool fetch, bool row_ops, bool smooth, bool split)
+{
+    if (fetch) return smooth ? kernel_with<true, true>(row_ops, split) : kernel_with<true, false>(row_ops, split);
+    return smooth ? kernel_with<false, true>(row_ops, split) : kernel_with<false, false>(row_ops, split);
+}
+WfKernel kernel_for(const WfParams &p) { return kernel_for(p.n_fetch > 0, p.row_ops != 0, p.smooth != 0, p.cluster > 1); }
+int threads_of(const WfParams &p) { return p.n_fetch > 0 ? WF_THREADS + 32 : WF_THREADS; }
 
 }  // namespace
 
@@ -1436,7 +1646,19 @@ cudaError_t wavefront_resident_ctas(const WfParams &p, int *ctas)
     const size_t smem = wavefront_smem_bytes(p);
     WfKernel k = kernel_for(p);
     if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024)) != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, p.n_fetch > 0 ? WF_THREADS + 32 : WF_THREADS, smem);
+    if (p.cluster > 1) {
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = (unsigned)p.cluster; attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)(sms / p.cluster * p.cluster)); cfg.blockDim = dim3((unsigned)threads_of(p)); cfg.dynamicSmemBytes = smem;
+        cfg.attrs = &attr; cfg.numAttrs = 1;
+        int clusters = 0;
+        if ((e = cudaOccupancyMaxActiveClusters(&clusters, k, &cfg)) != cudaSuccess) return e;
+        *ctas = clusters * p.cluster;
+        return cudaSuccess;
+    }
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads_of(p), smem);
     if (e != cudaSuccess) return e;
     *ctas = per_sm * sms;
     return cudaSuccess;
@@ -1451,8 +1673,8 @@ cudaError_t launch_wavefront(const WfParams &p, int grid, cudaStream_t s)
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64 || !configured[dev].load(std::memory_order_acquire)) {
-        for (int k = 0; k < 8; ++k) {
-            e = cudaFuncSetAttribute(kernel_for(k & 4, k & 2, k & 1), cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        for (int k = 0; k < 16; ++k) {
+            e = cudaFuncSetAttribute(kernel_for(k & 4, k & 2, k & 1, k & 8), cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
             if (e != cudaSuccess) return e;
         }
         if (dev >= 0 && dev < 64) configured[dev].store(true, std::memory_order_release);
@@ -1463,12 +1685,24 @@ cudaError_t launch_wavefront(const WfParams &p, int grid, cudaStream_t s)
 #endif
     // A program that fetches its input does not begin early: its CTAs would take the SMs in the order in which the previous
     // launch leaves them, which costs a long one more than the launch's two microseconds (ResNet-18 streamed 169.8 us so,
-    // 170.9 begun early; a ResNet-50 of batch 8 442.6 and 445.5).
-    if (p.n_fetch > 0) {
-        kernel_for(p)<<<grid, WF_THREADS + 32, smem, s>>>(p);
-        return cudaGetLastError();
+    // 170.9 begun early; a ResNet-50 of batch 8 442.6 and 445.5).  Nor do clusters of four, whose places on the chip are no
+    // whole number of its units of two SMs per cluster everywhere.
+    const bool early = p.n_fetch == 0 && p.cluster <= 2;
+    cudaLaunchAttribute attrs[2]{};
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3((unsigned)threads_of(p)); cfg.dynamicSmemBytes = smem; cfg.stream = s;
+    cfg.attrs = attrs;
+    if (early) {
+        attrs[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attrs[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
     }
-    return launch_after(kernel_for(p), dim3(grid), WF_THREADS, smem, s, p);
+    if (p.cluster > 1) {
+        attrs[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        attrs[cfg.numAttrs].val.clusterDim.x = (unsigned)p.cluster;
+        attrs[cfg.numAttrs].val.clusterDim.y = attrs[cfg.numAttrs].val.clusterDim.z = 1;
+        ++cfg.numAttrs;
+    }
+    return cudaLaunchKernelEx(&cfg, kernel_for(p), p);
 }
 
 }  // namespace lop

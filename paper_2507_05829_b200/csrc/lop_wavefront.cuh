@@ -19,7 +19,8 @@ namespace lop {
 // item is 1 << tr_log output rows of one image, tw_valid columns wide and BN channels deep (its receptive window is staged
 // in shared memory); a normalisation or concatenation item is one whole output row of one image; a gather or 3x3 pooling
 // item is 1 << tr_log of them.
-enum WfKind { WF_GATHER = 0, WF_CONV = 1, WF_POOL = 2, WF_FETCH = 3, WF_DWCONV = 4, WF_LAYERNORM = 5, WF_CONCAT = 6 };
+// WF_SPLIT is what the worker warps call a split tile of a WF_CONV stage.  WF_NONE: an item without work, in front of a split tile whose items have to start at a cluster's first CTA.
+enum WfKind { WF_GATHER = 0, WF_CONV = 1, WF_POOL = 2, WF_FETCH = 3, WF_DWCONV = 4, WF_LAYERNORM = 5, WF_CONCAT = 6, WF_NONE = 7, WF_SPLIT = 8 };
 // How a convolution stage feeds the tensor cores.
 //   WF_SLAB  one activation box per channel chunk: the output tile's receptive window (tile plus halo),
 //            laid out in shared memory as rows of P pixels; every filter tap is the same box read at a
@@ -61,7 +62,11 @@ struct WfStage {
     int out_map;              // tensor map of the output's rows below oh_hi (a unit is one bulk store), or -1: the workers store it
     int res_map;              // tensor map of the residual (a unit is one bulk load), or -1
     int keep_bytes;           // > 0: a tile's weights stay in shared memory (this many bytes at the ring's end) from tile to tile
-    int pad_[6];
+    // A split tile (s_log > 0): 1 << s_log consecutive items on as many CTAs of a cluster, each of which sums its share of the
+    // channel chunks (n_chunks of them) over all BN channels, hands the other CTAs their slices of the partial sums, and
+    // finishes the slice of BN >> s_log channels that is its own.  An item's cout_tile counts slices.
+    int s_log;
+    int pad_[5];
 };
 static_assert(sizeof(WfStage) == 256, "WfStage layout");
 
@@ -90,6 +95,7 @@ struct WfParams {
     void *fetch_dst;
     int n_fetch, fetch_window;
     int row_ops;              // the program has WF_DWCONV / WF_LAYERNORM / WF_CONCAT stages
+    int cluster;              // CTAs per cluster (1, 2 or 4): the most parts a tile of the program is split in
     int smooth;               // a convolution of the program is activated by SiLU or GELU
 };
 
@@ -103,6 +109,7 @@ constexpr int WF_ENTRIES = 16;                             // operand ring entri
 constexpr int WF_GROUPS = 8;                               // slab mode: box groups in flight at most (a power of two)
 constexpr int WF_UNITS = 4;                                // output units in flight (a power of two)
 constexpr uint32_t WF_FIXED_SMEM = 4096;                  // barriers, scale / shift and pixel tables
+constexpr uint32_t WF_SPLIT_BN = 64, WF_SPLIT_UNIT = 16 * 1024;     // channels of a split tile; bytes of an output unit that partial sums arrive in
 constexpr int WF_PUBQ = 4;                                 // finished items the publisher may lag behind the workers
 constexpr int WF_CTR_FIRST = 4;
 constexpr int WF_MAX_DEPS = 4095;

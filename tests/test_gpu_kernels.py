@@ -5,7 +5,7 @@ import torch
 
 import lop_inputs as li
 import paper_2507_05829_b200 as lop
-from lop_inputs.workloads import Segment, Workload, conv, pool
+from lop_inputs.workloads import NO_RESIDUAL, Segment, Workload, conv, pool
 from oracle import chain as ochain
 from paper_2507_05829_b200.chain import DeviceChain, to_host_f32
 from test_gpu_parity import TOL, check_workload, one_layer, rel_err
@@ -308,4 +308,37 @@ def test_calls_in_a_row_wait_for_what_they_read(dtype, C, H, W, flags):
         runs.append((a.outs[-1].clone(), b.outs[-1].clone()))
     assert torch.isfinite(runs[0][1].float()).all() and runs[0][1].float().abs().max() > 0
     assert torch.equal(runs[0][0], runs[1][0]) and torch.equal(runs[0][1], runs[1][1])
+
+
+# ------------------------------------------------------------------------------------ K summed in parts by the CTAs of a cluster
+SPLIT_CASES = [  # k, s, p, cin, cout, N, H, W, residual, activation
+    (3, 1, 1, 512, 512, 1, 7, 7, li.RES_PRE_ACT, li.ACT_RELU),          # four parts: one tile of pixels, every row of it in reach of padding
+    (3, 1, 1, 256, 256, 3, 11, 16, li.RES_POST_ACT, li.ACT_SILU),       # four parts, one chunk each; ragged tiles
+    (3, 2, 1, 256, 512, 2, 15, 13, li.RES_NONE, li.ACT_RELU),           # a box per tap, odd extents
+    (1, 1, 0, 2048, 512, 8, 7, 7, li.RES_NONE, li.ACT_NONE),            # pointwise
+    (3, 1, 1, 256, 256, 8, 14, 14, li.RES_PRE_ACT, li.ACT_GELU),        # two parts
+    (3, 1, 2, 128, 64, 1, 20, 18, li.RES_NONE, li.ACT_RELU),            # two chunks: two parts at most; one slice of channels per part
+]
+
+
+@pytest.mark.parametrize("case", SPLIT_CASES)
+def test_split_tiles(case):
+    """Against the oracle, and bit for bit between the executors: a chain of two such layers (several split tiles per CTA,
+    the second's partial sums behind the first's), one with a shortcut, in bands, streamed, into host memory."""
+    k, s, p, cin, cout, N, H, W, res, act = case
+    l0 = conv(cin, cout, k, s=s, p=p, act=act, input_from=-1)
+    layers = [l0, conv(cout, cout, 3, input_from=0, act=act, residual_from=0 if res != li.RES_NONE else NO_RESIDUAL, residual_pos=res)]
+    wl = Workload("split", "bf16", N, H, W, cin, [Segment(layers, 3)], seed=31)
+    li.fill_parameters(wl)
+    li.make_input(wl)
+    check_workload(wl, flags=lop.LOP_FLAG_REUSE_HALO, modes=("whole", "banded", "pipelined"))
+    dc, per = DeviceChain(wl, flags=lop.LOP_FLAG_REUSE_HALO), DeviceChain(wl, flags=lop.LOP_FLAG_PER_LAYER)
+    want = per.run_whole(per.input_tensor())
+    host = torch.empty(want.shape, dtype=want.dtype).pin_memory()
+    for _ in range(3):                                                  # calls in a row, too
+        got = dc.run_banded(dc.input_tensor())
+        dc.run_pipelined(dc.pinned_input(), out_pinned=host)
+    torch.cuda.synchronize()
+    dc.check_device()
+    assert torch.equal(got, want) and torch.equal(host, want.cpu())
 
