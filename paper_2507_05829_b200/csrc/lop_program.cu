@@ -882,9 +882,10 @@ int program_build(const std::vector<SegBind> &segs, std::vector<StageReq> reqs, 
         if (st.kind == WF_DWCONV || st.kind == WF_LAYERNORM || st.kind == WF_CONCAT) P.row_ops = 1;
         else if (st.kind == WF_CONV && (st.act == LOP_ACT_SILU || st.act == LOP_ACT_GELU)) P.smooth = 1;
     // entries in flight: about the link's bandwidth-delay product (some 25 GB/s x 3 us), at least a few warps' worth
+    long long bytes = 0;
+    for (const int4 &f : fetch_items) bytes += f.z;
+    P.fetch_bytes = bytes;
     if (P.n_fetch > 0) {
-        long long bytes = 0;
-        for (const int4 &f : fetch_items) bytes += f.z;
         // (a small input keeps the short window, which keeps its few bands in order; an input of megabytes is bound by
         // the link's rate, which needs more bytes on their way: measured 597 -> 577 us on a 2.4 MB batch)
         const long long window_bytes = std::min<long long>(LOP_FETCH_WINDOW_MAX_BYTES, std::max<long long>(LOP_FETCH_WINDOW_BYTES, bytes / 8));

@@ -1360,7 +1360,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
             if (lane == 0) {
                 tr(TRACE_FETCH0 + j, 1);
                 add_release(P.counters + rec.w);                   // the warp's stores, then the increments
-                add_release(P.counters + 3);
+                atomicAdd(P.counters + 3, 1u);                     // (the window orders nothing)
                 tr(TRACE_FETCH0 + j, 2);
             }
         }
@@ -1402,8 +1402,12 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 const bool staged = c < tw_valid;                      // the other anchors are the slab's halo gap
                 // staged rows are packed: image, row, column below tw_valid (the box of a bulk load or store)
                 const int srow = (((m >> (p_log + tr_log)) << tr_log) + r) * tw_valid + c;
+                int fuse_pool = 0;
+                void *yout = nullptr;
                 if (!bulk_out) {
                     const WfStage *sp = &P.stages[sidx];
+                    fuse_pool = __ldg(&sp->fuse_pool);
+                    yout = ldg_ptr<void *>(reinterpret_cast<const void *const *>(&sp->y));
                     const int oh_hi = __ldg(&sp->oh_hi), Ho = __ldg(&sp->Ho), Wo = __ldg(&sp->Wo), Cout = __ldg(&sp->Cout);
                     const int pool_Ho = __ldg(&sp->pool_Ho), pool_Wo = __ldg(&sp->pool_Wo), co0 = rec_cout(cur) * (units_n << sub_log);
                     const int ow = rec_tw(cur) * tw_valid + c;
@@ -1411,7 +1415,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                     const int n = rec_tn(cur) * (128 >> (p_log + tr_log)) + (m >> (p_log + tr_log));
                     const bool valid = staged && ow < Wo && oh < oh_hi && n < __ldg(&sp->N);
                     if (cgrp == 0 && staged) row_pix[srow] = valid ? (((long long)n * Ho + oh) * Wo + ow) * Cout + co0 : -1LL;
-                    if (__ldg(&sp->fuse_pool) && cgrp == 0 && !((r | c) & 1)) {
+                    if (fuse_pool && cgrp == 0 && !((r | c) & 1)) {
                         // top-left anchor of a 2x2 window: where its maximum goes, if the whole window is inside the stage
                         const int q = (((m >> (p_log + tr_log)) << (tr_log - 1)) + (r >> 1)) * ((1 << p_log) >> 1) + (c >> 1);
                         const bool ok = valid && c + 1 < tw_valid && ow + 1 < Wo && oh + 1 < oh_hi;
@@ -1485,9 +1489,6 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 }
                 ++cnt;
                 if (!bulk_out && !*epi_fail) {
-                    const WfStage *sp = &P.stages[sidx];
-                    const int fuse_pool = __ldg(&sp->fuse_pool);
-                    void *yout = ldg_ptr<void *>(reinterpret_cast<const void *const *>(&sp->y));
                     for (int u = 0; u < units_n; ++u) {
                         const uint8_t *unit = units + ((uc + u) & (WF_UNITS - 1)) * unit_bytes;
                         uint4 *y = static_cast<uint4 *>(yout) + (u << (sub_log - 3));
@@ -1683,11 +1684,12 @@ cudaError_t launch_wavefront(const WfParams &p, int grid, cudaStream_t s)
 #ifdef LOP_WF_TRACE
     g_last_params = p;
 #endif
-    // A program that fetches its input does not begin early: its CTAs would take the SMs in the order in which the previous
-    // launch leaves them, which costs a long one more than the launch's two microseconds (ResNet-18 streamed 169.8 us so,
-    // 170.9 begun early; a ResNet-50 of batch 8 442.6 and 445.5).  Nor do clusters of four, whose places on the chip are no
-    // whole number of its units of two SMs per cluster everywhere.
-    const bool early = p.n_fetch == 0 && p.cluster <= 2;
+    // A program that fetches much of its input does not begin early: its CTAs would take the SMs in the order in which the
+    // previous launch leaves them, and a long transfer suffers from that more than the launch's two microseconds (up to 300 KB:
+    // a VGG block streamed 33.5 us without, 31.9 begun early, a DenseNet layer 24.9 and 22.7; 0.8 MB: four images' VGG block
+    // 66.2 and 69.9; 1.6 MB: a ConvNeXt block 105 and 131).  Nor do clusters of four, which need not find their places while
+    // CTAs of another launch still hold some.
+    const bool early = p.fetch_bytes <= 512 * 1024 && p.cluster <= 2;
     cudaLaunchAttribute attrs[2]{};
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3((unsigned)threads_of(p)); cfg.dynamicSmemBytes = smem; cfg.stream = s;

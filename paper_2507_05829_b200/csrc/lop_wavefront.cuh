@@ -94,6 +94,7 @@ struct WfParams {
     const void *fetch_src;
     void *fetch_dst;
     int n_fetch, fetch_window;
+    long long fetch_bytes;    // of all entries
     int row_ops;              // the program has WF_DWCONV / WF_LAYERNORM / WF_CONCAT stages
     int cluster;              // CTAs per cluster (1, 2 or 4): the most parts a tile of the program is split in
     int smooth;               // a convolution of the program is activated by SiLU or GELU
