@@ -272,10 +272,19 @@ ConvTcGeom conv_tc_geometry(const ConvArgs &a, int rows, bool fill_sms)
     // with few pixel tiles, narrower channel tiles give more CTAs to fill the 148 SMs
     if (a.k_split > 1 && g.BN > 64) g.BN = 64;                // (an accumulator per part; Cout is a multiple of 64)
     while (fill_sms && best * (a.Cout / g.BN) < 148 && g.BN % 32 == 0 && g.BN > 32) g.BN /= 2;
-    const int stage = 128 * g.BK * 2 + ((g.BN * g.BK * 2 + 1023) / 1024) * 1024;
-    int stages = (100 * 1024) / stage;
+    // Ring stages: what lets as many CTAs share an SM as there are tiles for it (at most three, and no more than tensor memory
+    // holds), for one CTA's epilogue runs under another's loads; no more than the layer has steps.  (A VGG block's two layers
+    // of 392 tiles by two CTAs of 100 KB per SM, a third of a wave left over: 14.4 and 20.7 us; the block without
+    // allocation 40.7 us, so 34.6.)
+    const int stage = 128 * g.BK * 2 + ((g.BN * g.BK * 2 + 1023) / 1024) * 1024, steps = a.kh * a.kw * (a.Cin / g.BK);
+    const long long tiles = best * (a.Cout / g.BN);
+    long long per_sm = (tiles + 147) / 148;
+    per_sm = per_sm < 3 ? per_sm : 3;
+    while (per_sm > 1 && per_sm * g.BN * a.k_split > 512) --per_sm;
+    int stages = (int)((216 * 1024 / per_sm - 2048) / stage);
     if (stages > 8) stages = 8;
     if (stages < 2) stages = 2;
+    if (stages > steps) stages = steps;
     g.stages = stages;
     return g;
 }
@@ -353,7 +362,7 @@ cudaError_t launch_conv_tc(const ConvArgs &a, const ConvTcGeom &g, const ConvTcM
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64 || !configured[dev].load(std::memory_order_acquire)) {
-        e = cudaFuncSetAttribute(conv_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(200 * 1024));
+        e = cudaFuncSetAttribute(conv_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(220 * 1024));
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) configured[dev].store(true, std::memory_order_release);
     }
