@@ -1372,17 +1372,17 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
         const int cgrp = (warp - WF_FIRST_WORKER) >> 2;                     // which share of the tile's 16-column chunks is this warp's
         int item = blockIdx.x;
         int4 cur = item < NI ? __ldg(&P.items[item]) : zero4;
-        int4 nxt = item + G < NI ? __ldg(&P.items[item + G]) : zero4;
-        int2 dep_cur = (warp == WF_FIRST_WORKER && item < NI && lane < rec_ndep(cur)) ? __ldg(&P.deps[rec_dep0(cur) + lane]) : make_int2(0, 0);
+        // the dependency entry of this lane for the next item that has one to wait for here
+        auto dep_of = [&](const int4 &rec) { return warp == WF_FIRST_WORKER && lane < rec_ndep(rec) ? __ldg(&P.deps[rec_dep0(rec) + lane]) : make_int2(0, 0); };
+        int2 dep = dep_of(cur);
         int sidx = -1;
         uint32_t cnt = 0, done_items = 0, uc = 0;
         int sub_log = 6, units_n = 0;
         bool bulk_out = false;
         int kind = -1, p_log = 0, tr_log = 0, tw_valid = 0, act = 0, res_pos = 0;
         for (; item < NI; item += G) {
-            const int4 nn = item + 2 * G < NI ? __ldg(&P.items[item + 2 * G]) : zero4;
-            const int2 dep_nxt =
-                (warp == WF_FIRST_WORKER && item + G < NI && lane < rec_ndep(nxt)) ? __ldg(&P.deps[rec_dep0(nxt) + lane]) : make_int2(0, 0);
+            // (the record one item ahead, not two as for the loader: registers)
+            const int4 nxt = item + G < NI ? __ldg(&P.items[item + G]) : zero4;
             if (rec_stage(cur) != sidx) {
                 sidx = rec_stage(cur);
                 const WfStage *sp = &P.stages[sidx];
@@ -1500,12 +1500,14 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 }
                 if (tid == 0) tr(item, 12);
+                dep = dep_of(nxt);
             } else {
                 // an item of the worker warps alone: output rows of one image (or a depth-wise tile)
                 if (!SPLIT || kind < WF_NONE) {
-                    if (warp == WF_FIRST_WORKER && !wait_deps_warp(P, rec_dep0(cur), rec_ndep(cur), dep_cur, run, lane, [] {}) && lane == 0) *epi_fail = 1;
+                    if (warp == WF_FIRST_WORKER && !wait_deps_warp(P, rec_dep0(cur), rec_ndep(cur), dep, run, lane, [] {}) && lane == 0) *epi_fail = 1;
                     epi_bar();
                 }
+                dep = dep_of(nxt);                                     // on its way while the item is worked on
                 if (tid == 0) tr(item, 1);
                 const int n = rec_tn(cur), oh_lo = __ldg(&P.stages[sidx].oh_lo), oh = oh_lo + tile_r;
                 if (*epi_fail) {
@@ -1555,7 +1557,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 ++done_items;
             }
             if (tid == 0) tr(item, 6);
-            cur = nxt; dep_cur = dep_nxt; nxt = nn;
+            cur = nxt;
         }
     }
 
