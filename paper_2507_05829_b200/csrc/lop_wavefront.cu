@@ -21,11 +21,12 @@
 // later: the swizzle is a function of the address).  Anchors in the last (kw-1)*dw columns of a
 // pitch would wrap into the next row; they are computed and dropped.  K is walked as (channel chunk, kh,
 // kw, 16-channel step) whatever the tile, so a pixel's bits do not depend on who computes it.  (A gathered stem is a
-// pointwise layer here: its K is the order of the gathered values, lop_gather.cuh.)
+// pointwise layer here: its K is the order of the gathered values, lop_gather.cuh.)  Where the plan sums K in parts, a
+// tile's parts are items of neighbouring CTAs of a cluster, which exchange slices of their partial sums (split_item).
 //
 // Deadlock freedom: items are numbered in a topological order, every CTA is resident and takes its
-// items in increasing order, so the lowest unfinished item never waits on an unstarted one.  All
-// waits are bounded all the same; one that runs out raises the status word and the abort flag.
+// items in increasing order, so the lowest unfinished item never waits on an unstarted one (the parts of a split tile
+// wait for one another, and for nothing that has a higher number than the first of them).  All waits are bounded all the same; one that runs out raises the status word and the abort flag.
 #include <atomic>
 
 #include <cuda_bf16.h>
