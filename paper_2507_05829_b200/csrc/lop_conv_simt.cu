@@ -277,6 +277,7 @@ __global__ void __launch_bounds__(SMALL_THREADS) conv_simt_small_kernel(const __
         const unsigned n = live ? 16u : 0u;                    // 0: the sixteen bytes are zero-filled, nothing is read
         asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "r"(n) : "memory");
     };
+    grid_wait();                                               // before the weights too: the launch before this one may have written them
     // weights: K contiguous floats per output channel
     for (int i = threadIdx.x; i < SMALL_CO * (K >> 2); i += SMALL_THREADS) {
         const int r = i / (K >> 2), k4 = i - r * (K >> 2);
@@ -285,7 +286,6 @@ __global__ void __launch_bounds__(SMALL_THREADS) conv_simt_small_kernel(const __
         copy16(Bs + r * pitch + 4 * k4, live ? w + wo : w, live);
     }
     // patches: four threads per pixel, each every fourth filter tap
-    grid_wait();                                               // (no launch before this one writes weights)
     {
         const int px = threadIdx.x >> 2;
         const bool ok = m0 + px < M;

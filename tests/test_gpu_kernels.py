@@ -310,6 +310,36 @@ def test_calls_in_a_row_wait_for_what_they_read(dtype, C, H, W, flags):
     assert torch.equal(runs[0][0], runs[1][0]) and torch.equal(runs[0][1], runs[1][1])
 
 
+@pytest.mark.parametrize("dtype,C,flags", [("f32", 16, 0), ("bf16", 64, 0), ("bf16", 64, lop.LOP_FLAG_PER_LAYER), ("bf16", 64, lop.LOP_FLAG_FORCE_SIMT)])
+@pytest.mark.parametrize("streamed", [False, True])
+def test_parameters_that_the_calls_before_have_written(dtype, C, flags, streamed):
+    """A layer's filters are the output of the chain called before it, its scale and shift those of the one before that, other
+    values in every turn: the bits of calls with a synchronisation between them.  (Streamed: a launch that brings the input
+    stands between them.)"""
+    side = {16: 12, 64: 24}[C]                                          # side x side x C values are C filters of 3x3xC
+    makers = [one_layer(conv(C, C, 3, act=li.ACT_RELU), 1, side, side, dtype=dtype), one_layer(conv(16, C, 1, p=0), 1, 2, 1, dtype="f32"),
+              one_layer(conv(C, C, 3, act=li.ACT_NONE), 1, 20, 18, dtype=dtype)]
+    weights, affine, user = DeviceChain(makers[0], flags=flags), DeviceChain(makers[1]), DeviceChain(makers[2], flags=flags)
+    per_channel = affine.outs[-1].data_ptr()
+    user.plans[0].set_params(0, weights.outs[-1].data_ptr(), per_channel, per_channel + 4 * C)
+    xs = [(weights.input_tensor() * f, affine.input_tensor() * f) for f in (1.0, -0.5, 0.25)]
+    x, pinned = user.input_tensor(), user.pinned_input()
+    runs = []
+    for between in (torch.cuda.synchronize, lambda: None):
+        got = []
+        for turn in range(9):
+            xw, xa = xs[turn % 3]
+            for call in (lambda: affine.run_whole(xa), lambda: weights.run_whole(xw), lambda: user.run_pipelined(pinned) if streamed else user.run_whole(x)):
+                out = call()
+                between()
+            got.append(out.clone())
+        torch.cuda.synchronize()
+        runs.append(got)
+    assert all(torch.isfinite(t.float()).all() and t.float().abs().max() > 0 for t in runs[0])
+    assert not torch.equal(runs[0][0], runs[0][1]) and torch.equal(runs[0][0], runs[0][3])
+    assert all(torch.equal(a, b) for a, b in zip(*runs))
+
+
 # ------------------------------------------------------------------------------------ K summed in parts by the CTAs of a cluster
 SPLIT_CASES = [  # k, s, p, cin, cout, N, H, W, residual, activation
     (3, 1, 1, 512, 512, 1, 7, 7, li.RES_PRE_ACT, li.ACT_RELU),          # four parts: one tile of pixels, every row of it in reach of padding
