@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(SMALL_THREADS) conv_simt_small_kernel(const __
     if (m >= M) return;
     const Pixel q = pixel_of(p, m, M, rows);
     const long long o = (((long long)q.n * p.Ho + q.oh) * p.Wo + q.ow) * p.Cout;
-    const float *__restrict__ res = static_cast<const float *>(p.res);
+    const float *__restrict__ res = from_here(static_cast<const float *>(p.res));
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         const int co = n0 + cq + 4 * j;

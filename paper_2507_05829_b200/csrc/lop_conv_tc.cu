@@ -178,6 +178,7 @@ __global__ void __launch_bounds__(TC_THREADS) conv_tc_kernel(const __grid_consta
         if (ok) {
             __nv_bfloat16 *y = static_cast<__nv_bfloat16 *>(p.y);
             const __nv_bfloat16 *res = static_cast<const __nv_bfloat16 *>(p.res);
+            const float *scale = from_here(p.scale), *shift = from_here(p.shift);
             for (int j = 0; j < p.BN; j += 16) {
                 uint32_t r[16];
                 tmem_ld16(tmem_acc + ((uint32_t)(g * 32) << 16) + (uint32_t)j, r);
@@ -194,8 +195,8 @@ __global__ void __launch_bounds__(TC_THREADS) conv_tc_kernel(const __grid_consta
 #pragma unroll
                 for (int i = 0; i < 16; ++i) {
                     const int co = co0 + j + i;
-                    const float sc = p.scale ? __ldg(p.scale + co) : 1.0f;
-                    const float sf = p.shift ? __ldg(p.shift + co) : 0.0f;
+                    const float sc = scale ? __ldg(scale + co) : 1.0f;
+                    const float sf = shift ? __ldg(shift + co) : 0.0f;
                     v[i] = fmaf(sc, __uint_as_float(r[i]), sf);
                 }
                 float rv[16];

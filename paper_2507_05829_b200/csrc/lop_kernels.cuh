@@ -43,11 +43,12 @@ struct PoolArgs {
 #ifdef __CUDACC__
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-// A pointer whose loads the compiler must not take to before this place: those of read-only data move across grid_wait().
+// A pointer whose loads the compiler must not take to before this place: those of read-only data (__restrict__, __ldg) may move
+// across grid_wait(), but not in front of the place that the pointer comes from.
 template <typename T>
 __device__ __forceinline__ T *from_here(T *p)
 {
-    asm volatile("" : "+l"(p)::"memory");
+    asm volatile("" : "+l"(p));
     return p;
 }
 #endif

@@ -915,8 +915,8 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 const int co0 = SPLIT ? (rec_cout(cur) >> s_log) * BN : c0, ch0 = SPLIT ? (rec_cout(cur) & ((1 << s_log) - 1)) * n_chunks : 0;
                 if (ok && (((pc & 1u) ? ss_key[1] : ss_key[0]) != sidx || ((pc & 1u) ? ss_co[1] : ss_co[0]) != c0)) {
                     float *ds = s_scale + 128 * (pc & 1u), *dsh = s_shift + 128 * (pc & 1u);
-                    const float *scale = ldg_ptr<const float *>(reinterpret_cast<const void *const *>(&P.stages[sidx].scale));
-                    const float *shift = ldg_ptr<const float *>(reinterpret_cast<const void *const *>(&P.stages[sidx].shift));
+                    const float *scale = from_here(ldg_ptr<const float *>(reinterpret_cast<const void *const *>(&P.stages[sidx].scale)));
+                    const float *shift = from_here(ldg_ptr<const float *>(reinterpret_cast<const void *const *>(&P.stages[sidx].shift)));
                     if (pc & 1u) { ss_key[1] = sidx; ss_co[1] = c0; } else { ss_key[0] = sidx; ss_co[0] = c0; }
                     for (int i = lane; i < BN >> s_log; i += 32) {
                         ds[i] = scale ? __ldg(scale + c0 + i) : 1.0f;
