@@ -254,7 +254,8 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN)) conv_simt_kernel(const 
 // all there is, so both operands' whole K extent goes to shared memory in one go -- every load of the block in flight at
 // once, one barrier -- and a thread then walks its pixel's K for four output channels.  fp32 with Cin a multiple of
 // four.  Row pitch: an odd multiple of four floats, so that the eight pixels and the four channel rows a warp reads fall
-// into different banks.
+// into different banks.  Divisions and other index arithmetic stand before the wait for the launch in front, every read
+// behind it (with the divisions behind it, too, a 16-channel 3x3 layer of 32x32 called in a row takes 6.1 us, 4.6 so).
 // ---------------------------------------------------------------------------------------------
 constexpr int SMALL_PX = 16, SMALL_CO = 16, SMALL_THREADS = 64;
 
@@ -277,52 +278,49 @@ __global__ void __launch_bounds__(SMALL_THREADS) conv_simt_small_kernel(const __
         const unsigned n = live ? 16u : 0u;                    // 0: the sixteen bytes are zero-filled, nothing is read
         asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "r"(n) : "memory");
     };
+    // four threads per pixel (each every fourth filter tap) and per output channel (each every fourth group of four K values)
+    const int part = threadIdx.x & 3, r = threadIdx.x >> 2;
+    const bool ok = m0 + r < M, has_row = n0 + r < p.Cout;
+    const Pixel at = pixel_of(p, ok ? m0 + r : 0, M, rows);
+    const int ih0 = at.oh * p.sh - p.ph, iw0 = at.ow * p.sw - p.pw;
+    const long long x0 = (((long long)at.n * p.Hin + ih0) * p.Win + iw0) * p.Cin, w0 = (long long)(n0 + r) * K;
+    int a = part / p.kw, b = part - a * p.kw;
+    const int a4 = 4 / p.kw, b4 = 4 - a4 * p.kw;               // four taps further on
     grid_wait();                                               // before the weights too: the launch before this one may have written them
-    // weights: K contiguous floats per output channel
-    for (int i = threadIdx.x; i < SMALL_CO * (K >> 2); i += SMALL_THREADS) {
-        const int r = i / (K >> 2), k4 = i - r * (K >> 2);
-        const long long wo = (long long)(n0 + r) * K + 4 * k4;
-        const bool live = n0 + r < p.Cout && dbg_in_bounds(p.dbg, wo, 4, (long long)p.Cout * K);
-        copy16(Bs + r * pitch + 4 * k4, live ? w + wo : w, live);
+    for (int k = 4 * part; k < K; k += 16) {                   // K contiguous floats per output channel
+        const bool live = has_row && dbg_in_bounds(p.dbg, w0 + k, 4, (long long)p.Cout * K);
+        copy16(Bs + r * pitch + k, live ? w + w0 + k : w, live);
     }
-    // patches: four threads per pixel, each every fourth filter tap
-    {
-        const int px = threadIdx.x >> 2;
-        const bool ok = m0 + px < M;
-        const Pixel q = pixel_of(p, ok ? m0 + px : 0, M, rows);
-        for (int tap = threadIdx.x & 3; tap < taps; tap += 4) {
-            const int a = tap / p.kw, b = tap - a * p.kw;
-            const int ih = q.oh * p.sh - p.ph + a * p.dh, iw = q.ow * p.sw - p.pw + b * p.dw;
-            const long long xo = (((long long)q.n * p.Hin + ih) * p.Win + iw) * p.Cin;
-            const bool live = ok && ih >= 0 && ih < p.Hin && iw >= 0 && iw < p.Win && dbg_in_bounds(p.dbg, xo, p.Cin, x_elems);
-            for (int c = 0; c < c4n; ++c) copy16(As + px * pitch + tap * p.Cin + 4 * c, live ? x + xo + 4 * c : x, live);
-        }
+    for (int tap = part; tap < taps; tap += 4) {
+        const int ih = ih0 + a * p.dh, iw = iw0 + b * p.dw;
+        const long long xo = x0 + ((long long)a * p.dh * p.Win + b * p.dw) * p.Cin;
+        const bool live = ok && ih >= 0 && ih < p.Hin && iw >= 0 && iw < p.Win && dbg_in_bounds(p.dbg, xo, p.Cin, x_elems);
+        for (int c = 0; c < c4n; ++c) copy16(As + r * pitch + tap * p.Cin + 4 * c, live ? x + xo + 4 * c : x, live);
+        a += a4; b += b4;
+        if (b >= p.kw) { b -= p.kw; ++a; }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
 
-    const int px = threadIdx.x >> 2, cq = threadIdx.x & 3;
-    const float *xa = As + px * pitch;
+    const float *xa = As + r * pitch;
     float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll 4
     for (int k = 0; k < K; k += 4) {
         const float4 xv = *reinterpret_cast<const float4 *>(xa + k);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const float4 wv = *reinterpret_cast<const float4 *>(Bs + (cq + 4 * j) * pitch + k);
+            const float4 wv = *reinterpret_cast<const float4 *>(Bs + (part + 4 * j) * pitch + k);
             acc[j] = fmaf(xv.w, wv.w, fmaf(xv.z, wv.z, fmaf(xv.y, wv.y, fmaf(xv.x, wv.x, acc[j]))));
         }
     }
-    const long long m = m0 + px;
-    if (m >= M) return;
-    const Pixel q = pixel_of(p, m, M, rows);
-    const long long o = (((long long)q.n * p.Ho + q.oh) * p.Wo + q.ow) * p.Cout;
+    if (!ok) return;
+    const long long o = (((long long)at.n * p.Ho + at.oh) * p.Wo + at.ow) * p.Cout;
     const float *__restrict__ res = from_here(static_cast<const float *>(p.res));
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        const int co = n0 + cq + 4 * j;
-        if (co >= p.Cout || !dbg_in_bounds(p.dbg, o + co, 1, y_elems) || !dbg_in_bounds(p.dbg, q.oh - p.oh_lo, 1, rows)) continue;
+        const int co = n0 + part + 4 * j;
+        if (co >= p.Cout || !dbg_in_bounds(p.dbg, o + co, 1, y_elems) || !dbg_in_bounds(p.dbg, at.oh - p.oh_lo, 1, rows)) continue;
         static_cast<float *>(p.y)[o + co] = finish(p, res, o + co, co, acc[j]);
     }
 }
