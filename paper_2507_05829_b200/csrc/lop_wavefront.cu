@@ -1585,6 +1585,12 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
 
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    // A CTA that gave up may have copies on their way into its shared memory (operands, residual rows, the other parts' partial
+    // sums) or messages to other CTAs, and MMAs that read it.  Each takes microseconds: the memory is held for a hundred of them
+    // before another block may have it.  (Not a wait for the barriers that would tell: keeping the loader's counts for it to the
+    // end cost every run of a ResNet-50 0.3 to 0.6 %.  misc[1] is the same for all threads: every role has ended.)
+    if (misc[1])
+        for (int i = 0; i < 100; ++i) __nanosleep(1000);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (warp == 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
