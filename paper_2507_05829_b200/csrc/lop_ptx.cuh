@@ -64,6 +64,10 @@ __device__ __forceinline__ void st_async4(uint32_t remote, uint32_t a, uint32_t 
                  "r"(remote_bar)
                  : "memory");
 }
+__device__ __forceinline__ void st_cluster(uint32_t remote, uint32_t value)
+{
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote), "r"(value) : "memory");
+}
 __device__ __forceinline__ void cluster_sync()
 {
     asm volatile("barrier.cluster.arrive;" ::: "memory");

@@ -604,7 +604,8 @@ __device__ __forceinline__ uint32_t ld_shared(uint32_t addr)
     asm volatile("ld.volatile.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
     return v;
 }
-// Bounded wait on a barrier that other CTAs of the cluster may complete; gives up when this CTA's abort flag is raised.
+// Bounded wait on a barrier that other CTAs of the cluster may complete; gives up when this CTA's abort flag is raised (which a
+// CTA of the cluster that gives up does on its way out: what it was to send will not come).
 __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, uint32_t abort_at)
 {
     for (uint32_t i = 0; i < WAIT_LIMIT; ++i) {
@@ -1588,9 +1589,14 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
     // A CTA that gave up may have copies on their way into its shared memory (operands, residual rows, the other parts' partial
     // sums) or messages to other CTAs, and MMAs that read it.  Each takes microseconds: the memory is held for a hundred of them
     // before another block may have it.  (Not a wait for the barriers that would tell: keeping the loader's counts for it to the
-    // end cost every run of a ResNet-50 0.3 to 0.6 %.  misc[1] is the same for all threads: every role has ended.)
-    if (misc[1])
+    // end cost every run of a ResNet-50 0.3 to 0.6 %.)  Every role has ended: misc[1] changes now only by another CTA that gives
+    // up, and a warp sees one value of it.
+    if (misc[1]) {
+        // (the cluster's other CTAs hear of it first: a role of theirs may wait for this CTA's part of a tile, and for nothing
+        // else that would tell it.  Looks at the device-wide flag in those waits cost a ResNet-18 streamed one image 1.5 us.)
+        if (SPLIT && threadIdx.x < (unsigned)P.cluster) st_cluster(map_to_cta(bars + BAR_MISC + 4u, threadIdx.x), 1u);
         for (int i = 0; i < 100; ++i) __nanosleep(1000);
+    }
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (warp == 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");

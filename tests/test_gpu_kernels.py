@@ -372,3 +372,37 @@ def test_split_tiles(case):
     dc.check_device()
     assert torch.equal(got, want) and torch.equal(host, want.cpu())
 
+
+
+@pytest.mark.parametrize("case", [SPLIT_CASES[0], SPLIT_CASES[1], SPLIT_CASES[4]])
+def test_a_band_that_never_arrives_ends_a_launch_with_split_tiles(case):
+    """Band 1 is withheld (a dependency that the host never satisfies) with a limit of 4000 looks, about a millisecond: whoever
+    waits for a part of a tile that will not come gives up with the rest, long before a wait of its own would run out (0.2 s);
+    the status is reported once and the plan works again."""
+    k, s, p, cin, cout, N, H, W, res, act = case
+    layers = [conv(cin, cin, 1, p=0, input_from=-1), conv(cin, cout, k, s=s, p=p, act=act, input_from=0), conv(cout, cout, 3, act=act, input_from=1)]
+    wl = Workload("withheld", "bf16", N, H, W, cin, [Segment(layers, 3)], seed=32)
+    li.fill_parameters(wl)
+    li.make_input(wl)
+    dc = DeviceChain(wl, flags=lop.LOP_FLAG_REUSE_HALO | lop.LOP_FLAG_COPY_ENGINE)
+    plan, ws, out, x = dc.plans[0], dc.ws[0], dc.outs[0], dc.pinned_input()
+    good = dc.run_pipelined(x).clone()
+    torch.cuda.synchronize()
+    dc.check_device()
+    for _ in range(2):
+        plan.set_wait_limit(4000)
+        t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        t0.record()
+        plan.run_pipelined_withheld(1, x.data_ptr(), dc.staging.data_ptr(), out.data_ptr(), ws.data_ptr(), torch.cuda.current_stream().cuda_stream)
+        t1.record()
+        torch.cuda.synchronize()
+        assert t0.elapsed_time(t1) < 100.0
+        with pytest.raises(lop.LopError) as e:
+            plan.check_device(ws.data_ptr())
+        assert e.value.status == -7
+        plan.set_wait_limit(0)
+        out.zero_()
+        dc.run_pipelined(x)
+        torch.cuda.synchronize()
+        dc.check_device()
+        assert torch.equal(out, good)
