@@ -261,6 +261,9 @@ int lop_plan_layer_time(lop_plan_t *plan, int band, int layer, float *ms);
 /* Which kernel family serves a layer: 0 = pooling, 1 = CUDA-core convolution,
  * 2 = tcgen05 tensor-core convolution.  <0 on error. */
 int lop_plan_layer_kernel(const lop_plan_t *plan, int layer);
+/* HOST ONLY.  In how many parts (1, 2 or 4) a tensor-core convolution sums its channels: every part in float32 from zero, then
+ * the parts in order.  1 for all other layers.  <0 on error. */
+int lop_plan_layer_parts(const lop_plan_t *plan, int layer);
 /* Where the full-size output tensor of an intermediate layer (0 <= layer < n_layers - 1) lives: byte offset into the
  * workspace given to the lop_run_* calls; its shape is lop_plan_out_shape(layer), NHWC in the storage dtype.  The rows a
  * call has computed are there when the call's stream work is done (for inspection and tests; the last layer's tensor is

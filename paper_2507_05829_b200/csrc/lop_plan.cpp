@@ -466,6 +466,13 @@ int lop_plan_layer_kernel(const lop_plan_t *plan, int layer)
     return plan->layers[layer].kernel;
 }
 
+int lop_plan_layer_parts(const lop_plan_t *plan, int layer)
+{
+    if (!plan) { set_error("plan is NULL"); return LOP_EINVAL; }
+    if (layer < 0 || layer >= (int)plan->layers.size()) { set_error("lop_plan_layer_parts: layer %d out of range", layer); return LOP_EINVAL; }
+    return plan->layers[layer].k_split;
+}
+
 const char *lop_strerror(int status)
 {
     switch (status) {

@@ -48,7 +48,7 @@ constexpr int EPI_THREADS = 32 * WF_WORKER_WARPS;
 #define LOP_PREFETCH 32
 #endif
 constexpr int PREFETCH_BOXES = LOP_PREFETCH;                // weight boxes of a tile asked for ahead of its dependencies
-static_assert(8 * (2 * WF_ENTRIES + 4 + 2 * WF_PUBQ + 4 + 3 * WF_UNITS + 2 + WF_GROUPS + 2) + 128 + 2048 + 8 * (128 + 32) <= WF_FIXED_SMEM, "barriers and tables");
+static_assert(8 * (2 * WF_ENTRIES + 4 + 2 * WF_PUBQ + 4 + 3 * WF_UNITS + 2 + WF_GROUPS + 4) + 128 + 2048 + 8 * (128 + 32) <= WF_FIXED_SMEM, "barriers and tables");
 constexpr int COL_GROUPS = WF_WORKER_WARPS / 4;            // worker warps sharing a TMEM lane group split the columns
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned *p)
@@ -594,9 +594,12 @@ constexpr uint32_t BAR_ACCF = 16u * WF_ENTRIES;                                /
 constexpr uint32_t BAR_SSF = BAR_ACCF + 32u + 16u * WF_PUBQ;                   // scale / shift in place
 constexpr uint32_t BAR_UGRANT = BAR_SSF + 32u;                                 // output units: granted, ready, free
 constexpr uint32_t BAR_UREADY = BAR_UGRANT + 8u * WF_UNITS, BAR_UFREE = BAR_UREADY + 8u * WF_UNITS;
-constexpr uint32_t BAR_XOK = BAR_UFREE + 8u * WF_UNITS + 16u + 8u * WF_GROUPS; // the others take partial sums
-constexpr uint32_t BAR_XFULL = BAR_XOK + 8u;                                   // the others' partial sums are here
-constexpr uint32_t BAR_MISC = BAR_XFULL + 8u;                                  // words: [1] abort, [8 + q] the unit part q takes sums in
+// Tiles of two parts and of four have barriers and words of their own: a CTA two places away is a partner in the latter only,
+// may be ahead by a tile, and its word would count as the nearer partner's, which is still to come.
+constexpr uint32_t BAR_XOK = BAR_UFREE + 8u * WF_UNITS + 16u + 8u * WF_GROUPS; // the others take partial sums: of tiles of two parts, of four
+constexpr uint32_t BAR_XFULL = BAR_XOK + 16u;                                  // the others' partial sums are here
+constexpr uint32_t BAR_MISC = BAR_XFULL + 16u;                                 // words: [1] abort, [4] parity of the split tiles so far (bit 0: of
+                                                                               // two parts, 1: of four), [8 + q], [12 + q]: the unit part q takes sums in
 
 __device__ __forceinline__ uint32_t ld_shared(uint32_t addr)
 {
@@ -626,24 +629,24 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
 }
 
 // The loader's side, by its one thread: once the units that partial sums arrive in are free, the barriers are armed and the
-// other CTAs told where to write.  cout: the item's slice; uc: output units before these; n_split: split tiles before this one.
+// other CTAs told where to write.  cout: the item's slice; uc: output units before these; turn: parity of the tiles of as many
+// parts before this one.
 // (Barriers whose phase is not over cannot be armed again: with two parts the next tile's units are free before this one's
 // exchange is done.)
-__device__ __noinline__ bool take_partial_sums(uint32_t bars, uint32_t cout, uint32_t s_log, uint32_t uc, uint32_t n_split)
+__device__ __noinline__ bool take_partial_sums(uint32_t bars, uint32_t cout, uint32_t s_log, uint32_t uc, uint32_t turn)
 {
     const uint32_t others = (1u << s_log) - 1u, part = cout & others, base_rank = cta_rank() & ~others, abort_at = bars + BAR_MISC + 4u;
-    if (n_split > 0 && (!mbar_wait_cluster(bars + BAR_XOK, (n_split - 1u) & 1u, abort_at) || !mbar_wait_cluster(bars + BAR_XFULL, (n_split - 1u) & 1u, abort_at)))
-        return false;
+    const uint32_t xok = bars + BAR_XOK + 8u * (s_log - 1u), xfull = bars + BAR_XFULL + 8u * (s_log - 1u), words = bars + BAR_MISC + 16u * (s_log + 1u);
+    if (!mbar_wait_cluster(xok, turn ^ 1u, abort_at) || !mbar_wait_cluster(xfull, turn ^ 1u, abort_at)) return false;
     for (uint32_t u = uc; u < uc + ((others + 1u) >> 1); ++u) {
         const uint32_t sl = 8u * (u & (WF_UNITS - 1));
         if (!mbar_wait_cluster(bars + BAR_UFREE + sl, ((u / WF_UNITS) & 1u) ^ 1u, abort_at)) return false;
         mbar_arrive(bars + BAR_UGRANT + sl);                                   // (its phase; nobody waits for it)
     }
-    mbar_expect_tx(bars + BAR_XOK, 4u * others);
-    mbar_expect_tx(bars + BAR_XFULL, others * (512u * (WF_SPLIT_BN >> s_log)));
+    mbar_expect_tx(xok, 4u * others);
+    mbar_expect_tx(xfull, others * (512u * (WF_SPLIT_BN >> s_log)));
     for (uint32_t q = 0; q <= others; ++q)
-        if (q != part)
-            st_async(map_to_cta(bars + BAR_MISC + 4u * (8u + part), base_rank + q), uc & (WF_UNITS - 1), map_to_cta(bars + BAR_XOK, base_rank + q));
+        if (q != part) st_async(map_to_cta(words + 4u * part, base_rank + q), uc & (WF_UNITS - 1), map_to_cta(xok, base_rank + q));
     return true;
 }
 
@@ -659,8 +662,9 @@ __device__ __noinline__ bool take_partial_sums(uint32_t bars, uint32_t cout, uin
 template <bool SMOOTH>
 __device__ __noinline__ uint32_t split_item(const WfStage *sp, int4 rec, uint8_t *smem_bars, uint32_t unit0, uint32_t unit_bytes, uint32_t acc, uint32_t uc, uint32_t cnt)
 {
-    const uint32_t n_split = ld_shared(smem_u32(smem_bars) + BAR_MISC + 16u);  // split tiles before this one
     const uint32_t bars = smem_u32(smem_bars), s_log = (uint32_t)__ldg(&sp->s_log), parts = 1u << s_log, part = (uint32_t)rec_cout(rec) & (parts - 1u);
+    const uint32_t turn = ld_shared(bars + BAR_MISC + 16u) >> (s_log - 1u) & 1u;   // parity of the tiles of as many parts before this one
+    const uint32_t xok = bars + BAR_XOK + 8u * (s_log - 1u), xfull = bars + BAR_XFULL + 8u * (s_log - 1u), words = bars + BAR_MISC + 16u * (s_log + 1u);
     const uint32_t slice = WF_SPLIT_BN >> s_log, base_rank = cta_rank() & ~(parts - 1u), abort_at = bars + BAR_MISC + 4u, rx = uc + 1u;
     const uint32_t per_unit = parts >> 1, from_bytes = 512u * slice;           // senders per unit (two parts: one, four: two)
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u, row = (warp & 3u) * 32u + lane, cgrp = (warp - WF_FIRST_WORKER) >> 2, buf = cnt & 1u;
@@ -670,7 +674,7 @@ __device__ __noinline__ uint32_t split_item(const WfStage *sp, int4 rec, uint8_t
     const bool bulk_out = __ldg(&sp->out_map) >= 0;
     acc += ((warp & 3u) * 32u) << 16;
     bool ok = mbar_wait_cluster(bars + BAR_ACCF + 8u * buf, (cnt >> 1) & 1u, abort_at);
-    ok = ok && mbar_wait_cluster(bars + BAR_XOK, n_split & 1u, abort_at);
+    ok = ok && mbar_wait_cluster(xok, turn, abort_at);
     ok = __all_sync(0xffffffffu, ok);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     uint32_t r[8];                                                             // (eight columns at a time: what this needs, the kernel around the call has not)
@@ -680,8 +684,8 @@ __device__ __noinline__ uint32_t split_item(const WfStage *sp, int4 rec, uint8_t
         if (q == part) continue;
         if (((++k + 1u) >> 1 & 1u) != cgrp) continue;                          // (the first and third 16 columns: the warps without a chunk to finish)
         tmem_ld8(acc + c, r);
-        const uint32_t to = map_to_cta(sums_at(ld_shared(bars + BAR_MISC + 4u * (8u + q)), part < q ? part : part - 1u) + (c - q * slice) * 512u, base_rank + q);
-        const uint32_t bar = map_to_cta(bars + BAR_XFULL, base_rank + q);
+        const uint32_t to = map_to_cta(sums_at(ld_shared(words + 4u * q), part < q ? part : part - 1u) + (c - q * slice) * 512u, base_rank + q);
+        const uint32_t bar = map_to_cta(xfull, base_rank + q);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
         st_async4(to, r[0], r[1], r[2], r[3], bar);
         st_async4(to + 2048u, r[4], r[5], r[6], r[7], bar);
@@ -700,7 +704,7 @@ __device__ __noinline__ uint32_t split_item(const WfStage *sp, int4 rec, uint8_t
     const uint32_t sl = uc & (WF_UNITS - 1);
     ok = ok && mbar_wait_cluster(bars + BAR_UGRANT + 8u * sl, (uc / WF_UNITS) & 1u, abort_at);
     ok = ok && mbar_wait_cluster(bars + BAR_SSF + 8u * buf, (cnt >> 1) & 1u, abort_at);
-    ok = ok && mbar_wait_cluster(bars + BAR_XFULL, n_split & 1u, abort_at);
+    ok = ok && mbar_wait_cluster(xfull, turn, abort_at);
     ok = __all_sync(0xffffffffu, ok);
 #pragma unroll 1
     for (uint32_t j = 16u * cgrp; ok && j < min(slice, 16u * cgrp + 16u); j += 8) {
@@ -756,7 +760,7 @@ __device__ __noinline__ uint32_t split_item(const WfStage *sp, int4 rec, uint8_t
         mbar_arrive(bars + BAR_ACCF + 16u + 8u * buf);
         mbar_arrive(bars + BAR_SSF + 16u + 8u * buf);
         for (uint32_t u = rx; u < rx + (parts >> 1); ++u) mbar_arrive(bars + BAR_UFREE + 8u * (u & (WF_UNITS - 1)));
-        *reinterpret_cast<volatile uint32_t *>(smem_bars + BAR_MISC + 16) = n_split + 1u;
+        *reinterpret_cast<volatile uint32_t *>(smem_bars + BAR_MISC + 16) = ld_shared(bars + BAR_MISC + 16u) ^ (1u << (s_log - 1u));
     }
     if (!bulk_out && ld_shared(bars + BAR_MISC + 12) == 0u) {
         copy_unit(smem_bars - bars + unit0 + sl * unit_bytes, row_pix, static_cast<uint4 *>(ldg_ptr<void *>(reinterpret_cast<const void *const *>(&sp->y))),
@@ -789,10 +793,9 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
     const uint32_t uready0 = bars + BAR_UREADY, ufree0 = bars + BAR_UFREE;  // ... finished by the workers / read out
     const uint32_t wfull = ufree0 + 8u * WF_UNITS, wempty = wfull + 8u;  // kept weights: loaded / last used
     const uint32_t gfull0 = wempty + 8u;                                 // slab stages: a group of boxes is loaded
-    const uint32_t xok = bars + BAR_XOK, xfull = bars + BAR_XFULL;       // split tiles
     uint8_t *tail = smem + (bars + BAR_MISC - base);
     volatile uint32_t *misc = reinterpret_cast<volatile uint32_t *>(tail);      // [0] TMEM base, [1] abort, [2] run, [3] epilogue failure,
-                                                                                // [8..11] the units the other parts of a split tile take sums in
+                                                                                // [4], [8..15] split tiles (see BAR_MISC)
     volatile uint32_t *entry_at = misc + 16;                                     // [WF_ENTRIES]: where the ring's entries start (loader only)
     float *s_scale = reinterpret_cast<float *>(tail + 128);                      // [2][128]: per-channel scale of this and the next tile
     float *s_shift = s_scale + 256;                                              // [2][128]
@@ -824,8 +827,10 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
         mbar_init(wfull, 1);
         mbar_init(wempty, 1);
         for (int g = 0; g < WF_GROUPS; ++g) mbar_init(gfull0 + 8u * g, 1);
-        mbar_init(xok, 1);
-        mbar_init(xfull, 1);
+        for (uint32_t w = 0; w < 2; ++w) {
+            mbar_init(bars + BAR_XOK + 8u * w, 1);
+            mbar_init(bars + BAR_XFULL + 8u * w, 1);
+        }
         for (int q = 0; q < WF_PUBQ; ++q) {
             mbar_init(pubf0 + 8u * q, 1);
             mbar_init(pube0 + 8u * q, 1);
@@ -869,7 +874,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
         uint32_t a_bytes = 0, b_bytes = 0;
         const CUtensorMap *maps = nullptr;
         int s_log = 0;
-        uint32_t n_split = 0;                                  // split tiles so far
+        uint32_t split_turn = 0;                               // parity of the split tiles so far: bit 0 of two parts, bit 1 of four
         int first_offh = 0, first_offw = 0, first_mi = 0, cps = 1, units_n = 0, sub_log = 6, res_map = -1;
         bool first_have = true;
         uint32_t a_sz = 0, b_sz = 0, keep_bytes = 0;
@@ -1073,9 +1078,9 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                         }
                     }
                     if (SPLIT && s_log > 0 && !fail) {
-                        fail = !take_partial_sums(bars, (uint32_t)rec_cout(cur), (uint32_t)s_log, uc, n_split);
+                        fail = !take_partial_sums(bars, (uint32_t)rec_cout(cur), (uint32_t)s_log, uc, split_turn >> (s_log - 1) & 1u);
                         uc += (1u << s_log) >> 1;
-                        ++n_split;
+                        split_turn ^= 1u << (s_log - 1);
                     }
                     if (fail) atomicOr(P.status, 0x1u);
                     tr(item, 2);

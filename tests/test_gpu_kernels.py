@@ -351,6 +351,10 @@ SPLIT_CASES = [  # k, s, p, cin, cout, N, H, W, residual, activation
 ]
 
 
+def parts_of(dc):
+    return [[plan.layer_parts(i) for i in range(plan.num_layers())] for plan in dc.plans]
+
+
 @pytest.mark.parametrize("case", SPLIT_CASES)
 def test_split_tiles(case):
     """Against the oracle, and bit for bit between the executors: a chain of two such layers (several split tiles per CTA,
@@ -372,6 +376,33 @@ def test_split_tiles(case):
     dc.check_device()
     assert torch.equal(got, want) and torch.equal(host, want.cpu())
 
+
+MIXED_PARTS = [  # N, H, W, bands, segments of (k, s, cin, cout); the parts
+    (3, 14, 14, 7, [[(3, 1, 512, 512), (3, 1, 512, 256), (3, 1, 256, 256), (3, 1, 256, 512), (3, 1, 512, 512), (3, 1, 512, 256)]], [[2, 4, 4, 2, 2, 4]]),
+    (8, 7, 7, 3, [[(1, 1, 2048, 512), (3, 1, 512, 512), (1, 1, 512, 2048), (1, 1, 2048, 512), (3, 1, 512, 512)]], [[4, 2, 1, 4, 2]]),
+    (3, 28, 31, 4, [[(3, 2, 128, 256), (3, 1, 256, 256), (3, 1, 256, 256)], [(3, 2, 256, 512), (3, 1, 512, 512)]], [[2, 2, 2], [4, 4]]),
+]
+
+
+@pytest.mark.parametrize("N,H,W,bands,segments,parts", MIXED_PARTS)
+def test_tiles_of_two_parts_and_of_four_in_one_program(N, H, W, bands, segments, parts):
+    """A CTA takes part in a tile of two parts and then in one of four, whose other CTAs need not have finished theirs: the bits
+    of the per-layer kernels, in every one of many calls."""
+    segs = [Segment([conv(cin, cout, k, s=s, p=k // 2, act=li.ACT_RELU, input_from=i - 1) for i, (k, s, cin, cout) in enumerate(ls)], bands) for ls in segments]
+    wl = Workload("mixed", "bf16", N, H, W, segments[0][0][2], segs, seed=33)
+    li.fill_parameters(wl)
+    li.make_input(wl)
+    dc, per = DeviceChain(wl, flags=lop.LOP_FLAG_REUSE_HALO), DeviceChain(wl, flags=lop.LOP_FLAG_PER_LAYER)
+    assert parts_of(dc) == parts_of(per) == parts
+    want = per.run_whole(per.input_tensor()).clone()
+    assert torch.isfinite(want.float()).all() and want.float().abs().max() > 0
+    x, pinned = dc.input_tensor(), dc.pinned_input()
+    for _ in range(100):
+        for call in (lambda: dc.run_banded(x), lambda: dc.run_pipelined(pinned)):
+            dc.outs[-1].zero_()
+            got = call()
+            assert torch.equal(got, want)
+    dc.check_device()
 
 
 @pytest.mark.parametrize("case", [SPLIT_CASES[0], SPLIT_CASES[1], SPLIT_CASES[4]])
