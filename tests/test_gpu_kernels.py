@@ -341,13 +341,15 @@ def test_parameters_that_the_calls_before_have_written(dtype, C, flags, streamed
 
 
 # ------------------------------------------------------------------------------------ K summed in parts by the CTAs of a cluster
-SPLIT_CASES = [  # k, s, p, cin, cout, N, H, W, residual, activation
-    (3, 1, 1, 512, 512, 1, 7, 7, li.RES_PRE_ACT, li.ACT_RELU),          # four parts: one tile of pixels, every row of it in reach of padding
-    (3, 1, 1, 256, 256, 3, 11, 16, li.RES_POST_ACT, li.ACT_SILU),       # four parts, one chunk each; ragged tiles
-    (3, 2, 1, 256, 512, 2, 15, 13, li.RES_NONE, li.ACT_RELU),           # a box per tap, odd extents
-    (1, 1, 0, 2048, 512, 8, 7, 7, li.RES_NONE, li.ACT_NONE),            # pointwise
-    (3, 1, 1, 256, 256, 8, 14, 14, li.RES_PRE_ACT, li.ACT_GELU),        # two parts
-    (3, 1, 2, 128, 64, 1, 20, 18, li.RES_NONE, li.ACT_RELU),            # two chunks: two parts at most; one slice of channels per part
+SPLIT_CASES = [  # k, s, p, cin, cout, N, H, W, residual, activation; the parts that this layer and the 3x3 behind it are summed in
+    (3, 1, 1, 512, 512, 1, 7, 7, li.RES_PRE_ACT, li.ACT_RELU, [4, 4]),          # one tile of pixels, every row of it in reach of padding
+    (3, 1, 1, 256, 256, 3, 11, 16, li.RES_POST_ACT, li.ACT_SILU, [2, 2]),       # two chunks per part; ragged tiles
+    (3, 1, 1, 256, 256, 1, 11, 16, li.RES_POST_ACT, li.ACT_SILU, [4, 4]),       # one chunk per part
+    (3, 2, 1, 256, 512, 2, 15, 13, li.RES_NONE, li.ACT_RELU, [4, 4]),           # a box per tap, odd extents
+    (1, 1, 0, 2048, 512, 8, 7, 7, li.RES_NONE, li.ACT_NONE, [4, 2]),            # pointwise
+    (3, 1, 1, 256, 256, 8, 14, 14, li.RES_PRE_ACT, li.ACT_GELU, [2, 2]),
+    (3, 2, 1, 128, 256, 1, 28, 26, li.RES_NONE, li.ACT_RELU, [2, 4]),           # two chunks: two parts at most
+    (3, 1, 2, 128, 64, 1, 20, 18, li.RES_NONE, li.ACT_RELU, [1, 1]),            # too short a K: not split
 ]
 
 
@@ -359,7 +361,7 @@ def parts_of(dc):
 def test_split_tiles(case):
     """Against the oracle, and bit for bit between the executors: a chain of two such layers (several split tiles per CTA,
     the second's partial sums behind the first's), one with a shortcut, in bands, streamed, into host memory."""
-    k, s, p, cin, cout, N, H, W, res, act = case
+    k, s, p, cin, cout, N, H, W, res, act, parts = case
     l0 = conv(cin, cout, k, s=s, p=p, act=act, input_from=-1)
     layers = [l0, conv(cout, cout, 3, input_from=0, act=act, residual_from=0 if res != li.RES_NONE else NO_RESIDUAL, residual_pos=res)]
     wl = Workload("split", "bf16", N, H, W, cin, [Segment(layers, 3)], seed=31)
@@ -367,6 +369,7 @@ def test_split_tiles(case):
     li.make_input(wl)
     check_workload(wl, flags=lop.LOP_FLAG_REUSE_HALO, modes=("whole", "banded", "pipelined"))
     dc, per = DeviceChain(wl, flags=lop.LOP_FLAG_REUSE_HALO), DeviceChain(wl, flags=lop.LOP_FLAG_PER_LAYER)
+    assert parts_of(dc) == parts_of(per) == [parts]
     want = per.run_whole(per.input_tensor())
     host = torch.empty(want.shape, dtype=want.dtype).pin_memory()
     for _ in range(3):                                                  # calls in a row, too
@@ -405,12 +408,12 @@ def test_tiles_of_two_parts_and_of_four_in_one_program(N, H, W, bands, segments,
     dc.check_device()
 
 
-@pytest.mark.parametrize("case", [SPLIT_CASES[0], SPLIT_CASES[1], SPLIT_CASES[4]])
+@pytest.mark.parametrize("case", [SPLIT_CASES[0], SPLIT_CASES[1], SPLIT_CASES[5]])
 def test_a_band_that_never_arrives_ends_a_launch_with_split_tiles(case):
     """Band 1 is withheld (a dependency that the host never satisfies) with a limit of 4000 looks, about a millisecond: whoever
     waits for a part of a tile that will not come gives up with the rest, long before a wait of its own would run out (0.2 s);
     the status is reported once and the plan works again."""
-    k, s, p, cin, cout, N, H, W, res, act = case
+    k, s, p, cin, cout, N, H, W, res, act, parts = case
     layers = [conv(cin, cin, 1, p=0, input_from=-1), conv(cin, cout, k, s=s, p=p, act=act, input_from=0), conv(cout, cout, 3, act=act, input_from=1)]
     wl = Workload("withheld", "bf16", N, H, W, cin, [Segment(layers, 3)], seed=32)
     li.fill_parameters(wl)
