@@ -1538,8 +1538,13 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                 dep = dep_of(nxt);                                     // on its way while the item is worked on
                 if (tid == 0) tr(item, 1);
                 const int n = rec_tn(cur), oh_lo = __ldg(&P.stages[sidx].oh_lo), oh = oh_lo + tile_r;
-                if (*epi_fail) {
-                    // fall through to the common exit below
+                if (SPLIT && kind == WF_SPLIT) {
+                    // (also when a wait has run out: no barrier stands between the word's last write, behind the item before, and
+                    // this place, and warps that saw different values would meet at different barriers for good)
+                    uc += split_item<SMOOTH>(&P.stages[sidx], cur, smem + (bars - base), unit0, unit_bytes, tmem_base + (cnt & 1u) * 256u, uc, cnt);
+                    ++cnt;
+                } else if ((SPLIT && kind == WF_NONE) || *epi_fail) {
+                    // on to the barrier and the common exit below
                 } else if (kind == WF_POOL) {
                     const int oh0 = oh_lo + (tile_r << tr_log);
                     if (__ldg(&P.stages[sidx].mode)) pool3_item(&P.stages[sidx], n, oh0, min(1 << tr_log, __ldg(&P.stages[sidx].oh_hi) - oh0), tid);
@@ -1550,10 +1555,6 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
                     layernorm_item(&P.stages[sidx], n, oh, tid);
                 } else if (ROWOPS && kind == WF_CONCAT) {
                     concat_item(&P.stages[sidx], n, oh, tid);
-                } else if (SPLIT && kind == WF_SPLIT) {
-                    uc += split_item<SMOOTH>(&P.stages[sidx], cur, smem + (bars - base), unit0, unit_bytes, tmem_base + (cnt & 1u) * 256u, uc, cnt);
-                    ++cnt;
-                } else if (SPLIT && kind == WF_NONE) {
                 } else {
                     gather_item(&P.stages[sidx], n, tile_r, tid, stg);
                 }

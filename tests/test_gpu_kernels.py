@@ -408,20 +408,26 @@ def test_tiles_of_two_parts_and_of_four_in_one_program(N, H, W, bands, segments,
     dc.check_device()
 
 
-@pytest.mark.parametrize("case", [SPLIT_CASES[0], SPLIT_CASES[1], SPLIT_CASES[5]])
-def test_a_band_that_never_arrives_ends_a_launch_with_split_tiles(case):
+@pytest.mark.parametrize("case,pools", [(SPLIT_CASES[0], 0), (SPLIT_CASES[1], 0), (SPLIT_CASES[5], 0), (SPLIT_CASES[2], 3)])
+def test_a_band_that_never_arrives_ends_a_launch_with_split_tiles(case, pools):
     """Band 1 is withheld (a dependency that the host never satisfies) with a limit of 4000 looks, about a millisecond: whoever
     waits for a part of a tile that will not come gives up with the rest, long before a wait of its own would run out (0.2 s);
-    the status is reported once and the plan works again."""
+    the status is reported once and the plan works again.  With poolings between, whose single rows are many items that the
+    workers publish themselves, and the result stored to host memory, as split tiles are then, too: the workers may find their
+    way to the publisher closed in front of a split tile."""
     k, s, p, cin, cout, N, H, W, res, act, parts = case
-    layers = [conv(cin, cin, 1, p=0, input_from=-1), conv(cin, cout, k, s=s, p=p, act=act, input_from=0), conv(cout, cout, 3, act=act, input_from=1)]
+    layers = [conv(cin, cin, 1, p=0, input_from=-1)] + [pool(cin, 2, 1, 0, input_from=i) for i in range(pools)]
+    layers += [conv(cin, cout, k, s=s, p=p, act=act, input_from=pools), conv(cout, cout, 3, act=act, input_from=pools + 1)]
     wl = Workload("withheld", "bf16", N, H, W, cin, [Segment(layers, 3)], seed=32)
     li.fill_parameters(wl)
     li.make_input(wl)
     dc = DeviceChain(wl, flags=lop.LOP_FLAG_REUSE_HALO | lop.LOP_FLAG_COPY_ENGINE)
-    plan, ws, out, x = dc.plans[0], dc.ws[0], dc.outs[0], dc.pinned_input()
-    good = dc.run_pipelined(x).clone()
+    assert parts_of(dc)[0][-1] > 1
+    plan, ws, x = dc.plans[0], dc.ws[0], dc.pinned_input()
+    out = torch.empty_like(dc.outs[0], device="cpu").pin_memory() if pools else dc.outs[0]
+    dc.run_pipelined(x, out_pinned=out if pools else None)
     torch.cuda.synchronize()
+    good = out.clone()
     dc.check_device()
     for _ in range(2):
         plan.set_wait_limit(4000)
@@ -436,7 +442,7 @@ def test_a_band_that_never_arrives_ends_a_launch_with_split_tiles(case):
         assert e.value.status == -7
         plan.set_wait_limit(0)
         out.zero_()
-        dc.run_pipelined(x)
+        dc.run_pipelined(x, out_pinned=out if pools else None)
         torch.cuda.synchronize()
         dc.check_device()
         assert torch.equal(out, good)
