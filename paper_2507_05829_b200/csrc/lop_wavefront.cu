@@ -103,7 +103,8 @@ __device__ __forceinline__ int rec_dep0(const int4 &r) { return r.w; }
 // Bounded wait of a whole warp for an item's dependencies: lane j polls entry j of the list (its first
 // 32 entries were prefetched into `mine`).  Counters only grow (compare modulo 2^32).  The result is
 // uniform across the warp.  idle() runs once if the first look finds a producer unfinished: there is time then.  (No
-// sleep between two looks: a ResNet-50 of batch 8 442 us with 32 ns, 439 without.)
+// sleep between two looks: a ResNet-50 of batch 8 442 us with 32 ns, 439 without.  A long wait sleeps 2 us every 64 looks, which
+// keeps a look at 256 ns on average, as 32 ns after each do -- 210 without any: the limit is a number of looks and stands for a time.)
 template <typename Idle>
 __device__ __forceinline__ bool wait_deps_warp(const WfParams &P, int first, int count, int2 mine, unsigned run, int lane, Idle idle)
 {
@@ -121,7 +122,10 @@ __device__ __forceinline__ bool wait_deps_warp(const WfParams &P, int first, int
             if (__all_sync(0xffffffffu, done)) break;
             if (!idled) { idled = true; idle(); }
             if (i >= P.spin_limit) return false;
-            if ((i & 63u) == 63u && __any_sync(0xffffffffu, ld_relaxed(P.counters + 2) != 0u)) return false;
+            if ((i & 63u) == 63u) {
+                if (__any_sync(0xffffffffu, ld_relaxed(P.counters + 2) != 0u)) return false;
+                __nanosleep(2048);
+            }
         }
     }
     __syncwarp();            // every lane's acquire now orders the whole warp's later reads

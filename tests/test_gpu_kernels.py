@@ -446,3 +446,22 @@ def test_a_band_that_never_arrives_ends_a_launch_with_split_tiles(case, pools):
         torch.cuda.synchronize()
         dc.check_device()
         assert torch.equal(out, good)
+
+
+def test_a_wait_limit_covers_as_much_time_as_it_says():
+    """A band that never arrives with the largest limit that this call takes, 65536 looks of a quarter of a microsecond: 16.4 ms
+    (a look takes a little longer than 256 ns where the clocks are lower, so there is no sharp bound from above)."""
+    wl = li.build("vgg_block", H=44, W=36)
+    dc = DeviceChain(wl, flags=lop.LOP_FLAG_REUSE_HALO | lop.LOP_FLAG_COPY_ENGINE)
+    plan, ws, x = dc.plans[0], dc.ws[0], dc.pinned_input()
+    dc.run_pipelined(x)
+    torch.cuda.synchronize()
+    plan.set_wait_limit(65536)
+    t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    t0.record()
+    plan.run_pipelined_withheld(1, x.data_ptr(), dc.staging.data_ptr(), dc.outs[0].data_ptr(), ws.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    t1.record()
+    torch.cuda.synchronize()
+    assert 15.5 < t0.elapsed_time(t1) < 100.0
+    with pytest.raises(lop.LopError):
+        plan.check_device(ws.data_ptr())
