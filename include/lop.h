@@ -292,8 +292,9 @@ int lop_plan_check_device(lop_plan_t *plan, void *workspace);
  * invalid and lop_plan_check_device() reports LOP_EDEVICE and readies the plan for the next call.  The paper names the
  * failure of one unit as a risk of fine-grained partitioning (Sec. I) and answers it by tracking dependencies; this is
  * what happens here when a dependency is never satisfied.
- * lop_plan_set_wait_limit: polls (of about a quarter of a microsecond each) a wait for rows or for an arrival may
- * take; 0 restores the default (2^22, about a second).  Applies to the plan's later launches (for a chain: the first plan's). */
+ * lop_plan_set_wait_limit: polls (of a quarter to a third of a microsecond each) a wait for rows or for an arrival may
+ * take; 0 restores the default (2^22, more than a second).  Other waits of the kernel follow from it and end after some
+ * five seconds, so a larger limit than about 2^24 has no effect.  Applies to the plan's later launches (for a chain: the first plan's). */
 int lop_plan_set_wait_limit(lop_plan_t *plan, unsigned polls);
 /* lop_run_pipelined with the copy-engine transport, except that band `band` never arrives: neither its copy nor its
  * arrival write is enqueued.  Exists to exercise the failure path above without faulting anything: the kernel's wait

@@ -132,10 +132,14 @@ __device__ __forceinline__ bool wait_deps_warp(const WfParams &P, int first, int
     return true;
 }
 
+// What waits at a barrier may wait for the loader, which waits for rows: the limits below, five to eight seconds, are above
+// that wait's default of 1.5, and a role that gives up ends the others' waits by the abort flag.
+constexpr uint32_t BARRIER_TRIES = 8u * WAIT_LIMIT, BARRIER_TESTS = 64u * WAIT_LIMIT;
+
 // Bounded mbarrier wait that also gives up when the CTA's abort flag is raised.
 __device__ __forceinline__ bool mbar_wait_abortable(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag)
 {
-    for (uint32_t i = 0; i < WAIT_LIMIT; ++i) {
+    for (uint32_t i = 0; i < BARRIER_TRIES; ++i) {
         uint32_t done;
         asm volatile(
             "{\n"
@@ -156,7 +160,7 @@ __device__ __forceinline__ bool mbar_wait_abortable(uint32_t bar, uint32_t parit
 // wake up (a ResNet-50 of batch 32 795 us suspended, 790 so).
 __device__ __forceinline__ bool mbar_spin_abortable(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag)
 {
-    for (uint32_t i = 0; i < 8u * WAIT_LIMIT; ++i) {
+    for (uint32_t i = 0; i < BARRIER_TESTS; ++i) {
         uint32_t done;
         asm volatile(
             "{\n"
@@ -615,7 +619,7 @@ __device__ __forceinline__ uint32_t ld_shared(uint32_t addr)
 // CTA of the cluster that gives up does on its way out: what it was to send will not come).
 __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, uint32_t abort_at)
 {
-    for (uint32_t i = 0; i < WAIT_LIMIT; ++i) {
+    for (uint32_t i = 0; i < BARRIER_TRIES; ++i) {
         uint32_t done;
         asm volatile(
             "{\n"

@@ -465,3 +465,33 @@ def test_a_wait_limit_covers_as_much_time_as_it_says():
     assert 15.5 < t0.elapsed_time(t1) < 100.0
     with pytest.raises(lop.LopError):
         plan.check_device(ws.data_ptr())
+
+
+def test_a_late_band_is_waited_for_as_long_as_the_limit_says():
+    """The bands' copies queue behind others that keep the link busy for 1.2 s, more than the roles behind the one that waits for
+    rows used to wait (0.7 to 0.9 s); the limit is ten seconds."""
+    wl = li.build("vgg_block", H=44, W=36)
+    dc = DeviceChain(wl, flags=lop.LOP_FLAG_REUSE_HALO | lop.LOP_FLAG_COPY_ENGINE)
+    x = dc.pinned_input()
+    good = dc.run_pipelined(x).clone()
+    big = torch.empty(128 << 20, dtype=torch.uint8).pin_memory()
+    there, side = torch.empty_like(big, device="cuda"), torch.cuda.Stream()
+    t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+
+    def copies(n):
+        for _ in range(n):
+            there.copy_(big, non_blocking=True)
+    with torch.cuda.stream(side):
+        copies(2)
+        t0.record()
+        copies(8)
+        t1.record()
+    torch.cuda.synchronize()
+    dc.outs[-1].zero_()
+    dc.plans[0].set_wait_limit(1 << 25)
+    with torch.cuda.stream(side):
+        copies(int(1200.0 * 8 / t0.elapsed_time(t1)))
+    dc.run_pipelined(x)
+    torch.cuda.synchronize()
+    dc.check_device()
+    assert torch.equal(dc.outs[-1], good)
