@@ -1609,6 +1609,7 @@ __global__ void __launch_bounds__(FETCH ? WF_THREADS + 32 : WF_THREADS, 1) wavef
         // (the cluster's other CTAs hear of it first: a role of theirs may wait for this CTA's part of a tile, and for nothing
         // else that would tell it.  Looks at the device-wide flag in those waits cost a ResNet-18 streamed one image 1.5 us.)
         if (SPLIT && threadIdx.x < (unsigned)P.cluster) st_cluster(map_to_cta(bars + BAR_MISC + 4u, threadIdx.x), 1u);
+#pragma unroll 1
         for (int i = 0; i < 100; ++i) __nanosleep(1000);
     }
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
