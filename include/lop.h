@@ -262,7 +262,11 @@ int lop_plan_layer_time(lop_plan_t *plan, int band, int layer, float *ms);
  * 2 = tcgen05 tensor-core convolution.  <0 on error. */
 int lop_plan_layer_kernel(const lop_plan_t *plan, int layer);
 /* HOST ONLY.  In how many parts (1, 2 or 4) a tensor-core convolution sums its channels: every part in float32 from zero, then
- * the parts in order.  1 for all other layers.  <0 on error. */
+ * the parts in order.  1 for all other layers.  <0 on error.
+ * All functions that execute a plan, whole or in bands, by one launch or by many, sum in the plan's parts: their outputs are the
+ * same bits.  The parts are chosen at planning time from N, the layers' extents and channels and the plan's other layers, so a
+ * layer planned for another batch, or with other layers around it, may give other bits for the same values (float32 roundings
+ * of the sum, then the bf16 rounding of the output). */
 int lop_plan_layer_parts(const lop_plan_t *plan, int layer);
 /* Where the full-size output tensor of an intermediate layer (0 <= layer < n_layers - 1) lives: byte offset into the
  * workspace given to the lop_run_* calls; its shape is lop_plan_out_shape(layer), NHWC in the storage dtype.  The rows a

@@ -17,7 +17,8 @@
 // one tensor map per (row parity, column parity) whose base is offset by the parity and whose
 // strides are doubled, so each tap is again a dense box.  K is always walked in the order
 // (channel slab, kh, kw), whatever the tile position, and a plan that sums K in parts has one
-// accumulator per part, so a pixel's value does not depend on the band that computes it.  Every wait is bounded; a wait that runs out sets the status word.
+// accumulator per part, so a pixel's value does not depend on the band that computes it.  Every wait is bounded; a wait that
+// runs out sets the status word.
 #include <cuda.h>
 #include <atomic>
 

@@ -236,15 +236,14 @@ cudaError_t launch_maxpool(const PoolArgs &a, int dtype, cudaStream_t s)
         const long long vecs = pix * (a.C / 8);
         const bool aligned = (reinterpret_cast<uintptr_t>(a.x) & 15) == 0 && (reinterpret_cast<uintptr_t>(a.y) & 15) == 0;
         const unsigned blocks = (unsigned)((vecs + 255) / 256);
-        if (a.C % 8 == 0 && aligned && vecs < (1LL << 38) && a.kh == 2 && a.kw == 2) return launch_after(maxpool_bf16x8_kernel<2, 2>, dim3(blocks), 256, 0, s, a);
-        else if (a.C % 8 == 0 && aligned && vecs < (1LL << 38) && a.kh == 3 && a.kw == 3) return launch_after(maxpool_bf16x8_kernel<3, 3>, dim3(blocks), 256, 0, s, a);
-        else if (a.C % 8 == 0) return launch_after(maxpool_kernel<__nv_bfloat16, 8>, dim3(grid_for(pix * (a.C / 8), 256)), 256, 0, s, a);
-        else return launch_after(maxpool_kernel<__nv_bfloat16, 1>, dim3(grid_for(pix * a.C, 256)), 256, 0, s, a);
-    } else {
-        if (a.C % 4 == 0) return launch_after(maxpool_kernel<float, 4>, dim3(grid_for(pix * (a.C / 4), 256)), 256, 0, s, a);
-        return launch_after(maxpool_kernel<float, 1>, dim3(grid_for(pix * a.C, 256)), 256, 0, s, a);
+        const bool wide = a.C % 8 == 0 && aligned && vecs < (1LL << 38);
+        if (wide && a.kh == 2 && a.kw == 2) return launch_after(maxpool_bf16x8_kernel<2, 2>, dim3(blocks), 256, 0, s, a);
+        if (wide && a.kh == 3 && a.kw == 3) return launch_after(maxpool_bf16x8_kernel<3, 3>, dim3(blocks), 256, 0, s, a);
+        if (a.C % 8 == 0) return launch_after(maxpool_kernel<__nv_bfloat16, 8>, dim3(grid_for(pix * (a.C / 8), 256)), 256, 0, s, a);
+        return launch_after(maxpool_kernel<__nv_bfloat16, 1>, dim3(grid_for(pix * a.C, 256)), 256, 0, s, a);
     }
-    return cudaGetLastError();
+    if (a.C % 4 == 0) return launch_after(maxpool_kernel<float, 4>, dim3(grid_for(pix * (a.C / 4), 256)), 256, 0, s, a);
+    return launch_after(maxpool_kernel<float, 1>, dim3(grid_for(pix * a.C, 256)), 256, 0, s, a);
 }
 
 cudaError_t launch_stem_gather(const void *x, void *y, const GatherGeom &g, int lo, int hi, cudaStream_t s, unsigned *dbg, const StemWeights &wt)
@@ -257,8 +256,7 @@ cudaError_t launch_stem_gather(const void *x, void *y, const GatherGeom &g, int 
     uint16_t *yi = static_cast<uint16_t *>(y);
     // (a 64-bit division is a routine of several dozen instructions, and a thread has four of them)
     if (work < (1LL << 30)) return launch_after(stem_gather_kernel<int>, dim3(blocks), 256, 0, s, xi, yi, g, lo, hi, wt, dbg);
-    else return launch_after(stem_gather_kernel<long long>, dim3(blocks), 256, 0, s, xi, yi, g, lo, hi, wt, dbg);
-    return cudaGetLastError();
+    return launch_after(stem_gather_kernel<long long>, dim3(blocks), 256, 0, s, xi, yi, g, lo, hi, wt, dbg);
 }
 
 cudaError_t launch_fetch_rows(const void *src, void *dst, int N, int rows, long long row_bytes, int lo, int hi, cudaStream_t s)

@@ -208,7 +208,8 @@ static void plan_bands(lop_plan_t &pl)
 // In how many parts a tensor-core convolution sums its K.  Layers with few output tiles and a long K (the 7x7 maps of a
 // single image: eight tiles of 9 us each) leave the chip idle, so the persistent kernel gives the parts of a tile to the CTAs
 // of a cluster, which exchange their partial sums.  The choice is part of the plan, not of the launch: every executor sums in
-// the same parts, and a tensor's bits do not depend on which of them computed it, nor on the band.
+// the same parts, and a tensor's bits do not depend on which of them computed it, nor on the band.  They do depend on the plan's
+// shape and on its other layers, within the roundings of fp32 sums: the same image alone and in a batch may differ.
 // The estimate, in microseconds: a (64-channel chunk, filter tap) step takes 0.125 where one box serves all taps, 0.28 with a
 // box per tap, 0.19 for pointwise layers (what arrives per step at the 80-100 GB/s of an SM's operand loads); 2.2 go to the
 // first operands' latency and the epilogue, 1.7 to the exchange; 148 CTAs, of which clusters of four can use 132.

@@ -26,7 +26,8 @@
 //
 // Deadlock freedom: items are numbered in a topological order, every CTA is resident and takes its
 // items in increasing order, so the lowest unfinished item never waits on an unstarted one (the parts of a split tile
-// wait for one another, and for nothing that has a higher number than the first of them).  All waits are bounded all the same; one that runs out raises the status word and the abort flag.
+// wait for one another, and for nothing that has a higher number than the first of them).  All waits are bounded all the
+// same; one that runs out raises the status word and the abort flag.
 #include <atomic>
 
 #include <cuda_bf16.h>
@@ -669,7 +670,8 @@ __device__ __noinline__ bool take_partial_sums(uint32_t bars, uint32_t cout, uin
 // An epilogue of its own, out of line: with the exchange in front of the other tiles' epilogue, those took 0.2 us longer each
 // (a ResNet-50 of batch 32, which has no split tile, 830 -> 873 us).
 template <bool SMOOTH>
-__device__ __noinline__ uint32_t split_item(const WfStage *sp, int4 rec, uint8_t *smem_bars, uint32_t unit0, uint32_t unit_bytes, uint32_t acc, uint32_t uc, uint32_t cnt)
+__device__ __noinline__ uint32_t split_item(const WfStage *sp, int4 rec, uint8_t *smem_bars, uint32_t unit0, uint32_t unit_bytes, uint32_t acc,
+                                            uint32_t uc, uint32_t cnt)
 {
     const uint32_t bars = smem_u32(smem_bars), s_log = (uint32_t)__ldg(&sp->s_log), parts = 1u << s_log, part = (uint32_t)rec_cout(rec) & (parts - 1u);
     const uint32_t turn = ld_shared(bars + BAR_MISC + 16u) >> (s_log - 1u) & 1u;   // parity of the tiles of as many parts before this one
@@ -677,7 +679,9 @@ __device__ __noinline__ uint32_t split_item(const WfStage *sp, int4 rec, uint8_t
     const uint32_t slice = WF_SPLIT_BN >> s_log, base_rank = cta_rank() & ~(parts - 1u), abort_at = bars + BAR_MISC + 4u, rx = uc + 1u;
     const uint32_t per_unit = parts >> 1, from_bytes = 512u * slice;           // senders per unit (two parts: one, four: two)
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u, row = (warp & 3u) * 32u + lane, cgrp = (warp - WF_FIRST_WORKER) >> 2, buf = cnt & 1u;
-    auto sums_at = [&](uint32_t first_unit, uint32_t from) { return unit0 + ((first_unit + from / per_unit) & (WF_UNITS - 1)) * unit_bytes + (from & (per_unit - 1u)) * from_bytes + 16u * row; };
+    auto sums_at = [&](uint32_t first_unit, uint32_t from) {
+        return unit0 + ((first_unit + from / per_unit) & (WF_UNITS - 1)) * unit_bytes + (from & (per_unit - 1u)) * from_bytes + 16u * row;
+    };
     const int p_log = __ldg(&sp->p_log), tr_log = __ldg(&sp->tr_log), tw_valid = __ldg(&sp->tw_valid), sub_log = __ldg(&sp->sub_log);
     const int act = __ldg(&sp->act), res_pos = ldg_ptr<const void *>(&sp->res) ? __ldg(&sp->res_pos) : LOP_RES_NONE;
     const bool bulk_out = __ldg(&sp->out_map) >= 0;
@@ -686,7 +690,7 @@ __device__ __noinline__ uint32_t split_item(const WfStage *sp, int4 rec, uint8_t
     ok = ok && mbar_wait_cluster(xok, turn, abort_at);
     ok = __all_sync(0xffffffffu, ok);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    uint32_t r[8];                                                             // (eight columns at a time: what this needs, the kernel around the call has not)
+    uint32_t r[8];                                     // (eight columns at a time: what this needs, the kernel around the call has not)
 #pragma unroll 1
     for (uint32_t c = 0, k = 0; ok && c < WF_SPLIT_BN; c += 8) {
         const uint32_t q = c / slice;

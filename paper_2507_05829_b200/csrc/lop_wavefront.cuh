@@ -19,7 +19,8 @@ namespace lop {
 // item is 1 << tr_log output rows of one image, tw_valid columns wide and BN channels deep (its receptive window is staged
 // in shared memory); a normalisation or concatenation item is one whole output row of one image; a gather or 3x3 pooling
 // item is 1 << tr_log of them.
-// WF_SPLIT is what the worker warps call a split tile of a WF_CONV stage.  WF_NONE: an item without work, in front of a split tile whose items have to start at a cluster's first CTA.
+// WF_SPLIT is what the worker warps call a split tile of a WF_CONV stage.  WF_NONE: an item without work, in front of a split
+// tile whose items have to start at a cluster's first CTA.
 enum WfKind { WF_GATHER = 0, WF_CONV = 1, WF_POOL = 2, WF_FETCH = 3, WF_DWCONV = 4, WF_LAYERNORM = 5, WF_CONCAT = 6, WF_NONE = 7, WF_SPLIT = 8 };
 // How a convolution stage feeds the tensor cores.
 //   WF_SLAB  one activation box per channel chunk: the output tile's receptive window (tile plus halo),
