@@ -286,6 +286,29 @@ def test_gelu_over_its_whole_range(flags):
     assert np.isposinf(got[np.isposinf(x)]).all()
 
 
+@pytest.mark.parametrize("flags", [0, lop.LOP_FLAG_PER_LAYER])
+def test_gelu_rounds_as_the_exact_function(flags):
+    """Four million values of t in (-1, 0), where the result is small and its error shows: an fp32 value that is off by e is
+    rounded to another bf16 than the exact one for a share of e over the spacing, which is 2^-8 to 2^-7 of the value, 0.0056 on
+    the mean.  The bound is that of a mean error of one unit in fp32's last place, 6e-8 (measured: 7.9e-6; with a polynomial whose
+    error was half as large again 1.4e-5)."""
+    C, n = 64, 256
+    rng = np.random.default_rng(11)
+    x = li.round_to_bf16(rng.uniform(-0.9, -0.05, (1, n, n, C)).astype(np.float32))
+    l = conv(C, C, 1, p=0, act=li.ACT_GELU)
+    wl = one_layer(l, 1, n, n, dtype="bf16")
+    w = np.eye(C) + 2.0 ** -9 * np.roll(np.eye(C), 1, axis=0)                  # two terms that the sum holds exactly: many values of t
+    l.weight = w.astype(np.float32).reshape(l.weight.shape)
+    l.scale, l.shift = rng.uniform(0.95, 1.05, C).astype(np.float32), rng.uniform(-0.04, 0.04, C).astype(np.float32)
+    got = to_host_f32((lambda dc: dc.run_whole(dc.input_tensor(x)))(DeviceChain(wl, flags=flags)))
+    t = torch.from_numpy(((x.astype(np.float64) @ w.T) * l.scale + l.shift).astype(np.float32)).double()    # (one rounding, as fmaf)
+    want, e = np.frexp((0.5 * t * torch.erfc(-t / 2.0 ** 0.5)).numpy())
+    want = np.ldexp(np.rint(want * 256.0) / 256.0, e)
+    wrong = float((got != want).mean())
+    assert (np.abs(got - want) <= 2.0 ** -7 * np.abs(want)).all()
+    assert wrong < 6e-8 / 0.0056, wrong
+
+
 # ------------------------------------------------------------------------------------ launches that begin before the previous one ended
 @pytest.mark.parametrize("dtype,C,H,W,flags", [("bf16", 64, 40, 36, 0), ("bf16", 64, 40, 36, lop.LOP_FLAG_PER_LAYER), ("f32", 16, 32, 32, 0),
                                                ("f32", 64, 70, 61, 0), ("bf16", 5, 19, 23, lop.LOP_FLAG_FORCE_SIMT)])
