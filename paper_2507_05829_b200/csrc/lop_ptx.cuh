@@ -214,7 +214,7 @@ __device__ __forceinline__ float exp2_approx(float x)
 // fitted for this purpose (least squares reweighted towards the largest relative error, which is 3e-8 up to u = 3 before
 // rounding, 1e-6 at 5, 1e-5 at 9).  In v, which is small where u is, and not in 1 - v, whose rounding would weigh twice its
 // size in Q(0).  Norm of the error over the result's against 64 bits, for normal t of deviation 1, 2, 3: 3.5, 3.1, 2.6e-8;
-// 0.5 t (1 + erf(t / sqrt 2)) in fp32 has 3.8, 3.7, 3.1e-8; relative to a single value of |t| < 1 at most 3.3e-7 and 2.2e-7.
+// 0.5 t (1 + erf(t / sqrt 2)) in fp32 has 3.8, 3.7, 3.1e-8; relative to a single value of |t| < 1 at most 3.1e-7 and 2.2e-7.
 // It keeps its relative accuracy in the lower tail, where that form cancels.  It has neither branches nor the library
 // erf's two polynomials, which took 5.5 us of a 128x128 tile's epilogue (a ConvNeXt block 45.0 -> 41.0 us).
 // u is clamped at 16, where Q is 0 in fp32, so that an infinite t has no 0 * infinity on the way.
@@ -229,7 +229,8 @@ __device__ __forceinline__ float2 gelu2(float t0, float t1)
     float d0, d1;
     rowop::unpack2(den, d0, d1);
     const f32x2 v = mul2(mul2(u, both(0.33f)), rowop::pack2(rcp_approx(d0), rcp_approx(d1)));
-    const float coeff[7] = {0.10439056158065796f, 0.030913464725017548f, -0.145896777510643f, -0.3189733922481537f, 1.086843490600586f, -1.2089178562164307f, 0.5f};
+    const float coeff[7] = {0.10439056158065796f, 0.030913464725017548f, -0.145896777510643f, -0.3189733922481537f,
+                            1.086843490600586f, -1.2089178562164307f, 0.5f};
     f32x2 r = both(-0.04851029813289642f);
 #pragma unroll
     for (int i = 0; i < 7; ++i) {
