@@ -302,8 +302,8 @@ int lop_plan_check_device(lop_plan_t *plan, void *workspace);
 int lop_plan_set_wait_limit(lop_plan_t *plan, unsigned polls);
 /* lop_run_pipelined with the copy-engine transport, except that band `band` never arrives: neither its copy nor its
  * arrival write is enqueued.  Exists to exercise the failure path above without faulting anything: the kernel's wait
- * for that band runs out after the plan's wait limit -- which must have been set, to at most 65536 polls, a few
- * milliseconds -- and the call's stream work ends normally with the status word raised (bit 0x10). */
+ * for that band runs out after the plan's wait limit -- which must have been set, to at most 65536 polls, some
+ * twenty milliseconds -- and the call's stream work ends normally with the status word raised (bit 0x10). */
 int lop_run_pipelined_withheld(lop_plan_t *plan, int band, const void *in_host_pinned, void *staging_dev, void *out_dev,
                                void *workspace, void *stream);
 

@@ -433,7 +433,7 @@ def test_tiles_of_two_parts_and_of_four_in_one_program(N, H, W, bands, segments,
 
 @pytest.mark.parametrize("case,pools", [(SPLIT_CASES[0], 0), (SPLIT_CASES[1], 0), (SPLIT_CASES[5], 0), (SPLIT_CASES[2], 3)])
 def test_a_band_that_never_arrives_ends_a_launch_with_split_tiles(case, pools):
-    """Band 1 is withheld (a dependency that the host never satisfies) with a limit of 4000 looks, about a millisecond: whoever
+    """Band 1 is withheld (a dependency that the host never satisfies) with a limit of 4000 looks, one to two milliseconds: whoever
     waits for a part of a tile that will not come gives up with the rest, long before a wait of its own would run out (seconds);
     the status is reported once and the plan works again.  With poolings between, whose single rows are many items that the
     workers publish themselves, and the result stored to host memory, as split tiles are then, too: the workers may find their
